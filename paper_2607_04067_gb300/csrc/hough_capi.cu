@@ -95,9 +95,8 @@ static int round16(int x) { return (x + 15) & ~15; }
 // Shared-memory layout for a shape; returns false if it does not fit.
 static bool layout(Plan& pl) {
   const int wpad = pl.groups * 32;
-  const int cell = pl.acc32 ? 4 : 2;
   // mirror-pair: groups / 2 word groups of 32 lanes (the last may be part idle) x rows_phys
-  const int acc_bytes = pl.mp ? (pl.groups / 2) * 32 * pl.rows_phys * 4 : wpad * pl.nrho_pad * cell;
+  const int acc_bytes = pl.mp ? (pl.groups / 2) * 32 * pl.rows_phys * 4 : wpad * pl.nrho_pad * 2;
   const int sel_bytes = (2 * pl.n_theta + 64) * 4 + pl.n_theta * 16 + pl.n_theta * pl.nrb_g * 4;
   int o = 0;
   pl.off_acc = o;
@@ -191,8 +190,8 @@ static void mp_consts(Plan& pl, int n_rho) {
   pl.mp_lsq = (long long)std::floor(L * L);
 }
 
-// Launch shape for parameters p; acc32 < 0 lets the planner choose the cell width.
-int make_plan(const hough_params* p, Plan& pl, int acc32 = -1) {
+// Launch shape for parameters p.
+int make_plan(const hough_params* p, Plan& pl) {
   int rc = check_params(p);
   if (rc) return rc;
   std::memset(&pl, 0, sizeof(pl));
@@ -211,19 +210,16 @@ int make_plan(const hough_params* p, Plan& pl, int acc32 = -1) {
   pl.grab = p->events_per_cta > 0 ? p->events_per_cta : 1;
   {
     const double nr = p->n_rho, delta = nr * std::ldexp(1.0, -20);
-    pl.fpbin = 1;
     pl.fp_scale = (float)(nr / (2.0 * (double)kH));
     pl.fp_c0 = (float)(0.5 * nr);
     pl.fp_khi = (float)(nr - 0.5);
     pl.fp_dlo = (float)(delta - 0.5);
     pl.fp_dhi = (float)(-delta - 0.5);
   }
-  const int cell_choice = acc32 < 0 ? 0 : acc32;
   // Mirror pairs (columns j and N-1-j in one word) need an even N_theta and a table with
-  // c[N-1-j] = -c[j], s[N-1-j] = s[j] (true for round-half-away-from-zero), int16 cells and
-  // the float row estimate.
+  // c[N-1-j] = -c[j], s[N-1-j] = s[j] (true for round-half-away-from-zero).
   bool sym = false;
-  if (p->n_theta % 2 == 0 && !cell_choice && pl.fpbin) {
+  if (p->n_theta % 2 == 0) {
     TrigTable tt;
     host_trig(p->n_theta, &tt);
     sym = true;
@@ -246,8 +242,7 @@ int make_plan(const hough_params* p, Plan& pl, int acc32 = -1) {
     }
     pl.tiles = T;
     pl.tile_w = W;
-    pl.acc32 = cell_choice;
-    pl.nrho_pad = pl.acc32 ? p->n_rho : ((p->n_rho + 1) & ~1);
+    pl.nrho_pad = (p->n_rho + 1) & ~1;
     const int halo = T > 1 ? 32 : 0;
     if (p->block) {
       const int work = p->block - halo;
@@ -268,15 +263,14 @@ int make_plan(const hough_params* p, Plan& pl, int acc32 = -1) {
       if (p->theta_tiles) return HOUGH_EPARAM;
       continue;
     }
-    pl.mirror = sym ? 1 : 0;
-    pl.mp = pl.mirror;
+    pl.mp = sym ? 1 : 0;
     if (pl.mp) mp_consts(pl, p->n_rho);
     // row ranges of the peak scan: the power of two that minimises the slowest warp's row
     // steps, each unit (30 columns x one range) paying two extra rows to prime its window and
     // about 16 rows' worth of setup (measured at 256 x 256, 1024 threads: 4 ranges scan in
     // 9.4 k cycles an event, 8 in 9.5 k, 16 in 10.3 k, 32 in 12.6 k)
     {
-      const bool packed = !pl.mp && !pl.acc32 && (p->n_rho & 1) == 0;
+      const bool packed = !pl.mp && (p->n_rho & 1) == 0;
       const int cols = pl.mp ? pl.tile_w / 2 : pl.tile_w;
       const int nblk = (cols + 29) / 30, nwarps = pl.threads / 32;
       const int rows = packed ? p->n_rho / 2 : p->n_rho;

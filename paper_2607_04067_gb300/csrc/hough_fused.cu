@@ -6,9 +6,9 @@
 //     does not fit one CTA's shared memory;
 //   - every lane of a "worker" warp owns theta columns of the tile for the whole vote.
 //     Lane l's cells live in shared-memory bank l only: word ((g * rows + row) * 32 + l),
-//     rows = N_rho / 2 packed int16 pairs (or N_rho int32 cells), so the column-parallel
+//     rows = N_rho / 2 packed int16 pairs, so the column-parallel
 //     vote is free of bank conflicts whatever rho bins the hits hit; warps sharing
-//     columns split the hits and add with red.shared. In mirror mode a lane owns
+//     columns split the hits and add with red.shared. With an even N_theta a lane owns
 //     column j and its mirror N_theta-1-j (th -> pi - th: c -> -c, s -> s), so one pair
 //     of products gives both rho values;
 //   - for tiled events one extra warp votes the two neighbour columns of the tile
@@ -41,30 +41,21 @@ __device__ __forceinline__ uint32_t vmax2(uint32_t a, uint32_t b) {
 
 __device__ __forceinline__ uint32_t swap16(uint32_t x) { return __funnelshift_l(x, x, 16); }
 
-template <bool A32>
 __device__ __forceinline__ int acc_index(int c, int k, int nrp) {
-  return A32 ? ((((c >> 5) * nrp + k) << 5) + (c & 31)) : ((((c >> 5) * (nrp >> 1) + (k >> 1)) << 5) + (c & 31));
+  return (((c >> 5) * (nrp >> 1) + (k >> 1)) << 5) + (c & 31);
 }
 
-template <bool A32>
 __device__ __forceinline__ int acc_get(const uint32_t* acc, int c, int k, int nrp) {
-  const uint32_t w = acc[acc_index<A32>(c, k, nrp)];
-  return A32 ? (int)w : (int)((w >> ((k & 1) << 4)) & 0xffffu);
+  const uint32_t w = acc[acc_index(c, k, nrp)];
+  return (int)((w >> ((k & 1) << 4)) & 0xffffu);
 }
 
 // One vote for row k of the column whose row-0 word is at shared address `colbase`.
 // No memory clobber: the accumulator is only read after a barrier, and leaving the hit
 // loads free to move above the atomics lets consecutive hits overlap.
-template <bool A32>
 __device__ __forceinline__ void vote_cell(uint32_t colbase, int k) {
-  uint32_t addr, inc;
-  if (A32) {
-    addr = colbase + ((uint32_t)k << 7);
-    inc = 1u;
-  } else {
-    addr = colbase + (((uint32_t)k >> 1) << 7);
-    inc = 1u << (((uint32_t)k & 1u) << 4);
-  }
+  const uint32_t addr = colbase + (((uint32_t)k >> 1) << 7);
+  const uint32_t inc = 1u << (((uint32_t)k & 1u) << 4);
   asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(inc));
 }
 
@@ -130,7 +121,7 @@ __device__ unsigned long long block_sum_u64(unsigned long long v, unsigned long 
 // (compacted, order not kept). Valid hits beyond int32 set bit 0 of *s_flags, bad
 // hits bit 1.
 __device__ void stage_vote32(const int2* __restrict__ xy, long long base, int cn, int2* hb, int* s_nv, int* s_flags,
-                             bool as_float, long long lsq, uint16_t* idx) {
+                             long long lsq, uint16_t* idx) {
   const int lane = threadIdx.x & 31;
   // each thread's next hit is loaded one pass ahead, so the loads overlap the mapping
   int2 hn = threadIdx.x < cn ? xy[base + threadIdx.x] : make_int2(0, 0);
@@ -162,7 +153,7 @@ __device__ void stage_vote32(const int2* __restrict__ xy, long long base, int cn
           fp[2] = (float)v;
           idx[at] = (uint16_t)i;
         } else {
-          hb[at] = as_float ? make_int2(__float_as_int((float)u), __float_as_int((float)v)) : make_int2((int)u, (int)v);
+          hb[at] = make_int2(__float_as_int((float)u), __float_as_int((float)v));
         }
       }
     }
@@ -225,11 +216,10 @@ __device__ void stage_sel64(const int2* __restrict__ xy, long long base, int cn,
 struct VoteLane {
   bool on;          // lane votes
   bool halo;        // lane of the halo warp (tiles > 1)
-  bool mirror;      // lane also votes the mirror column
   int p, P;         // hit partition of this warp, partitions per column set
   int cj, sj;       // trig of the (first) column
   uint32_t col1;    // shared address of column 1, row 0
-  uint32_t col2;    // mirror column (mirror mode) or halo column
+  uint32_t col2;    // halo column
 };
 
 // Bin of the float estimate kf = u A + v B + N_rho/2 of k* = (u c + v s + H) N_rho / 2H, where
@@ -256,7 +246,6 @@ __device__ __forceinline__ int bin_fp(float kf, const FpBin& K, float uf, float 
   return r;
 }
 
-template <bool A32>
 __device__ __forceinline__ void vote32_fp(const Plan& pl, const VoteLane& L, const int2* hb, int nv) {
   if (!L.on) return;
   const BinMagic m = pl.magic;
@@ -274,84 +263,18 @@ __device__ __forceinline__ void vote32_fp(const Plan& pl, const VoteLane& L, con
   }
   const float4* hb4 = reinterpret_cast<const float4*>(hb);
   const int np = nv >> 1, P = L.P;
-  if (L.mirror) {
-#pragma unroll 2
-    for (int q = L.p; q < np; q += P) {
-      const float4 h = hb4[q];
-      const float v0 = __fmaf_rn(h.y, B, c0), v1 = __fmaf_rn(h.w, B, c0);
-      vote_cell<A32>(L.col1, bin_fp(__fmaf_rn(h.x, A, v0), K, h.x, h.y, cj, sj, m));
-      vote_cell<A32>(L.col2, bin_fp(__fmaf_rn(-h.x, A, v0), K, h.x, h.y, -cj, sj, m));
-      vote_cell<A32>(L.col1, bin_fp(__fmaf_rn(h.z, A, v1), K, h.z, h.w, cj, sj, m));
-      vote_cell<A32>(L.col2, bin_fp(__fmaf_rn(-h.z, A, v1), K, h.z, h.w, -cj, sj, m));
-    }
-    if ((nv & 1) && L.p == np % P) {
-      const float2 h = reinterpret_cast<const float2*>(hb)[nv - 1];
-      const float v0 = __fmaf_rn(h.y, B, c0);
-      vote_cell<A32>(L.col1, bin_fp(__fmaf_rn(h.x, A, v0), K, h.x, h.y, cj, sj, m));
-      vote_cell<A32>(L.col2, bin_fp(__fmaf_rn(-h.x, A, v0), K, h.x, h.y, -cj, sj, m));
-    }
-  } else {
 #pragma unroll 4
-    for (int q = L.p; q < np; q += P) {
-      const float4 h = hb4[q];
-      vote_cell<A32>(L.col1, bin_fp(__fmaf_rn(h.x, A, __fmaf_rn(h.y, B, c0)), K, h.x, h.y, cj, sj, m));
-      vote_cell<A32>(L.col1, bin_fp(__fmaf_rn(h.z, A, __fmaf_rn(h.w, B, c0)), K, h.z, h.w, cj, sj, m));
-    }
-    if ((nv & 1) && L.p == np % P) {
-      const float2 h = reinterpret_cast<const float2*>(hb)[nv - 1];
-      vote_cell<A32>(L.col1, bin_fp(__fmaf_rn(h.x, A, __fmaf_rn(h.y, B, c0)), K, h.x, h.y, cj, sj, m));
-    }
+  for (int q = L.p; q < np; q += P) {
+    const float4 h = hb4[q];
+    vote_cell(L.col1, bin_fp(__fmaf_rn(h.x, A, __fmaf_rn(h.y, B, c0)), K, h.x, h.y, cj, sj, m));
+    vote_cell(L.col1, bin_fp(__fmaf_rn(h.z, A, __fmaf_rn(h.w, B, c0)), K, h.z, h.w, cj, sj, m));
+  }
+  if ((nv & 1) && L.p == np % P) {
+    const float2 h = reinterpret_cast<const float2*>(hb)[nv - 1];
+    vote_cell(L.col1, bin_fp(__fmaf_rn(h.x, A, __fmaf_rn(h.y, B, c0)), K, h.x, h.y, cj, sj, m));
   }
 }
 
-template <bool A32>
-__device__ __forceinline__ void vote32(const Plan& pl, const VoteLane& L, const int2* hb, int nv) {
-  if (!L.on) return;
-  const int Hh = (int)kH;
-  const BinMagic m = pl.magic;
-  const int cj = L.cj, sj = L.sj;
-  if (L.halo) {
-    const int lane = threadIdx.x & 31;
-    for (int i = lane & 15; i < nv; i += 16) {
-      const int2 h = hb[i];
-      vote_halo(L.col2, rho_bin32(h.x * cj + (h.y * sj + Hh), m));
-    }
-    return;
-  }
-  const int4* hb4 = reinterpret_cast<const int4*>(hb);
-  const int np = nv >> 1, P = L.P;
-  if (L.mirror) {
-#pragma unroll 2
-    for (int q = L.p; q < np; q += P) {
-      const int4 h = hb4[q];
-      const int v0 = h.y * sj + Hh, u0 = h.x * cj;
-      const int v1 = h.w * sj + Hh, u1 = h.z * cj;
-      vote_cell<A32>(L.col1, rho_bin32(v0 + u0, m));
-      vote_cell<A32>(L.col2, rho_bin32(v0 - u0, m));
-      vote_cell<A32>(L.col1, rho_bin32(v1 + u1, m));
-      vote_cell<A32>(L.col2, rho_bin32(v1 - u1, m));
-    }
-    if ((nv & 1) && L.p == np % P) {
-      const int2 h = hb[nv - 1];
-      const int v0 = h.y * sj + Hh, u0 = h.x * cj;
-      vote_cell<A32>(L.col1, rho_bin32(v0 + u0, m));
-      vote_cell<A32>(L.col2, rho_bin32(v0 - u0, m));
-    }
-  } else {
-#pragma unroll 4
-    for (int q = L.p; q < np; q += P) {
-      const int4 h = hb4[q];
-      vote_cell<A32>(L.col1, rho_bin32(h.x * cj + (h.y * sj + Hh), m));
-      vote_cell<A32>(L.col1, rho_bin32(h.z * cj + (h.w * sj + Hh), m));
-    }
-    if ((nv & 1) && L.p == np % P) {
-      const int2 h = hb[nv - 1];
-      vote_cell<A32>(L.col1, rho_bin32(h.x * cj + (h.y * sj + Hh), m));
-    }
-  }
-}
-
-template <bool A32>
 __device__ __forceinline__ void vote64(const Plan& pl, const VoteLane& L, const longlong2* hw, int nv) {
   if (!L.on) return;
   const BinMagic m = pl.magic;
@@ -367,8 +290,7 @@ __device__ __forceinline__ void vote64(const Plan& pl, const VoteLane& L, const 
   for (int q = L.p; q < nv; q += L.P) {
     const longlong2 h = hw[q];
     const long long vs = h.y * sj + kH, uc = h.x * cj;
-    vote_cell<A32>(L.col1, rho_bin64(vs + uc, m));
-    if (L.mirror) vote_cell<A32>(L.col2, rho_bin64(vs - uc, m));
+    vote_cell(L.col1, rho_bin64(vs + uc, m));
   }
 }
 
@@ -392,9 +314,8 @@ __device__ __forceinline__ int mp_get(const uint32_t* acc, int c, int k, int Wd,
 }
 
 // Cells of the CTA's accumulator for the iterative finder (one tile): read, and suppress by a
-// 16-bit store of zero into the cell's half of its word (a 32-bit store with int32 cells), which
-// leaves the other half of the word alone.
-template <bool A32, bool MP>
+// 16-bit store of zero into the cell's half of its word, which leaves the other half of the word alone.
+template <bool MP>
 struct FusedCells {
   static constexpr bool kPairs = MP;  // word w holds columns w and 2 Wd - 1 - w
   uint32_t* acc;
@@ -413,16 +334,14 @@ struct FusedCells {
       const uint32_t x = acc[mp_word(hi ? 2 * Wd - 1 - j : j, k + 1, rp)];
       return hi ? (int)(x >> 16) : (int)(x & 0xffffu);
     }
-    return acc_get<A32>(acc, j, k, nrp);
+    return acc_get(acc, j, k, nrp);
   }
   __device__ void clear(int j, int k) {
     if (MP) {
       const bool hi = j >= Wd;
       reinterpret_cast<uint16_t*>(acc)[2 * mp_word(hi ? 2 * Wd - 1 - j : j, k + 1, rp) + (hi ? 1 : 0)] = 0;
-    } else if (A32) {
-      acc[acc_index<true>(j, k, nrp)] = 0u;
     } else {
-      reinterpret_cast<uint16_t*>(acc)[2 * acc_index<false>(j, k, nrp) + (k & 1)] = 0;
+      reinterpret_cast<uint16_t*>(acc)[2 * acc_index(j, k, nrp) + (k & 1)] = 0;
     }
   }
 };
@@ -852,8 +771,7 @@ __device__ void scan_packed(const Plan& pl, const uint32_t* acc, const uint32_t*
   }
 }
 
-// Scalar scan for the int32-cell layout or an odd N_rho: one row per step.
-template <bool A32>
+// Scalar scan for an odd N_rho: one row per step.
 __device__ void scan_scalar(const Plan& pl, const uint32_t* acc, const uint32_t* halo, uint32_t* pbits,
                             int wt, int T, int j0, bool do_cs, unsigned long long& csum) {
   const int NT = pl.n_theta, NR = pl.n_rho, nrp = pl.nrho_pad, R = pl.scan_ranges;
@@ -868,7 +786,7 @@ __device__ void scan_scalar(const Plan& pl, const uint32_t* acc, const uint32_t*
     auto fetch = [&](int kk) -> int {
       const int rr = s.mir ? NR - 1 - kk : kk;
       if (s.kind == 3 || rr < 0 || rr >= NR) return -1;
-      if (s.kind == 0) return acc_get<A32>(acc, s.col, rr, nrp);
+      if (s.kind == 0) return acc_get(acc, s.col, rr, nrp);
       return (int)((halo[(s.kind - 1) * (nrp >> 1) + (rr >> 1)] >> ((rr & 1) << 4)) & 0xffffu);
     };
     const bool tested = lane >= 1 && lane <= 30 && c >= 0 && c < wt;
@@ -1210,7 +1128,6 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
 
 // Maximum (returned to every thread; *s_max must be 0 beforehand) and, with do_cs, this thread's
 // part of the accumulator checksum over the tile's own cells.
-template <bool A32>
 __device__ int tile_max_cs(const Plan& pl, const uint32_t* acc, int Wd, int aw, int wt, int j0, bool do_cs,
                            int* s_max, unsigned long long& cs) {
   const int NT = pl.n_theta, NR = pl.n_rho, lane = threadIdx.x & 31, warp = threadIdx.x >> 5,
@@ -1230,7 +1147,7 @@ __device__ int tile_max_cs(const Plan& pl, const uint32_t* acc, int Wd, int aw, 
   } else {
     for (int k = warp; k < NR; k += nwarps)
       for (int c = lane; c < wt; c += 32) {
-        const int v = acc_get<A32>(acc, c, k, pl.nrho_pad);
+        const int v = acc_get(acc, c, k, pl.nrho_pad);
         m = max(m, v);
         if (do_cs && v) cs += (unsigned long long)v * mix64((unsigned long long)(j0 + c) * NR + k + 1);
       }
@@ -1244,7 +1161,6 @@ __device__ int tile_max_cs(const Plan& pl, const uint32_t* acc, int Wd, int aw, 
 // Bit k of word (c, k >> 5) of pbits for every tile-local column c whose cell k holds >= tq votes
 // (tile-local columns as in the peak records: mirror-pair word w's low half is column w, its
 // high half column 2 Wd - 1 - w).
-template <bool A32>
 __device__ void tile_candidate_bits(const Plan& pl, const uint32_t* acc, uint32_t* pbits, int Wd, int wt, int tq) {
   const int NR = pl.n_rho, nrb = pl.nrb, lane = threadIdx.x & 31, warp = threadIdx.x >> 5,
             nwarps = blockDim.x >> 5;
@@ -1258,7 +1174,7 @@ __device__ void tile_candidate_bits(const Plan& pl, const uint32_t* acc, uint32_
   } else {
     for (int k = warp; k < NR; k += nwarps)
       for (int c = lane; c < wt; c += 32)
-        if (acc_get<A32>(acc, c, k, pl.nrho_pad) >= tq) atomicOr(&pbits[c * nrb + (k >> 5)], 1u << (k & 31));
+        if (acc_get(acc, c, k, pl.nrho_pad) >= tq) atomicOr(&pbits[c * nrb + (k >> 5)], 1u << (k & 31));
   }
 }
 
@@ -1557,7 +1473,6 @@ __device__ int merge_iterative(const Plan& pl, const FusedIO& io, unsigned char*
 
 // Steps 1-2 of a work item: clears the CTA's accumulator of theta tile t (with the halo columns,
 // the peak bitmap and the flags) and votes the event's hits [a, a + n) into it, chunk by chunk.
-template <bool A32>
 __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, long long a, int n,
                           int t) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
@@ -1572,14 +1487,13 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
   const int wt = min(pl.tile_w, NT - j0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
   const int wpad = pl.groups * 32;
-  const int rows_w = A32 ? nrp : (nrp >> 1);  // words per column
+  const int rows_w = nrp >> 1;  // words per column
   // mirror-pair tiles: words [aw, aw + Wd), i.e. columns [aw, aw + Wd) and their mirrors
   // (full tiles own tile_w / 2 words, the last one possibly fewer)
   const int Wd = pl.mp ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
 
   // lane roles of the vote
   VoteLane L;
-  L.mirror = pl.mirror != 0;
   L.halo = warp >= pl.groups * pl.split;
   L.on = false;
   L.cj = L.sj = 0;
@@ -1606,23 +1520,17 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     L.col2 = (uint32_t)__cvta_generic_to_shared(halo) + (uint32_t)((lane >> 4) * (nrp >> 1)) * 4u;
     L.p = 0;
     L.P = 1;
-  } else if (L.mirror) {
-    const int P2 = 2 * pl.split;
-    const int gpair = warp / P2, g2 = pl.groups - 1 - gpair;
+  } else if (pl.mp) {
+    const int P2 = 2 * pl.split, gpair = warp / P2;
     L.p = warp % P2;
     L.P = P2;
     const int c1 = gpair * 32 + lane;
-    L.on = !pl.mp || c1 < Wd;  // lanes past the tile's last word idle
+    L.on = c1 < Wd;  // lanes past the tile's last word idle
     if (L.on) {
-      L.cj = tc[(pl.mp ? aw : j0) + c1];
-      L.sj = ts[(pl.mp ? aw : j0) + c1];
+      L.cj = tc[aw + c1];
+      L.sj = ts[aw + c1];
     }
-    if (pl.mp) {
-      L.col1 = acc_s + (uint32_t)mp_word(c1, 0, pl.rows_phys) * 4u;
-    } else {
-      L.col1 = acc_s + (uint32_t)(((gpair * rows_w) << 5) + lane) * 4u;
-      L.col2 = acc_s + (uint32_t)(((g2 * rows_w) << 5) + (31 - lane)) * 4u;
-    }
+    L.col1 = acc_s + (uint32_t)mp_word(c1, 0, pl.rows_phys) * 4u;
   } else {
     const int g = warp / pl.split;
     L.p = warp % pl.split;
@@ -1663,7 +1571,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
       sh.wide = 0;
     }
     __syncthreads();
-    stage_vote32(io.xy, a + h0, cn, hb, &sh.nv, &sh.wide, pl.fpbin != 0, pl.mp ? pl.mp_lsq : 0,
+    stage_vote32(io.xy, a + h0, cn, hb, &sh.nv, &sh.wide, pl.mp ? pl.mp_lsq : 0,
                  pl.mp ? reinterpret_cast<uint16_t*>(smem + pl.off_idx) : nullptr);
     __syncthreads();
     HOUGH_PHASE(HOUGH_PHASE_STAGE);
@@ -1674,10 +1582,8 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     if (!(sh.wide & 1)) {
       if (pl.mp)
         vote_mp32(pl, L, hb, sh.nv);
-      else if (pl.fpbin)
-        vote32_fp<A32>(pl, L, hb, sh.nv);
       else
-        vote32<A32>(pl, L, hb, sh.nv);
+        vote32_fp(pl, L, hb, sh.nv);
     } else {
       const int half = pl.hit_cap >> 1;
       for (int s0 = 0; s0 < cn; s0 += half) {
@@ -1690,7 +1596,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
         if (pl.mp)
           vote_mp64(pl, L, hw, sh.nv);
         else
-          vote64<A32>(pl, L, hw, sh.nv);
+          vote64(pl, L, hw, sh.nv);
       }
     }
   }
@@ -1699,7 +1605,6 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
 
 }
 
-template <bool A32>
 __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, long long item,
                          bool do_cs) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
@@ -1721,7 +1626,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
   const int Wd = pl.mp ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
 
-  vote_tile<A32>(pl, io, smem, sh, a, n, t);
+  vote_tile(pl, io, smem, sh, a, n, t);
 
   // 3-4. peaks
   const int maxp = pl.max_peaks;
@@ -1753,24 +1658,24 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
                                maxp, pbits, pl.iter_cap, nullptr, st_words, io.peaks + e * (long long)maxp, sh.tmp,
                                reinterpret_cast<uint16_t*>(pbits + pl.iter_cap + st_words), pl.iter_act);
     };
-    total = pl.mp ? iterative(FusedCells<A32, true>{acc, Wd, nrp, pl.rows_phys})
-                  : iterative(FusedCells<A32, false>{acc, Wd, nrp, pl.rows_phys});
+    total = pl.mp ? iterative(FusedCells<true>{acc, Wd, nrp, pl.rows_phys})
+                  : iterative(FusedCells<false>{acc, Wd, nrp, pl.rows_phys});
     n_low = total;
   } else {
     // 3. peak scan, or (the iterative finder on theta tiles) the tile's candidates: every cell
     // at or above the tile's own relative threshold, a superset of the cells the event's
     // threshold admits (the event's maximum is at least the tile's)
     unsigned long long csum = 0;
-    const bool packed = !pl.mp && !A32 && (NR & 1) == 0;
+    const bool packed = !pl.mp && (NR & 1) == 0;
     if (pl.peak_mode == HOUGH_PEAK_ITERATIVE) {
       if (pl.mp) {
         mp_fold(pl, acc, Wd, nullptr);
         __syncthreads();
         HOUGH_PHASE(HOUGH_PHASE_FOLD);
       }
-      tmax = tile_max_cs<A32>(pl, acc, Wd, aw, wt, j0, do_cs, &sh.it_max, csum);
+      tmax = tile_max_cs(pl, acc, Wd, aw, wt, j0, do_cs, &sh.it_max, csum);
       const long long need = ((long long)pl.rel_num * tmax + pl.rel_den - 1) / pl.rel_den;
-      tile_candidate_bits<A32>(pl, acc, pbits, Wd, wt, (int)max((long long)pl.threshold, need));
+      tile_candidate_bits(pl, acc, pbits, Wd, wt, (int)max((long long)pl.threshold, need));
     } else if (pl.mp) {
       mp_fold(pl, acc, Wd, T > 1 ? halo : nullptr);
       __syncthreads();
@@ -1779,7 +1684,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     } else if (packed) {
       scan_packed(pl, acc, halo, pbits, wt, T, j0, do_cs, csum);
     } else {
-      scan_scalar<A32>(pl, acc, halo, pbits, wt, T, j0, do_cs, csum);
+      scan_scalar(pl, acc, halo, pbits, wt, T, j0, do_cs, csum);
     }
     __syncthreads();
     HOUGH_PHASE(HOUGH_PHASE_SCAN);
@@ -1832,7 +1737,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
           if (o < P1) {
             const int kl = kb + l, c = kl >> pl.key_shift;
             const int k = ((kl & (KG - 1)) << 5) + (int)__fns(wd, 0u, r + 1);
-            const int votes = pl.mp ? mp_get(acc, c, k, Wd, pl) : acc_get<A32>(acc, c, k, nrp);
+            const int votes = pl.mp ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
             const int col = pl.mp ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
             dst2[o] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes);
           }
@@ -1848,7 +1753,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
             const int bb = __ffs(bits) - 1;
             bits &= bits - 1u;
             const int k = (w << 5) + bb;
-            const int votes = pl.mp ? mp_get(acc, c, k, Wd, pl) : acc_get<A32>(acc, c, k, nrp);
+            const int votes = pl.mp ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
             const int col = pl.mp ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
             dst2[pos] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes);
             ++pos;
@@ -1965,7 +1870,6 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
 }
 
-template <bool A32>
 __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ItemShared sh;
@@ -1979,7 +1883,7 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
   __syncthreads();  // the table is read before run_item's first barrier
   const bool do_cs = io.checksum != nullptr;
   if (!io.persistent) {
-    run_item<A32>(pl, io, smem, sh, blockIdx.x, do_cs);
+    run_item(pl, io, smem, sh, blockIdx.x, do_cs);
     return;
   }
   for (;;) {
@@ -1989,7 +1893,7 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
     const long long base = s_item;
     if (base >= io.n_items) break;
     const long long end = min(base + pl.grab, io.n_items);
-    for (long long it = base; it < end; ++it) run_item<A32>(pl, io, smem, sh, it, do_cs);
+    for (long long it = base; it < end; ++it) run_item(pl, io, smem, sh, it, do_cs);
   }
 }
 
@@ -2016,7 +1920,6 @@ struct SpillCells {
 // memory exactly as the fused kernel does and stores the cells to its slot, runs the iterative
 // finder there (the stepwise form, any size) and selects the hits. Count and list were written
 // by the fused kernel before this launch on the same stream.
-template <bool A32>
 __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ItemShared sh;
@@ -2038,7 +1941,7 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
     const int n = nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll;  // a too-large event is never deferred
     int flags = 0;
     for (int t = 0; t < T; ++t) {
-      vote_tile<A32>(pl, io, smem, sh, a, n, t);
+      vote_tile(pl, io, smem, sh, a, n, t);
       const int j0 = t * pl.tile_w, wt = min(pl.tile_w, NT - j0), Wd = pl.mp ? (wt >> 1) : 0,
                 aw = t * (pl.tile_w >> 1);
       if (pl.mp) {
@@ -2053,7 +1956,7 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
       } else {
         for (int i = tid; i < wt * NR; i += bd) {
           const int c = i / NR, k = i - c * NR;
-          A[(j0 + c) * NR + k] = acc_get<A32>(acc, c, k, pl.nrho_pad);
+          A[(j0 + c) * NR + k] = acc_get(acc, c, k, pl.nrho_pad);
         }
       }
       flags |= sh.flags;
@@ -2215,7 +2118,7 @@ static cudaError_t set_smem(const void* fn, int bytes) {
 }
 
 int fused_max_ctas_per_sm(const Plan& pl) {
-  const void* fn = pl.acc32 ? (const void*)fused_kernel<true> : (const void*)fused_kernel<false>;
+  const void* fn = (const void*)fused_kernel;
   if (set_smem(fn, pl.smem_bytes) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, pl.threads, pl.smem_bytes) != cudaSuccess) return 0;
@@ -2223,21 +2126,12 @@ int fused_max_ctas_per_sm(const Plan& pl) {
 }
 
 cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st) {
-  cudaError_t err;
   const bool deferred = pl.peak_mode == HOUGH_PEAK_ITERATIVE && pl.tiles > 1;
-  if (pl.acc32) {
-    err = set_smem((const void*)fused_kernel<true>, pl.smem_bytes);
-    if (err == cudaSuccess && deferred) err = set_smem((const void*)deferred_kernel<true>, pl.smem_bytes);
-    if (err != cudaSuccess) return err;
-    fused_kernel<true><<<grid, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
-    if (deferred) deferred_kernel<true><<<io.n_spill, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
-  } else {
-    err = set_smem((const void*)fused_kernel<false>, pl.smem_bytes);
-    if (err == cudaSuccess && deferred) err = set_smem((const void*)deferred_kernel<false>, pl.smem_bytes);
-    if (err != cudaSuccess) return err;
-    fused_kernel<false><<<grid, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
-    if (deferred) deferred_kernel<false><<<io.n_spill, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
-  }
+  cudaError_t err = set_smem((const void*)fused_kernel, pl.smem_bytes);
+  if (err == cudaSuccess && deferred) err = set_smem((const void*)deferred_kernel, pl.smem_bytes);
+  if (err != cudaSuccess) return err;
+  fused_kernel<<<grid, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
+  if (deferred) deferred_kernel<<<io.n_spill, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
   return cudaGetLastError();
 }
 

@@ -24,7 +24,6 @@ struct Plan {
   int groups;     // 32-column groups per tile
   int split;      // warps voting each column group (hit partitions)
   int threads;    // CTA size: groups * split * 32 (+ 32 halo lanes when tiles > 1)
-  int acc32;      // 1: one int32 cell per shared word; 0: two int16 cells per word
   int nrho_pad;   // rows allocated per column
   int nrb;        // 32-bit bitmap words per column
   int nrb_g;      // bitmap words per column with one guard bit on each side
@@ -35,8 +34,6 @@ struct Plan {
   int key_shift;    // log2(key_groups)
   int key_words;    // bitmap words per key
   int grab;       // persistent queue: items per pop
-  int mirror;     // 1: each vote lane owns column j and its mirror N_theta-1-j
-  int fpbin;      // 1: fast-path bins from a float estimate, exact integer path when ambiguous
   int mp;         // 1: mirror-pair word layout (column j low half, N_theta-1-j high half, guard rows)
   int rows_phys;  // mirror-pair layout: physical rows per column (N_rho + 2)
   int mp_F, mp_rmask, mp_amask, mp_k7;  // float row estimate: fraction bits, row mask, ambiguity mask,

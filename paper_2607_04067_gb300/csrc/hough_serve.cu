@@ -28,7 +28,7 @@
 
 namespace hgpu {
 
-int make_plan(const hough_params* p, Plan& pl, int acc32);
+int make_plan(const hough_params* p, Plan& pl);
 
 namespace {
 
@@ -470,7 +470,7 @@ static int serve_sizes(const hough_serve_config* c, SlotLayout& L, Plan& pl) {
       c->queue_capacity < 1)
     return HOUGH_EINVAL;
   if (c->max_batch_hits > (int64_t)1 << 31) return HOUGH_EINVAL;
-  int rc = make_plan(&c->params, pl, -1);
+  int rc = make_plan(&c->params, pl);
   if (rc) return rc;
   slot_layout(*c, pl, L);
   return HOUGH_OK;
