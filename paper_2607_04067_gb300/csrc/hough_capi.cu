@@ -123,6 +123,9 @@ static bool layout(Plan& pl) {
   }
   pl.off_cnt = o;  // record keys of the local-maximum scan or of a tile's candidates
   if (!it_whole) o += round16(wpad * pl.key_groups * 4);
+  // the vote's list lies in a region that is first written after the vote
+  pl.off_amb = it_whole ? pl.off_pbits : pl.off_cnt;
+  pl.amb_cap = std::min(1024, (o - pl.off_amb) / 4);
   pl.off_unres = o;
   o += round16((pl.hit_cap + 1024) / 32 * 4);
   pl.off_trig = o;
@@ -179,6 +182,7 @@ static void mp_consts(Plan& pl, int n_rho) {
   pl.rows_phys = n_rho + 2;
   pl.mp_F = F;
   pl.mp_rmask = (1 << b) - 1;
+  pl.mp_zoff = 0x4B400000 + (1 << b);
   const double E = (n_rho + 1) * std::ldexp(1.0, F - 23) * (1.0 + std::ldexp(1.0, -20)) + 1.0;
   const int e_min = (int)std::ceil(E);
   int W = 2;

@@ -384,106 +384,225 @@ __device__ __forceinline__ float2 staged_hit(const float* f, int i) {
   return make_float2(q[0], q[2]);
 }
 
-// The four votes of one staged pair of hits (u0, u1, v0, v1) into a word's two columns: row
-// estimates of column j (+A) and of its mirror (-A), packed two hits at a time.
-struct PairEst {
-  float2 k02, k13;  // (hit 0, hit 1) in the low column, then in the high column
+// d = a + b on pairs of floats, rounded down.
+__device__ __forceinline__ float2 add2_rm(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "add.rm.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+
+// Adding 1.5 2^23 rounded down leaves the integer part of a row estimate in the low bits of the
+// sum's pattern: row = pattern - mp_zoff.
+constexpr float kMagic = 12582912.0f;
+
+// Votes of a staged pair of hits (u0, u1, v0, v1) in one word whose estimates lay in the ambiguous
+// window: where the exact row differs from the estimated one that was voted, minus one there and
+// plus one at the exact row. (The packed sums are modulo 2^32, so the order of the adds is free.)
+__device__ __forceinline__ void pair_fix(const Plan& pl, float4 h, int cj, int sj, uint32_t base) {
+  const float A = __fmul_rn((float)cj, pl.fp_scale), B = __fmul_rn((float)sj, pl.fp_scale);
+#pragma unroll 1
+  for (int i = 0; i < 4; ++i) {
+    const float u = i & 2 ? h.y : h.x, v = i & 2 ? h.w : h.z;
+    const float kf = __fmaf_rn(i & 1 ? -u : u, A, __fmaf_rn(v, B, pl.mp_c0));
+    const uint32_t y = __float_as_uint(kf);
+    if ((y & (uint32_t)pl.mp_amask) != 0u) continue;
+    const uint32_t r0 = (y >> pl.mp_F) & (uint32_t)pl.mp_rmask;
+    const int ui = __float2int_rn(u), vi = __float2int_rn(v);
+    const uint32_t r1 = (uint32_t)rho_bin32(ui * (i & 1 ? -cj : cj) + (vi * sj + (int)kH), pl.magic) + 1u;
+    if (r0 != r1) {
+      const uint32_t inc = i & 1 ? 0x10000u : 1u;
+      red_u32(base + (r0 << 7), 0u - inc);
+      red_u32(base + (r1 << 7), inc);
+    }
+  }
+}
+
+// Shared list of (pair of hits, word) steps with an estimate in the ambiguous window.
+struct AmbList {
+  uint32_t* e;  // first pair << 10 | first word
+  int* n;
+  int cap;
 };
 
-__device__ __forceinline__ PairEst pair_est(float4 h, float2 AA, float2 NAA, float2 BB, float2 CC) {
-  const float2 V = fma2(make_float2(h.z, h.w), BB, CC);
-  return PairEst{fma2(make_float2(h.x, h.y), AA, V), fma2(make_float2(h.x, h.y), NAA, V)};
-}
-
-__device__ __forceinline__ bool pair_clear(const PairEst& e, uint32_t am) {
-  return ((__float_as_uint(e.k02.x) & am) != 0u) & ((__float_as_uint(e.k13.x) & am) != 0u) &
-         ((__float_as_uint(e.k02.y) & am) != 0u) & ((__float_as_uint(e.k13.y) & am) != 0u);
-}
-
-__device__ __forceinline__ void pair_red_fast(const PairEst& e, uint32_t base2, int F) {
-  red_u32(base2 + ((__float_as_uint(e.k02.x) >> F) << 7), 1u);
-  red_u32(base2 + ((__float_as_uint(e.k13.x) >> F) << 7), 0x10000u);
-  red_u32(base2 + ((__float_as_uint(e.k02.y) >> F) << 7), 1u);
-  red_u32(base2 + ((__float_as_uint(e.k13.y) >> F) << 7), 0x10000u);
-}
-
-__device__ __forceinline__ void pair_red_exact(const PairEst& e, float4 h, const Plan& pl, uint32_t base,
-                                               uint32_t base2, int cj, int sj) {
-  red_u32(mp_addr(e.k02.x, pl, base, base2, h.x, h.z, cj, sj), 1u);
-  red_u32(mp_addr(e.k13.x, pl, base, base2, h.x, h.z, -cj, sj), 0x10000u);
-  red_u32(mp_addr(e.k02.y, pl, base, base2, h.y, h.w, cj, sj), 1u);
-  red_u32(mp_addr(e.k13.y, pl, base, base2, h.y, h.w, -cj, sj), 0x10000u);
-}
-
-__device__ __forceinline__ void vote_mp32(const Plan& pl, const VoteLane& L, const int2* hb, int nv) {
-  const int cj = L.cj, sj = L.sj;
-  const float* hf = reinterpret_cast<const float*>(hb);
-  if (L.halo) {
-    // A halo word of a tile (columns j and N-1-j), 16 lanes: the same float row estimate as
-    // the tile's own words, into a contiguous column (4 bytes per row, guard rows folded
-    // like the accumulator's), exact bins when ambiguous.
-    if (!L.on) return;
-    const float A = __fmul_rn((float)cj, pl.fp_scale), B = __fmul_rn((float)sj, pl.fp_scale);
-    const float c0 = pl.mp_c0;
-    const uint32_t am = (uint32_t)pl.mp_amask, base2 = L.col2 - ((uint32_t)pl.mp_k7 >> 5);
-    const int F = pl.mp_F;
-#pragma unroll 2
-    for (int i = L.p; i < nv; i += L.P) {
-      const float2 h = staged_hit(hf, i);
-      const float v0 = __fmaf_rn(h.y, B, c0);
-      const uint32_t y0 = (uint32_t)__float_as_int(__fmaf_rn(h.x, A, v0));
-      const uint32_t y1 = (uint32_t)__float_as_int(__fmaf_rn(-h.x, A, v0));
-      if (((y0 & am) != 0u) & ((y1 & am) != 0u)) {
-        red_u32(base2 + ((y0 >> F) << 2), 1u);
-        red_u32(base2 + ((y1 >> F) << 2), 0x10000u);
-      } else {
-        const int u = __float2int_rn(h.x), vs = __float2int_rn(h.y) * sj + (int)kH;
-        red_u32(L.col2 + ((uint32_t)(rho_bin32(u * cj + vs, pl.magic) + 1) << 2), 1u);
-        red_u32(L.col2 + ((uint32_t)(rho_bin32(vs - u * cj, pl.magic) + 1) << 2), 0x10000u);
+// The vote of a warp's share of the hit pairs (p, p + P, ...) into W words a lane: words w0, w0 + 32, ...
+// The loop runs straight through: every estimate votes at once, and a step of U pairs x W words with an
+// estimate in the ambiguous window (2e-4 of the votes at 256 rows) is listed for vote_fix, so that a
+// warp does not run the exact path's ~100 instructions for one lane. The loop is bound by issue: a vote's
+// estimate, floor, address, add and test take 5.5 slots (a packed f32x2 operation takes two), and by
+// the unit that takes the atomics (one warp a cycle) and the broadcast loads (an LDS.128 two cycles), which
+// is why a lane's two words share their loads. Alone, 2,022 hits at 256 x 256, 1,024 threads: 33.5 k cycles with
+// one word and a branch a pair; straight through 28.3 k with one word, 26.8 k with two, 27.6 k with four;
+// 19.4 k with no test, 16.2 k for the atomics alone. A test on the distance from the rounded estimate (two more
+// packed operations instead of the masks) took 30.4 k. In the kernel (batched events): 39.9 k -> 32.7 k
+// cycles; four words a lane spill there (33.0 k).
+template <int W, int U>
+__device__ __forceinline__ void vote_words(const Plan& pl, const int16_t* tc, const int16_t* ts, uint32_t acc_s,
+                                           int aw, int w0, bool on, int p, int P, const int2* hb, int nv,
+                                           const AmbList& L) {
+  if (!on) return;
+  float2 AA[W], BB[W];
+  uint32_t bs[W];
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    const int j = aw + w0 + 32 * w;
+    const float A = __fmul_rn((float)tc[j], pl.fp_scale), B = __fmul_rn((float)ts[j], pl.fp_scale);
+    AA[w] = make_float2(A, A);
+    BB[w] = make_float2(B, B);
+    bs[w] = acc_s + (uint32_t)mp_word(w0 + 32 * w, 0, pl.rows_phys) * 4u - ((uint32_t)pl.mp_zoff << 7);
+  }
+  const float2 CC = make_float2(pl.mp_c0, pl.mp_c0), MM = make_float2(kMagic, kMagic);
+  const uint32_t am = (uint32_t)pl.mp_amask;
+  const float4* hb4 = reinterpret_cast<const float4*>(hb);
+  auto vote_pair = [&](float4 h) {
+    const float2 uu = make_float2(h.x, h.y), nu = make_float2(-h.x, -h.y), vv = make_float2(h.z, h.w);
+    bool ok = true;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      const float2 V = fma2(vv, BB[w], CC);
+      const float2 k0 = fma2(uu, AA[w], V), k1 = fma2(nu, AA[w], V);
+      const float2 z0 = add2_rm(k0, MM), z1 = add2_rm(k1, MM);
+      red_u32(bs[w] + (__float_as_uint(z0.x) << 7), 1u);
+      red_u32(bs[w] + (__float_as_uint(z1.x) << 7), 0x10000u);
+      red_u32(bs[w] + (__float_as_uint(z0.y) << 7), 1u);
+      red_u32(bs[w] + (__float_as_uint(z1.y) << 7), 0x10000u);
+      ok = ok & ((__float_as_uint(k0.x) & am) != 0u) & ((__float_as_uint(k1.x) & am) != 0u) &
+           ((__float_as_uint(k0.y) & am) != 0u) & ((__float_as_uint(k1.y) & am) != 0u);
+    }
+    return ok;
+  };
+  auto list = [&](int q, int n) {
+    const int at = atomicAdd(L.n, 1);
+    if (at < L.cap) {
+      L.e[at] = ((uint32_t)q << 10) | (uint32_t)w0;
+    } else {  // no room: now
+      for (int i = 0; i < n; ++i)
+        for (int w = 0; w < W; ++w) {
+          const int x = w0 + 32 * w;
+          pair_fix(pl, hb4[q + i * P], tc[aw + x], ts[aw + x], acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u);
+        }
+    }
+  };
+  const int np = nv >> 1;
+  int q = p;
+#pragma unroll 1
+  for (; q + (U - 1) * P < np; q += U * P) {
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < U; ++i) ok = vote_pair(hb4[q + i * P]) & ok;
+    if (!ok) list(q, U);
+  }
+#pragma unroll 1
+  for (; q < np; q += P) {
+    if (!vote_pair(hb4[q])) {
+      for (int w = 0; w < W; ++w) {
+        const int x = w0 + 32 * w;
+        pair_fix(pl, hb4[q], tc[aw + x], ts[aw + x], acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u);
       }
     }
-    return;
   }
-  const float A = __fmul_rn((float)cj, pl.fp_scale), B = __fmul_rn((float)sj, pl.fp_scale);
-  if (!L.on) return;
-  const float2 AA = make_float2(A, A), NAA = make_float2(-A, -A), BB = make_float2(B, B);
-  const float2 CC = make_float2(pl.mp_c0, pl.mp_c0);
-  const uint32_t base = L.col1, base2 = L.col1 - (uint32_t)pl.mp_k7;
+  if ((nv & 1) && p == np % P) {
+    const float2 h = staged_hit(reinterpret_cast<const float*>(hb), nv - 1);
+    for (int w = 0; w < W; ++w) {
+      const int x = w0 + 32 * w, cj = tc[aw + x], sj = ts[aw + x];
+      const uint32_t base = acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u, base2 = base - (uint32_t)pl.mp_k7;
+      const float v0 = __fmaf_rn(h.y, BB[w].x, pl.mp_c0);
+      red_u32(mp_addr(__fmaf_rn(h.x, AA[w].x, v0), pl, base, base2, h.x, h.y, cj, sj), 1u);
+      red_u32(mp_addr(__fmaf_rn(-h.x, AA[w].x, v0), pl, base, base2, h.x, h.y, -cj, sj), 0x10000u);
+    }
+  }
+}
+
+// The listed steps' exact rows, a thread a (pair, word).
+template <int W, int U>
+__device__ __forceinline__ void vote_fix(const Plan& pl, const int16_t* tc, const int16_t* ts, uint32_t acc_s, int aw,
+                                         int P, const int2* hb, const AmbList& L) {
+  const int n = min(*L.n, L.cap) * (W * U);
   const float4* hb4 = reinterpret_cast<const float4*>(hb);
-  const int np = nv >> 1, P = L.P;
-  const uint32_t am = (uint32_t)pl.mp_amask;
-  const int F = pl.mp_F;
-  // One pair of hits (4 votes) a step and one exactness test for the 4: the rare step with an
-  // estimate in the ambiguous window takes the exact path vote by vote. (Two pairs a step with one
-  // test for 8 votes measured slower inside this kernel: 43.4 k against 39.6 k cycles an event.)
-#pragma unroll 4
-  for (int q = L.p; q < np; q += P) {
-    const float4 g = hb4[q];
-    const PairEst eg = pair_est(g, AA, NAA, BB, CC);
-    if (pair_clear(eg, am)) pair_red_fast(eg, base2, F);
-    else pair_red_exact(eg, g, pl, base, base2, cj, sj);
+  for (int it = threadIdx.x; it < n; it += blockDim.x) {
+    const uint32_t e = L.e[it / (W * U)];
+    const int q = (int)(e >> 10) + (it % U) * P, x = (int)(e & 1023u) + 32 * (it / U % W);
+    pair_fix(pl, hb4[q], tc[aw + x], ts[aw + x], acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u);
   }
-  if ((nv & 1) && L.p == np % P) {
-    const float2 h = staged_hit(hf, nv - 1);
+}
+
+// All of a chunk's votes into a mirror-pair tile of Wd words (every thread calls it; the votes are
+// complete after the next barrier).
+__device__ __forceinline__ void vote_mp32(const Plan& pl, const int16_t* tc, const int16_t* ts, uint32_t acc_s, int aw,
+                                          int Wd, const int2* hb, int nv, const AmbList& L) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = pl.groups >> 1, P2 = 2 * pl.split;
+  const bool worker = warp < G * P2;
+  auto go = [&](auto wc, auto uc) {
+    constexpr int W = decltype(wc)::value, U = decltype(uc)::value;
+    const int P = P2 * W, w0 = (warp / P) * (32 * W) + lane;
+    vote_words<W, U>(pl, tc, ts, acc_s, aw, w0, worker && w0 < Wd, warp % P, P, hb, nv, L);
+    __syncthreads();
+    vote_fix<W, U>(pl, tc, ts, acc_s, aw, P, hb, L);
+  };
+  using std::integral_constant;
+  // two words a lane only where every lane has both
+  if ((Wd & 63) == 0) go(integral_constant<int, 2>{}, integral_constant<int, 2>{});
+  else go(integral_constant<int, 1>{}, integral_constant<int, 4>{});
+}
+
+// Halo words of a mirror-pair tile: the words before and after its own (none at the theta wrap or at the
+// middle word), each a contiguous column of 4-byte rows (guard rows folded like the accumulator's). Every
+// thread of the CTA takes hits, even threads for the word before, odd ones for the word after: a warp
+// of its own finished last (the vote of stress events at 512 x 512 took 313 k cycles with it, 207 k without
+// any halo).
+struct HaloLane {
+  bool on;
+  int c, s;
+  uint32_t col;  // shared address of row 0
+};
+
+__device__ __forceinline__ HaloLane halo_lane(const Plan& pl, const int16_t* tc, const int16_t* ts,
+                                              const uint32_t* halo, int aw, int Wd) {
+  const int side = threadIdx.x & 1, w = side ? aw + Wd : aw - 1;
+  HaloLane h;
+  h.on = side ? w < (pl.n_theta >> 1) : w >= 0;
+  h.c = h.on ? tc[w] : 0;
+  h.s = h.on ? ts[w] : 0;
+  h.col = (uint32_t)__cvta_generic_to_shared(halo) + (uint32_t)(side * pl.rows_phys) * 4u;
+  return h;
+}
+
+__device__ __forceinline__ void halo_mp32(const Plan& pl, const HaloLane& H, const int2* hb, int nv) {
+  if (!H.on) return;
+  const float A = __fmul_rn((float)H.c, pl.fp_scale), B = __fmul_rn((float)H.s, pl.fp_scale);
+  const uint32_t am = (uint32_t)pl.mp_amask, base2 = H.col - ((uint32_t)pl.mp_k7 >> 5);
+  const int F = pl.mp_F;
+#pragma unroll 2
+  for (int i = threadIdx.x >> 1; i < nv; i += blockDim.x >> 1) {
+    const float2 h = staged_hit(reinterpret_cast<const float*>(hb), i);
     const float v0 = __fmaf_rn(h.y, B, pl.mp_c0);
-    red_u32(mp_addr(__fmaf_rn(h.x, A, v0), pl, base, base2, h.x, h.y, cj, sj), 1u);
-    red_u32(mp_addr(__fmaf_rn(-h.x, A, v0), pl, base, base2, h.x, h.y, -cj, sj), 0x10000u);
+    const uint32_t y0 = __float_as_uint(__fmaf_rn(h.x, A, v0)), y1 = __float_as_uint(__fmaf_rn(-h.x, A, v0));
+    if (((y0 & am) != 0u) & ((y1 & am) != 0u)) {
+      red_u32(base2 + ((y0 >> F) << 2), 1u);
+      red_u32(base2 + ((y1 >> F) << 2), 0x10000u);
+    } else {
+      const int uc = __float2int_rn(h.x) * H.c, vs = __float2int_rn(h.y) * H.s + (int)kH;
+      red_u32(H.col + ((uint32_t)(rho_bin32(vs + uc, pl.magic) + 1) << 2), 1u);
+      red_u32(H.col + ((uint32_t)(rho_bin32(vs - uc, pl.magic) + 1) << 2), 0x10000u);
+    }
+  }
+}
+
+__device__ __forceinline__ void halo_mp64(const Plan& pl, const HaloLane& H, const longlong2* hw, int nv) {
+  if (!H.on) return;
+  for (int i = threadIdx.x >> 1; i < nv; i += blockDim.x >> 1) {
+    const long long vs = hw[i].y * H.s + kH, uc = hw[i].x * H.c;
+    red_u32(H.col + ((uint32_t)(rho_bin64(vs + uc, pl.magic) + 1) << 2), 1u);
+    red_u32(H.col + ((uint32_t)(rho_bin64(vs - uc, pl.magic) + 1) << 2), 0x10000u);
   }
 }
 
 __device__ __forceinline__ void vote_mp64(const Plan& pl, const VoteLane& L, const longlong2* hw, int nv) {
   const BinMagic m = pl.magic;
   const long long cj = L.cj, sj = L.sj;
-  if (L.halo) {
-    if (!L.on) return;
-    for (int i = L.p; i < nv; i += L.P) {
-      const longlong2 h = hw[i];
-      const long long vs = h.y * sj + kH, uc = h.x * cj;
-      red_u32(L.col2 + ((uint32_t)(rho_bin64(vs + uc, m) + 1) << 2), 1u);
-      red_u32(L.col2 + ((uint32_t)(rho_bin64(vs - uc, m) + 1) << 2), 0x10000u);
-    }
-    return;
-  }
   if (!L.on) return;
   for (int q = L.p; q < nv; q += L.P) {
     const longlong2 h = hw[q];
@@ -968,7 +1087,7 @@ __device__ int select_staged(const Plan& pl, const int2* hb, const uint16_t* idx
 }
 
 struct ItemShared {
-  int nv, flags, wide, last, total, D, reuse;
+  int nv, flags, wide, last, total, D, reuse, n_amb;
   int kept_tot;
   long long tstart[128];  // segment starts of the tile merge (2 segments a mirror-pair tile)
   int tmp[32];
@@ -1501,17 +1620,8 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
   const uint32_t acc_s = (uint32_t)__cvta_generic_to_shared(acc);
   const bool want_halo = pl.peak_mode != HOUGH_PEAK_ITERATIVE;  // only the 3x3 test reads the halo
   if (L.halo && pl.mp) {
-    // lanes 0-15: word aw - 1, lanes 16-31: word aw + Wd (both of its columns), each lane
-    // a sixteenth of the hits; none at the theta wrap or at the middle word
-    const int hs = lane >> 4, wg = hs ? aw + Wd : aw - 1;
-    L.on = want_halo && (hs ? (aw + Wd < (NT >> 1)) : (aw > 0));
-    if (L.on) {
-      L.cj = tc[wg];
-      L.sj = ts[wg];
-    }
-    L.col2 = (uint32_t)__cvta_generic_to_shared(halo) + (uint32_t)(hs * pl.rows_phys) * 4u;
-    L.p = lane & 15;
-    L.P = 16;
+    L.p = 0;  // no words of its own (every thread votes halo hits)
+    L.P = 1;
   } else if (L.halo) {
     const int jh = lane < 16 ? (j0 - 1 + NT) % NT : (j0 + wt) % NT;
     L.on = want_halo;
@@ -1544,6 +1654,11 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     L.col1 = acc_s + (uint32_t)(((g * rows_w) << 5) + lane) * 4u;
   }
 
+  const bool mp_halo = pl.mp && T > 1 && want_halo;
+  HaloLane HL{false, 0, 0, 0u};
+  if (mp_halo) HL = halo_lane(pl, tc, ts, halo, aw, Wd);
+  const AmbList amb{reinterpret_cast<uint32_t*>(smem + pl.off_amb), &sh.n_amb, pl.amb_cap};
+
   // 1. clear accumulator, halo columns, peak bitmap and counters
   __syncthreads();
   HOUGH_PHASE_START();
@@ -1569,6 +1684,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     if (tid == 0) {
       sh.nv = 0;
       sh.wide = 0;
+      sh.n_amb = 0;
     }
     __syncthreads();
     stage_vote32(io.xy, a + h0, cn, hb, &sh.nv, &sh.wide, pl.mp ? pl.mp_lsq : 0,
@@ -1580,8 +1696,9 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
       if (sh.wide & 1) sh.reuse = 0;  // wide hits are not in the staged list
     }
     if (!(sh.wide & 1)) {
+      if (mp_halo) halo_mp32(pl, HL, hb, sh.nv);
       if (pl.mp)
-        vote_mp32(pl, L, hb, sh.nv);
+        vote_mp32(pl, tc, ts, acc_s, aw, Wd, hb, sh.nv, amb);
       else
         vote32_fp(pl, L, hb, sh.nv);
     } else {
@@ -1593,6 +1710,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
         __syncthreads();
         stage_vote64(io.xy, a + h0 + s0, sn, hw, &sh.nv);
         __syncthreads();
+        if (mp_halo) halo_mp64(pl, HL, hw, sh.nv);
         if (pl.mp)
           vote_mp64(pl, L, hw, sh.nv);
         else

@@ -36,6 +36,7 @@ struct Plan {
   int grab;       // persistent queue: items per pop
   int mp;         // 1: mirror-pair word layout (column j low half, N_theta-1-j high half, guard rows)
   int rows_phys;  // mirror-pair layout: physical rows per column (N_rho + 2)
+  int mp_zoff;    // pattern of 1.5 2^23, plus 2^b
   int mp_F, mp_rmask, mp_amask, mp_k7;  // float row estimate: fraction bits, row mask, ambiguity mask,
                                         // exponent bits of (y >> F) << 7
   float mp_c0;    // N_rho/2 + 1 + 2^b + W/2 2^-F
@@ -44,6 +45,7 @@ struct Plan {
   // iterative finder on theta tiles: candidate keys the merging CTA holds; slice height and
   // candidate keys of the deferred kernel's finder
   int merge_cap, def_sh, def_cap;
+  int off_amb, amb_cap;  // list of ambiguous vote steps (shares a region that the vote leaves free) and its entries
   // shared-memory layout in bytes
   int off_acc, region_bytes, off_halo, off_hits, off_idx, off_pbits, off_cnt, off_unres, off_trig, smem_bytes;
   BinMagic magic;

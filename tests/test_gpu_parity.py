@@ -325,6 +325,40 @@ def test_non_default_stream_and_graph_replay(h):
         assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
 
 
+# ---------------------------------------------------------------- the mirror-pair vote at its edges
+
+def near_boundary_hits(ev, n_theta, n_rho, n_hits):
+    """The hits of ev with the most theta columns whose exact bin position lies within 5e-5 of a boundary."""
+    x, y = ev.xy[:, 0].astype(np.int64), ev.xy[:, 1].astype(np.int64)
+    r2 = x * x + y * y
+    u, v = (x << 33) // r2, (y << 33) // r2
+    th = (np.arange(n_theta) + 0.5) * np.pi / n_theta
+    c, s = np.rint(16384 * np.cos(th)), np.rint(16384 * np.sin(th))
+    k = (u[:, None] * c + v[:, None] * s + 703687442) * n_rho / (2.0 * 703687442)
+    near = (np.abs(k - np.rint(k)) < 5e-5).sum(axis=1)
+    return ev.xy[np.argsort(-near, kind="stable")[:n_hits]]
+
+
+@pytest.mark.parametrize("n_theta,n_rho,tiles", [(64, 64, 1), (128, 100, 1), (130, 64, 1), (256, 256, 1), (256, 256, 2),
+                                                 (512, 512, 4), (1000, 500, 8), (258, 256, 3)])
+def test_vote_edges(h, n_theta, n_rho, tiles):
+    """One and two words a lane; events of 0, 1, 2, 3, ... hits (fewer pairs than warps, odd counts, one
+    staging chunk and one hit more); hits repeated so that their near-boundary columns overflow the
+    list of ambiguous steps. Accumulators by checksum, and every output."""
+    ev = gen.generate("batched", 12)
+    near = near_boundary_hits(ev, n_theta, n_rho, 3)
+    parts = [ev.xy[i:i + n] for i, n in enumerate([0, 1, 2, 3, 7, 31, 64, 65, 127, 130, 257, 4096, 4097])]
+    parts += [np.repeat(near[i:i + 1], 3001 + i, axis=0) for i in range(3)]
+    off = np.concatenate([[0], np.cumsum([len(p) for p in parts])]).astype(np.int64)
+    xy = np.ascontiguousarray(np.concatenate(parts))
+    ref = oracle.run(xy, off, oracle.params(n_theta, n_rho, 3, 1, 16384), threads=THREADS)
+    d_xy, d_off = torch.from_numpy(xy).cuda(), torch.from_numpy(off).cuda()
+    for batched in (False, True):
+        out = h.run(d_xy, d_off, h.params(n_theta, n_rho, 3, 1, 16384, theta_tiles=tiles), checksum=True, batched=batched)
+        assert h.status(out.status) == ref.status
+        assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
+
+
 # ---------------------------------------------------------------- exhaustive bin function
 
 @pytest.mark.parametrize("n_rho", [4, 63, 64, 256, 512, 1000, 1024])
