@@ -98,7 +98,7 @@ static bool layout(Plan& pl) {
   // mirror-pair: groups / 2 word groups of 32 lanes (the last may be part idle) x rows_phys
   const int acc_bytes = pl.mp ? (pl.groups / 2) * 32 * pl.rows_phys * 4 : wpad * pl.nrho_pad * 2;
   const int sel_bytes = (2 * pl.n_theta + 64) * 4 + pl.n_theta * 16 + pl.n_theta * pl.nrb_g * 4;
-  int o = 0;
+  int o = 1024;  // the scan of a wrapped word may read up to seven rows (of 128 bytes) below row 0
   pl.off_acc = o;
   pl.region_bytes = round16(acc_bytes > sel_bytes ? acc_bytes : sel_bytes);
   o += pl.region_bytes;
@@ -119,7 +119,7 @@ static bool layout(Plan& pl) {
       iter_words = iter_scratch_words(pl.n_theta, pl.n_rho, kIterSliceRows);
       if (pl.iter_cap > 0 && cand_words > iter_words) iter_words = cand_words;
     }
-    o += round16((wpad * pl.nrb > iter_words ? wpad * pl.nrb : iter_words) * 4);
+    o += round16((wpad * pl.nrb_p > iter_words ? wpad * pl.nrb_p : iter_words) * 4);
   }
   pl.off_cnt = o;  // record keys of the local-maximum scan or of a tile's candidates
   if (!it_whole) o += round16(wpad * pl.key_groups * 4);
@@ -209,7 +209,8 @@ int make_plan(const hough_params* p, Plan& pl) {
   pl.rel_den = p->rel_den;
   pl.nms_radius = p->nms_radius;
   pl.nrb = (p->n_rho + 31) / 32;
-  pl.nrb_g = (p->n_rho + 2 + 31) / 32;
+  pl.nrb_p = pl.nrb | 1;
+  pl.nrb_g = ((p->n_rho + 2 + 31) / 32) | 1;
   pl.magic = host_magic(p->n_rho);
   pl.grab = p->events_per_cta > 0 ? p->events_per_cta : 1;
   {
@@ -269,14 +270,13 @@ int make_plan(const hough_params* p, Plan& pl) {
     }
     pl.mp = sym ? 1 : 0;
     if (pl.mp) mp_consts(pl, p->n_rho);
-    // row ranges of the peak scan: the power of two that minimises the slowest warp's row
-    // steps, each unit (30 columns x one range) paying two extra rows to prime its window and
-    // about 16 rows' worth of setup (measured at 256 x 256, 1024 threads: 4 ranges scan in
-    // 9.4 k cycles an event, 8 in 9.5 k, 16 in 10.3 k, 32 in 12.6 k)
+    if (!pl.mp)
+    // Column layout: the power of two of row ranges that minimises the slowest warp's row steps, each
+    // unit (30 columns x one range) paying two extra rows to prime its window and about 16 rows' worth
+    // of setup.
     {
-      const bool packed = !pl.mp && (p->n_rho & 1) == 0;
-      const int cols = pl.mp ? pl.tile_w / 2 : pl.tile_w;
-      const int nblk = (cols + 29) / 30, nwarps = pl.threads / 32;
+      const bool packed = (p->n_rho & 1) == 0;
+      const int nblk = (pl.tile_w + 29) / 30, nwarps = pl.threads / 32;
       const int rows = packed ? p->n_rho / 2 : p->n_rho;
       long best = -1;
       for (int Rs = 0; (1 << Rs) <= 64 && (rows >> Rs) >= 2; ++Rs) {

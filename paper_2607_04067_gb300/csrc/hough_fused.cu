@@ -632,141 +632,129 @@ __device__ void mp_fold(const Plan& pl, uint32_t* acc, int n_words, uint32_t* ha
   }
 }
 
-// Peak scan of the mirror-pair layout: one row per step, both columns of a word at once.
-// For word lane w, lane w-1 holds the left neighbour of column w and the right neighbour of
-// column N-1-w; lane w+1 the other two. Lane w = -1 supplies the theta wrap (word lane 0, rows
-// mirrored, halves swapped) and lane w = N/2 the middle (word lane N/2-1, halves swapped).
-// A tile owns words [aw, aw + half) (columns aw.. and their mirrors); its neighbour words
-// aw - 1 and aw + half come from the halo (two contiguous columns of rows_phys words, no
-// mirroring) unless the tile starts at word 0 (theta wrap) or ends at the middle word.
-__device__ void scan_mp(const Plan& pl, const uint32_t* acc, const uint32_t* halo, int aw, int half,
-                        uint32_t* pbits, bool do_cs, unsigned long long& csum) {
-  const int NT = pl.n_theta, NR = pl.n_rho, R = pl.scan_ranges, rp = pl.rows_phys;
-  const bool first = aw == 0, last = aw + half == (NT >> 1);
+// Where the word before (side 0) or after (side 1) a 32-word group of the tile lies: its row -1 as a word
+// offset into the CTA's shared memory, the words from row to row, and whether its halves are swapped.
+struct EdgeWord {
+  int at;
+  short step, swap;
+};
+
+// Edge words of the tile's groups (the CTA's last 2 G threads). Before word 0 lies the theta wrap (word 0, rows mirrored:
+// from the top down, halves swapped), after the middle word itself (halves swapped), else the halo
+// (two contiguous columns of rows_phys words, of the words aw - 1 and aw + half; a tile owns words
+// [aw, aw + half), columns aw.. and their mirrors).
+__device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, EdgeWord* ew) {
+  const int G = (half + 31) >> 5, i = (int)(blockDim.x - 1 - threadIdx.x), rp = pl.rows_phys, acc0 = pl.off_acc >> 2, halo0 = pl.off_halo >> 2;
+  if (i >= 2 * G) return;
+  const int w = i & 1 ? min((i >> 1) * 32 + 32, half) : (i >> 1) * 32 - 1;
+  EdgeWord e{acc0, 32, 0};
+  if (w >= 0 && w < half) {
+    e.at += mp_word(w, 0, rp);
+  } else if (w < 0 ? aw == 0 : aw + half == (pl.n_theta >> 1)) {
+    e.at += w < 0 ? mp_word(0, pl.n_rho + 1, rp) : mp_word(half - 1, 0, rp);
+    e.step = w < 0 ? -32 : 32;
+    e.swap = 1;
+  } else {
+    e.at = halo0 + (w < 0 ? 0 : rp);
+    e.step = 1;
+  }
+  ew[i] = e;
+}
+
+// Peak scan of the mirror-pair layout, both columns of a word at once, in two passes. (1) Row groups (32
+// words x 4 rows: one 16-byte load a lane) in which some cell reaches the threshold are listed; about a
+// third of them at 256 x 256 and T = 16, a few per cent at 1000 x 1000 and T = 12. (2) Warps take listed
+// groups in turn, lane l word l, and set the flags of their peaks in the cleared bitmap.
+// For word lane w, lane w-1 holds the left neighbour of column w and the right neighbour of column
+// N-1-w; lane w+1 the other two; lane 0 and lane n (lane 31 with a full group of n = 32) also read the
+// words beyond the group (edge_words).
+// Both passes are bound by the integer ALU, which takes a warp instruction every two cycles of a scheduler (so
+// 100 instructions of set-up in each of 32 warps are about 1.3 k cycles): the first takes 11 instructions a
+// group, the second about 125. One pass in units of 30 words x 64 rows took 9.3 k cycles an event at 256 x 256
+// (the central rows' candidates fell to a few warps) and 10.0 k a tile at 1000 x 1000; units of 8 rows
+// 9.6 k and 7.5 k; this form 9.9 k and 3.9 k.
+// list: room for (half + 31) / 32 * ((N_rho + 3) / 4) entries; *n_list zero beforehand.
+__device__ void scan_mp(const Plan& pl, const unsigned char* smem, int aw, int half, const EdgeWord* ew,
+                        uint32_t* pbits, uint16_t* list, int* n_list, bool do_cs, unsigned long long& csum) {
+  const int NT = pl.n_theta, NR = pl.n_rho, rp = pl.rows_phys;
+  const uint32_t* const sw = reinterpret_cast<const uint32_t*>(smem);
+  const uint32_t* const acc = sw + (pl.off_acc >> 2);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int nblk = (half + 29) / 30;
+  const int G = (half + 31) >> 5, n4 = (NR + 3) >> 2;  // groups of words, of rows
   const uint32_t TT = (uint32_t)pl.threshold | ((uint32_t)pl.threshold << 16);
-  for (int u = warp; u < nblk * R; u += nwarps) {
-    const int b = u >> pl.scan_shift, r = u & (R - 1);
-    const int k0 = (NR * r) >> pl.scan_shift, k1 = (NR * (r + 1)) >> pl.scan_shift;
-    const int w = b * 30 + lane - 1;
-    // Source word of this lane for logical row k: physical row k + 1 (or N_rho - k when the
-    // rows are mirrored); the zeroed guard rows supply the missing rows -1 and N_rho.
-    int sw = w, p0 = k0, step = 32;
-    unsigned sel = 0x3210u;  // byte permutation: identity, or swap of the two halves
-    const uint32_t* hcol = nullptr;
-    if (w < 0) {
-      if (first) {
-        sw = 0;
-        p0 = NR - (k0 - 1);
-        step = -32;
-        sel = 0x1032u;
-      } else {
-        hcol = halo;
+  // (1) A half reaches T iff bit 15 of C - T + 0x8000 is set (cells are at most 32767: no borrow across
+  // the halves). Rows past the last one may be read (they only list a group in vain), inside the CTA's
+  // shared memory.
+  for (int g = 0; g < G; ++g) {
+    const uint4* row = reinterpret_cast<const uint4*>(acc + mp_word(32 * g, 1, rp)) + lane;
+    uint32_t hit = 0;
+    int q0 = warp, c = 0;
+    for (int q = warp; q < n4; q += nwarps, ++c) {
+      if (c == 32) {  // a warp's mask of 32 groups is full (only small CTAs)
+        if ((hit >> lane) & 1u) list[atomicAdd(n_list, 1)] = (uint16_t)(g << 8 | (q0 + lane * nwarps));
+        hit = 0;
+        q0 = q;
+        c = 0;
       }
-    } else if (w >= half) {
-      if (w == half && last) {
-        sw = half - 1;
-        sel = 0x1032u;
-      } else if (w == half) {
-        hcol = halo + rp;
-      } else {
-        sw = 0;  // nothing: read guard row 0 (zero) throughout
-        p0 = 0;
-        step = 0;
-      }
-    }
-    const uint32_t* ptr = hcol ? hcol + k0 : acc + mp_word(sw, p0, rp);  // row k0 - 1
-    if (hcol) step = 1;
-    const bool tested = lane >= 1 && lane <= 30 && w >= 0 && w < half;
-    // Raster order runs over theta, then rho: the row above and the preceding column are
-    // "before" a cell (strictly below it at a peak), the rest "after" (at most equal). The
-    // preceding column of the low half (column aw+w) is lane w-1's low half (the wrapped
-    // column N-1 at word 0: after, not before); of the high half (column N-1-aw-w) lane w+1's
-    // high half; lane w-1's high half follows it (except at word 0: the wrapped column 0).
-    // Strictness becomes +1 on that neighbour, so a cell is a peak iff C >= max(U + 1, D,
-    // VU + addU, VD + 0x10000, T) per half; cells are at most 32767, so nothing carries.
-    const uint32_t addU = (w != 0 || !first) ? 1u : 0x10000u;
-    const int clo = w, chi = 2 * half - 1 - w;                // tile-local columns
-    const int glo = aw + w, ghi = NT - 1 - aw - w;             // event columns
-    uint32_t U = __byte_perm(ptr[0], 0u, sel);
-    ptr += step;
-    uint32_t C = __byte_perm(ptr[0], 0u, sel);
-    ptr += step;
-    for (int ks = k0; ks < k1;) {
-      const int ke = min(k1, (ks | 31) + 1);  // rows of one bitmap word
-      uint32_t bl = 0, bh = 0;                // peak flags, newest row in bit 0
-      int k = ks;
-      // Groups of four rows: the loads and the candidate test run straight through, and the
-      // neighbour test only for a group where some tested cell reaches T (bit 15 of a half of
-      // 0x8000 - (max(C, T) - C) is set iff C >= T); most groups have none.
-      for (; k + 4 <= ke; k += 4) {
-        uint32_t R4[4];
+      const uint4 x = row[q << 5];
+      const uint32_t top = vmax2(vmax2(x.x, x.y), vmax2(x.z, x.w));
+      if (__any_sync(kFull, ((top - TT + 0x80008000u) & 0x80008000u) != 0u)) hit |= 1u << c;
+      if (do_cs) {
+        const int k = 4 * q + (lane >> 3), w = 32 * g + 4 * (lane & 7);
+        const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          R4[i] = __byte_perm(ptr[0], 0u, sel);
-          ptr += step;
-        }
-        const uint32_t c1 = R4[0], c2 = R4[1], c3 = R4[2];
-        const uint32_t cand = ((0x80008000u - vmax2(C, TT) + C) | (0x80008000u - vmax2(c1, TT) + c1) |
-                               (0x80008000u - vmax2(c2, TT) + c2) | (0x80008000u - vmax2(c3, TT) + c3)) &
-                              0x80008000u;
-        if (__any_sync(kFull, tested && cand != 0u)) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const uint32_t Cc = i == 0 ? C : R4[i - 1], Uu = i == 0 ? U : (i == 1 ? C : R4[i - 2]), Dd = R4[i];
-            const uint32_t VM = vmax2(vmax2(Uu, Cc), Dd);
-            const uint32_t VU = __shfl_up_sync(kFull, VM, 1);
-            const uint32_t VD = __shfl_down_sync(kFull, VM, 1);
-            const uint32_t X = vmax2(vmax2(vmax2(Uu + 0x00010001u, Dd), vmax2(VU + addU, VD + 0x10000u)), TT);
-            const uint32_t Z = 0x80008000u - vmax2(X, Cc) + Cc;
-            bh = __funnelshift_l(Z, bh, 1);
-            bl = __funnelshift_l(Z << 16, bl, 1);
-          }
-        } else {
-          bh <<= 4;
-          bl <<= 4;
-        }
-        if (do_cs && tested) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const uint32_t Cc = i == 0 ? C : R4[i - 1];
-            const unsigned a0 = Cc & 0xffffu, a1 = Cc >> 16;
-            if (a0) csum += (unsigned long long)a0 * mix64((unsigned long long)glo * NR + k + i + 1);
-            if (a1) csum += (unsigned long long)a1 * mix64((unsigned long long)ghi * NR + k + i + 1);
+          const unsigned a0 = xs[i] & 0xffffu, a1 = xs[i] >> 16;
+          if (k < NR && w + i < half) {
+            if (a0) csum += (unsigned long long)a0 * mix64((unsigned long long)(aw + w + i) * NR + k + 1);
+            if (a1) csum += (unsigned long long)a1 * mix64((unsigned long long)(NT - 1 - aw - w - i) * NR + k + 1);
           }
         }
-        U = R4[2];
-        C = R4[3];
       }
-#pragma unroll 4
-      for (; k < ke; ++k) {
-        const uint32_t D = __byte_perm(ptr[0], 0u, sel);
-        ptr += step;
-        const uint32_t VM = vmax2(vmax2(U, C), D);
-        const uint32_t VU = __shfl_up_sync(kFull, VM, 1);
-        const uint32_t VD = __shfl_down_sync(kFull, VM, 1);
-        const uint32_t X = vmax2(vmax2(vmax2(U + 0x00010001u, D), vmax2(VU + addU, VD + 0x10000u)), TT);
-        // half of Z has bit 15 set iff C >= X there: 0x8000 - (max(X, C) - C), no borrow
-        const uint32_t Z = 0x80008000u - vmax2(X, C) + C;
-        bh = __funnelshift_l(Z, bh, 1);
-        bl = __funnelshift_l(Z << 16, bl, 1);
-        if (do_cs && tested) {
-          const unsigned a0 = C & 0xffffu, a1 = C >> 16;
-          if (a0) csum += (unsigned long long)a0 * mix64((unsigned long long)glo * NR + k + 1);
-          if (a1) csum += (unsigned long long)a1 * mix64((unsigned long long)ghi * NR + k + 1);
-        }
-        U = C;
-        C = D;
-      }
-      if (tested) {
-        const int sh = 32 - (ke - ks) - (ks & 31);  // row ks to bit ks & 31
-        bl = __brev(bl) >> sh;
-        bh = __brev(bh) >> sh;
-        if (bl) atomicOr(&pbits[clo * pl.nrb + (ks >> 5)], bl);
-        if (bh) atomicOr(&pbits[chi * pl.nrb + (ks >> 5)], bh);
-      }
-      ks = ke;
+    }
+    if ((hit >> lane) & 1u) list[atomicAdd(n_list, 1)] = (uint16_t)(g << 8 | (q0 + lane * nwarps));
+  }
+  __syncthreads();
+  // (2) Raster order runs over theta, then rho: the row above and the preceding column are
+  // "before" a cell (strictly below it at a peak), the rest "after" (at most equal). The
+  // preceding column of the low half (column aw+w) is lane w-1's low half (the wrapped
+  // column N-1 at word 0: after, not before); of the high half (column N-1-aw-w) lane w+1's
+  // high half; lane w-1's high half follows it (except at word 0: the wrapped column 0).
+  // Strictness becomes +1 on that neighbour, so a cell is a peak iff C >= max(U + 1, D,
+  // VU + addU, VD + 0x10000, T) per half.
+  const int nl = *n_list;
+  for (int it = warp; it < nl; it += nwarps) {
+    const int en = list[it], g = en >> 8, k = (en & 255) << 2, n = min(32, half - 32 * g), w = 32 * g + lane;
+    const uint32_t addU = (w != 0 || aw != 0) ? 1u : 0x10000u;
+    const uint32_t* ptr = acc + mp_word(w, k, rp);  // row k - 1 (lanes past the last word: zero words)
+    const uint32_t R[6] = {ptr[0], ptr[32], ptr[64], ptr[96], ptr[128], ptr[160]};
+    uint32_t EV[4] = {0u, 0u, 0u, 0u};  // 3-row maxima of the word beyond the group
+    if (lane == 0 || lane == min(n, 31)) {  // (n == 1: lanes 0 and 1)
+      const EdgeWord ed = ew[2 * g + (lane != 0)];
+      const int st = ed.step;
+      const uint32_t* q = sw + ed.at + st * k;
+      uint32_t e[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) e[i] = q[st * i];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) EV[i] = __byte_perm(vmax2(vmax2(e[i], e[i + 1]), e[i + 2]), 0u, ed.swap ? 0x1032u : 0x3210u);
+    }
+    uint32_t fl = 0u;  // flags, the low column's in the low half, the newest row at bit 15 of each half
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint32_t VM = vmax2(vmax2(R[i], R[i + 1]), R[i + 2]);
+      if (n < 32 && lane == n) VM = EV[i];
+      uint32_t VU = __shfl_up_sync(kFull, VM, 1), VD = __shfl_down_sync(kFull, VM, 1);
+      if (lane == 0) VU = EV[i];
+      if (lane == 31 && n == 32) VD = EV[i];
+      const uint32_t X = vmax2(vmax2(vmax2(R[i] + 0x00010001u, R[i + 2]), vmax2(VU + addU, VD + 0x10000u)), TT);
+      fl = (fl >> 1) | ((R[i + 1] - X + 0x80008000u) & 0x80008000u);
+    }
+    if (NR - k < 4) fl &= ((1u << (NR - k)) - 1u) * 0x10001000u;  // rows past the last one
+    if (lane < n) {
+      const uint32_t lo = (fl >> 12) & 15u, hi = fl >> 28;
+      if (lo) atomicOr(&pbits[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
+      if (hi) atomicOr(&pbits[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
     }
   }
 }
@@ -884,7 +872,7 @@ __device__ void scan_packed(const Plan& pl, const uint32_t* acc, const uint32_t*
         P = C;
         C = N;
       }
-      if (tested && bits) atomicOr(&pbits[c * pl.nrb + (ws >> 4)], bits);
+      if (tested && bits) atomicOr(&pbits[c * pl.nrb_p + (ws >> 4)], bits);
       ws = we;
     }
   }
@@ -920,7 +908,7 @@ __device__ void scan_scalar(const Plan& pl, const uint32_t* acc, const uint32_t*
       const int vmR = __shfl_down_sync(kFull, vm, 1);
       if (tested && vc >= pl.threshold && vc > vp && vc >= vn && (lstrict ? vc > vmL : vc >= vmL) &&
           (rstrict ? vc > vmR : vc >= vmR)) {
-        atomicOr(&pbits[c * pl.nrb + (k >> 5)], 1u << (k & 31));
+        atomicOr(&pbits[c * pl.nrb_p + (k >> 5)], 1u << (k & 31));
       }
       if (do_cs && tested && vc > 0) csum += (unsigned long long)vc * mix64(cell0 + k + 1);
       vp = vc;
@@ -1087,7 +1075,8 @@ __device__ int select_staged(const Plan& pl, const int2* hb, const uint16_t* idx
 }
 
 struct ItemShared {
-  int nv, flags, wide, last, total, D, reuse, n_amb;
+  EdgeWord edge[32];  // of at most 16 word groups
+  int nv, flags, wide, last, total, D, reuse, n_amb, n_low;
   int kept_tot;
   long long tstart[128];  // segment starts of the tile merge (2 segments a mirror-pair tile)
   int tmp[32];
@@ -1128,7 +1117,7 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
   if (from_bits) {
     for (int j = tid; j < NT; j += bd) {
       int cc = 0;
-      for (int w = 0; w < pl.nrb; ++w) cc += __popc(pbits[j * pl.nrb + w]);
+      for (int w = 0; w < pl.nrb; ++w) cc += __popc(pbits[j * pl.nrb_p + w]);
       colcnt[j] = cc;
     }
   } else {
@@ -1170,7 +1159,7 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
   if (from_bits) {
     for (int j = tid; j < NT; j += bd) {
       if (colcnt[j] == 0) continue;
-      const uint32_t* P = pbits + j * pl.nrb;
+      const uint32_t* P = pbits + j * pl.nrb_p;
       uint32_t* out = bm + colidx[j] * nrb;
       if (!staged) {
         for (int W = 0; W < nrb; ++W) out[W] = dilated_word(P, W, pl.nrb, NR, hw);
@@ -1281,7 +1270,7 @@ __device__ int tile_max_cs(const Plan& pl, const uint32_t* acc, int Wd, int aw, 
 // (tile-local columns as in the peak records: mirror-pair word w's low half is column w, its
 // high half column 2 Wd - 1 - w).
 __device__ void tile_candidate_bits(const Plan& pl, const uint32_t* acc, uint32_t* pbits, int Wd, int wt, int tq) {
-  const int NR = pl.n_rho, nrb = pl.nrb, lane = threadIdx.x & 31, warp = threadIdx.x >> 5,
+  const int NR = pl.n_rho, nrb = pl.nrb_p, lane = threadIdx.x & 31, warp = threadIdx.x >> 5,
             nwarps = blockDim.x >> 5;
   if (pl.mp) {
     for (int k = warp; k < NR; k += nwarps)
@@ -1668,7 +1657,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     for (int i = tid; i < nz; i += bd) z[i] = make_uint4(0u, 0u, 0u, 0u);
     if (T > 1)
       for (int i = tid; i < (pl.mp ? 2 * pl.rows_phys : nrp); i += bd) halo[i] = 0u;
-    for (int i = tid; i < wpad * pl.nrb; i += bd) pbits[i] = 0;
+    for (int i = tid; i < wpad * pl.nrb_p; i += bd) pbits[i] = 0;
     if (tid == 0) {
       sh.flags = 0;
       sh.it_max = 0;
@@ -1695,6 +1684,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
       if (sh.wide & 2) sh.flags |= HOUGH_F_BAD_HIT;
       if (sh.wide & 1) sh.reuse = 0;  // wide hits are not in the staged list
     }
+    if (pl.mp && want_halo && h0 == 0) edge_words(pl, aw, Wd, sh.edge);  // for the scan (no hits: no candidates)
     if (!(sh.wide & 1)) {
       if (mp_halo) halo_mp32(pl, HL, hb, sh.nv);
       if (pl.mp)
@@ -1796,9 +1786,10 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       tile_candidate_bits(pl, acc, pbits, Wd, wt, (int)max((long long)pl.threshold, need));
     } else if (pl.mp) {
       mp_fold(pl, acc, Wd, T > 1 ? halo : nullptr);
+      if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
       __syncthreads();
       HOUGH_PHASE(HOUGH_PHASE_FOLD);
-      scan_mp(pl, acc, halo, aw, Wd, pbits, do_cs, csum);
+      scan_mp(pl, smem, aw, Wd, sh.edge, pbits, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb, do_cs, csum);
     } else if (packed) {
       scan_packed(pl, acc, halo, pbits, wt, T, j0, do_cs, csum);
     } else {
@@ -1810,55 +1801,67 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // 4. raster-order positions and peak records: keys (column, group of key_words bitmap words)
     // in raster order, counted from the peak bitmap
     const int KG = pl.key_groups, G = pl.key_words, nkeys = wt * KG;
-    for (int key = tid; key < nkeys; key += bd) {
-      const int c = key >> pl.key_shift, w0 = (key & (KG - 1)) * G, w1 = min(pl.nrb, w0 + G);
+    const int nwarps = bd >> 5, kpw = ((nkeys + 32 * nwarps - 1) / (32 * nwarps)) * 32;  // keys a warp
+    const int key0 = warp * kpw, key1 = min(nkeys, key0 + kpw);
+    auto key_word = [&](int key) {  // one word a key
+      const int w = key & (KG - 1);
+      return w < pl.nrb ? pbits[(key >> pl.key_shift) * pl.nrb_p + w] : 0u;
+    };
+    int base = 0;  // records before this warp's keys
+    if (G == 1) {
+      // A warp counts and then writes one run of keys; its first position is the sum of the counts of
+      // the warps before it: one barrier, where a block scan of the keys and a second read took five
+      // and 3.3 k + 4.7 k cycles an event (batched).
       int np = 0;
-      for (int w = w0; w < w1; ++w) np += __popc(pbits[c * pl.nrb + w]);
-      cnt[key] = np;
+      for (int key = key0 + lane; key < key1; key += 32) np += __popc(key_word(key));
+      np = __reduce_add_sync(kFull, np);
+      if (lane == 0) sh.tmp[warp] = np;
+      __syncthreads();
+      const int x = lane < nwarps ? sh.tmp[lane] : 0;
+      base = __reduce_add_sync(kFull, lane < warp ? x : 0);
+      total = __reduce_add_sync(kFull, x);
+    } else {
+      for (int key = tid; key < nkeys; key += bd) {
+        const int c = key >> pl.key_shift, w0 = (key & (KG - 1)) * G, w1 = min(pl.nrb, w0 + G);
+        int np = 0;
+        for (int w = w0; w < w1; ++w) np += __popc(pbits[c * pl.nrb_p + w]);
+        cnt[key] = np;
+      }
+      __syncthreads();
+      total = block_exscan(cnt, nkeys, sh.tmp);
     }
-    __syncthreads();
-    total = block_exscan(cnt, nkeys, sh.tmp);
     HOUGH_PHASE(HOUGH_PHASE_EXSCAN);
     // peaks of the tile's low columns (mirror-pair tiles: the high columns follow them)
-    n_low = (pl.mp && Wd < wt) ? cnt[Wd << pl.key_shift] : total;
+    const int key_hi = Wd << pl.key_shift;  // first key of the high columns
+    n_low = (pl.mp && Wd < wt && G > 1) ? cnt[key_hi] : total;
     // event column of tile-local column c: mirror-pair tiles hold [aw, aw + Wd) then
     // [N - aw - Wd, N - aw), both ascending; other tiles [j0, j0 + wt)
     const int hi0 = NT - aw - 2 * Wd;
     hough_peak* dst = (T == 1) ? io.peaks + e * (long long)maxp : io.tile_peaks + (e * T + t) * (long long)maxp;
     uint2* dst2 = reinterpret_cast<uint2*>(dst);  // records are 8-byte aligned (checked on the host)
-    const int nwarps = bd >> 5;
     if (G == 1) {
-      // A warp takes 32 consecutive keys (one bitmap word each) and writes their peaks to
-      // consecutive positions: lane i of a pass finds the key owning position P0 + i (the last
-      // lane whose start is <= it) by a shuffle search and the bit by its rank in that word.
-      for (int kb = warp * 32; kb < nkeys; kb += nwarps * 32) {
+      // a lane takes a key: its word's peaks, one a step, to the positions after the lanes before it
+      for (int kb = key0; kb < key1; kb += 32) {
         const int key = kb + lane;
-        uint32_t word = 0;
-        int start = total;
-        if (key < nkeys) {
-          const int w = key & (KG - 1);
-          word = (w < pl.nrb) ? pbits[(key >> pl.key_shift) * pl.nrb + w] : 0u;
-          start = cnt[key];
+        uint32_t bits = key < key1 ? key_word(key) : 0u;
+        const int np = __popc(bits);
+        int pos = np;  // inclusive scan
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(kFull, pos, o);
+          if (lane >= o) pos += y;
         }
-        const int P0 = __shfl_sync(kFull, start, 0);
-        const int P1 = min(__shfl_sync(kFull, start + __popc(word), 31), maxp);
-        for (int o0 = P0; o0 < P1; o0 += 32) {
-          const int o = o0 + lane;
-          int l = 0;
-  #pragma unroll
-          for (int st = 16; st > 0; st >>= 1) {
-            const int sc = __shfl_sync(kFull, start, l + st);
-            if (sc <= o) l += st;
-          }
-          const int r = o - __shfl_sync(kFull, start, l);
-          const uint32_t wd = __shfl_sync(kFull, word, l);
-          if (o < P1) {
-            const int kl = kb + l, c = kl >> pl.key_shift;
-            const int k = ((kl & (KG - 1)) << 5) + (int)__fns(wd, 0u, r + 1);
-            const int votes = pl.mp ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
-            const int col = pl.mp ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
-            dst2[o] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes);
-          }
+        const int step = __shfl_sync(kFull, pos, 31);
+        pos += base - np;
+        base += step;
+        if (pl.mp && T > 1 && key == key_hi) sh.n_low = pos;
+        const int c = key >> pl.key_shift, k0 = (key & (KG - 1)) << 5;
+        const int col = pl.mp ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
+        while (bits && pos < maxp) {
+          const int k = k0 + __ffs(bits) - 1;
+          bits &= bits - 1u;
+          const int votes = pl.mp ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
+          dst2[pos++] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes);
         }
       }
     } else {
@@ -1866,7 +1869,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         const int c = key >> pl.key_shift, w0 = (key & (KG - 1)) * G, w1 = min(pl.nrb, w0 + G);
         int pos = cnt[key];
         for (int w = w0; w < w1 && pos < maxp; ++w) {
-          uint32_t bits = pbits[c * pl.nrb + w];
+          uint32_t bits = pbits[c * pl.nrb_p + w];
           while (bits && pos < maxp) {
             const int bb = __ffs(bits) - 1;
             bits &= bits - 1u;
@@ -1881,6 +1884,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     }
     cs_tile = do_cs ? block_sum_u64(csum, sh.red) : 0ull;
     __syncthreads();
+    if (G == 1 && pl.mp && Wd < wt && T > 1) n_low = sh.n_low;
     HOUGH_PHASE(HOUGH_PHASE_RECORDS);
   }
 

@@ -26,9 +26,12 @@ struct Plan {
   int threads;    // CTA size: groups * split * 32 (+ 32 halo lanes when tiles > 1)
   int nrho_pad;   // rows allocated per column
   int nrb;        // 32-bit bitmap words per column
-  int nrb_g;      // bitmap words per column with one guard bit on each side
+  int nrb_p;      // words a column takes in the peak bitmap: nrb made odd, so that neighbouring columns' words of
+                  // the same rows lie in different banks
+  int nrb_g;      // bitmap words per column with one guard bit on each side, odd (lanes that test different
+                  // columns at nearby rows would meet in one bank: 32 words a column at 1000 rows)
   int hit_cap;    // hits staged in shared memory per chunk
-  int scan_ranges;  // row ranges of the peak scan (a power of two)
+  int scan_ranges;  // row ranges of the peak scan (a power of two), column layout
   int scan_shift;   // log2(scan_ranges)
   int key_groups;   // peak-record keys per column (a power of two)
   int key_shift;    // log2(key_groups)
