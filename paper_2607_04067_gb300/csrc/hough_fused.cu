@@ -421,42 +421,50 @@ __device__ __forceinline__ void pair_fix(const Plan& pl, float4 h, int cj, int s
   }
 }
 
-// Shared list of (pair of hits, word) steps with an estimate in the ambiguous window.
+// Shared list of vote steps with an estimate in the ambiguous window.
 struct AmbList {
   uint32_t* e;  // first pair << 10 | first word
-  int* n;
+  int* n;       // counts on past cap
   int cap;
 };
 
-// The vote of a warp's share of the hit pairs (p, p + P, ...) into W words a lane: words w0, w0 + 32, ...
-// The loop runs straight through: every estimate votes at once, and a step of U pairs x W words with an
-// estimate in the ambiguous window (2e-4 of the votes at 256 rows) is listed for vote_fix, so that a
-// warp does not run the exact path's ~100 instructions for one lane. The loop is bound by issue: a vote's
-// estimate, floor, address, add and test take 5.5 slots (a packed f32x2 operation takes two), and by
-// the unit that takes the atomics (one warp a cycle) and the broadcast loads (an LDS.128 two cycles), which
-// is why a lane's two words share their loads. Alone, 2,022 hits at 256 x 256, 1,024 threads: 33.5 k cycles with
-// one word and a branch a pair; straight through 28.3 k with one word, 26.8 k with two, 27.6 k with four;
-// 19.4 k with no test, 16.2 k for the atomics alone. A test on the distance from the rounded estimate (two more
-// packed operations instead of the masks) took 30.4 k. In the kernel (batched events): 39.9 k -> 32.7 k
-// cycles; four words a lane spill there (33.0 k).
+// Constants of one lane's vote loop (offsets in bytes into the CTA's dynamic shared memory).
+template <int W>
+struct VoteArgs {
+  float A[W], B[W];   // its words' coefficients
+  uint32_t bs[W];     // shared address of its words' row "pattern 0"
+  float c0;
+  uint32_t am;
+  int p, P, np;       // pairs p, p + P, ... below np
+  int hits;           // staged pairs
+  uint32_t tag;       // first word
+  int list, n, cap;   // ambiguous steps, their count, room
+};
+
+// The vote of a lane's share of the hit pairs into its W words. The loop runs straight through: every
+// estimate votes at once, and a step of U pairs x W words with an estimate in the ambiguous window (2e-4
+// of the votes at 256 rows) is listed for vote_fix, so that a warp does not run the exact path's ~100
+// instructions for one lane. The loop is bound by issue: a vote's estimate, floor, address, add and test
+// take 5.5 slots (a packed f32x2 operation takes two), and by the unit that takes the atomics (one warp a
+// cycle) and the broadcast loads (an LDS.128 two cycles), which is why a lane's two words share their loads.
+// Alone, 2,022 hits at 256 x 256, 1,024 threads: 33.5 k cycles with one word and a branch a pair; straight through
+// 28.3 k with one word, 26.8 k with two, 27.6 k with four; 19.4 k with no test, 16.2 k for the atomics alone. A
+// test on the distance from the rounded estimate (two more packed operations instead of the masks) took
+// 30.4 k. A function of its own, with its arguments in registers: inlined, its registers and schedule
+// changed with unrelated code around it (33 k to 40 k cycles an event).
 template <int W, int U>
-__device__ __forceinline__ void vote_words(const Plan& pl, const int16_t* tc, const int16_t* ts, uint32_t acc_s,
-                                           int aw, int w0, bool on, int p, int P, const int2* hb, int nv,
-                                           const AmbList& L) {
-  if (!on) return;
+__device__ __noinline__ void vote_loop(const VoteArgs<W> v) {
+  extern __shared__ __align__(16) unsigned char smem[];
   float2 AA[W], BB[W];
-  uint32_t bs[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) {
-    const int j = aw + w0 + 32 * w;
-    const float A = __fmul_rn((float)tc[j], pl.fp_scale), B = __fmul_rn((float)ts[j], pl.fp_scale);
-    AA[w] = make_float2(A, A);
-    BB[w] = make_float2(B, B);
-    bs[w] = acc_s + (uint32_t)mp_word(w0 + 32 * w, 0, pl.rows_phys) * 4u - ((uint32_t)pl.mp_zoff << 7);
+    AA[w] = make_float2(v.A[w], v.A[w]);
+    BB[w] = make_float2(v.B[w], v.B[w]);
   }
-  const float2 CC = make_float2(pl.mp_c0, pl.mp_c0), MM = make_float2(kMagic, kMagic);
-  const uint32_t am = (uint32_t)pl.mp_amask;
-  const float4* hb4 = reinterpret_cast<const float4*>(hb);
+  const float2 CC = make_float2(v.c0, v.c0), MM = make_float2(kMagic, kMagic);
+  const uint32_t am = v.am;
+  const float4* hb4 = reinterpret_cast<const float4*>(smem + v.hits);
+  const int np = v.np, P = v.P;
   auto vote_pair = [&](float4 h) {
     const float2 uu = make_float2(h.x, h.y), nu = make_float2(-h.x, -h.y), vv = make_float2(h.z, h.w);
     bool ok = true;
@@ -465,87 +473,98 @@ __device__ __forceinline__ void vote_words(const Plan& pl, const int16_t* tc, co
       const float2 V = fma2(vv, BB[w], CC);
       const float2 k0 = fma2(uu, AA[w], V), k1 = fma2(nu, AA[w], V);
       const float2 z0 = add2_rm(k0, MM), z1 = add2_rm(k1, MM);
-      red_u32(bs[w] + (__float_as_uint(z0.x) << 7), 1u);
-      red_u32(bs[w] + (__float_as_uint(z1.x) << 7), 0x10000u);
-      red_u32(bs[w] + (__float_as_uint(z0.y) << 7), 1u);
-      red_u32(bs[w] + (__float_as_uint(z1.y) << 7), 0x10000u);
+      red_u32(v.bs[w] + (__float_as_uint(z0.x) << 7), 1u);
+      red_u32(v.bs[w] + (__float_as_uint(z1.x) << 7), 0x10000u);
+      red_u32(v.bs[w] + (__float_as_uint(z0.y) << 7), 1u);
+      red_u32(v.bs[w] + (__float_as_uint(z1.y) << 7), 0x10000u);
       ok = ok & ((__float_as_uint(k0.x) & am) != 0u) & ((__float_as_uint(k1.x) & am) != 0u) &
            ((__float_as_uint(k0.y) & am) != 0u) & ((__float_as_uint(k1.y) & am) != 0u);
     }
     return ok;
   };
-  auto list = [&](int q, int n) {
-    const int at = atomicAdd(L.n, 1);
-    if (at < L.cap) {
-      L.e[at] = ((uint32_t)q << 10) | (uint32_t)w0;
-    } else {  // no room: now
-      for (int i = 0; i < n; ++i)
-        for (int w = 0; w < W; ++w) {
-          const int x = w0 + 32 * w;
-          pair_fix(pl, hb4[q + i * P], tc[aw + x], ts[aw + x], acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u);
-        }
-    }
+  auto list = [&](int q) {
+    const int at = atomicAdd(reinterpret_cast<int*>(smem + v.n), 1);
+    if (at < v.cap) reinterpret_cast<uint32_t*>(smem + v.list)[at] = ((uint32_t)q << 10) | v.tag;
   };
-  const int np = nv >> 1;
-  int q = p;
+  int q = v.p;
 #pragma unroll 1
   for (; q + (U - 1) * P < np; q += U * P) {
     bool ok = true;
 #pragma unroll
     for (int i = 0; i < U; ++i) ok = vote_pair(hb4[q + i * P]) & ok;
-    if (!ok) list(q, U);
+    if (!ok) list(q);
   }
 #pragma unroll 1
-  for (; q < np; q += P) {
-    if (!vote_pair(hb4[q])) {
-      for (int w = 0; w < W; ++w) {
-        const int x = w0 + 32 * w;
-        pair_fix(pl, hb4[q], tc[aw + x], ts[aw + x], acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u);
-      }
-    }
-  }
-  if ((nv & 1) && p == np % P) {
-    const float2 h = staged_hit(reinterpret_cast<const float*>(hb), nv - 1);
-    for (int w = 0; w < W; ++w) {
-      const int x = w0 + 32 * w, cj = tc[aw + x], sj = ts[aw + x];
-      const uint32_t base = acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u, base2 = base - (uint32_t)pl.mp_k7;
-      const float v0 = __fmaf_rn(h.y, BB[w].x, pl.mp_c0);
-      red_u32(mp_addr(__fmaf_rn(h.x, AA[w].x, v0), pl, base, base2, h.x, h.y, cj, sj), 1u);
-      red_u32(mp_addr(__fmaf_rn(-h.x, AA[w].x, v0), pl, base, base2, h.x, h.y, -cj, sj), 0x10000u);
-    }
-  }
+  for (; q < np; q += P)
+    if (!vote_pair(hb4[q])) list(q);
 }
 
-// The listed steps' exact rows, a thread a (pair, word).
-template <int W, int U>
-__device__ __forceinline__ void vote_fix(const Plan& pl, const int16_t* tc, const int16_t* ts, uint32_t acc_s, int aw,
-                                         int P, const int2* hb, const AmbList& L) {
-  const int n = min(*L.n, L.cap) * (W * U);
-  const float4* hb4 = reinterpret_cast<const float4*>(hb);
-  for (int it = threadIdx.x; it < n; it += blockDim.x) {
-    const uint32_t e = L.e[it / (W * U)];
-    const int q = (int)(e >> 10) + (it % U) * P, x = (int)(e & 1023u) + 32 * (it / U % W);
-    pair_fix(pl, hb4[q], tc[aw + x], ts[aw + x], acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u);
-  }
+// The last hit of an odd count, a word a thread of the first warp of each word group.
+__device__ __forceinline__ void vote_last(const Plan& pl, const int16_t* tc, const int16_t* ts, uint32_t acc_s, int aw,
+                                          int x, float2 h) {
+  const int cj = tc[aw + x], sj = ts[aw + x];
+  const float A = __fmul_rn((float)cj, pl.fp_scale), v0 = __fmaf_rn(h.y, __fmul_rn((float)sj, pl.fp_scale), pl.mp_c0);
+  const uint32_t base = acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u, base2 = base - (uint32_t)pl.mp_k7;
+  red_u32(mp_addr(__fmaf_rn(h.x, A, v0), pl, base, base2, h.x, h.y, cj, sj), 1u);
+  red_u32(mp_addr(__fmaf_rn(-h.x, A, v0), pl, base, base2, h.x, h.y, -cj, sj), 0x10000u);
 }
 
 // All of a chunk's votes into a mirror-pair tile of Wd words (every thread calls it; the votes are
 // complete after the next barrier).
-__device__ __forceinline__ void vote_mp32(const Plan& pl, const int16_t* tc, const int16_t* ts, uint32_t acc_s, int aw,
-                                          int Wd, const int2* hb, int nv, const AmbList& L) {
+template <int W, int U>
+__device__ __forceinline__ void vote_words(const Plan& pl, unsigned char* smem, const int16_t* tc, const int16_t* ts,
+                                           uint32_t acc_s, int aw, int Wd, int nv, const AmbList& L) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = pl.groups >> 1, P2 = 2 * pl.split;
-  const bool worker = warp < G * P2;
-  auto go = [&](auto wc, auto uc) {
-    constexpr int W = decltype(wc)::value, U = decltype(uc)::value;
-    const int P = P2 * W, w0 = (warp / P) * (32 * W) + lane;
-    vote_words<W, U>(pl, tc, ts, acc_s, aw, w0, worker && w0 < Wd, warp % P, P, hb, nv, L);
-    __syncthreads();
-    vote_fix<W, U>(pl, tc, ts, acc_s, aw, P, hb, L);
-  };
-  using std::integral_constant;
-  // two words a lane only where every lane has both
-  if ((Wd & 63) == 0) go(integral_constant<int, 2>{}, integral_constant<int, 2>{});
-  else go(integral_constant<int, 1>{}, integral_constant<int, 4>{});
+  const int P = P2 * W, w0 = (warp / P) * (32 * W) + lane, np = nv >> 1;
+  const float4* hb4 = reinterpret_cast<const float4*>(smem + pl.off_hits);
+  if (warp < G * P2 && w0 < Wd) {
+    VoteArgs<W> v;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      const int x = w0 + 32 * w;
+      v.A[w] = __fmul_rn((float)tc[aw + x], pl.fp_scale);
+      v.B[w] = __fmul_rn((float)ts[aw + x], pl.fp_scale);
+      v.bs[w] = acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u - ((uint32_t)pl.mp_zoff << 7);
+    }
+    v.c0 = pl.mp_c0;
+    v.am = (uint32_t)pl.mp_amask;
+    v.p = warp % P;
+    v.P = P;
+    v.np = np;
+    v.hits = pl.off_hits;
+    v.tag = (uint32_t)w0;
+    v.list = (int)(reinterpret_cast<unsigned char*>(L.e) - smem);
+    v.n = (int)((uint32_t)__cvta_generic_to_shared(L.n) - (uint32_t)__cvta_generic_to_shared(smem));
+    v.cap = L.cap;
+    vote_loop<W, U>(v);
+    if ((nv & 1) && warp % P == np % P)
+      for (int w = 0; w < W; ++w)
+        vote_last(pl, tc, ts, acc_s, aw, w0 + 32 * w, staged_hit(reinterpret_cast<const float*>(hb4), nv - 1));
+  }
+  __syncthreads();
+  // the listed steps' exact rows, a thread a (pair, word); with more steps than the list holds, every one's
+  const int nl = *L.n;
+  if (nl <= L.cap) {
+    for (int it = threadIdx.x; it < nl * (W * U); it += blockDim.x) {
+      const uint32_t e = L.e[it / (W * U)];
+      const int q = (int)(e >> 10) + (it % U) * P, x = (int)(e & 1023u) + 32 * (it / U % W);
+      // a single step at the end of a lane's share stands for one pair
+      if (it % U == 0 || (int)(e >> 10) + (U - 1) * P < np)
+        pair_fix(pl, hb4[q], tc[aw + x], ts[aw + x], acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u);
+    }
+  } else {
+    for (long long it = threadIdx.x; it < (long long)np * Wd; it += blockDim.x) {
+      const int q = (int)(it / Wd), x = (int)(it - (long long)q * Wd);
+      pair_fix(pl, hb4[q], tc[aw + x], ts[aw + x], acc_s + (uint32_t)mp_word(x, 0, pl.rows_phys) * 4u);
+    }
+  }
+}
+
+// Two words a lane only where every lane has both.
+__device__ __forceinline__ void vote_mp32(const Plan& pl, unsigned char* smem, const int16_t* tc, const int16_t* ts,
+                                          uint32_t acc_s, int aw, int Wd, int nv, const AmbList& L) {
+  if ((Wd & 63) == 0) vote_words<2, 2>(pl, smem, tc, ts, acc_s, aw, Wd, nv, L);
+  else vote_words<1, 4>(pl, smem, tc, ts, acc_s, aw, Wd, nv, L);
 }
 
 // Halo words of a mirror-pair tile: the words before and after its own (none at the theta wrap or at the
@@ -1074,7 +1093,25 @@ __device__ int select_staged(const Plan& pl, const int2* hb, const uint16_t* idx
   return kept;
 }
 
+// A work item: tile item % T of event `event`, whose hits are [off[0], off[1]). Two of them in shared
+// memory, the current one and the next: in a persistent launch the next is popped before the current one's
+// vote, and its event's index and offsets are read by asynchronous copies issued between the phases, so that
+// no barrier waits for their latency (3.5 k cycles an event in a chain after the last item).
+struct WorkItem {
+  long long off[2];
+  int item;  // >= n_items: none
+  int event;
+};
+
+__device__ __forceinline__ void copy_async(void* smem, const void* gmem, int bytes) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+  if (bytes == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(gmem) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(a), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 struct ItemShared {
+  WorkItem it[2];
   EdgeWord edge[32];  // of at most 16 word groups
   int nv, flags, wide, last, total, D, reuse, n_amb, n_low;
   int kept_tot;
@@ -1581,6 +1618,7 @@ __device__ int merge_iterative(const Plan& pl, const FusedIO& io, unsigned char*
 
 // Steps 1-2 of a work item: clears the CTA's accumulator of theta tile t (with the halo columns,
 // the peak bitmap and the flags) and votes the event's hits [a, a + n) into it, chunk by chunk.
+template <bool MP, bool ITER>
 __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, long long a, int n,
                           int t) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
@@ -1598,7 +1636,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
   const int rows_w = nrp >> 1;  // words per column
   // mirror-pair tiles: words [aw, aw + Wd), i.e. columns [aw, aw + Wd) and their mirrors
   // (full tiles own tile_w / 2 words, the last one possibly fewer)
-  const int Wd = pl.mp ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
+  const int Wd = MP ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
 
   // lane roles of the vote
   VoteLane L;
@@ -1607,8 +1645,8 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
   L.cj = L.sj = 0;
   L.col1 = L.col2 = 0;
   const uint32_t acc_s = (uint32_t)__cvta_generic_to_shared(acc);
-  const bool want_halo = pl.peak_mode != HOUGH_PEAK_ITERATIVE;  // only the 3x3 test reads the halo
-  if (L.halo && pl.mp) {
+  const bool want_halo = !ITER;  // only the 3x3 test reads the halo
+  if (L.halo && MP) {
     L.p = 0;  // no words of its own (every thread votes halo hits)
     L.P = 1;
   } else if (L.halo) {
@@ -1619,7 +1657,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     L.col2 = (uint32_t)__cvta_generic_to_shared(halo) + (uint32_t)((lane >> 4) * (nrp >> 1)) * 4u;
     L.p = 0;
     L.P = 1;
-  } else if (pl.mp) {
+  } else if (MP) {
     const int P2 = 2 * pl.split, gpair = warp / P2;
     L.p = warp % P2;
     L.P = P2;
@@ -1643,7 +1681,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     L.col1 = acc_s + (uint32_t)(((g * rows_w) << 5) + lane) * 4u;
   }
 
-  const bool mp_halo = pl.mp && T > 1 && want_halo;
+  const bool mp_halo = MP && T > 1 && want_halo;
   HaloLane HL{false, 0, 0, 0u};
   if (mp_halo) HL = halo_lane(pl, tc, ts, halo, aw, Wd);
   const AmbList amb{reinterpret_cast<uint32_t*>(smem + pl.off_amb), &sh.n_amb, pl.amb_cap};
@@ -1656,7 +1694,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     const int nz = pl.region_bytes >> 4;
     for (int i = tid; i < nz; i += bd) z[i] = make_uint4(0u, 0u, 0u, 0u);
     if (T > 1)
-      for (int i = tid; i < (pl.mp ? 2 * pl.rows_phys : nrp); i += bd) halo[i] = 0u;
+      for (int i = tid; i < (MP ? 2 * pl.rows_phys : nrp); i += bd) halo[i] = 0u;
     for (int i = tid; i < wpad * pl.nrb_p; i += bd) pbits[i] = 0;
     if (tid == 0) {
       sh.flags = 0;
@@ -1665,7 +1703,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
   }
 
   // 2. map + vote, chunk by chunk
-  if (tid == 0) sh.reuse = (pl.mp && n > 0 && n <= pl.hit_cap) ? 1 : 0;
+  if (tid == 0) sh.reuse = (MP && n > 0 && n <= pl.hit_cap) ? 1 : 0;
   for (int h0 = 0; h0 < n; h0 += pl.hit_cap) {
     const int cn = min(pl.hit_cap, n - h0);
     __syncthreads();
@@ -1676,19 +1714,19 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
       sh.n_amb = 0;
     }
     __syncthreads();
-    stage_vote32(io.xy, a + h0, cn, hb, &sh.nv, &sh.wide, pl.mp ? pl.mp_lsq : 0,
-                 pl.mp ? reinterpret_cast<uint16_t*>(smem + pl.off_idx) : nullptr);
+    stage_vote32(io.xy, a + h0, cn, hb, &sh.nv, &sh.wide, MP ? pl.mp_lsq : 0,
+                 MP ? reinterpret_cast<uint16_t*>(smem + pl.off_idx) : nullptr);
     __syncthreads();
     HOUGH_PHASE(HOUGH_PHASE_STAGE);
     if (tid == 0) {
       if (sh.wide & 2) sh.flags |= HOUGH_F_BAD_HIT;
       if (sh.wide & 1) sh.reuse = 0;  // wide hits are not in the staged list
     }
-    if (pl.mp && want_halo && h0 == 0) edge_words(pl, aw, Wd, sh.edge);  // for the scan (no hits: no candidates)
+    if (MP && want_halo && h0 == 0) edge_words(pl, aw, Wd, sh.edge);  // for the scan (no hits: no candidates)
     if (!(sh.wide & 1)) {
       if (mp_halo) halo_mp32(pl, HL, hb, sh.nv);
-      if (pl.mp)
-        vote_mp32(pl, tc, ts, acc_s, aw, Wd, hb, sh.nv, amb);
+      if (MP)
+        vote_mp32(pl, smem, tc, ts, acc_s, aw, Wd, sh.nv, amb);
       else
         vote32_fp(pl, L, hb, sh.nv);
     } else {
@@ -1701,7 +1739,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
         stage_vote64(io.xy, a + h0 + s0, sn, hw, &sh.nv);
         __syncthreads();
         if (mp_halo) halo_mp64(pl, HL, hw, sh.nv);
-        if (pl.mp)
+        if (MP)
           vote_mp64(pl, L, hw, sh.nv);
         else
           vote64(pl, L, hw, sh.nv);
@@ -1713,7 +1751,15 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
 
 }
 
-__device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, long long item,
+// Takes n items from the queue; the first one's index (at most INT_MAX, which is past the last item).
+__device__ __forceinline__ int pop_items(const FusedIO& io, int n) {
+  return (int)min(atomicAdd(io.queue, (unsigned long long)n), (unsigned long long)INT_MAX);
+}
+
+// The work item sh.it[cur]. more: the index of the item after it if that is known already (popped
+// together, or none), else -1 (popped here); sh.it[cur ^ 1] receives it.
+template <bool MP, bool ITER>
+__device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, int cur, int more,
                          bool do_cs) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
   uint32_t* halo = reinterpret_cast<uint32_t*>(smem + pl.off_halo);
@@ -1723,28 +1769,55 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   const int16_t* ts = tc + pl.n_theta;
 
   const int T = pl.tiles, NT = pl.n_theta, NR = pl.n_rho, nrp = pl.nrho_pad;
-  const long long e = io.order ? (long long)io.order[item / T] : item / T;
-  const int t = (int)(item % T);
-  const long long a = io.off[e];
-  const long long nll = io.off[e + 1] - a;
-  const bool too_large = nll > HOUGH_MAX_EVENT_HITS;
-  const int n = too_large ? 0 : (int)nll;
+  const long long e = sh.it[cur].event;
+  const int t = sh.it[cur].item % T;
   const int j0 = t * pl.tile_w;
   const int wt = min(pl.tile_w, NT - j0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
-  const int Wd = pl.mp ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
+  const int Wd = MP ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
 
-  vote_tile(pl, io, smem, sh, a, n, t);
+  // the next item, in steps whose latencies pass behind the phases between them (thread 0)
+  WorkItem& next = sh.it[cur ^ 1];
+  const bool fetch = io.persistent && tid == 0;
+  if (fetch && more < 0) more = pop_items(io, pl.grab);
+  bool other = false;  // the next item exists and belongs to another event
+  auto fetch_event = [&]() {
+    if (!fetch) return;
+    next.item = more;
+    other = more < io.n_items;
+    if (other && more - sh.it[cur].item + t < T) {  // items are popped in ascending order
+      other = false;
+      next.event = sh.it[cur].event;
+      next.off[0] = sh.it[cur].off[0];
+      next.off[1] = sh.it[cur].off[1];
+    }
+    if (other) copy_async(&next.event, io.order + (T == 1 ? more : more / T), 4);
+  };
+  auto fetch_offsets = [&]() {
+    if (!fetch || !other) return;
+    copy_async_wait();
+    copy_async(&next.off[0], io.off + next.event, 8);
+    copy_async(&next.off[1], io.off + next.event + 1, 8);
+  };
+  auto fetch_done = [&]() {
+    if (fetch && other) copy_async_wait();
+  };
+
+  {
+    const long long a = sh.it[cur].off[0], nll = sh.it[cur].off[1] - a;
+    vote_tile<MP, ITER>(pl, io, smem, sh, a, nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll, t);
+  }
+  fetch_event();
 
   // 3-4. peaks
   const int maxp = pl.max_peaks;
   int total = 0, n_low = 0;
   unsigned long long cs_tile = 0;
   int tmax = 0;
-  if (pl.peak_mode == HOUGH_PEAK_ITERATIVE && T == 1) {
+  if (ITER && T == 1) {
     // the paper's iterative finder on a whole accumulator: the checksum first, then the
     // extraction, which clears the cells it suppresses; records in extraction order
-    if (pl.mp) {
+    if (MP) {
       mp_fold(pl, acc, Wd, nullptr);
       __syncthreads();
       HOUGH_PHASE(HOUGH_PHASE_FOLD);
@@ -1760,13 +1833,13 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       }
       __syncthreads();
       HOUGH_PHASE(HOUGH_PHASE_SCAN);
-      HOUGH_PHASE(HOUGH_PHASE_SCAN);
+      fetch_offsets();
       const int st_words = (((NT * NR + 15) >> 4) + 31) & ~31;  // 2 bits a cell, whole 32-word blocks
       return extract_iterative(cells, NT, NR, kIterSliceRows, pl.threshold, pl.rel_num, pl.rel_den, pl.nms_radius,
                                maxp, pbits, pl.iter_cap, nullptr, st_words, io.peaks + e * (long long)maxp, sh.tmp,
                                reinterpret_cast<uint16_t*>(pbits + pl.iter_cap + st_words), pl.iter_act);
     };
-    total = pl.mp ? iterative(FusedCells<true>{acc, Wd, nrp, pl.rows_phys})
+    total = MP ? iterative(FusedCells<true>{acc, Wd, nrp, pl.rows_phys})
                   : iterative(FusedCells<false>{acc, Wd, nrp, pl.rows_phys});
     n_low = total;
   } else {
@@ -1774,9 +1847,9 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // at or above the tile's own relative threshold, a superset of the cells the event's
     // threshold admits (the event's maximum is at least the tile's)
     unsigned long long csum = 0;
-    const bool packed = !pl.mp && (NR & 1) == 0;
-    if (pl.peak_mode == HOUGH_PEAK_ITERATIVE) {
-      if (pl.mp) {
+    const bool packed = !MP && (NR & 1) == 0;
+    if (ITER) {
+      if (MP) {
         mp_fold(pl, acc, Wd, nullptr);
         __syncthreads();
         HOUGH_PHASE(HOUGH_PHASE_FOLD);
@@ -1784,7 +1857,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       tmax = tile_max_cs(pl, acc, Wd, aw, wt, j0, do_cs, &sh.it_max, csum);
       const long long need = ((long long)pl.rel_num * tmax + pl.rel_den - 1) / pl.rel_den;
       tile_candidate_bits(pl, acc, pbits, Wd, wt, (int)max((long long)pl.threshold, need));
-    } else if (pl.mp) {
+    } else if (MP) {
       mp_fold(pl, acc, Wd, T > 1 ? halo : nullptr);
       if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
       __syncthreads();
@@ -1797,6 +1870,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     }
     __syncthreads();
     HOUGH_PHASE(HOUGH_PHASE_SCAN);
+    fetch_offsets();
 
     // 4. raster-order positions and peak records: keys (column, group of key_words bitmap words)
     // in raster order, counted from the peak bitmap
@@ -1833,7 +1907,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     HOUGH_PHASE(HOUGH_PHASE_EXSCAN);
     // peaks of the tile's low columns (mirror-pair tiles: the high columns follow them)
     const int key_hi = Wd << pl.key_shift;  // first key of the high columns
-    n_low = (pl.mp && Wd < wt && G > 1) ? cnt[key_hi] : total;
+    n_low = (MP && Wd < wt && G > 1) ? cnt[key_hi] : total;
     // event column of tile-local column c: mirror-pair tiles hold [aw, aw + Wd) then
     // [N - aw - Wd, N - aw), both ascending; other tiles [j0, j0 + wt)
     const int hi0 = NT - aw - 2 * Wd;
@@ -1854,13 +1928,13 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         const int step = __shfl_sync(kFull, pos, 31);
         pos += base - np;
         base += step;
-        if (pl.mp && T > 1 && key == key_hi) sh.n_low = pos;
+        if (MP && T > 1 && key == key_hi) sh.n_low = pos;
         const int c = key >> pl.key_shift, k0 = (key & (KG - 1)) << 5;
-        const int col = pl.mp ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
+        const int col = MP ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
         while (bits && pos < maxp) {
           const int k = k0 + __ffs(bits) - 1;
           bits &= bits - 1u;
-          const int votes = pl.mp ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
+          const int votes = MP ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
           dst2[pos++] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes);
         }
       }
@@ -1874,8 +1948,8 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
             const int bb = __ffs(bits) - 1;
             bits &= bits - 1u;
             const int k = (w << 5) + bb;
-            const int votes = pl.mp ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
-            const int col = pl.mp ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
+            const int votes = MP ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
+            const int col = MP ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
             dst2[pos] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes);
             ++pos;
           }
@@ -1884,9 +1958,11 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     }
     cs_tile = do_cs ? block_sum_u64(csum, sh.red) : 0ull;
     __syncthreads();
-    if (G == 1 && pl.mp && Wd < wt && T > 1) n_low = sh.n_low;
+    if (G == 1 && MP && Wd < wt && T > 1) n_low = sh.n_low;
     HOUGH_PHASE(HOUGH_PHASE_RECORDS);
   }
+
+  fetch_done();
 
   // 5. tiles: publish, and let the last tile of the event merge
   int ev_total = total;
@@ -1910,8 +1986,8 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // Raster order of the event: the tiles' low segments in tile order, then (mirror-pair
     // tiles) their high segments in reverse tile order. Segment s < T is tile s's records
     // [0, lo); segment T + i is tile T-1-i's records [lo, all).
-    const int nseg = pl.mp ? 2 * T : T;
-    if (pl.peak_mode == HOUGH_PEAK_ITERATIVE) {
+    const int nseg = MP ? 2 * T : T;
+    if (ITER) {
       ev_total = merge_iterative(pl, io, smem, sh, e);
       if (tid == 0) {
         unsigned long long csa = 0;
@@ -1964,6 +2040,9 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
 
   // 6. event outputs and selection (single tile, or the last tile)
+  const long long a = sh.it[cur].off[0], nll = sh.it[cur].off[1] - a;
+  const bool too_large = nll > HOUGH_MAX_EVENT_HITS;
+  const int n = too_large ? 0 : (int)nll;
   if (tid == 0) {
     io.npeaks[e] = ev_total;
     if (io.checksum) io.checksum[e] = ev_cs;
@@ -1972,12 +2051,16 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_MERGE);
+  if (io.persistent && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
+    const long long i = next.off[0] + 16LL * tid;
+    if (i < next.off[1]) asm volatile("prefetch.global.L2 [%0];" ::"l"(io.xy + i));
+  }
   int kept = 0;
   if (too_large) {
     for (long long i = tid; i < nll; i += bd) io.mask[a + i] = 0;
   } else {
     kept = select_event(pl, io, smem, sh, tc, ts, a, n, io.peaks + e * (long long)maxp, min(ev_total, maxp),
-                        pl.peak_mode == HOUGH_PEAK_LOCAL_MAX && T == 1 && ev_total <= maxp && pl.keep_hw < 32);
+                        !ITER && T == 1 && ev_total <= maxp && pl.keep_hw < 32);
   }
   if (tid == 0) sh.kept_tot = 0;
   __syncthreads();
@@ -1992,10 +2075,11 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
 }
 
+// One instance a layout (MP: mirror pairs) and peak finder, so that none carries the others' registers.
+template <bool MP, bool ITER>
 __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ItemShared sh;
-  __shared__ long long s_item;
   if (io.status[1] != 0) return;  // offsets of this call failed validation
   int16_t* tc = reinterpret_cast<int16_t*>(smem + pl.off_trig);
   for (int j = threadIdx.x; j < pl.n_theta; j += blockDim.x) {
@@ -2004,18 +2088,25 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
   }
   __syncthreads();  // the table is read before run_item's first barrier
   const bool do_cs = io.checksum != nullptr;
-  if (!io.persistent) {
-    run_item(pl, io, smem, sh, blockIdx.x, do_cs);
-    return;
+  const bool queue = io.persistent && io.n_items > gridDim.x;  // else an item a CTA, and none after it
+  if (threadIdx.x == 0) {
+    const int it = queue ? pop_items(io, pl.grab) : (int)blockIdx.x;
+    sh.it[0].item = it;
+    if (it < io.n_items) {
+      const int e = io.order ? io.order[it / pl.tiles] : it / pl.tiles;
+      sh.it[0].event = e;
+      sh.it[0].off[0] = io.off[e];
+      sh.it[0].off[1] = io.off[e + 1];
+    }
   }
-  for (;;) {
+  int left = 0;  // items popped together with the current one and still to come
+  for (int cur = 0;; cur ^= 1) {
     __syncthreads();
-    if (threadIdx.x == 0) s_item = (long long)atomicAdd(io.queue, (unsigned long long)pl.grab);
-    __syncthreads();
-    const long long base = s_item;
-    if (base >= io.n_items) break;
-    const long long end = min(base + pl.grab, io.n_items);
-    for (long long it = base; it < end; ++it) run_item(pl, io, smem, sh, it, do_cs);
+    const int it = sh.it[cur].item;
+    if (it >= io.n_items) break;
+    left = left > 0 ? left - 1 : pl.grab - 1;
+    run_item<MP, ITER>(pl, io, smem, sh, cur, !queue ? INT_MAX : left > 0 ? it + 1 : -1, do_cs);
+    if (!io.persistent) break;
   }
 }
 
@@ -2042,6 +2133,7 @@ struct SpillCells {
 // memory exactly as the fused kernel does and stores the cells to its slot, runs the iterative
 // finder there (the stepwise form, any size) and selects the hits. Count and list were written
 // by the fused kernel before this launch on the same stream.
+template <bool MP>
 __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ItemShared sh;
@@ -2063,10 +2155,10 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
     const int n = nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll;  // a too-large event is never deferred
     int flags = 0;
     for (int t = 0; t < T; ++t) {
-      vote_tile(pl, io, smem, sh, a, n, t);
-      const int j0 = t * pl.tile_w, wt = min(pl.tile_w, NT - j0), Wd = pl.mp ? (wt >> 1) : 0,
+      vote_tile<MP, true>(pl, io, smem, sh, a, n, t);
+      const int j0 = t * pl.tile_w, wt = min(pl.tile_w, NT - j0), Wd = MP ? (wt >> 1) : 0,
                 aw = t * (pl.tile_w >> 1);
-      if (pl.mp) {
+      if (MP) {
         mp_fold(pl, const_cast<uint32_t*>(acc), Wd, nullptr);
         __syncthreads();
         for (int i = tid; i < Wd * NR; i += bd) {
@@ -2239,8 +2331,17 @@ static cudaError_t set_smem(const void* fn, int bytes) {
   return e;
 }
 
+namespace {
+using FusedKernel = void (*)(const Plan, const FusedIO, const TrigTable);
+FusedKernel fused_of(const Plan& pl) {
+  const bool it = pl.peak_mode == HOUGH_PEAK_ITERATIVE;
+  return pl.mp ? (it ? fused_kernel<true, true> : fused_kernel<true, false>)
+               : (it ? fused_kernel<false, true> : fused_kernel<false, false>);
+}
+}  // namespace
+
 int fused_max_ctas_per_sm(const Plan& pl) {
-  const void* fn = (const void*)fused_kernel;
+  const void* fn = (const void*)fused_of(pl);
   if (set_smem(fn, pl.smem_bytes) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, pl.threads, pl.smem_bytes) != cudaSuccess) return 0;
@@ -2249,11 +2350,12 @@ int fused_max_ctas_per_sm(const Plan& pl) {
 
 cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st) {
   const bool deferred = pl.peak_mode == HOUGH_PEAK_ITERATIVE && pl.tiles > 1;
-  cudaError_t err = set_smem((const void*)fused_kernel, pl.smem_bytes);
-  if (err == cudaSuccess && deferred) err = set_smem((const void*)deferred_kernel, pl.smem_bytes);
+  const FusedKernel fused = fused_of(pl), def = pl.mp ? deferred_kernel<true> : deferred_kernel<false>;
+  cudaError_t err = set_smem((const void*)fused, pl.smem_bytes);
+  if (err == cudaSuccess && deferred) err = set_smem((const void*)def, pl.smem_bytes);
   if (err != cudaSuccess) return err;
-  fused_kernel<<<grid, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
-  if (deferred) deferred_kernel<<<io.n_spill, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
+  fused<<<grid, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
+  if (deferred) def<<<io.n_spill, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
   return cudaGetLastError();
 }
 
