@@ -98,7 +98,12 @@ static bool layout(Plan& pl) {
   // mirror-pair: groups / 2 word groups of 32 lanes (the last may be part idle) x rows_phys
   const int acc_bytes = pl.mp ? (pl.groups / 2) * 32 * pl.rows_phys * 4 : wpad * pl.nrho_pad * 2;
   const int sel_bytes = (2 * pl.n_theta + 64) * 4 + pl.n_theta * 16 + pl.n_theta * pl.nrb_g * 4;
-  int o = 1024;  // the scan of a wrapped word may read up to seven rows (of 128 bytes) below row 0
+  int o = 0;
+  pl.off_trig = o;
+  o += round16(2 * pl.n_theta * 2);
+  pl.off_unres = o;
+  o += round16((pl.hit_cap + 1024) / 32 * 4);
+  if (pl.mp) o = std::max(o, 384);  // the scan of a wrapped word may read up to three rows (of 128 bytes) below row 0
   pl.off_acc = o;
   pl.region_bytes = round16(acc_bytes > sel_bytes ? acc_bytes : sel_bytes);
   o += pl.region_bytes;
@@ -113,10 +118,12 @@ static bool layout(Plan& pl) {
   {
     int iter_words = 0;
     if (it_whole) {
-      // candidate keys, then 2 state bits a cell (also room for the walk's 1-bit bitmap), then
-      // two lists of undecided candidates (16-bit indices)
-      const int cand_words = pl.iter_cap + (((pl.n_theta * pl.n_rho + 15) / 16 + 31) & ~31) + pl.iter_act;
       iter_words = iter_scratch_words(pl.n_theta, pl.n_rho, kIterSliceRows);
+      // Mirror pairs: the candidates' and the local maxima's bitmaps, then three lists (undecided
+      // candidates, the cells that block them, those to look at again). Columns: candidate keys, 2 state bits a cell (also room for
+      // the walk's 1-bit bitmap), two lists of undecided candidates (16-bit indices).
+      const int cand_words = pl.mp ? 2 * wpad * pl.nrb_p + 2 * pl.iter_cap + pl.iter_cap / 2
+                                   : pl.iter_cap + (((pl.n_theta * pl.n_rho + 15) / 16 + 31) & ~31) + pl.iter_act;
       if (pl.iter_cap > 0 && cand_words > iter_words) iter_words = cand_words;
     }
     o += round16((wpad * pl.nrb_p > iter_words ? wpad * pl.nrb_p : iter_words) * 4);
@@ -124,21 +131,17 @@ static bool layout(Plan& pl) {
   pl.off_cnt = o;  // record keys of the local-maximum scan or of a tile's candidates
   if (!it_whole) o += round16(wpad * pl.key_groups * 4);
   // the vote's list lies in a region that is first written after the vote
-  pl.off_amb = it_whole ? pl.off_pbits : pl.off_cnt;
+  pl.off_amb = !it_whole ? pl.off_cnt : pl.off_pbits + (pl.mp && pl.iter_cap > 0 ? 8 * wpad * pl.nrb_p : 0);
   pl.amb_cap = std::min(1024, (o - pl.off_amb) / 4);
-  pl.off_unres = o;
-  o += round16((pl.hit_cap + 1024) / 32 * 4);
-  pl.off_trig = o;
-  o += round16(2 * pl.n_theta * 2);
   pl.smem_bytes = o;
   if (o > kSmemBudget) return false;
   if (pl.peak_mode == HOUGH_PEAK_ITERATIVE && pl.tiles > 1) {
     // the merging CTA's candidates (a key and a state byte each, after the column starts) in
-    // [off_acc, off_unres); the deferred kernel's finder (scratch, then a bitmap of every cell)
-    // below the trig table
-    const int free_bytes = pl.off_unres - pl.off_acc - 4 * ((pl.n_theta + 4) & ~3);
+    // [off_acc, smem_bytes); the deferred kernel's finder (scratch, then a bitmap of every cell)
+    // after the trig table
+    const int free_bytes = pl.smem_bytes - pl.off_acc - 4 * ((pl.n_theta + 4) & ~3);
     pl.merge_cap = std::min(65520, free_bytes / 5) & ~15;  // key and state a candidate (16-bit indices)
-    const int avail = pl.off_trig / 4, gone = (pl.n_theta * pl.n_rho + 31) / 32;
+    const int avail = (pl.smem_bytes - pl.off_unres) / 4, gone = (pl.n_theta * pl.n_rho + 31) / 32;
     int sh = kIterSliceRows;
     while (sh < pl.n_rho && iter_scratch_words(pl.n_theta, pl.n_rho, sh) + gone > avail) sh *= 2;
     const int sw = iter_scratch_words(pl.n_theta, pl.n_rho, sh);
@@ -209,7 +212,6 @@ int make_plan(const hough_params* p, Plan& pl) {
   pl.rel_den = p->rel_den;
   pl.nms_radius = p->nms_radius;
   pl.nrb = (p->n_rho + 31) / 32;
-  pl.nrb_p = pl.nrb | 1;
   pl.nrb_g = ((p->n_rho + 2 + 31) / 32) | 1;
   pl.magic = host_magic(p->n_rho);
   pl.grab = p->events_per_cta > 0 ? p->events_per_cta : 1;
@@ -306,16 +308,22 @@ int make_plan(const hough_params* p, Plan& pl) {
       pl.key_shift = ks;
       pl.key_words = gw;
     }
-    // the most staged hits, then (iterative finder) the most candidate keys of its candidate form
-    for (int cap = 4096; cap >= 512; cap >>= 1) {
-      pl.hit_cap = cap;
-      const int icap0 = pl.peak_mode == HOUGH_PEAK_ITERATIVE && T == 1 ? 8192 : 0;
-      for (int icap = icap0; icap >= 0; icap = icap > 1024 ? icap / 2 : icap - 1024) {
-        pl.iter_cap = icap;
-        for (int act = icap > 0 ? 2048 : 0; act >= 0;
-             act = act > 1024 ? act - 512 : act > 256 ? act / 2 : act - 256) {  // 2048, 1536, 1024, 512, 256, 0
-          pl.iter_act = act;
-          if (layout(pl)) return HOUGH_OK;
+    // the most staged hits, then (iterative finder on a whole accumulator) the longest lists: mirror pairs,
+    // 4,096 to 256 undecided candidates; columns, 8,192 to 1,024 candidate keys and 2,048 to 256 undecided
+    // ones. No lists (one pass a peak) only where no number of staged hits leaves room for any.
+    const bool whole = pl.peak_mode == HOUGH_PEAK_ITERATIVE && T == 1;
+    for (int lists = whole ? 1 : 0; lists >= 0; --lists) {
+      for (int cap = 4096; cap >= 512; cap >>= 1) {
+        pl.hit_cap = cap;
+        for (int icap = !lists ? 0 : pl.mp ? 4096 : 8192; icap >= (!lists ? 0 : pl.mp ? 256 : 1024);
+             icap = pl.mp && icap > 1024 ? icap - 512 : icap > 0 ? icap / 2 : -1) {
+          pl.iter_cap = icap;
+          for (int act = icap > 0 && !pl.mp ? 2048 : 0; act >= 0;
+               act = act > 1024 ? act - 512 : act > 256 ? act / 2 : act - 256) {  // 2048, 1536, 1024, 512, 256, 0
+            pl.iter_act = act;
+            for (pl.nrb_p = pl.nrb | 1; pl.nrb_p >= pl.nrb; --pl.nrb_p)  // odd where there is room
+              if (layout(pl)) return HOUGH_OK;
+          }
         }
       }
     }

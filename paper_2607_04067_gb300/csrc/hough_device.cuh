@@ -874,6 +874,256 @@ __device__ int resolve_rounds(Cells& cells, int NT, int NR, int R, int tq, int m
   return nk;
 }
 
+// The cells (j << 16 | k) of a bitmap (word(i) of word i = j stride + (k >> 5)) appended to list, of which *n
+// counts all, past its room too. A warp takes word w of 32 consecutive columns, whose counts are alike
+// (candidates crowd in the central rows of every column), and the warps of all column groups take one w after
+// the other. All threads call it.
+template <class Word>
+__device__ __forceinline__ void list_cells(int NT, int NR, int stride, Word&& word, uint32_t* list, int room, int* n) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int NG = (NT + 31) >> 5, NRW = (NR + 31) >> 5, dq = nwarps / NG, dr = nwarps - dq * NG;
+  int w = warp / NG, g = warp - w * NG;
+#pragma unroll 1
+  for (; w < NRW; w += dq, g += dr) {
+    if (g >= NG) {
+      g -= NG;
+      if (++w >= NRW) break;
+    }
+    const int j = 32 * g + lane;
+    uint32_t bits = j < NT ? word(j * stride + w) : 0u;
+    if (!__any_sync(0xffffffffu, bits != 0u)) continue;
+    const int c = __popc(bits);
+    int at = c;  // inclusive scan over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += y;
+    }
+    int base = 0;
+    if (lane == 31) base = atomicAdd(n, at);
+    at += __shfl_sync(0xffffffffu, base, 31) - c;
+#pragma unroll 1
+    while (bits) {
+      const int b = 31 - __clz(bits);
+      bits ^= 1u << b;
+      if (at < room) list[at] = ((uint32_t)j << 16) | (uint32_t)(32 * w + b);
+      ++at;
+    }
+  }
+}
+
+// The kept set of the iterative finder (Sec. 2: the best unsuppressed cell is the next peak and suppresses
+// its window) from its candidates. A candidate is kept iff every higher-ranked candidate of its window is
+// dropped, and dropped by a kept cell whose window covers it. Cells are only ever dropped, and only by kept
+// ones, so the order in which threads look does not matter: a stale reading delays a decision, it never makes
+// a wrong one. Each undecided candidate remembers the highest-ranked live cell that it found in its window
+// (its blocker); until that cell is dropped a look at it suffices, and if it is kept it drops the candidate.
+// Whenever nobody's blocker was dropped, nobody is left undecided: the best undecided candidate's blocker can
+// only be a kept cell, which has dropped it.
+// Fields: columns NT, rows NR, R; alive: bit k & 31 of word j stride + (k >> 5) set for candidate (j, k) until
+// it is dropped (a kept cell keeps its bit); surv: likewise the candidates to look at first, among them all that
+// rank above their whole window (the 3x3 local maxima); it ends as the kept cells, whose number is returned:
+// they are in list (j << 16 | k) if it holds them. list: room for 2 ucap words, redo for ucap entries.
+// look(jk, on, win, at): a group of G lanes (8 where a window has at most 8 columns, else 16 or 32; every lane
+// of the warp calls it, `on` alike in a group's lanes) looks at the window of jk. True if no live cell there
+// ranks above it: then jk is kept, and its window's other candidates have been dropped. Else `at` of the lane
+// with win set is the highest-ranked one. live(jk): not dropped. All threads call it. s[0], s[1], s[2] used.
+struct KeptSet {
+  int NT, NR, R, stride, ucap;
+  uint32_t *alive, *surv, *list;
+  uint16_t* redo;
+  int* s;
+  __device__ int lg() const { return 2 * R + 1 <= 8 ? 3 : 2 * R + 1 <= 16 ? 4 : 5; }
+};
+
+template <class Look, class Live>
+__device__ __forceinline__ int resolve_kept(const KeptSet& K, Look&& look, Live&& live) {
+  const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, stride = K.stride, nw = K.NT * stride, ucap = K.ucap;
+  const int lg = K.lg(), sub = lane & ((1 << lg) - 1), lead = lane & ~((1 << lg) - 1);
+  uint32_t *const alive = K.alive, *const surv = K.surv, *const list = K.list;
+  uint16_t* const redo = K.redo;
+  int* const s = K.s;
+  auto word_of = [&](uint32_t jk) { return (int)(jk >> 16) * stride + (int)((jk & 0xffffu) >> 5); };
+  if (tid == 0) s[0] = s[1] = s[2] = 0;
+  __syncthreads();
+  if (K.R > 0) {
+    const int t0 = (tid >> 5) << (5 - lg), grp = lane >> lg, dt = (bd >> 5) << (5 - lg);  // groups of a warp, of the CTA
+    // first the local maxima: those with no live cell above them in their window are kept
+    list_cells(K.NT, K.NR, stride, [&](int i) { return surv[i]; }, list, 2 * ucap, &s[0]);
+    __syncthreads();
+    const int ns = s[0];
+    if (ns <= 2 * ucap) {
+#pragma unroll 1
+      for (int t = t0; t < ns; t += dt) {  // uniform a warp
+        const bool on = t + grp < ns;
+        const uint32_t jk = list[min(t + grp, ns - 1)];
+        bool win;
+        uint32_t at;
+        if (!look(jk, on, win, at) && on && sub == 0) atomicAnd(&surv[word_of(jk)], ~(1u << (jk & 31u)));  // not kept yet
+      }
+    } else {
+#pragma unroll 1
+      for (int i = tid; i < nw; i += bd) surv[i] = 0u;  // no room: look at all candidates alike
+    }
+    __syncthreads();
+    HOUGH_PHASE(HOUGH_PHASE_IT_COLLECT);
+    // then the candidates left undecided
+    list_cells(K.NT, K.NR, stride, [&](int i) { return alive[i] & ~surv[i]; }, list, 2 * ucap, &s[1]);
+    __syncthreads();
+    const int nu = s[1];
+    if (nu <= ucap) {
+      uint32_t* blk = list + ucap;  // the blocker; the candidate itself once it is decided
+#pragma unroll 1
+      for (int n = nu, first = 1;; first = 0) {
+        if (!first) {  // whose blocker has been dropped (and who has not)
+#pragma unroll 1
+          for (int i0 = tid - lane; i0 < nu; i0 += bd) {  // uniform a warp
+            const int i = min(i0 + lane, nu - 1);
+            const uint32_t jk = list[i], b = blk[i];
+            const bool open = i0 + lane < nu && b != jk;
+            const bool dropped = open && !live(jk);
+            const bool again = open && !dropped && !live(b);
+            if (dropped) blk[i] = jk;
+            const int pos = warp_append(&s[2], again);
+            if (again) redo[pos] = (uint16_t)i;
+          }
+          __syncthreads();
+          n = s[2];
+          if (n == 0) break;  // uniform
+        }
+#pragma unroll 1
+        for (int t = t0; t < n; t += dt) {
+          const bool in = t + grp < n;
+          const int i = first ? min(t + grp, nu - 1) : (int)redo[min(t + grp, n - 1)];
+          const uint32_t jk = list[i];
+          // one reading for the group
+          const bool on = __shfl_sync(0xffffffffu, in && live(jk) ? 1 : 0, lead) != 0;
+          bool win;
+          uint32_t at;
+          if (look(jk, on, win, at)) {
+            if (sub == 0) atomicOr(&surv[word_of(jk)], 1u << (jk & 31u));
+            at = jk;
+          }
+          if (win || (in && !on && sub == 0)) blk[i] = on ? at : jk;  // (dropped meanwhile: decided)
+        }
+        __syncthreads();
+        if (tid == 0) s[2] = 0;
+        __syncthreads();
+      }
+    } else {  // more than the list holds: by bitmap words, a group a word
+#pragma unroll 1
+      for (;;) {
+        bool pending = false;
+#pragma unroll 1
+        for (int t = t0; t < nw; t += dt) {
+          const int i = min(t + grp, nw - 1);
+          uint32_t u = __shfl_sync(0xffffffffu, t + grp < nw ? alive[i] & ~surv[i] : 0u, lead);  // one reading
+          const uint32_t j = (uint32_t)(i / stride), k0 = (uint32_t)(i - (int)j * stride) << 5;
+#pragma unroll 1
+          while (__any_sync(0xffffffffu, u != 0u)) {
+            const uint32_t k = k0 + (u ? 31u - (uint32_t)__clz(u) : 0u), jk = (j << 16) | k;
+            const bool on = __shfl_sync(0xffffffffu, u && live(jk) ? 1 : 0, lead) != 0;
+            bool win;
+            uint32_t at;
+            const bool kept = look(jk, on, win, at);
+            if (kept && sub == 0) atomicOr(&surv[i], 1u << (k & 31u));
+            pending = pending || (on && !kept);
+            u &= ~(1u << (k & 31u));
+          }
+        }
+        if (!__syncthreads_or(pending)) break;
+      }
+    }
+  } else {
+#pragma unroll 1
+    for (int i = tid; i < nw; i += bd) surv[i] = alive[i];  // no window: every candidate is kept
+    __syncthreads();
+  }
+  HOUGH_PHASE(HOUGH_PHASE_IT_RESOLVE);
+  if (tid == 0) s[0] = 0;
+  __syncthreads();
+  list_cells(K.NT, K.NR, stride, [&](int i) { return surv[i]; }, list, 2 * ucap, &s[0]);
+  __syncthreads();
+  return s[0];
+}
+
+// Most kept cells that store_ranked orders in a list of `room` words.
+__host__ __device__ inline int ranked_room(int room) {
+  int n = 32;
+  while (2 * n <= room) n <<= 1;
+  return n;
+}
+
+// Stores the n cells of list (j << 16 | k; n <= ranked_room(room), its words) as peaks in rank order:
+// votes, then raster order. vmax, vmin: bounds of their votes. Up to room / 4 cells whose votes span at most
+// room / 4 values are put into one bucket a value first, and then ranked within their bucket (250 of 256 x 256
+// cells, each counting the cells above it: 9.1 k cycles an event; so 4.0 k); else sorted. All threads call it.
+template <class Cells>
+__device__ void store_ranked(const Cells& cells, int NR, uint32_t* list, int room, int n, int vmax, int vmin,
+                             int cell_bits, int maxp, hough_peak* dst) {
+  const int tid = threadIdx.x, bd = blockDim.x;
+  const uint32_t cm = (1u << cell_bits) - 1u;
+  const int q = room >> 2, B = vmax - vmin + 1;
+  const bool buckets = n <= q && B < q;
+  int N = 32;
+  while (N < n) N <<= 1;
+  uint32_t* start = list + q;     // of bucket vmax - votes; B + 1 of them
+  uint32_t* sorted = list + 2 * q;
+  if (buckets)
+    for (int i = tid; i <= B; i += bd) start[i] = 0u;
+  for (int i = tid; i < (buckets ? n : N); i += bd) {  // in place: votes, then the smaller cell
+    uint32_t key = 0u;
+    if (i < n) {
+      const int j = (int)(list[i] >> 16), k = (int)(list[i] & 0xffffu);
+      key = ((uint32_t)cells.votes(j, k) << cell_bits) | (cm - (uint32_t)(j * NR + k));
+    }
+    list[i] = key;
+  }
+  __syncthreads();
+  auto store = [&](int r, uint32_t key) {
+    const int cell = (int)(cm - (key & cm)), j = cell / NR;
+    hough_peak pk;
+    pk.theta_bin = (int16_t)j;
+    pk.rho_bin = (int16_t)(cell - j * NR);
+    pk.votes = (int16_t)(key >> cell_bits);
+    pk.flags = 0;
+    dst[r] = pk;
+  };
+  if (buckets) {
+    for (int i = tid; i < n; i += bd) atomicAdd(&start[vmax - (int)(list[i] >> cell_bits) + 1], 1u);
+    __syncthreads();
+    if (tid < 32) {  // counts of the buckets before, in place
+      const int per = (B + 32) / 32, i0 = min(tid * per, B + 1), i1 = min(i0 + per, B + 1);
+      uint32_t sum = 0u;
+      for (int i = i0; i < i1; ++i) sum += start[i];
+      uint32_t x = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (tid >= o) x += y;
+      }
+      x -= sum;
+      for (int i = i0; i < i1; ++i) start[i] = x += start[i];
+    }
+    __syncthreads();
+    // start[b]: first place of bucket b; filling it moves start[b] on to start[b + 1] as it was
+    for (int i = tid; i < n; i += bd) sorted[atomicAdd(&start[vmax - (int)(list[i] >> cell_bits)], 1u)] = list[i];
+    __syncthreads();
+    for (int i = tid; i < n; i += bd) {
+      const uint32_t key = sorted[i];
+      const int b = vmax - (int)(key >> cell_bits), lo = b ? (int)start[b - 1] : 0, hi = (int)start[b];
+      int r = lo;
+      for (int m = lo; m < hi; ++m) r += sorted[m] > key;
+      if (r < maxp) store(r, key);
+    }
+  } else {
+    bitonic_desc(list, N);
+    for (int i = tid; i < min(n, maxp); i += bd) store(i, list[i]);
+  }
+  __syncthreads();
+  HOUGH_PHASE(HOUGH_PHASE_IT_ORDER);
+}
+
 // Stage 2, as one walk (sup: a shared bitmap of NT NR bits, cell (j, k) bit j NR + k): the CTA
 // sorts the keys (cap words, past C free), then warp 0 walks them 32 at a time: lanes drop
 // candidates covered by earlier chunks' windows, then the lowest remaining lane is kept and the

@@ -346,6 +346,105 @@ struct FusedCells {
   }
 };
 
+// The iterative finder's kept set on a whole mirror-pair accumulator: dropped candidates' cells are set to
+// zero beside their bits, so a look is a plain maximum over the window's votes (cells that are no candidates
+// rank below every candidate). A column of the window a lane, its rows read independently: one
+// thread took ~9 k cycles a look at R = 3, its bits and votes one after the other; a group of 8 lanes that
+// tests the bits 3.1 k a round of 128 looks. Batched events at 256 x 256 (half the maximum, R = 3; 2,300
+// candidates, 490 local maxima, 250 kept), kept set in all, local maxima included: 57 k cycles with rounds on two
+// state bits a cell where a thread scans a window at every visit, 64 k with blockers and a thread a look, 46 k
+// with groups and bits, 38 k so.
+struct WholeWindow {
+  uint32_t* acc;
+  int half, rp, tq;
+  KeptSet K;
+  __device__ uint16_t* cell(int j, int k) const {
+    const bool hi = j >= half;
+    return reinterpret_cast<uint16_t*>(acc + mp_word(hi ? 2 * half - 1 - j : j, k + 1, rp)) + (hi ? 1 : 0);
+  }
+  __device__ int votes(int j, int k) const { return (int)*cell(j, k); }
+  __device__ bool live(uint32_t jk) const { return *cell((int)(jk >> 16), (int)(jk & 0xffffu)) != 0; }
+  // Rank within a window in 32 bits: votes (15 bits), then the place of the column in raster order (9 bits; a
+  // column from across the wrap, where rho is mirrored, comes after the others at the low end, before them at
+  // the high end), then the row (8 bits, from the column's first row).
+  __device__ bool look(uint32_t jk, bool on, bool& win, uint32_t& at) const {
+    const int lane = threadIdx.x & 31, G = 1 << K.lg(), sub = lane & (G - 1), R = K.R, W = 2 * R + 1, NT = K.NT;
+    const int j = (int)(jk >> 16), k = (int)(jk & 0xffffu), c0 = max(0, k - R), c1 = min(K.NR - 1, k + R), n = c1 - c0 + 1;
+    uint32_t m = 0u;
+    if (on) {
+#pragma unroll 1
+      for (int a = sub - R; a <= R; a += G) {
+        int jj = j + a, r0 = c0, place = 511 - (a + R + W);
+        if ((unsigned)jj >= (unsigned)NT) {
+          place -= jj < 0 ? W : -W;
+          jj += jj < 0 ? NT : -NT;
+          r0 = K.NR - 1 - c1;
+        }
+        const uint16_t* col = cell(jj, r0);
+        uint32_t t = 0u;  // votes << 8 | 255 - row from the first
+        if (n == 7) {
+#pragma unroll
+          for (int i = 0; i < 7; ++i) t = max(t, (uint32_t)col[i << 6] * 256u + (uint32_t)(255 - i));
+        } else {
+#pragma unroll 4
+          for (int i = 0; i < n; ++i) t = max(t, (uint32_t)col[i << 6] * 256u + (uint32_t)(255 - i));
+        }
+        const uint32_t x = ((t & ~255u) << 9) | (uint32_t)(place << 8) | (t & 255u);
+        if (x > m) {
+          m = x;
+          at = ((uint32_t)jj << 16) | (uint32_t)(r0 + 255 - (int)(t & 255u));
+        }
+      }
+    }
+    uint32_t top = m;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) top = max(top, __shfl_xor_sync(kFull, top, o));
+    if (G > 8)
+      for (int o = 8; o < G; o <<= 1) top = max(top, __shfl_xor_sync(kFull, top, o));
+    win = on && m == top;  // ranks are distinct: one lane
+    const unsigned self = __ballot_sync(kFull, win && at == jk);
+    if (!((self >> (lane & ~(G - 1))) & (0xffffffffu >> (32 - G)))) return false;
+#pragma unroll 1
+    for (int a = sub - R; a <= R; a += G) {
+      int jj = j + a, r0 = c0;
+      if ((unsigned)jj >= (unsigned)NT) {
+        jj += jj < 0 ? NT : -NT;
+        r0 = K.NR - 1 - c1;
+      }
+      const int r1 = r0 + n - 1, own = a == 0 ? k : -1;
+      uint16_t* col = cell(jj, r0);
+#pragma unroll 4
+      for (int i = 0; i < n; ++i)
+        if (r0 + i != own) col[i << 6] = 0;
+#pragma unroll 1
+      for (int w = r0 >> 5; w <= (r1 >> 5); ++w) {
+        uint32_t x = 0xffffffffu;
+        if (w == (r0 >> 5)) x &= 0xffffffffu << (r0 & 31);
+        if (w == (r1 >> 5)) x &= 0xffffffffu >> (31 - (r1 & 31));
+        if (a == 0 && w == (k >> 5)) x &= ~(1u << (k & 31));
+        if (K.alive[jj * K.stride + w] & x) atomicAnd(&K.alive[jj * K.stride + w], ~x);
+      }
+    }
+    return true;
+  }
+};
+
+// Maximum of a mirror-pair accumulator's cells (its words lie in one run; guard rows and lanes past the
+// last word are zero), to every thread; *s_max must be 0 beforehand.
+__device__ int acc_max_mp(const Plan& pl, const uint32_t* acc, int half, int* s_max) {
+  const uint4* x4 = reinterpret_cast<const uint4*>(acc);
+  const int n4 = ((half + 31) >> 5) * pl.rows_phys * 8;
+  uint32_t m = 0u;
+  for (int i = threadIdx.x; i < n4; i += blockDim.x) {
+    const uint4 x = x4[i];
+    m = vmax2(m, vmax2(vmax2(x.x, x.y), vmax2(x.z, x.w)));
+  }
+  const int top = __reduce_max_sync(kFull, (int)max(m & 0xffffu, m >> 16));
+  if ((threadIdx.x & 31) == 0 && top) atomicMax(s_max, top);
+  __syncthreads();
+  return *s_max;
+}
+
 // Shared address of the vote whose float row estimate, shifted by 1 + 2^b + e (2^b > N_rho + 1,
 // e = W/2 units of 2^-F, W a power of two), is kfp. In [2^b, 2^(b+1)) a float's low F = 23 - b
 // bits are the fraction and the bits above them (127 + b) 2^b + integer part, so
@@ -693,45 +792,70 @@ __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, Edg
 // (the central rows' candidates fell to a few warps) and 10.0 k a tile at 1000 x 1000; units of 8 rows
 // 9.6 k and 7.5 k; this form 9.9 k and 3.9 k.
 // list: room for (half + 31) / 32 * ((N_rho + 3) / 4) entries; *n_list zero beforehand.
-__device__ void scan_mp(const Plan& pl, const unsigned char* smem, int aw, int half, const EdgeWord* ew,
-                        uint32_t* pbits, uint16_t* list, int* n_list, bool do_cs, unsigned long long& csum) {
+// cand (nullable): a second cleared bitmap for all cells that reach the threshold (the iterative finder's
+// candidates, of which the peaks are the 3x3 local maxima).
+template <bool CAND>
+__device__ void scan_mp(const Plan& pl, const unsigned char* smem, int thr, int aw, int half, const EdgeWord* ew,
+                        uint32_t* pbits, uint32_t* cand, uint16_t* list, int* n_list, bool do_cs,
+                        unsigned long long& csum) {
   const int NT = pl.n_theta, NR = pl.n_rho, rp = pl.rows_phys;
   const uint32_t* const sw = reinterpret_cast<const uint32_t*>(smem);
   const uint32_t* const acc = sw + (pl.off_acc >> 2);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int G = (half + 31) >> 5, n4 = (NR + 3) >> 2;  // groups of words, of rows
-  const uint32_t TT = (uint32_t)pl.threshold | ((uint32_t)pl.threshold << 16);
+  const uint32_t TT = (uint32_t)thr | ((uint32_t)thr << 16);
   // (1) A half reaches T iff bit 15 of C - T + 0x8000 is set (cells are at most 32767: no borrow across
   // the halves). Rows past the last one may be read (they only list a group in vain), inside the CTA's
   // shared memory.
-  for (int g = 0; g < G; ++g) {
-    const uint4* row = reinterpret_cast<const uint4*>(acc + mp_word(32 * g, 1, rp)) + lane;
-    uint32_t hit = 0;
-    int q0 = warp, c = 0;
-    for (int q = warp; q < n4; q += nwarps, ++c) {
-      if (c == 32) {  // a warp's mask of 32 groups is full (only small CTAs)
-        if ((hit >> lane) & 1u) list[atomicAdd(n_list, 1)] = (uint16_t)(g << 8 | (q0 + lane * nwarps));
-        hit = 0;
-        q0 = q;
-        c = 0;
-      }
-      const uint4 x = row[q << 5];
-      const uint32_t top = vmax2(vmax2(x.x, x.y), vmax2(x.z, x.w));
-      if (__any_sync(kFull, ((top - TT + 0x80008000u) & 0x80008000u) != 0u)) hit |= 1u << c;
-      if (do_cs) {
-        const int k = 4 * q + (lane >> 3), w = 32 * g + 4 * (lane & 7);
-        const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+  {
+    int g = 0, q = warp, c = 0;
+    uint32_t hit = 0, mine = 0;  // bit c of hit: the warp's c-th group; lane c keeps which one that is
+    while (q >= n4 && g < G) {
+      q -= n4;
+      ++g;
+    }
+    while (g < G) {
+      uint4 x[4];
+      int gs[4], qs[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const unsigned a0 = xs[i] & 0xffffu, a1 = xs[i] >> 16;
-          if (k < NR && w + i < half) {
-            if (a0) csum += (unsigned long long)a0 * mix64((unsigned long long)(aw + w + i) * NR + k + 1);
-            if (a1) csum += (unsigned long long)a1 * mix64((unsigned long long)(NT - 1 - aw - w - i) * NR + k + 1);
+      for (int i = 0; i < 4; ++i) {  // four independent loads (past the last group: row group 0, not counted)
+        gs[i] = g;
+        qs[i] = g < G ? q : 0;
+        x[i] = *(reinterpret_cast<const uint4*>(acc + mp_word(32 * (g < G ? g : 0), 1 + 4 * qs[i], rp)) + lane);
+        q += nwarps;
+        while (q >= n4 && g < G) {
+          q -= n4;
+          ++g;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t top = vmax2(vmax2(x[i].x, x[i].y), vmax2(x[i].z, x[i].w));
+        if (__any_sync(kFull, gs[i] < G && ((top - TT + 0x80008000u) & 0x80008000u) != 0u)) hit |= 1u << c;
+        if (lane == c) mine = (uint32_t)(gs[i] << 8 | qs[i]);
+        ++c;
+        if (do_cs && gs[i] < G) {
+          const int k = 4 * qs[i] + (lane >> 3), w = 32 * gs[i] + 4 * (lane & 7);
+          const uint32_t xs[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const unsigned a0 = xs[m] & 0xffffu, a1 = xs[m] >> 16;
+            if (k < NR && w + m < half) {
+              if (a0) csum += (unsigned long long)a0 * mix64((unsigned long long)(aw + w + m) * NR + k + 1);
+              if (a1) csum += (unsigned long long)a1 * mix64((unsigned long long)(NT - 1 - aw - w - m) * NR + k + 1);
+            }
           }
         }
       }
+      if (c == 32 || g >= G) {
+        int at = 0;
+        if (lane == 0 && hit) at = atomicAdd(n_list, __popc(hit));
+        at = __shfl_sync(kFull, at, 0) + __popc(hit & lanemask_lt());
+        if ((hit >> lane) & 1u) list[at] = (uint16_t)mine;
+        hit = 0;
+        c = 0;
+      }
     }
-    if ((hit >> lane) & 1u) list[atomicAdd(n_list, 1)] = (uint16_t)(g << 8 | (q0 + lane * nwarps));
   }
   __syncthreads();
   // (2) Raster order runs over theta, then rho: the row above and the preceding column are
@@ -758,9 +882,10 @@ __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int aw, int h
 #pragma unroll
       for (int i = 0; i < 4; ++i) EV[i] = __byte_perm(vmax2(vmax2(e[i], e[i + 1]), e[i + 2]), 0u, ed.swap ? 0x1032u : 0x3210u);
     }
-    uint32_t fl = 0u;  // flags, the low column's in the low half, the newest row at bit 15 of each half
+    uint32_t fl = 0u, cf = 0u;  // flags, the low column's in the low half, the newest row at bit 15 of each half
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
+      if (CAND) cf = (cf >> 1) | ((R[i + 1] - TT + 0x80008000u) & 0x80008000u);
       uint32_t VM = vmax2(vmax2(R[i], R[i + 1]), R[i + 2]);
       if (n < 32 && lane == n) VM = EV[i];
       uint32_t VU = __shfl_up_sync(kFull, VM, 1), VD = __shfl_down_sync(kFull, VM, 1);
@@ -769,7 +894,16 @@ __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int aw, int h
       const uint32_t X = vmax2(vmax2(vmax2(R[i] + 0x00010001u, R[i + 2]), vmax2(VU + addU, VD + 0x10000u)), TT);
       fl = (fl >> 1) | ((R[i + 1] - X + 0x80008000u) & 0x80008000u);
     }
-    if (NR - k < 4) fl &= ((1u << (NR - k)) - 1u) * 0x10001000u;  // rows past the last one
+    if (NR - k < 4) {  // rows past the last one
+      const uint32_t valid = ((1u << (NR - k)) - 1u) * 0x10001000u;
+      fl &= valid;
+      cf &= valid;
+    }
+    if (CAND && lane < n) {
+      const uint32_t lo = (cf >> 12) & 15u, hi = cf >> 28;
+      if (lo) atomicOr(&cand[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
+      if (hi) atomicOr(&cand[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
+    }
     if (lane < n) {
       const uint32_t lo = (fl >> 12) & 15u, hi = fl >> 28;
       if (lo) atomicOr(&pbits[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
@@ -1600,7 +1734,7 @@ __device__ int merge_iterative(const Plan& pl, const FusedIO& io, unsigned char*
   block_exscan(colstart, NT + 1, sh.tmp);
   const SparseCands sc{keys, colstart, C};
   unsigned char* work = reinterpret_cast<unsigned char*>(keys + C);
-  const int work_bytes = (int)(smem + pl.off_unres - work);
+  const int work_bytes = (int)(smem + pl.smem_bytes - work);
   hough_peak* dst = io.peaks + e * (long long)maxp;
   // the rounds on a 2-bit state per cell of the event where that map fits (512 x 512: 64 KB);
   // the rank of an undecided neighbour comes from its key, found by binary search in its column
@@ -1695,7 +1829,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     for (int i = tid; i < nz; i += bd) z[i] = make_uint4(0u, 0u, 0u, 0u);
     if (T > 1)
       for (int i = tid; i < (MP ? 2 * pl.rows_phys : nrp); i += bd) halo[i] = 0u;
-    for (int i = tid; i < wpad * pl.nrb_p; i += bd) pbits[i] = 0;
+    for (int i = tid; i < (ITER && MP && T == 1 && pl.iter_cap > 0 ? 2 : 1) * wpad * pl.nrb_p; i += bd) pbits[i] = 0;
     if (tid == 0) {
       sh.flags = 0;
       sh.it_max = 0;
@@ -1722,7 +1856,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
       if (sh.wide & 2) sh.flags |= HOUGH_F_BAD_HIT;
       if (sh.wide & 1) sh.reuse = 0;  // wide hits are not in the staged list
     }
-    if (MP && want_halo && h0 == 0) edge_words(pl, aw, Wd, sh.edge);  // for the scan (no hits: no candidates)
+    if (MP && (want_halo || T == 1) && h0 == 0) edge_words(pl, aw, Wd, sh.edge);  // for the scan (no hits: no candidates)
     if (!(sh.wide & 1)) {
       if (mp_halo) halo_mp32(pl, HL, hb, sh.nv);
       if (MP)
@@ -1778,7 +1912,9 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
 
   // the next item, in steps whose latencies pass behind the phases between them (thread 0)
   WorkItem& next = sh.it[cur ^ 1];
-  const bool fetch = io.persistent && tid == 0;
+  // Not for the iterative finder on tiles: there an event's last tile takes much longer than the others, and an
+  // item popped before it would wait for it instead of going to another CTA.
+  const bool fetch = io.persistent && tid == 0 && !(ITER && T > 1);
   if (fetch && more < 0) more = pop_items(io, pl.grab);
   bool other = false;  // the next item exists and belongs to another event
   auto fetch_event = [&]() {
@@ -1819,28 +1955,54 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // extraction, which clears the cells it suppresses; records in extraction order
     if (MP) {
       mp_fold(pl, acc, Wd, nullptr);
+      if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
       __syncthreads();
       HOUGH_PHASE(HOUGH_PHASE_FOLD);
     }
-    auto iterative = [&](auto cells) {
-      if (do_cs) {
-        unsigned long long cs = 0;
-        for (int c = tid; c < NT * NR; c += bd) {
-          const int v = cells.get(c / NR, c % NR);
-          if (v) cs += (unsigned long long)v * mix64((unsigned long long)c + 1);
-        }
-        cs_tile = block_sum_u64(cs, sh.red);
+    if (do_cs) {
+      unsigned long long cs = 0;
+      for (int c = tid; c < NT * NR; c += bd) {
+        const int j = c / NR, k = c - j * NR, v = MP ? mp_get(acc, j, k, Wd, pl) : acc_get(acc, j, k, nrp);
+        if (v) cs += (unsigned long long)v * mix64((unsigned long long)c + 1);
       }
+      cs_tile = block_sum_u64(cs, sh.red);
       __syncthreads();
-      HOUGH_PHASE(HOUGH_PHASE_SCAN);
-      fetch_offsets();
-      const int st_words = (((NT * NR + 15) >> 4) + 31) & ~31;  // 2 bits a cell, whole 32-word blocks
-      return extract_iterative(cells, NT, NR, kIterSliceRows, pl.threshold, pl.rel_num, pl.rel_den, pl.nms_radius,
-                               maxp, pbits, pl.iter_cap, nullptr, st_words, io.peaks + e * (long long)maxp, sh.tmp,
-                               reinterpret_cast<uint16_t*>(pbits + pl.iter_cap + st_words), pl.iter_act);
-    };
-    total = MP ? iterative(FusedCells<true>{acc, Wd, nrp, pl.rows_phys})
-                  : iterative(FusedCells<false>{acc, Wd, nrp, pl.rows_phys});
+    }
+    HOUGH_PHASE(HOUGH_PHASE_SCAN);
+    fetch_offsets();
+    hough_peak* dst = io.peaks + e * (long long)maxp;
+    total = -1;
+    if (MP && pl.iter_cap > 0) {
+      // candidates and their 3x3 local maxima as bitmaps (cleared with the accumulator), then the kept set
+      const int amax = acc_max_mp(pl, acc, Wd, &sh.it_max);
+      HOUGH_PHASE(HOUGH_PHASE_IT_MAX);
+      const int tq = (int)max((long long)pl.threshold, ((long long)pl.rel_num * amax + pl.rel_den - 1) / pl.rel_den);
+      uint32_t* cand = pbits + pl.groups * 32 * pl.nrb_p;
+      uint32_t* list = cand + pl.groups * 32 * pl.nrb_p;
+      unsigned long long none = 0;
+      scan_mp<true>(pl, smem, tq, 0, Wd, sh.edge, pbits, cand, reinterpret_cast<uint16_t*>(list), &sh.n_amb, false, none);
+      __syncthreads();
+      const WholeWindow ww{acc, Wd, pl.rows_phys, tq,
+                           KeptSet{NT, NR, pl.nms_radius, pl.nrb_p, pl.iter_cap, cand, pbits, list,
+                                   reinterpret_cast<uint16_t*>(list + 2 * pl.iter_cap), sh.tmp}};
+      const int nk = resolve_kept(ww.K, [&](uint32_t jk, bool on, bool& win, uint32_t& at) { return ww.look(jk, on, win, at); },
+                                  [&](uint32_t jk) { return ww.live(jk); });
+      if (nk <= ranked_room(2 * pl.iter_cap)) {
+        store_ranked(ww, NR, list, 2 * pl.iter_cap, nk, amax, tq, 17, maxp, dst);  // at most 227 KB / 2 cells: 17 bits, and 15 of votes
+        total = nk;
+      }
+    }
+    // No bitmaps, or more peaks than the list ranks. (One pass a peak lists a kept set's cells in rank order
+    // too: the dropped candidates are zero, the cells that are none below the threshold.)
+    if (total < 0) {
+      auto general = [&](auto cells) {
+        const int st_words = (((NT * NR + 15) >> 4) + 31) & ~31;  // 2 bits a cell, whole 32-word blocks
+        return extract_iterative(cells, NT, NR, kIterSliceRows, pl.threshold, pl.rel_num, pl.rel_den, pl.nms_radius,
+                                 maxp, pbits, MP ? 0 : pl.iter_cap, nullptr, st_words, dst, sh.tmp,
+                                 reinterpret_cast<uint16_t*>(pbits + pl.iter_cap + st_words), pl.iter_act);
+      };
+      total = MP ? general(FusedCells<true>{acc, Wd, nrp, pl.rows_phys}) : general(FusedCells<false>{acc, Wd, nrp, pl.rows_phys});
+    }
     n_low = total;
   } else {
     // 3. peak scan, or (the iterative finder on theta tiles) the tile's candidates: every cell
@@ -1862,7 +2024,8 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
       __syncthreads();
       HOUGH_PHASE(HOUGH_PHASE_FOLD);
-      scan_mp(pl, smem, aw, Wd, sh.edge, pbits, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb, do_cs, csum);
+      scan_mp<false>(pl, smem, pl.threshold, aw, Wd, sh.edge, pbits, nullptr, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb,
+                     do_cs, csum);
     } else if (packed) {
       scan_packed(pl, acc, halo, pbits, wt, T, j0, do_cs, csum);
     } else {
@@ -2051,7 +2214,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_MERGE);
-  if (io.persistent && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
+  if (io.persistent && !(ITER && T > 1) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
     const long long i = next.off[0] + 16LL * tid;
     if (i < next.off[1]) asm volatile("prefetch.global.L2 [%0];" ::"l"(io.xy + i));
   }
@@ -2089,24 +2252,26 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
   __syncthreads();  // the table is read before run_item's first barrier
   const bool do_cs = io.checksum != nullptr;
   const bool queue = io.persistent && io.n_items > gridDim.x;  // else an item a CTA, and none after it
-  if (threadIdx.x == 0) {
-    const int it = queue ? pop_items(io, pl.grab) : (int)blockIdx.x;
-    sh.it[0].item = it;
-    if (it < io.n_items) {
-      const int e = io.order ? io.order[it / pl.tiles] : it / pl.tiles;
-      sh.it[0].event = e;
-      sh.it[0].off[0] = io.off[e];
-      sh.it[0].off[1] = io.off[e + 1];
-    }
-  }
+  auto fetch_item = [&](WorkItem& w, int it) {  // thread 0
+    w.item = it;
+    if (it >= io.n_items) return;
+    const int e = io.order ? io.order[it / pl.tiles] : it / pl.tiles;
+    w.event = e;
+    w.off[0] = io.off[e];
+    w.off[1] = io.off[e + 1];
+  };
+  if (threadIdx.x == 0) fetch_item(sh.it[0], queue ? pop_items(io, pl.grab) : (int)blockIdx.x);
   int left = 0;  // items popped together with the current one and still to come
+#pragma unroll 1
   for (int cur = 0;; cur ^= 1) {
     __syncthreads();
     const int it = sh.it[cur].item;
     if (it >= io.n_items) break;
     left = left > 0 ? left - 1 : pl.grab - 1;
-    run_item<MP, ITER>(pl, io, smem, sh, cur, !queue ? INT_MAX : left > 0 ? it + 1 : -1, do_cs);
+    const int more = !queue ? INT_MAX : left > 0 ? it + 1 : -1;
+    run_item<MP, ITER>(pl, io, smem, sh, cur, more, do_cs);
     if (!io.persistent) break;
+    if (ITER && pl.tiles > 1 && threadIdx.x == 0) fetch_item(sh.it[cur ^ 1], more < 0 ? pop_items(io, pl.grab) : more);
   }
 }
 
@@ -2177,8 +2342,8 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
       __syncthreads();
     }
     __threadfence_block();
-    // the finder: its scratch first, then the suppression bitmap, below the trig table
-    uint32_t* scratch = reinterpret_cast<uint32_t*>(smem);
+    // the finder: its scratch first, then the suppression bitmap, after the trig table
+    uint32_t* scratch = reinterpret_cast<uint32_t*>(smem + pl.off_unres);
     const int sw = iter_scratch_words(NT, NR, pl.def_sh);
     uint32_t* gone = scratch + (sw > pl.def_cap ? sw : pl.def_cap);
     for (int i = tid; i < (NT * NR + 31) >> 5; i += bd) gone[i] = 0u;

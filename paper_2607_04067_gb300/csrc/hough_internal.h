@@ -17,8 +17,9 @@ constexpr int kIterSliceRows = 32;
 struct Plan {
   int n_theta, n_rho, threshold, keep_hw, max_peaks;
   int peak_mode, rel_num, rel_den, nms_radius;  // peak finder (0: 3x3 local maxima, 1: iterative)
-  int iter_cap;   // iterative finder: candidate keys of its candidate form (0: one pass per peak only)
-  int iter_act;   // iterative finder: entries of each of its two lists of undecided candidates
+  // iterative finder on a whole accumulator (0: one pass a peak only). Mirror pairs: undecided candidates that
+  // are listed; columns: candidate keys, and entries of each of two lists of undecided candidates
+  int iter_cap, iter_act;
   int tiles;      // theta tiles per event
   int tile_w;     // columns per tile (last tile may be narrower)
   int groups;     // 32-column groups per tile
@@ -26,8 +27,8 @@ struct Plan {
   int threads;    // CTA size: groups * split * 32 (+ 32 halo lanes when tiles > 1)
   int nrho_pad;   // rows allocated per column
   int nrb;        // 32-bit bitmap words per column
-  int nrb_p;      // words a column takes in the peak bitmap: nrb made odd, so that neighbouring columns' words of
-                  // the same rows lie in different banks
+  int nrb_p;      // words a column takes in the peak bitmap: nrb made odd where there is room, so that
+                  // neighbouring columns' words of the same rows lie in different banks
   int nrb_g;      // bitmap words per column with one guard bit on each side, odd (lanes that test different
                   // columns at nearby rows would meet in one bank: 32 words a column at 1000 rows)
   int hit_cap;    // hits staged in shared memory per chunk
