@@ -93,7 +93,7 @@ static constexpr int kSmemBudget = 227 * 1024 - 2048;  // dynamic bytes; static 
 static int round16(int x) { return (x + 15) & ~15; }
 
 // Shared-memory layout for a shape; returns false if it does not fit.
-static bool layout(Plan& pl) {
+static bool layout(Plan& pl, bool local) {
   const int wpad = pl.groups * 32;
   // mirror-pair: groups / 2 word groups of 32 lanes (the last may be part idle) x rows_phys
   const int acc_bytes = pl.mp ? (pl.groups / 2) * 32 * pl.rows_phys * 4 : wpad * pl.nrho_pad * 2;
@@ -130,6 +130,10 @@ static bool layout(Plan& pl) {
   }
   pl.off_cnt = o;  // record keys of the local-maximum scan or of a tile's candidates
   if (!it_whole) o += round16(wpad * pl.key_groups * 4);
+  // the record keys' counts are not needed where a key is one word: the local maxima's bitmap may lie there
+  const bool it_tiled = pl.peak_mode == HOUGH_PEAK_ITERATIVE && pl.tiles > 1;
+  pl.off_local = it_tiled && pl.mp && local ? (pl.key_words == 1 ? pl.off_cnt : o) : 0;
+  if (pl.off_local) o = std::max(o, pl.off_local + round16(wpad * pl.nrb_p * 4));
   // the vote's list lies in a region that is first written after the vote
   pl.off_amb = !it_whole ? pl.off_cnt : pl.off_pbits + (pl.mp && pl.iter_cap > 0 ? 8 * wpad * pl.nrb_p : 0);
   pl.amb_cap = std::min(1024, (o - pl.off_amb) / 4);
@@ -321,8 +325,10 @@ int make_plan(const hough_params* p, Plan& pl) {
           for (int act = icap > 0 && !pl.mp ? 2048 : 0; act >= 0;
                act = act > 1024 ? act - 512 : act > 256 ? act / 2 : act - 256) {  // 2048, 1536, 1024, 512, 256, 0
             pl.iter_act = act;
-            for (pl.nrb_p = pl.nrb | 1; pl.nrb_p >= pl.nrb; --pl.nrb_p)  // odd where there is room
-              if (layout(pl)) return HOUGH_OK;
+            // odd bitmap strides and the tiles' local maxima where there is room
+            for (bool local : {true, false})
+              for (pl.nrb_p = pl.nrb | 1; pl.nrb_p >= pl.nrb; --pl.nrb_p)
+                if (layout(pl, local)) return HOUGH_OK;
           }
         }
       }

@@ -10,18 +10,10 @@
 #pragma once
 
 #include <cstdint>
-#include <type_traits>
 
 #include "hough.h"
 
 namespace hgpu {
-
-// Cells given as a sorted candidate list (kSorted: lower(j, k), end(j), key(p), rows ascending in
-// a column) let the rounds walk a column instead of looking every cell up.
-template <class C, class = void>
-struct sorted_cells : std::false_type {};
-template <class C>
-struct sorted_cells<C, std::void_t<decltype(C::kSorted)>> : std::bool_constant<C::kSorted> {};
 
 // Phase timers (builds with HOUGH_PHASE_TIMERS defined): thread 0 of a CTA adds the clock64()
 // cycles since its previous mark to the counter of the phase that just ended (HOUGH_PHASE_*).
@@ -537,11 +529,6 @@ __device__ int resolve_rounds(Cells& cells, int NT, int NR, int R, int tq, int m
       }
       // the states of rows r0 .. r1 of column jj, 16 cells at a time
       const int b0 = (jj * NR + r0) << 1, nb = (r1 - r0 + 1) << 1;
-      int p = 0, e_col = 0;  // sorted lists: a walk down column jj's list
-      if constexpr (sorted_cells<Cells>::value) {
-        p = cells.lower(jj, r0);
-        e_col = cells.end(jj);
-      }
       for (int off = 0; off < nb && !drop && all; off += 32) {
         const int bb = b0 + off, w = bb >> 5, sh = bb & 31, len = min(32, nb - off);
         uint32_t f = st[swz(w)] >> sh;
@@ -554,13 +541,7 @@ __device__ int resolve_rounds(Cells& cells, int NT, int NR, int R, int tq, int m
         uint32_t m = f & ~(f >> 1) & 0x55555555u;  // undecided cells
         while (m && all) {
           const int kr = r0 + ((off + __ffs(m) - 1) >> 1);
-          uint32_t kd;
-          if constexpr (sorted_cells<Cells>::value) {  // an undecided cell is in its column's list
-            while (p < e_col && 1023 - (int)(cells.key(p) & 1023u) < kr) ++p;
-            kd = p < e_col ? cells.key(p) : 0u;
-          } else {
-            kd = ((uint32_t)cells.get(jj, kr) << 20) | ((uint32_t)(1023 - jj) << 10) | (uint32_t)(1023 - kr);
-          }
+          const uint32_t kd = ((uint32_t)cells.get(jj, kr) << 20) | ((uint32_t)(1023 - jj) << 10) | (uint32_t)(1023 - kr);
           if (kd > key) all = false;  // an undecided cell ranked above (the cell itself is equal)
           m &= m - 1u;
         }
@@ -598,24 +579,7 @@ __device__ int resolve_rounds(Cells& cells, int NT, int NR, int R, int tq, int m
     for (int t0 = threadIdx.x - lane; t0 < C; t0 += bd) {  // slots of a warp: uniform
       const int t = t0 + lane;
       bool sv = t < C;
-      if (sv && R > 0 && sorted_cells<Cells>::value) {  // three column walks
-        const uint32_t key = keys[t];
-        const int j = 1023 - (int)((key >> 10) & 1023u), k = 1023 - (int)(key & 1023u);
-        for (int da = -1; da <= 1; ++da) {
-          int jj = j + da, r0 = max(0, k - 1), r1 = min(NR - 1, k + 1);
-          if (jj < 0 || jj >= NT) {  // across the theta wrap: the other end, rho mirrored
-            jj = jj < 0 ? jj + NT : jj - NT;
-            const int t0 = NR - 1 - r1;
-            r1 = NR - 1 - r0;
-            r0 = t0;
-          }
-          if constexpr (sorted_cells<Cells>::value) {
-            const int e_col = cells.end(jj);
-            for (int p = cells.lower(jj, r0); p < e_col && 1023 - (int)(cells.key(p) & 1023u) <= r1; ++p)
-              sv = sv && cells.key(p) <= key;
-          }
-        }
-      } else if (sv && R > 0) {
+      if (sv && R > 0) {
         const uint32_t key = keys[t];
         const int j = 1023 - (int)((key >> 10) & 1023u), k = 1023 - (int)(key & 1023u);
 #pragma unroll
@@ -655,15 +619,9 @@ __device__ int resolve_rounds(Cells& cells, int NT, int NR, int R, int tq, int m
             r0 = NR - 1 - k1;
             r1 = NR - 1 - k0;
           }
-          if constexpr (sorted_cells<Cells>::value) {
-            const int e_col = cells.end(jj);
-            for (int p = cells.lower(jj, r0); p < e_col && 1023 - (int)(cells.key(p) & 1023u) <= r1; ++p)
-              top &= cells.key(p) <= key;
-          } else {
 #pragma unroll 4
-            for (int kr = r0; kr <= r1; ++kr)
-              top &= (((uint32_t)cells.get(jj, kr) << 20) | ((uint32_t)(1023 - jj) << 10) | (uint32_t)(1023 - kr)) <= key;
-          }
+          for (int kr = r0; kr <= r1; ++kr)
+            top &= (((uint32_t)cells.get(jj, kr) << 20) | ((uint32_t)(1023 - jj) << 10) | (uint32_t)(1023 - kr)) <= key;
         }
         if (top) atomicOr(&st[swz(c >> 4)], 2u << ((c & 15) << 1));  // 1 -> 3
       }
@@ -765,20 +723,9 @@ __device__ int resolve_rounds(Cells& cells, int NT, int NR, int R, int tq, int m
           if (nb < 32) f &= (1u << nb) - 1u;
           kept_seen = ((f & (f >> 1)) & 0x55555555u) != 0u;
           uint32_t m = f & ~(f >> 1) & 0x55555555u;  // undecided cells
-          int p = 0, e_col = 0;
-          if constexpr (sorted_cells<Cells>::value) {
-            p = cells.lower(jj, r0);
-            e_col = cells.end(jj);
-          }
           while (m && !above) {
             const int kr = r0 + ((__ffs(m) - 1) >> 1);
-            uint32_t kd;
-            if constexpr (sorted_cells<Cells>::value) {
-              while (p < e_col && 1023 - (int)(cells.key(p) & 1023u) < kr) ++p;
-              kd = p < e_col ? cells.key(p) : 0u;
-            } else {
-              kd = ((uint32_t)cells.get(jj, kr) << 20) | ((uint32_t)(1023 - jj) << 10) | (uint32_t)(1023 - kr);
-            }
+            const uint32_t kd = ((uint32_t)cells.get(jj, kr) << 20) | ((uint32_t)(1023 - jj) << 10) | (uint32_t)(1023 - kr);
             above = kd > key;  // an undecided cell ranked above (the cell itself is equal)
             m &= m - 1u;
           }
@@ -874,6 +821,157 @@ __device__ int resolve_rounds(Cells& cells, int NT, int NR, int R, int tq, int m
   return nk;
 }
 
+// The kept set of the iterative finder (Sec. 2: the best unsuppressed cell is the next peak and suppresses
+// its window) from its candidates. A candidate is kept iff every higher-ranked candidate of its window is
+// dropped, and dropped by a kept cell whose window covers it. Cells are only ever dropped, and only by kept
+// ones, so the order in which threads look does not matter: a stale reading delays a decision, it never makes
+// a wrong one. Each undecided candidate remembers the highest-ranked live cell that it found in its window
+// (its blocker); until that cell is dropped a look at it suffices, and if it is kept it drops the candidate.
+// Whenever nobody's blocker was dropped, nobody is left undecided: the best undecided candidate's blocker can
+// only be a kept cell, which has dropped it.
+// P, the candidates: each has an id, and a bit `alive` until it is dropped (a kept cell keeps its bit), and a bit
+// `surv`. surv marks those to look at first (any of them; best those that the 3x3 test leaves) and ends as the
+// kept cells, whose number is returned: they are in list if it holds them.
+//   radius(), lg(): the window's half-width; log2 of the lanes of a group that looks at one
+//   words(), id(i, b): bitmap words, and the candidate of bit b of word i; alive, surv: the bitmaps
+//   bit(id, w): the word w and the mask of a candidate's bit
+//   list_bits(word, list, room, n): appends the candidates whose bit is set in word(i), counting all of them
+//   live(id): not dropped
+//   look(id, on, win, at): a group of lanes (every lane of the warp calls it, `on` alike in a group's) looks
+//     at a candidate's window. True if no live cell there ranks above it: then it is kept, and the others of
+//     its window have been dropped. Else `at` of the lane with win set is the highest-ranked one.
+// list: room for 2 ucap words, redo for ucap entries. All threads call it. s[0], s[1], s[2] used.
+template <class P>
+__device__ __forceinline__ int resolve_kept(const P& p, uint32_t* list, int ucap, uint16_t* redo, int* s) {
+  const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, nw = p.words();
+  const int lg = p.lg(), sub = lane & ((1 << lg) - 1), lead = lane & ~((1 << lg) - 1);
+  uint32_t *const alive = p.alive, *const surv = p.surv;
+  if (tid == 0) s[0] = s[1] = s[2] = 0;
+  __syncthreads();
+  if (p.radius() > 0) {
+    const int t0 = (tid >> 5) << (5 - lg), grp = lane >> lg, dt = (bd >> 5) << (5 - lg);  // groups of a warp, of the CTA
+    // first the local maxima: those with no live cell above them in their window are kept
+    p.list_bits([&](int i) { return surv[i]; }, list, 2 * ucap, &s[0]);
+    __syncthreads();
+    const int ns = s[0];
+    if (ns <= 2 * ucap) {
+#pragma unroll 1
+      for (int t = t0; t < ns; t += dt) {  // uniform a warp
+        const bool on = t + grp < ns;
+        const uint32_t id = list[min(t + grp, ns - 1)];
+        bool win;
+        uint32_t at;
+        if (!p.look(id, on, win, at) && on && sub == 0) {  // not kept yet
+          int w;
+          const uint32_t m = p.bit(id, w);
+          atomicAnd(&surv[w], ~m);
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int i = tid; i < nw; i += bd) surv[i] = 0u;  // no room: look at all candidates alike
+    }
+    __syncthreads();
+    HOUGH_PHASE(HOUGH_PHASE_IT_COLLECT);
+    // then the candidates left undecided
+    p.list_bits([&](int i) { return alive[i] & ~surv[i]; }, list, 2 * ucap, &s[1]);
+    __syncthreads();
+    const int nu = s[1];
+    if (nu <= ucap) {
+      uint32_t* blk = list + ucap;  // the blocker; the candidate itself once it is decided
+#pragma unroll 1
+      for (int n = nu, first = 1;; first = 0) {
+        if (!first) {  // whose blocker has been dropped (and who has not)
+#pragma unroll 1
+          for (int i0 = tid - lane; i0 < nu; i0 += bd) {  // uniform a warp
+            const int i = min(i0 + lane, nu - 1);
+            const uint32_t id = list[i], b = blk[i];
+            const bool open = i0 + lane < nu && b != id;
+            const bool dropped = open && !p.live(id);
+            const bool again = open && !dropped && !p.live(b);
+            if (dropped) blk[i] = id;
+            const int pos = warp_append(&s[2], again);
+            if (again) redo[pos] = (uint16_t)i;
+          }
+          __syncthreads();
+          n = s[2];
+          if (n == 0) break;  // uniform
+        }
+#pragma unroll 1
+        for (int t = t0; t < n; t += dt) {
+          const bool in = t + grp < n;
+          const int i = first ? min(t + grp, nu - 1) : (int)redo[min(t + grp, n - 1)];
+          const uint32_t id = list[i];
+          // one reading for the group
+          const bool on = __shfl_sync(0xffffffffu, in && p.live(id) ? 1 : 0, lead) != 0;
+          bool win;
+          uint32_t at;
+          if (p.look(id, on, win, at)) {
+            if (sub == 0) {
+              int w;
+              const uint32_t m = p.bit(id, w);
+              atomicOr(&surv[w], m);
+            }
+            at = id;
+          }
+          if (win || (in && !on && sub == 0)) blk[i] = on ? at : id;  // (dropped meanwhile: decided)
+        }
+        __syncthreads();
+        if (tid == 0) s[2] = 0;
+        __syncthreads();
+      }
+    } else {  // more than the list holds: by bitmap words, a group a word
+#pragma unroll 1
+      for (;;) {
+        bool pending = false;
+#pragma unroll 1
+        for (int t = t0; t < nw; t += dt) {
+          const int i = min(t + grp, nw - 1);
+          uint32_t u = __shfl_sync(0xffffffffu, t + grp < nw ? alive[i] & ~surv[i] : 0u, lead);  // one reading
+#pragma unroll 1
+          while (__any_sync(0xffffffffu, u != 0u)) {
+            const int b = u ? 31 - __clz(u) : 0;
+            const uint32_t id = p.id(i, b);
+            const bool on = __shfl_sync(0xffffffffu, u && p.live(id) ? 1 : 0, lead) != 0;
+            bool win;
+            uint32_t at;
+            const bool kept = p.look(id, on, win, at);
+            if (kept && sub == 0) atomicOr(&surv[i], 1u << b);
+            pending = pending || (on && !kept);
+            u &= ~(1u << b);
+          }
+        }
+        if (!__syncthreads_or(pending)) break;
+      }
+    }
+  } else {
+#pragma unroll 1
+    for (int i = tid; i < nw; i += bd) surv[i] = alive[i];  // no window: every candidate is kept
+    __syncthreads();
+  }
+  HOUGH_PHASE(HOUGH_PHASE_IT_RESOLVE);
+  if (tid == 0) s[0] = 0;
+  __syncthreads();
+  p.list_bits([&](int i) { return surv[i]; }, list, 2 * ucap, &s[0]);
+  __syncthreads();
+  return s[0];
+}
+
+// Positions in a list counted by *n for the bits of a warp's 32 words: the first one of this lane's c bits (an
+// inclusive scan over the lanes, one atomic a warp). Every lane calls it.
+__device__ __forceinline__ int warp_positions(int c, int* n) {
+  const int lane = threadIdx.x & 31;
+  int at = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, at, o);
+    if (lane >= o) at += y;
+  }
+  int base = 0;
+  if (lane == 31) base = atomicAdd(n, at);
+  return at + __shfl_sync(0xffffffffu, base, 31) - c;
+}
+
 // The cells (j << 16 | k) of a bitmap (word(i) of word i = j stride + (k >> 5)) appended to list, of which *n
 // counts all, past its room too. A warp takes word w of 32 consecutive columns, whose counts are alike
 // (candidates crowd in the central rows of every column), and the warps of all column groups take one w after
@@ -892,16 +990,7 @@ __device__ __forceinline__ void list_cells(int NT, int NR, int stride, Word&& wo
     const int j = 32 * g + lane;
     uint32_t bits = j < NT ? word(j * stride + w) : 0u;
     if (!__any_sync(0xffffffffu, bits != 0u)) continue;
-    const int c = __popc(bits);
-    int at = c;  // inclusive scan over the lanes
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, at, o);
-      if (lane >= o) at += y;
-    }
-    int base = 0;
-    if (lane == 31) base = atomicAdd(n, at);
-    at += __shfl_sync(0xffffffffu, base, 31) - c;
+    int at = warp_positions(__popc(bits), n);
 #pragma unroll 1
     while (bits) {
       const int b = 31 - __clz(bits);
@@ -912,141 +1001,6 @@ __device__ __forceinline__ void list_cells(int NT, int NR, int stride, Word&& wo
   }
 }
 
-// The kept set of the iterative finder (Sec. 2: the best unsuppressed cell is the next peak and suppresses
-// its window) from its candidates. A candidate is kept iff every higher-ranked candidate of its window is
-// dropped, and dropped by a kept cell whose window covers it. Cells are only ever dropped, and only by kept
-// ones, so the order in which threads look does not matter: a stale reading delays a decision, it never makes
-// a wrong one. Each undecided candidate remembers the highest-ranked live cell that it found in its window
-// (its blocker); until that cell is dropped a look at it suffices, and if it is kept it drops the candidate.
-// Whenever nobody's blocker was dropped, nobody is left undecided: the best undecided candidate's blocker can
-// only be a kept cell, which has dropped it.
-// Fields: columns NT, rows NR, R; alive: bit k & 31 of word j stride + (k >> 5) set for candidate (j, k) until
-// it is dropped (a kept cell keeps its bit); surv: likewise the candidates to look at first, among them all that
-// rank above their whole window (the 3x3 local maxima); it ends as the kept cells, whose number is returned:
-// they are in list (j << 16 | k) if it holds them. list: room for 2 ucap words, redo for ucap entries.
-// look(jk, on, win, at): a group of G lanes (8 where a window has at most 8 columns, else 16 or 32; every lane
-// of the warp calls it, `on` alike in a group's lanes) looks at the window of jk. True if no live cell there
-// ranks above it: then jk is kept, and its window's other candidates have been dropped. Else `at` of the lane
-// with win set is the highest-ranked one. live(jk): not dropped. All threads call it. s[0], s[1], s[2] used.
-struct KeptSet {
-  int NT, NR, R, stride, ucap;
-  uint32_t *alive, *surv, *list;
-  uint16_t* redo;
-  int* s;
-  __device__ int lg() const { return 2 * R + 1 <= 8 ? 3 : 2 * R + 1 <= 16 ? 4 : 5; }
-};
-
-template <class Look, class Live>
-__device__ __forceinline__ int resolve_kept(const KeptSet& K, Look&& look, Live&& live) {
-  const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, stride = K.stride, nw = K.NT * stride, ucap = K.ucap;
-  const int lg = K.lg(), sub = lane & ((1 << lg) - 1), lead = lane & ~((1 << lg) - 1);
-  uint32_t *const alive = K.alive, *const surv = K.surv, *const list = K.list;
-  uint16_t* const redo = K.redo;
-  int* const s = K.s;
-  auto word_of = [&](uint32_t jk) { return (int)(jk >> 16) * stride + (int)((jk & 0xffffu) >> 5); };
-  if (tid == 0) s[0] = s[1] = s[2] = 0;
-  __syncthreads();
-  if (K.R > 0) {
-    const int t0 = (tid >> 5) << (5 - lg), grp = lane >> lg, dt = (bd >> 5) << (5 - lg);  // groups of a warp, of the CTA
-    // first the local maxima: those with no live cell above them in their window are kept
-    list_cells(K.NT, K.NR, stride, [&](int i) { return surv[i]; }, list, 2 * ucap, &s[0]);
-    __syncthreads();
-    const int ns = s[0];
-    if (ns <= 2 * ucap) {
-#pragma unroll 1
-      for (int t = t0; t < ns; t += dt) {  // uniform a warp
-        const bool on = t + grp < ns;
-        const uint32_t jk = list[min(t + grp, ns - 1)];
-        bool win;
-        uint32_t at;
-        if (!look(jk, on, win, at) && on && sub == 0) atomicAnd(&surv[word_of(jk)], ~(1u << (jk & 31u)));  // not kept yet
-      }
-    } else {
-#pragma unroll 1
-      for (int i = tid; i < nw; i += bd) surv[i] = 0u;  // no room: look at all candidates alike
-    }
-    __syncthreads();
-    HOUGH_PHASE(HOUGH_PHASE_IT_COLLECT);
-    // then the candidates left undecided
-    list_cells(K.NT, K.NR, stride, [&](int i) { return alive[i] & ~surv[i]; }, list, 2 * ucap, &s[1]);
-    __syncthreads();
-    const int nu = s[1];
-    if (nu <= ucap) {
-      uint32_t* blk = list + ucap;  // the blocker; the candidate itself once it is decided
-#pragma unroll 1
-      for (int n = nu, first = 1;; first = 0) {
-        if (!first) {  // whose blocker has been dropped (and who has not)
-#pragma unroll 1
-          for (int i0 = tid - lane; i0 < nu; i0 += bd) {  // uniform a warp
-            const int i = min(i0 + lane, nu - 1);
-            const uint32_t jk = list[i], b = blk[i];
-            const bool open = i0 + lane < nu && b != jk;
-            const bool dropped = open && !live(jk);
-            const bool again = open && !dropped && !live(b);
-            if (dropped) blk[i] = jk;
-            const int pos = warp_append(&s[2], again);
-            if (again) redo[pos] = (uint16_t)i;
-          }
-          __syncthreads();
-          n = s[2];
-          if (n == 0) break;  // uniform
-        }
-#pragma unroll 1
-        for (int t = t0; t < n; t += dt) {
-          const bool in = t + grp < n;
-          const int i = first ? min(t + grp, nu - 1) : (int)redo[min(t + grp, n - 1)];
-          const uint32_t jk = list[i];
-          // one reading for the group
-          const bool on = __shfl_sync(0xffffffffu, in && live(jk) ? 1 : 0, lead) != 0;
-          bool win;
-          uint32_t at;
-          if (look(jk, on, win, at)) {
-            if (sub == 0) atomicOr(&surv[word_of(jk)], 1u << (jk & 31u));
-            at = jk;
-          }
-          if (win || (in && !on && sub == 0)) blk[i] = on ? at : jk;  // (dropped meanwhile: decided)
-        }
-        __syncthreads();
-        if (tid == 0) s[2] = 0;
-        __syncthreads();
-      }
-    } else {  // more than the list holds: by bitmap words, a group a word
-#pragma unroll 1
-      for (;;) {
-        bool pending = false;
-#pragma unroll 1
-        for (int t = t0; t < nw; t += dt) {
-          const int i = min(t + grp, nw - 1);
-          uint32_t u = __shfl_sync(0xffffffffu, t + grp < nw ? alive[i] & ~surv[i] : 0u, lead);  // one reading
-          const uint32_t j = (uint32_t)(i / stride), k0 = (uint32_t)(i - (int)j * stride) << 5;
-#pragma unroll 1
-          while (__any_sync(0xffffffffu, u != 0u)) {
-            const uint32_t k = k0 + (u ? 31u - (uint32_t)__clz(u) : 0u), jk = (j << 16) | k;
-            const bool on = __shfl_sync(0xffffffffu, u && live(jk) ? 1 : 0, lead) != 0;
-            bool win;
-            uint32_t at;
-            const bool kept = look(jk, on, win, at);
-            if (kept && sub == 0) atomicOr(&surv[i], 1u << (k & 31u));
-            pending = pending || (on && !kept);
-            u &= ~(1u << (k & 31u));
-          }
-        }
-        if (!__syncthreads_or(pending)) break;
-      }
-    }
-  } else {
-#pragma unroll 1
-    for (int i = tid; i < nw; i += bd) surv[i] = alive[i];  // no window: every candidate is kept
-    __syncthreads();
-  }
-  HOUGH_PHASE(HOUGH_PHASE_IT_RESOLVE);
-  if (tid == 0) s[0] = 0;
-  __syncthreads();
-  list_cells(K.NT, K.NR, stride, [&](int i) { return surv[i]; }, list, 2 * ucap, &s[0]);
-  __syncthreads();
-  return s[0];
-}
-
 // Most kept cells that store_ranked orders in a list of `room` words.
 __host__ __device__ inline int ranked_room(int room) {
   int n = 32;
@@ -1054,15 +1008,15 @@ __host__ __device__ inline int ranked_room(int room) {
   return n;
 }
 
-// Stores the n cells of list (j << 16 | k; n <= ranked_room(room), its words) as peaks in rank order:
-// votes, then raster order. vmax, vmin: bounds of their votes. Up to room / 4 cells whose votes span at most
+// Stores the n candidates of list (n <= ranked_room(room), its words) as peaks in rank order: p.key(id), whose
+// upper bits from p.kVotes on are the votes and the rest the raster order; p.cell(key, j, k). vmax, vmin: bounds of
+// their votes. Up to room / 4 cells whose votes span at most
 // room / 4 values are put into one bucket a value first, and then ranked within their bucket (250 of 256 x 256
 // cells, each counting the cells above it: 9.1 k cycles an event; so 4.0 k); else sorted. All threads call it.
-template <class Cells>
-__device__ void store_ranked(const Cells& cells, int NR, uint32_t* list, int room, int n, int vmax, int vmin,
-                             int cell_bits, int maxp, hough_peak* dst) {
+template <class P>
+__device__ void store_ranked(const P& p, uint32_t* list, int room, int n, int vmax, int vmin, int maxp, hough_peak* dst) {
   const int tid = threadIdx.x, bd = blockDim.x;
-  const uint32_t cm = (1u << cell_bits) - 1u;
+  constexpr int cell_bits = P::kVotes;
   const int q = room >> 2, B = vmax - vmin + 1;
   const bool buckets = n <= q && B < q;
   int N = 32;
@@ -1071,20 +1025,14 @@ __device__ void store_ranked(const Cells& cells, int NR, uint32_t* list, int roo
   uint32_t* sorted = list + 2 * q;
   if (buckets)
     for (int i = tid; i <= B; i += bd) start[i] = 0u;
-  for (int i = tid; i < (buckets ? n : N); i += bd) {  // in place: votes, then the smaller cell
-    uint32_t key = 0u;
-    if (i < n) {
-      const int j = (int)(list[i] >> 16), k = (int)(list[i] & 0xffffu);
-      key = ((uint32_t)cells.votes(j, k) << cell_bits) | (cm - (uint32_t)(j * NR + k));
-    }
-    list[i] = key;
-  }
+  for (int i = tid; i < (buckets ? n : N); i += bd) list[i] = i < n ? p.key(list[i]) : 0u;  // in place
   __syncthreads();
   auto store = [&](int r, uint32_t key) {
-    const int cell = (int)(cm - (key & cm)), j = cell / NR;
+    int j, k;
+    p.cell(key, j, k);
     hough_peak pk;
     pk.theta_bin = (int16_t)j;
-    pk.rho_bin = (int16_t)(cell - j * NR);
+    pk.rho_bin = (int16_t)k;
     pk.votes = (int16_t)(key >> cell_bits);
     pk.flags = 0;
     dst[r] = pk;

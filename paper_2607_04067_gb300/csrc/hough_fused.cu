@@ -354,22 +354,47 @@ struct FusedCells {
 // candidates, 490 local maxima, 250 kept), kept set in all, local maxima included: 57 k cycles with rounds on two
 // state bits a cell where a thread scans a window at every visit, 64 k with blockers and a thread a look, 46 k
 // with groups and bits, 38 k so.
+// Ids: j << 16 | k; bitmap word of cell (j, k): j stride + (k >> 5).
 struct WholeWindow {
+  static constexpr int kVotes = 17;  // at most 227 KB / 2 cells: 17 bits, and 15 of votes
   uint32_t* acc;
-  int half, rp, tq;
-  KeptSet K;
+  int half, rp, NT, NR, R, stride;
+  uint32_t *alive, *surv;
+  __device__ int radius() const { return R; }
+  __device__ int lg() const { return 2 * R + 1 <= 8 ? 3 : 2 * R + 1 <= 16 ? 4 : 5; }
+  __device__ int words() const { return NT * stride; }
+  __device__ uint32_t id(int i, int b) const {
+    const int j = i / stride;
+    return ((uint32_t)j << 16) | (uint32_t)(32 * (i - j * stride) + b);
+  }
+  __device__ uint32_t bit(uint32_t jk, int& w) const {
+    w = (int)(jk >> 16) * stride + (int)((jk & 0xffffu) >> 5);
+    return 1u << (jk & 31u);
+  }
+  template <class Word>
+  __device__ void list_bits(Word&& word, uint32_t* list, int room, int* n) const {
+    list_cells(NT, NR, stride, word, list, room, n);
+  }
+  __device__ uint32_t key(uint32_t jk) const {
+    const int j = (int)(jk >> 16), k = (int)(jk & 0xffffu);
+    return ((uint32_t)*cell(j, k) << kVotes) | (uint32_t)((1 << kVotes) - 1 - (j * NR + k));
+  }
+  __device__ void cell(uint32_t key, int& j, int& k) const {
+    const int c = (1 << kVotes) - 1 - (int)(key & ((1u << kVotes) - 1u));
+    j = c / NR;
+    k = c - j * NR;
+  }
   __device__ uint16_t* cell(int j, int k) const {
     const bool hi = j >= half;
     return reinterpret_cast<uint16_t*>(acc + mp_word(hi ? 2 * half - 1 - j : j, k + 1, rp)) + (hi ? 1 : 0);
   }
-  __device__ int votes(int j, int k) const { return (int)*cell(j, k); }
   __device__ bool live(uint32_t jk) const { return *cell((int)(jk >> 16), (int)(jk & 0xffffu)) != 0; }
   // Rank within a window in 32 bits: votes (15 bits), then the place of the column in raster order (9 bits; a
   // column from across the wrap, where rho is mirrored, comes after the others at the low end, before them at
   // the high end), then the row (8 bits, from the column's first row).
   __device__ bool look(uint32_t jk, bool on, bool& win, uint32_t& at) const {
-    const int lane = threadIdx.x & 31, G = 1 << K.lg(), sub = lane & (G - 1), R = K.R, W = 2 * R + 1, NT = K.NT;
-    const int j = (int)(jk >> 16), k = (int)(jk & 0xffffu), c0 = max(0, k - R), c1 = min(K.NR - 1, k + R), n = c1 - c0 + 1;
+    const int lane = threadIdx.x & 31, G = 1 << lg(), sub = lane & (G - 1), W = 2 * R + 1;
+    const int j = (int)(jk >> 16), k = (int)(jk & 0xffffu), c0 = max(0, k - R), c1 = min(NR - 1, k + R), n = c1 - c0 + 1;
     uint32_t m = 0u;
     if (on) {
 #pragma unroll 1
@@ -378,7 +403,7 @@ struct WholeWindow {
         if ((unsigned)jj >= (unsigned)NT) {
           place -= jj < 0 ? W : -W;
           jj += jj < 0 ? NT : -NT;
-          r0 = K.NR - 1 - c1;
+          r0 = NR - 1 - c1;
         }
         const uint16_t* col = cell(jj, r0);
         uint32_t t = 0u;  // votes << 8 | 255 - row from the first
@@ -409,7 +434,7 @@ struct WholeWindow {
       int jj = j + a, r0 = c0;
       if ((unsigned)jj >= (unsigned)NT) {
         jj += jj < 0 ? NT : -NT;
-        r0 = K.NR - 1 - c1;
+        r0 = NR - 1 - c1;
       }
       const int r1 = r0 + n - 1, own = a == 0 ? k : -1;
       uint16_t* col = cell(jj, r0);
@@ -422,7 +447,7 @@ struct WholeWindow {
         if (w == (r0 >> 5)) x &= 0xffffffffu << (r0 & 31);
         if (w == (r1 >> 5)) x &= 0xffffffffu >> (31 - (r1 & 31));
         if (a == 0 && w == (k >> 5)) x &= ~(1u << (k & 31));
-        if (K.alive[jj * K.stride + w] & x) atomicAnd(&K.alive[jj * K.stride + w], ~x);
+        if (alive[jj * stride + w] & x) atomicAnd(&alive[jj * stride + w], ~x);
       }
     }
     return true;
@@ -760,8 +785,8 @@ struct EdgeWord {
 // Edge words of the tile's groups (the CTA's last 2 G threads). Before word 0 lies the theta wrap (word 0, rows mirrored:
 // from the top down, halves swapped), after the middle word itself (halves swapped), else the halo
 // (two contiguous columns of rows_phys words, of the words aw - 1 and aw + half; a tile owns words
-// [aw, aw + half), columns aw.. and their mirrors).
-__device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, EdgeWord* ew) {
+// [aw, aw + half), columns aw.. and their mirrors); without a halo, nothing (guard row 0, zero, throughout).
+__device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, bool halo, EdgeWord* ew) {
   const int G = (half + 31) >> 5, i = (int)(blockDim.x - 1 - threadIdx.x), rp = pl.rows_phys, acc0 = pl.off_acc >> 2, halo0 = pl.off_halo >> 2;
   if (i >= 2 * G) return;
   const int w = i & 1 ? min((i >> 1) * 32 + 32, half) : (i >> 1) * 32 - 1;
@@ -772,9 +797,11 @@ __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, Edg
     e.at += w < 0 ? mp_word(0, pl.n_rho + 1, rp) : mp_word(half - 1, 0, rp);
     e.step = w < 0 ? -32 : 32;
     e.swap = 1;
-  } else {
+  } else if (halo) {
     e.at = halo0 + (w < 0 ? 0 : rp);
     e.step = 1;
+  } else {
+    e.step = 0;
   }
   ew[i] = e;
 }
@@ -796,9 +823,8 @@ __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, Edg
 // candidates, of which the peaks are the 3x3 local maxima).
 template <bool CAND>
 __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int thr, int aw, int half, const EdgeWord* ew,
-                        uint32_t* pbits, uint32_t* cand, uint16_t* list, int* n_list, bool do_cs,
-                        unsigned long long& csum) {
-  const int NT = pl.n_theta, NR = pl.n_rho, rp = pl.rows_phys;
+                        uint32_t* pbits, uint32_t* cand, uint16_t* list, int* n_list) {
+  const int NR = pl.n_rho, rp = pl.rows_phys;
   const uint32_t* const sw = reinterpret_cast<const uint32_t*>(smem);
   const uint32_t* const acc = sw + (pl.off_acc >> 2);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -834,18 +860,6 @@ __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int thr, int 
         if (__any_sync(kFull, gs[i] < G && ((top - TT + 0x80008000u) & 0x80008000u) != 0u)) hit |= 1u << c;
         if (lane == c) mine = (uint32_t)(gs[i] << 8 | qs[i]);
         ++c;
-        if (do_cs && gs[i] < G) {
-          const int k = 4 * qs[i] + (lane >> 3), w = 32 * gs[i] + 4 * (lane & 7);
-          const uint32_t xs[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const unsigned a0 = xs[m] & 0xffffu, a1 = xs[m] >> 16;
-            if (k < NR && w + m < half) {
-              if (a0) csum += (unsigned long long)a0 * mix64((unsigned long long)(aw + w + m) * NR + k + 1);
-              if (a1) csum += (unsigned long long)a1 * mix64((unsigned long long)(NT - 1 - aw - w - m) * NR + k + 1);
-            }
-          }
-        }
       }
       if (c == 32 || g >= G) {
         int at = 0;
@@ -1246,13 +1260,18 @@ __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_
 
 struct ItemShared {
   WorkItem it[2];
-  EdgeWord edge[32];  // of at most 16 word groups
   int nv, flags, wide, last, total, D, reuse, n_amb, n_low;
   int kept_tot;
-  long long tstart[128];  // segment starts of the tile merge (2 segments a mirror-pair tile)
+  int tstart[129], tfrom[128];  // segments of the tile merge (2 a mirror-pair tile): starts, first records
   int tmp[32];
-  unsigned long long red[32];
-  int it_max, it_tq, it_ok, it_C, it_kept;  // iterative finder on theta tiles
+  union {
+    struct {
+      EdgeWord edge[32];  // of at most 16 word groups, for the scan
+      unsigned long long red[32];
+    };
+    int cnt4[128];  // the merge's counts (after both have been read)
+  };
+  int it_max, it_ok;  // iterative finder
 };
 
 // Word W of column P's peak rows dilated by +-hw (hw < 32) and cut to [0, N_rho): bit k is
@@ -1405,349 +1424,301 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
 
 // ---- the iterative finder (Sec. 2) on theta tiles ----
 
-// Maximum (returned to every thread; *s_max must be 0 beforehand) and, with do_cs, this thread's
-// part of the accumulator checksum over the tile's own cells.
-__device__ int tile_max_cs(const Plan& pl, const uint32_t* acc, int Wd, int aw, int wt, int j0, bool do_cs,
-                           int* s_max, unsigned long long& cs) {
-  const int NT = pl.n_theta, NR = pl.n_rho, lane = threadIdx.x & 31, warp = threadIdx.x >> 5,
-            nwarps = blockDim.x >> 5;
-  int m = 0;
-  if (pl.mp) {
-    for (int k = warp; k < NR; k += nwarps)
-      for (int w = lane; w < Wd; w += 32) {
-        const uint32_t x = acc[mp_word(w, k + 1, pl.rows_phys)];
-        const unsigned lo = x & 0xffffu, hi = x >> 16;
-        m = max(m, (int)max(lo, hi));
-        if (do_cs) {
-          if (lo) cs += (unsigned long long)lo * mix64((unsigned long long)(aw + w) * NR + k + 1);
-          if (hi) cs += (unsigned long long)hi * mix64((unsigned long long)(NT - 1 - aw - w) * NR + k + 1);
-        }
-      }
-  } else {
-    for (int k = warp; k < NR; k += nwarps)
-      for (int c = lane; c < wt; c += 32) {
-        const int v = acc_get(acc, c, k, pl.nrho_pad);
-        m = max(m, v);
-        if (do_cs && v) cs += (unsigned long long)v * mix64((unsigned long long)(j0 + c) * NR + k + 1);
-      }
+// This thread's part of the accumulator checksum over a mirror-pair tile's own cells.
+__device__ __noinline__ unsigned long long tile_checksum(const uint32_t* acc, int NT, int NR, int rp, int aw, int half) {
+  unsigned long long cs = 0;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < half * NR; i += blockDim.x) {
+    const int k = i / half, w = i - k * half;
+    const uint32_t x = acc[mp_word(w, k + 1, rp)];
+    cs += (unsigned long long)(x & 0xffffu) * mix64((unsigned long long)(aw + w) * NR + k + 1) +
+          (unsigned long long)(x >> 16) * mix64((unsigned long long)(NT - 1 - aw - w) * NR + k + 1);
   }
+  return cs;
+}
+
+// Maximum of a column tile (returned to every thread; *s_max must be 0 beforehand) and, with do_cs, this
+// thread's part of the accumulator checksum over the tile's own cells.
+__device__ int tile_max_cs(const Plan& pl, const uint32_t* acc, int wt, int j0, bool do_cs, int* s_max,
+                           unsigned long long& cs) {
+  const int NR = pl.n_rho, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  int m = 0;
+  for (int k = warp; k < NR; k += nwarps)
+    for (int c = lane; c < wt; c += 32) {
+      const int v = acc_get(acc, c, k, pl.nrho_pad);
+      m = max(m, v);
+      if (do_cs && v) cs += (unsigned long long)v * mix64((unsigned long long)(j0 + c) * NR + k + 1);
+    }
   m = __reduce_max_sync(kFull, m);
   if (lane == 0 && m) atomicMax(s_max, m);
   __syncthreads();
   return *s_max;
 }
 
-// Bit k of word (c, k >> 5) of pbits for every tile-local column c whose cell k holds >= tq votes
-// (tile-local columns as in the peak records: mirror-pair word w's low half is column w, its
-// high half column 2 Wd - 1 - w).
-__device__ void tile_candidate_bits(const Plan& pl, const uint32_t* acc, uint32_t* pbits, int Wd, int wt, int tq) {
-  const int NR = pl.n_rho, nrb = pl.nrb_p, lane = threadIdx.x & 31, warp = threadIdx.x >> 5,
-            nwarps = blockDim.x >> 5;
-  if (pl.mp) {
-    for (int k = warp; k < NR; k += nwarps)
-      for (int w = lane; w < Wd; w += 32) {
-        const uint32_t x = acc[mp_word(w, k + 1, pl.rows_phys)];
-        if ((int)(x & 0xffffu) >= tq) atomicOr(&pbits[w * nrb + (k >> 5)], 1u << (k & 31));
-        if ((int)(x >> 16) >= tq) atomicOr(&pbits[(2 * Wd - 1 - w) * nrb + (k >> 5)], 1u << (k & 31));
-      }
-  } else {
-    for (int k = warp; k < NR; k += nwarps)
-      for (int c = lane; c < wt; c += 32)
-        if (acc_get(acc, c, k, pl.nrho_pad) >= tq) atomicOr(&pbits[c * nrb + (k >> 5)], 1u << (k & 31));
-  }
+// Bit k of word (c, k >> 5) of pbits for every column c of a column tile whose cell k holds >= tq votes.
+__device__ void tile_candidate_bits(const Plan& pl, const uint32_t* acc, uint32_t* pbits, int wt, int tq) {
+  const int NR = pl.n_rho, nrb = pl.nrb_p, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  for (int k = warp; k < NR; k += nwarps)
+    for (int c = lane; c < wt; c += 32)
+      if (acc_get(acc, c, k, pl.nrho_pad) >= tq) atomicOr(&pbits[c * nrb + (k >> 5)], 1u << (k & 31));
 }
 
 __device__ __forceinline__ uint32_t cand_key(int v, int j, int k) {
   return ((uint32_t)v << 20) | ((uint32_t)(1023 - j) << 10) | (uint32_t)(1023 - k);
 }
 
-// Candidates of the iterative finder in sparse form: keys (cand_key) in raster order, colstart[j]
-// the first candidate of column j and colstart[NT] = C.
-struct SparseCands {
-  uint32_t* keys;
-  const int* colstart;
-  int C;
-};
-
-// Votes of a cell that is a candidate of a sparse list (the dense rounds only ask for candidates):
-// the row within its column's list by binary search.
-struct ListCells {
-  static constexpr bool kSorted = true;  // the rounds walk a column's list instead of searching each cell
+// The iterative finder's candidates as a list of keys (cand_key) in raster order, colstart[j] the first
+// one of column j and colstart[NT] = C, for resolve_kept: ids are places in the list, a window's column is a run of it
+// found by binary search over rows, and a key is a rank (votes, then raster order). A column a lane.
+struct ListWindow {
+  static constexpr int kVotes = 20;
   const uint32_t* keys;
   const int* colstart;
-  // first candidate of column j at row k or below it in the list (rows ascend), else the column's end
-  __device__ int lower(int j, int k) const {
-    int lo = colstart[j], hi = colstart[j + 1];
+  int NT, NR, R, C;
+  uint32_t *alive, *surv;  // a bit a candidate; alive has a word past its last
+  __device__ int radius() const { return R; }
+  __device__ int lg() const { return 2 * R + 1 <= 8 ? 3 : 2 * R + 1 <= 16 ? 4 : 5; }
+  __device__ int words() const { return (C + 31) >> 5; }
+  __device__ uint32_t id(int i, int b) const { return (uint32_t)(32 * i + b); }
+  __device__ uint32_t bit(uint32_t c, int& w) const {
+    w = (int)(c >> 5);
+    return 1u << (c & 31u);
+  }
+  template <class Word>
+  __device__ void list_bits(Word&& word, uint32_t* list, int room, int* n) const {
+    const int lane = threadIdx.x & 31, nw = words();
+#pragma unroll 1
+    for (int i0 = threadIdx.x - lane; i0 < nw; i0 += blockDim.x) {  // uniform a warp
+      const int i = i0 + lane;
+      uint32_t bits = i < nw ? word(i) : 0u;
+      int at = warp_positions(__popc(bits), n);
+#pragma unroll 1
+      while (bits) {
+        const int b = 31 - __clz(bits);
+        bits ^= 1u << b;
+        if (at < room) list[at] = (uint32_t)(32 * i + b);
+        ++at;
+      }
+    }
+  }
+  __device__ uint32_t key(uint32_t c) const { return keys[c]; }
+  __device__ void cell(uint32_t key, int& j, int& k) const {
+    j = 1023 - (int)((key >> 10) & 1023u);
+    k = 1023 - (int)(key & 1023u);
+  }
+  __device__ bool live(uint32_t c) const { return (alive[c >> 5] >> (c & 31u)) & 1u; }
+  // column j + a of the window of (j, k): its first candidate at or past the window's first row, the last of
+  // the window's rows, and the column's end
+  __device__ void column(int j, int k, int a, int& lo, int& r1, int& end) const {
+    int jj = j + a, r0 = max(0, k - R);
+    r1 = min(NR - 1, k + R);
+    if ((unsigned)jj >= (unsigned)NT) {  // across the theta wrap: the other end, rho mirrored
+      jj += jj < 0 ? NT : -NT;
+      const int t0 = NR - 1 - r1;
+      r1 = NR - 1 - r0;
+      r0 = t0;
+    }
+    lo = colstart[jj];
+    end = colstart[jj + 1];
+    int hi = end;
+#pragma unroll 1
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (1023 - (int)(keys[mid] & 1023u) < k) lo = mid + 1;
+      if (1023 - (int)(keys[mid] & 1023u) < r0) lo = mid + 1;
       else hi = mid;
     }
-    return lo;
   }
-  __device__ int end(int j) const { return colstart[j + 1]; }
-  __device__ uint32_t key(int p) const { return keys[p]; }
-  __device__ int get(int j, int k) const {
-    const int lo = lower(j, k);
-    return (lo < colstart[j + 1] && 1023 - (int)(keys[lo] & 1023u) == k) ? (int)(keys[lo] >> 20) : 0;
+  __device__ bool look(uint32_t c, bool on, bool& win, uint32_t& at) const {
+    const int lane = threadIdx.x & 31, G = 1 << lg(), sub = lane & (G - 1);
+    uint32_t m = 0u;
+    int j = 0, k = 0, lo = 0, n = 0;  // of this lane's last column: its run in the window
+    if (on) {
+      cell(keys[c], j, k);
+#pragma unroll 1
+      for (int a = sub - R; a <= R; a += G) {
+        int r1, end;
+        column(j, k, a, lo, r1, end);
+        n = 0;
+#pragma unroll 1
+        for (bool in = true; in; n += 4) {  // four independent reads (past the run: not counted)
+          const uint32_t f = __funnelshift_r(alive[(lo + n) >> 5], alive[((lo + n) >> 5) + 1], (lo + n) & 31);
+          uint32_t x[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) x[i] = keys[min(lo + n + i, C - 1)];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            in = in && lo + n + i < end && 1023 - (int)(x[i] & 1023u) <= r1;
+            if (in && ((f >> i) & 1u) && x[i] > m) {
+              m = x[i];
+              at = (uint32_t)(lo + n + i);
+            }
+          }
+        }
+      }
+    }
+    uint32_t top = m;
+    for (int o = 1; o < G; o <<= 1) top = max(top, __shfl_xor_sync(kFull, top, o));
+    win = on && m == top;  // keys are distinct: one lane
+    const unsigned self = __ballot_sync(kFull, win && at == c);
+    if (!((self >> (lane & ~(G - 1))) & (0xffffffffu >> (32 - G)))) return false;
+#pragma unroll 1
+    for (int a = sub - R; a <= R; a += G) {
+      int r1, end;
+      column(j, k, a, lo, r1, end);
+#pragma unroll 1
+      for (int i = lo; i < end && 1023 - (int)(keys[i] & 1023u) <= r1; ++i)
+        if (i != (int)c) atomicAnd(&alive[i >> 5], ~(1u << (i & 31)));
+    }
+    return true;
   }
 };
 
-// Visits every other candidate in the suppression window of candidate i (columns j - R .. j + R
-// and rows k - R .. k + R; a column past either end of the theta range is taken from the other end
-// with the rows mirrored, rows beyond the rho edges do not exist), each column's rows found by a
-// binary search; visit(m, key_m) returns false to stop.
-template <class V>
-__device__ __forceinline__ void visit_window(const SparseCands& s, int NT, int NR, int R, int i, V&& visit) {
-  const uint32_t key = s.keys[i];
-  const int j = 1023 - (int)((key >> 10) & 1023u), k = 1023 - (int)(key & 1023u);
-  for (int d = -R; d <= R; ++d) {
-    int jj = j + d, r0 = max(0, k - R), r1 = min(NR - 1, k + R);
-    if (jj < 0 || jj >= NT) {
-      jj = jj < 0 ? jj + NT : jj - NT;
-      const int q0 = NR - 1 - r1;
-      r1 = NR - 1 - r0;
-      r0 = q0;
-    }
-    int lo = s.colstart[jj];
-    const int end = s.colstart[jj + 1];
-    int hi = end;
-    while (lo < hi) {  // first candidate of column jj at a row >= r0
-      const int mid = (lo + hi) >> 1;
-      if (1023 - (int)(s.keys[mid] & 1023u) < r0) lo = mid + 1;
-      else hi = mid;
-    }
-    for (int m = lo; m < end; ++m) {
-      const uint32_t km = s.keys[m];
-      if (1023 - (int)(km & 1023u) > r1) break;
-      if (m != i && !visit(m, km)) return;
-    }
-  }
-}
-
-// The iterative finder's peaks from its candidates (Sec. 2: the best unsuppressed cell is the next
-// peak and suppresses its window, until the best fails the threshold). The passes keep exactly the
-// candidates that no kept higher-ranked candidate covers, listed by rank; the window relation is
-// symmetric, so a candidate's dominators are the higher-ranked candidates in its own window. They
-// are listed once per candidate (CSR, in work when it fits; else every round rescans the window).
-// Rounds then settle the candidates in parallel: dropped once a dominator is kept, kept once every
-// dominator is dropped; every round settles at least the best undecided one. The kept keys,
-// compacted into the front of keys and ordered by rank (bitonic within keys_room, else by
-// counting), are stored to dst (the first maxp); returns their count. All threads call it.
-__device__ int resolve_sparse(const Plan& pl, const SparseCands& s, int keys_room, unsigned char* work,
-                              int work_bytes, hough_peak* dst, ItemShared& sh) {
-  const int NT = pl.n_theta, NR = pl.n_rho, R = pl.nms_radius, maxp = pl.max_peaks, C = s.C;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x, nwarps = bd >> 5;
-  volatile uint8_t* st = work;  // 1 undecided, 2 dropped, 3 kept
-  const int st_bytes = (C + 15) & ~15, doff_words = (C + 4) & ~3;
-  int* doff = reinterpret_cast<int*>(work + st_bytes);
-  uint16_t* dom = reinterpret_cast<uint16_t*>(doff + doff_words);  // candidate indices (C < 65536)
-  const long long dom_cap = ((long long)work_bytes - st_bytes - 4LL * doff_words) / 2;
-  bool csr = dom_cap >= 0;
-  if (csr) {
-    for (int i = tid; i < C; i += bd) {
-      const uint32_t key = s.keys[i];
-      int cnt = 0;
-      visit_window(s, NT, NR, R, i, [&](int, uint32_t km) {
-        cnt += km > key;
-        return true;
-      });
-      doff[i] = cnt;
-    }
-    __syncthreads();
-    const int E = block_exscan(doff, C, sh.tmp);
-    if (tid == 0) doff[C] = E;
-    csr = E <= dom_cap;  // uniform
-    __syncthreads();
-  }
-  if (csr) {
-    for (int i = tid; i < C; i += bd) {
-      const uint32_t key = s.keys[i];
-      int t = doff[i];
-      visit_window(s, NT, NR, R, i, [&](int m, uint32_t km) {
-        if (km > key) dom[t++] = (uint16_t)m;
-        return true;
-      });
-      st[i] = doff[i + 1] == doff[i] ? 3 : 1;  // no dominator: kept at once
-    }
-  } else {
-    for (int i = tid; i < C; i += bd) st[i] = 1;
-  }
-  if (tid < 3) sh.tmp[tid] = 0;
-  __syncthreads();
-  for (int round = 0;; ++round) {
-    int und = 0;
-    for (int i = tid; i < C; i += bd) {
-      if (st[i] != 1) continue;
-      bool drop = false, all = true;
-      if (csr) {
-        for (int t = doff[i], t1 = doff[i + 1]; t < t1; ++t) {
-          const uint8_t sd = st[dom[t]];
-          if (sd == 3) {
-            drop = true;
-            break;
-          }
-          all = all && sd != 1;
-        }
-      } else {
-        const uint32_t key = s.keys[i];
-        visit_window(s, NT, NR, R, i, [&](int m, uint32_t km) {
-          const uint8_t sm = st[m];
-          if (sm == 3) {  // a kept candidate in the window always ranks above this one
-            drop = true;
-            return false;
-          }
-          if (sm == 1 && km > key) all = false;
-          return true;
-        });
+// The segments that the last tile CTA of an event merges: starts of the low segments in tile order, then
+// (mirror-pair tiles) of the high ones in reverse tile order, in sh.tstart (nseg + 1 of them, the last the event's total),
+// each segment's first record in its tile's slot in sh.tfrom; the event's checksum in sh.red[0], the tiles' largest
+// cell in sh.it_max, and in sh.it_ok whether every tile's records fit its slot. One warp reads all counts
+// at once (a thread alone: a chain of 2 to 6 L2 reads a tile).
+template <bool MP>
+__device__ void merge_segments(const Plan& pl, const FusedIO& io, ItemShared& sh, long long e, bool do_cs) {
+  const int T = pl.tiles, nseg = MP ? 2 * T : T, lane = threadIdx.x & 31;
+  if (threadIdx.x >= 32) return;
+  int ct[4], sum = 0, top = 0;
+  bool ok = true;
+  unsigned long long cs = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int sg = 4 * lane + i, tt = sg < T ? sg : 2 * T - 1 - sg;
+    ct[i] = 0;
+    if (sg < nseg) {
+      const int2 c = __ldcg(reinterpret_cast<const int2*>(io.tile_cnt) + e * T + tt);  // records, low ones
+      ct[i] = sg < T ? c.y : c.x - c.y;
+      sh.tfrom[sg] = sg < T ? 0 : c.y;
+      ok = ok && c.x <= pl.max_peaks;
+      if (sg < T) {
+        if (do_cs) cs += __ldcg(io.tile_cs + e * T + tt);
+        if (io.tile_max) top = max(top, __ldcg(io.tile_max + e * T + tt));
       }
-      if (drop) st[i] = 2;
-      else if (all) st[i] = 3;
-      else ++und;
     }
-    // undecided count: three rotating counters, so that one barrier a round suffices
-    const int r3 = round % 3;
-    und = __reduce_add_sync(kFull, und);
-    if (lane == 0 && und) atomicAdd(&sh.tmp[r3], und);
-    if (tid == 0) sh.tmp[(r3 + 1) % 3] = 0;
-    __syncthreads();
-    if (sh.tmp[r3] == 0) break;
+    sum += ct[i];
   }
-  HOUGH_PHASE(HOUGH_PHASE_IT_RESOLVE);
-  // the kept keys, compacted in place into the front of keys
-  if (tid == 0) sh.it_kept = 0;
-  __syncthreads();
-  for (int i0 = 0; i0 < C; i0 += bd) {
-    const int i = i0 + tid;
-    const bool kept = i < C && st[i] == 3;
-    const uint32_t key = kept ? s.keys[i] : 0u;
-    const unsigned bal = __ballot_sync(kFull, kept);
-    if (lane == 0) sh.tmp[warp] = __popc(bal);
-    __syncthreads();
-    int before = 0, chunk = 0;
-    for (int w = 0; w < nwarps; ++w) {
-      const int c = sh.tmp[w];
-      before += w < warp ? c : 0;
-      chunk += c;
-    }
-    if (kept) s.keys[sh.it_kept + before + __popc(bal & lanemask_lt())] = key;
-    __syncthreads();
-    if (tid == 0) sh.it_kept += chunk;
-    __syncthreads();
+  int at = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(kFull, at, o);
+    if (lane >= o) at += y;
   }
-  const int nk = sh.it_kept;
-  int N = 32;
-  while (N < nk) N <<= 1;
-  if (nk > 256 && N <= keys_room) {
-    for (int i = nk + tid; i < N; i += bd) s.keys[i] = 0u;
-    __syncthreads();
-    bitonic_desc(s.keys, N);
-    for (int i = tid; i < min(nk, maxp); i += bd) store_peak(dst + i, s.keys[i]);
-  } else {  // rank = the kept keys above it (keys are distinct)
-    for (int i = tid; i < nk; i += bd) {
-      const uint32_t key = s.keys[i];
-      int r = 0;
-      for (int m = 0; m < nk; ++m) r += s.keys[m] > key;
-      if (r < maxp) store_peak(dst + r, key);
-    }
+  at -= sum;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (4 * lane + i <= nseg) sh.tstart[4 * lane + i] = at;
+    at += ct[i];
   }
-  __syncthreads();
-  HOUGH_PHASE(HOUGH_PHASE_IT_ORDER);
-  return nk;
+  if (lane == 31 && nseg == 128) sh.tstart[128] = at;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) cs += __shfl_xor_sync(kFull, cs, o);
+  top = __reduce_max_sync(kFull, top);
+  ok = __all_sync(kFull, ok);
+  if (lane == 0) {
+    sh.red[0] = cs;
+    sh.it_max = top;
+    sh.it_ok = ok;
+  }
 }
 
-// The event's peaks from its tiles' candidate lists, in the last tile CTA of the event. The
-// event's threshold tq = max(T, ceil(rel max)) comes from the tiles' maxima. The candidates (cells
-// >= tq) are gathered in raster order, with the first candidate of every column (colstart), into
-// the CTA's free shared memory, and settled in rounds as in the untiled finder (a candidate is
-// dropped once a kept candidate lies in its window, kept once every higher-ranked candidate in
-// its window is dropped), each window looked up column by column by binary search over rows.
-// The kept ones, sorted by rank, are the peaks in extraction order. Returns their count, or -1
-// (nothing written) when a tile could not publish all its candidates or they exceed the room.
+// Record i of the event's merged segments: where it lies in the tiles' slots.
+__device__ __forceinline__ const hough_peak* merged_record(const Plan& pl, const FusedIO& io, const ItemShared& sh,
+                                                           long long e, int nseg, int i) {
+  int lo = 0, hi = nseg - 1;  // the last segment that starts at or before i
+#pragma unroll 1
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (sh.tstart[mid] <= i) lo = mid;
+    else hi = mid - 1;
+  }
+  const int tt = lo < pl.tiles ? lo : 2 * pl.tiles - 1 - lo;
+  return io.tile_peaks + (e * pl.tiles + tt) * (long long)pl.max_peaks + sh.tfrom[lo] + (i - sh.tstart[lo]);
+}
+
+// The event's peaks from its tiles' candidate lists, in the last tile CTA of the event (after
+// merge_segments). The event's threshold tq = max(T, ceil(rel max)) comes from the tiles' maxima. The
+// candidates (cells >= tq) are gathered in raster order, with the first candidate of every column (colstart),
+// into the CTA's free shared memory, and their kept set is found and ranked there (resolve_kept; the tiles
+// marked the local maxima among them). Returns their count, or -1 (nothing written) when a tile could
+// not publish all its candidates, a cell has more votes than a key holds, or there is no room.
+// Stress events (512 x 512, 16,100 candidates): 730 k cycles with rounds on two state bits a cell, their ranking included; so
+// 389 k.
+template <bool MP>
 __device__ int merge_iterative(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, long long e) {
-  const int T = pl.tiles, NT = pl.n_theta, NR = pl.n_rho, R = pl.nms_radius, maxp = pl.max_peaks;
+  const int T = pl.tiles, NT = pl.n_theta, NR = pl.n_rho, maxp = pl.max_peaks, cap = pl.merge_cap;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x, nwarps = bd >> 5;
-  const int nseg = pl.mp ? 2 * T : T, cap = pl.merge_cap;
+  const int nseg = MP ? 2 * T : T, total = sh.tstart[nseg], amax = sh.it_max;
+  if (!sh.it_ok || amax > 4095) return -1;  // uniform; a key holds votes in 12 bits
+  const int tq = (int)max((long long)pl.threshold, ((long long)pl.rel_num * amax + pl.rel_den - 1) / pl.rel_den);
   int* colstart = reinterpret_cast<int*>(smem + pl.off_acc);  // NT + 1
-  uint32_t* keys = reinterpret_cast<uint32_t*>(colstart + ((NT + 4) & ~3));
-  if (tid == 0) {
-    int M = 0;
-    bool ok = true;
-    long long run = 0;
-    for (int tt = 0; tt < T; ++tt) {
-      M = max(M, __ldcg(io.tile_max + e * T + tt));
-      ok = ok && __ldcg(io.tile_cnt + 2 * (e * T + tt)) <= maxp;
+  uint32_t* surv = reinterpret_cast<uint32_t*>(colstart + ((NT + 4) & ~3));
+  const int bw = (cap + 63) >> 5;  // bitmap words, one past the last
+  uint32_t* alive = surv + bw;
+  uint32_t* keys = alive + bw;
+  for (int i = tid; i < bw; i += bd) surv[i] = 0u;
+  // gather the candidates >= tq, in order, four a thread at a time (their reads go to the L2 together)
+  int C = 0;
+#pragma unroll 1
+  for (int i0 = 0; i0 < total; i0 += 4 * bd) {
+    uint32_t key[4];
+    bool keep[4], local[4];
+    int before[4];
+    __syncthreads();  // surv is zero, sh.tmp free
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int i = i0 + m * bd + tid;
+      int2 r = make_int2(0, 0);
+      if (i < total) r = __ldcg(reinterpret_cast<const int2*>(merged_record(pl, io, sh, e, nseg, i)));
+      const int j = r.x & 0xffff, k = (r.x >> 16) & 0xffff, v = r.y & 0xffff;
+      keep[m] = i < total && v >= tq;
+      local[m] = (r.y >> 16) != 0;
+      key[m] = cand_key(v, j, k);
     }
-    for (int sg = 0; sg < nseg; ++sg) {
-      const int tt = sg < T ? sg : 2 * T - 1 - sg;
-      const int all = __ldcg(io.tile_cnt + 2 * (e * T + tt)), lo = __ldcg(io.tile_cnt + 2 * (e * T + tt) + 1);
-      sh.tstart[sg] = run;
-      run += sg < T ? lo : all - lo;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const unsigned bal = __ballot_sync(kFull, keep[m]);
+      before[m] = __popc(bal & lanemask_lt());
+      if (lane == 0) sh.cnt4[m * 32 + warp] = __popc(bal);
     }
-    const long long need = ((long long)pl.rel_num * M + pl.rel_den - 1) / pl.rel_den;
-    sh.it_tq = (int)max((long long)pl.threshold, need);
-    sh.it_ok = ok && M <= 4095 ? 1 : 0;  // a key holds votes in 12 bits
-    sh.it_C = 0;
-  }
-  __syncthreads();
-  if (!sh.it_ok) return -1;  // uniform
-  const int tq = sh.it_tq;
-  // gather the candidates >= tq, in order
-  for (int sg = 0; sg < nseg; ++sg) {
-    const int tt = sg < T ? sg : 2 * T - 1 - sg;
-    const int all = __ldcg(io.tile_cnt + 2 * (e * T + tt)), lo = __ldcg(io.tile_cnt + 2 * (e * T + tt) + 1);
-    const int from = sg < T ? 0 : lo, ct = sg < T ? lo : all - lo;
-    const hough_peak* src = io.tile_peaks + (e * T + tt) * (long long)maxp + from;
-    for (int i0 = 0; i0 < ct; i0 += bd) {
-      const int i = i0 + tid;
-      uint32_t key = 0;
-      bool keep = false;
-      if (i < ct) {
-        const int2 r = __ldcg(reinterpret_cast<const int2*>(src) + i);
-        const int j = r.x & 0xffff, k = (r.x >> 16) & 0xffff, v = r.y & 0xffff;
-        keep = v >= tq;
-        key = cand_key(v, j, k);
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int c = lane < nwarps ? sh.cnt4[m * 32 + lane] : 0;
+      const int pos = C + __reduce_add_sync(kFull, lane < warp ? c : 0) + before[m];
+      C += __reduce_add_sync(kFull, c);
+      if (keep[m] && pos < cap) {
+        keys[pos] = key[m];
+        if (local[m]) atomicOr(&surv[pos >> 5], 1u << (pos & 31));
       }
-      const unsigned bal = __ballot_sync(kFull, keep);
-      if (lane == 0) sh.tmp[warp] = __popc(bal);
-      __syncthreads();
-      int before = 0, chunk = 0;
-      for (int w = 0; w < nwarps; ++w) {
-        const int c = sh.tmp[w];
-        before += w < warp ? c : 0;
-        chunk += c;
-      }
-      const int pos = sh.it_C + before + __popc(bal & lanemask_lt());
-      if (keep && pos < cap) keys[pos] = key;
-      __syncthreads();
-      if (tid == 0) sh.it_C += chunk;
-      __syncthreads();
     }
   }
-  const int C = sh.it_C;
   if (C > cap) return -1;  // uniform
-  // first candidate of every column (keys are in raster order)
-  for (int j = tid; j <= NT; j += bd) colstart[j] = 0;
   __syncthreads();
-  for (int i = tid; i < C; i += bd) atomicAdd(&colstart[1023 - (int)((keys[i] >> 10) & 1023u)], 1);
-  __syncthreads();
-  block_exscan(colstart, NT + 1, sh.tmp);
-  const SparseCands sc{keys, colstart, C};
-  unsigned char* work = reinterpret_cast<unsigned char*>(keys + C);
-  const int work_bytes = (int)(smem + pl.smem_bytes - work);
-  hough_peak* dst = io.peaks + e * (long long)maxp;
-  // the rounds on a 2-bit state per cell of the event where that map fits (512 x 512: 64 KB);
-  // the rank of an undecided neighbour comes from its key, found by binary search in its column
-  int stw = 32;
-  while (stw < ((NT * NR + 15) >> 4)) stw <<= 1;
-  if (4LL * stw <= work_bytes) {
-    ListCells lc{keys, colstart};
-    const int act_cap = (int)min(2048LL, (work_bytes - 4LL * stw) / 4);  // two lists of 16-bit indices
-    const int n = resolve_rounds(lc, NT, NR, R, 0, maxp, keys, C, reinterpret_cast<uint32_t*>(work), stw,
-                                 reinterpret_cast<uint16_t*>(work + 4LL * stw), act_cap, dst, sh.tmp);
-    if (n >= 0) return n;  // else (past 64 rounds) the sparse form, which needs only keys and colstart
+  for (int i = tid; i < bw; i += bd) alive[i] = 32 * i + 32 <= C ? 0xffffffffu : 32 * i < C ? (1u << (C & 31)) - 1u : 0u;
+  // first candidate of every column (keys are in raster order): where the column changes
+  for (int i = tid; i <= C; i += bd) {
+    const int j1 = i < C ? 1023 - (int)((keys[i] >> 10) & 1023u) : NT;
+    const int j0 = i > 0 ? 1023 - (int)((keys[i - 1] >> 10) & 1023u) : -1;
+    for (int j = j0 + 1; j <= j1; ++j) colstart[j] = i;
   }
-  return resolve_sparse(pl, sc, cap, work, work_bytes, dst, sh);
+  __syncthreads();
+  uint32_t* list = reinterpret_cast<uint32_t*>((reinterpret_cast<uintptr_t>(keys + C) + 15) & ~(uintptr_t)15);
+  // the lists up to the staged hits, which the selection reads again; over them only where they would be short
+  int ucap = (int)((smem + pl.off_hits - reinterpret_cast<unsigned char*>(list)) / 10);
+  if (ucap < max(1024, C >> 1)) {
+    ucap = (int)((smem + pl.smem_bytes - reinterpret_cast<unsigned char*>(list)) / 10);
+    if (tid == 0) sh.reuse = 0;  // (read after the barriers below)
+  }
+  ucap = min(32768, ucap) & ~15;
+  const ListWindow lw{keys, colstart, NT, NR, pl.nms_radius, C, alive, surv};
+  const int nk = resolve_kept(lw, list, ucap, reinterpret_cast<uint16_t*>(list + 2 * ucap), sh.tmp);
+  if (nk > ranked_room(2 * ucap)) return -1;  // uniform
+  store_ranked(lw, list, 2 * ucap, nk, amax, tq, maxp, io.peaks + e * (long long)maxp);
+  return nk;
 }
 
 // Steps 1-2 of a work item: clears the CTA's accumulator of theta tile t (with the halo columns,
@@ -1856,7 +1827,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
       if (sh.wide & 2) sh.flags |= HOUGH_F_BAD_HIT;
       if (sh.wide & 1) sh.reuse = 0;  // wide hits are not in the staged list
     }
-    if (MP && (want_halo || T == 1) && h0 == 0) edge_words(pl, aw, Wd, sh.edge);  // for the scan (no hits: no candidates)
+    if (MP && h0 == 0) edge_words(pl, aw, Wd, want_halo, sh.edge);  // for the scan (no hits: no candidates)
     if (!(sh.wide & 1)) {
       if (mp_halo) halo_mp32(pl, HL, hb, sh.nv);
       if (MP)
@@ -1979,16 +1950,12 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       const int tq = (int)max((long long)pl.threshold, ((long long)pl.rel_num * amax + pl.rel_den - 1) / pl.rel_den);
       uint32_t* cand = pbits + pl.groups * 32 * pl.nrb_p;
       uint32_t* list = cand + pl.groups * 32 * pl.nrb_p;
-      unsigned long long none = 0;
-      scan_mp<true>(pl, smem, tq, 0, Wd, sh.edge, pbits, cand, reinterpret_cast<uint16_t*>(list), &sh.n_amb, false, none);
+      scan_mp<true>(pl, smem, tq, 0, Wd, sh.edge, pbits, cand, reinterpret_cast<uint16_t*>(list), &sh.n_amb);
       __syncthreads();
-      const WholeWindow ww{acc, Wd, pl.rows_phys, tq,
-                           KeptSet{NT, NR, pl.nms_radius, pl.nrb_p, pl.iter_cap, cand, pbits, list,
-                                   reinterpret_cast<uint16_t*>(list + 2 * pl.iter_cap), sh.tmp}};
-      const int nk = resolve_kept(ww.K, [&](uint32_t jk, bool on, bool& win, uint32_t& at) { return ww.look(jk, on, win, at); },
-                                  [&](uint32_t jk) { return ww.live(jk); });
+      const WholeWindow ww{acc, Wd, pl.rows_phys, NT, NR, pl.nms_radius, pl.nrb_p, cand, pbits};
+      const int nk = resolve_kept(ww, list, pl.iter_cap, reinterpret_cast<uint16_t*>(list + 2 * pl.iter_cap), sh.tmp);
       if (nk <= ranked_room(2 * pl.iter_cap)) {
-        store_ranked(ww, NR, list, 2 * pl.iter_cap, nk, amax, tq, 17, maxp, dst);  // at most 227 KB / 2 cells: 17 bits, and 15 of votes
+        store_ranked(ww, list, 2 * pl.iter_cap, nk, amax, tq, maxp, dst);
         total = nk;
       }
     }
@@ -2008,24 +1975,32 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // 3. peak scan, or (the iterative finder on theta tiles) the tile's candidates: every cell
     // at or above the tile's own relative threshold, a superset of the cells the event's
     // threshold admits (the event's maximum is at least the tile's)
+    // (mirror pairs: with the 3x3 local maxima among them marked; at a tile's edges some that are none, since
+    // the neighbour columns of other tiles count as empty there)
     unsigned long long csum = 0;
     const bool packed = !MP && (NR & 1) == 0;
-    if (ITER) {
-      if (MP) {
-        mp_fold(pl, acc, Wd, nullptr);
-        __syncthreads();
-        HOUGH_PHASE(HOUGH_PHASE_FOLD);
-      }
-      tmax = tile_max_cs(pl, acc, Wd, aw, wt, j0, do_cs, &sh.it_max, csum);
-      const long long need = ((long long)pl.rel_num * tmax + pl.rel_den - 1) / pl.rel_den;
-      tile_candidate_bits(pl, acc, pbits, Wd, wt, (int)max((long long)pl.threshold, need));
+    uint32_t* local = pl.off_local ? reinterpret_cast<uint32_t*>(smem + pl.off_local) : pbits;  // no room: none marked
+    if (ITER && MP) {
+      mp_fold(pl, acc, Wd, nullptr);
+      if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
+      if (pl.off_local)
+        for (int i = tid; i < pl.groups * 32 * pl.nrb_p; i += bd) local[i] = 0u;
+      __syncthreads();
+      HOUGH_PHASE(HOUGH_PHASE_FOLD);
+      tmax = acc_max_mp(pl, acc, Wd, &sh.it_max);
+      if (do_cs) csum = tile_checksum(acc, NT, NR, pl.rows_phys, aw, Wd);
+      const int tq = (int)max((long long)pl.threshold, ((long long)pl.rel_num * tmax + pl.rel_den - 1) / pl.rel_den);
+      scan_mp<true>(pl, smem, tq, aw, Wd, sh.edge, local, pbits, reinterpret_cast<uint16_t*>(halo), &sh.n_amb);
+    } else if (ITER) {
+      tmax = tile_max_cs(pl, acc, wt, j0, do_cs, &sh.it_max, csum);
+      tile_candidate_bits(pl, acc, pbits, wt, (int)max((long long)pl.threshold, ((long long)pl.rel_num * tmax + pl.rel_den - 1) / pl.rel_den));
     } else if (MP) {
       mp_fold(pl, acc, Wd, T > 1 ? halo : nullptr);
       if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
       __syncthreads();
       HOUGH_PHASE(HOUGH_PHASE_FOLD);
-      scan_mp<false>(pl, smem, pl.threshold, aw, Wd, sh.edge, pbits, nullptr, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb,
-                     do_cs, csum);
+      if (do_cs) csum = tile_checksum(acc, NT, NR, pl.rows_phys, aw, Wd);
+      scan_mp<false>(pl, smem, pl.threshold, aw, Wd, sh.edge, pbits, nullptr, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb);
     } else if (packed) {
       scan_packed(pl, acc, halo, pbits, wt, T, j0, do_cs, csum);
     } else {
@@ -2098,7 +2073,9 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
           const int k = k0 + __ffs(bits) - 1;
           bits &= bits - 1u;
           const int votes = MP ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
-          dst2[pos++] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes);
+          uint32_t lm = 0u;
+          if (ITER && MP && pl.off_local) lm = (local[c * pl.nrb_p + (k >> 5)] >> (k & 31)) & 1u;
+          dst2[pos++] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes | (lm << 16));
         }
       }
     } else {
@@ -2113,7 +2090,9 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
             const int k = (w << 5) + bb;
             const int votes = MP ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
             const int col = MP ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
-            dst2[pos] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes);
+            uint32_t lm = 0u;
+            if (ITER && MP && pl.off_local) lm = (local[c * pl.nrb_p + w] >> bb) & 1u;
+            dst2[pos] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes | (lm << 16));
             ++pos;
           }
         }
@@ -2150,16 +2129,11 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // tiles) their high segments in reverse tile order. Segment s < T is tile s's records
     // [0, lo); segment T + i is tile T-1-i's records [lo, all).
     const int nseg = MP ? 2 * T : T;
+    merge_segments<MP>(pl, io, sh, e, do_cs);
+    __syncthreads();
+    ev_cs = sh.red[0];
     if (ITER) {
-      ev_total = merge_iterative(pl, io, smem, sh, e);
-      if (tid == 0) {
-        unsigned long long csa = 0;
-        if (do_cs)
-          for (int tt = 0; tt < T; ++tt) csa += __ldcg(io.tile_cs + e * T + tt);
-        sh.red[0] = csa;
-      }
-      __syncthreads();
-      ev_cs = sh.red[0];
+      ev_total = merge_iterative<MP>(pl, io, smem, sh, e);
       if (ev_total < 0) {  // deferred: the fallback kernel writes this event's outputs
         if (tid == 0) {
           if (io.checksum) io.checksum[e] = ev_cs;
@@ -2169,36 +2143,11 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         return;
       }
     } else {
-    if (tid == 0) {
-      long long run = 0;
-      unsigned long long csa = 0;
-      for (int sg = 0; sg < nseg; ++sg) {
-        const int tt = sg < T ? sg : 2 * T - 1 - sg;
-        const int all = __ldcg(io.tile_cnt + 2 * (e * T + tt)), lo = __ldcg(io.tile_cnt + 2 * (e * T + tt) + 1);
-        sh.tstart[sg] = run;
-        run += sg < T ? lo : all - lo;
-        if (do_cs && sg < T) csa += __ldcg(io.tile_cs + e * T + tt);
-      }
-      sh.total = (int)run;
-      sh.red[0] = csa;
-    }
-    __syncthreads();
-    ev_total = sh.total;
-    ev_cs = sh.red[0];
-    hough_peak* out = io.peaks + e * (long long)maxp;
-    for (int sg = 0; sg < nseg; ++sg) {
-      const int tt = sg < T ? sg : 2 * T - 1 - sg;
-      const int all = __ldcg(io.tile_cnt + 2 * (e * T + tt)), lo = __ldcg(io.tile_cnt + 2 * (e * T + tt) + 1);
-      const int from = sg < T ? 0 : lo, ct = sg < T ? lo : all - lo;
-      const long long st0 = sh.tstart[sg];
-      const int ncopy = (int)max(0LL, min((long long)ct, (long long)maxp - st0));
-      const hough_peak* src = io.tile_peaks + (e * T + tt) * (long long)maxp + from;
-      for (int i = tid; i < ncopy; i += bd) {
-        const int2 v = __ldcg(reinterpret_cast<const int2*>(src) + i);
-        reinterpret_cast<int2*>(out)[st0 + i] = v;
-      }
-    }
-    __syncthreads();
+      ev_total = sh.tstart[nseg];
+      hough_peak* out = io.peaks + e * (long long)maxp;
+      for (int i = tid; i < min(ev_total, maxp); i += bd)
+        reinterpret_cast<int2*>(out)[i] = __ldcg(reinterpret_cast<const int2*>(merged_record(pl, io, sh, e, nseg, i)));
+      __syncthreads();
     }
   }
 

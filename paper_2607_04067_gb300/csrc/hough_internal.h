@@ -49,6 +49,7 @@ struct Plan {
   // iterative finder on theta tiles: candidate keys the merging CTA holds; slice height and
   // candidate keys of the deferred kernel's finder
   int merge_cap, def_sh, def_cap;
+  int off_local;  // iterative finder on mirror-pair tiles: bitmap of the candidates' 3x3 local maxima (0: no room)
   int off_amb, amb_cap;  // list of ambiguous vote steps (shares a region that the vote leaves free) and its entries
   // shared-memory layout in bytes
   int off_acc, region_bytes, off_halo, off_hits, off_idx, off_pbits, off_cnt, off_unres, off_trig, smem_bytes;

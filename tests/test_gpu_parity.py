@@ -580,6 +580,25 @@ def test_iterative_stepwise_large_accumulator(h):
         assert np.array_equal(got[e][: min(n[e], 256)], exp[e][: min(n[e], 256)])
 
 
+@pytest.mark.parametrize("nt,nr,thr,num,den,R,tiles", [
+    (256, 256, 1, 0, 1, 1, 1),    # more undecided candidates than are listed, more peaks than are ranked at once
+    (256, 256, 2, 0, 1, 8, 1),    # a window of more than 16 columns; candidates by bitmap words
+    (130, 90, 4, 1, 3, 20, 1),    # more columns than lanes, taller than a bitmap word
+    (256, 256, 60, 1, 1, 3, 1),   # the maximum's own votes: few candidates, or none
+    (256, 256, 2, 0, 1, 2, 4),    # candidate lists that leave no room beside the staged hits
+    (256, 200, 4, 1, 4, 8, 64),   # 128 segments to merge
+    (250, 64, 3, 1, 3, 1, 8),     # tiles of uneven width
+    (255, 64, 3, 1, 3, 4, 5),     # column tiles: no local maxima marked
+])
+def test_iterative_edges(h, nt, nr, thr, num, den, R, tiles):
+    """Whole and tiled finders where their lists, windows and merges have their edges; two events of one and
+    no hits among the others."""
+    ev = gen.generate(gen.CONFIGS["plain_paper"], 3)
+    a = int(ev.off[1])
+    xy, off = ev.xy, np.array([0, a, a, a + 1, int(ev.off[2]), int(ev.off[3])], np.int64)
+    run_iterative_tiled(h, xy, off, nt, nr, thr, num, den, R, 20000, tiles)
+
+
 # ---------------------------------------------------------------- iterative finder on theta tiles
 
 ITER_TILED = [  # (workload, events, n_theta, n_rho, threshold, rel_num, rel_den, nms_radius, max_peaks, tiles)
