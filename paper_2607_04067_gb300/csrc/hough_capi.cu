@@ -93,6 +93,18 @@ static constexpr int kSmemBudget = 227 * 1024 - 2048;  // dynamic bytes; static 
 static int round16(int x) { return (x + 15) & ~15; }
 
 // Shared-memory layout for a shape; returns false if it does not fit.
+static bool layout(Plan& pl, bool local);
+
+// The layout with more hits staged whole (up to 7,168, so that events above 4,096 hits take one chunk and their
+// selection reads the staged ones) where a CTA fills an SM in any case.
+static void stage_more(Plan& pl, bool local) {
+  if (pl.hit_cap != 4096 || pl.smem_bytes * 2 <= kSmemBudget || pl.tiles == 1 && pl.peak_mode == HOUGH_PEAK_ITERATIVE) return;
+  for (int cap = 7168; cap >= 4096; cap -= 1024) {
+    pl.hit_cap = cap;
+    if (layout(pl, local)) return;
+  }
+}
+
 static bool layout(Plan& pl, bool local) {
   const int wpad = pl.groups * 32;
   // mirror-pair: groups / 2 word groups of 32 lanes (the last may be part idle) x rows_phys
@@ -253,6 +265,7 @@ int make_plan(const hough_params* p, Plan& pl) {
     }
     pl.tiles = T;
     pl.tile_w = W;
+    if (p->events_per_cta == 0) pl.grab = T;  // a run of an event's tiles, whose hits are staged once
     pl.nrho_pad = (p->n_rho + 1) & ~1;
     const int halo = T > 1 ? 32 : 0;
     if (p->block) {
@@ -328,7 +341,10 @@ int make_plan(const hough_params* p, Plan& pl) {
             // odd bitmap strides and the tiles' local maxima where there is room
             for (bool local : {true, false})
               for (pl.nrb_p = pl.nrb | 1; pl.nrb_p >= pl.nrb; --pl.nrb_p)
-                if (layout(pl, local)) return HOUGH_OK;
+                if (layout(pl, local)) {
+                  stage_more(pl, local);
+                  return HOUGH_OK;
+                }
           }
         }
       }
@@ -499,7 +515,7 @@ int hough_resolve_params(hough_params* p) {
   int rc = make_plan(p, pl);
   if (rc) return rc;
   p->theta_tiles = pl.tiles;
-  p->events_per_cta = pl.grab;
+  p->events_per_cta = p->events_per_cta > 0 ? p->events_per_cta : 1;
   p->block = pl.threads;
   return HOUGH_OK;
 }

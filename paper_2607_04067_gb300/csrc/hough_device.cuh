@@ -9,6 +9,7 @@
 //              (rho range [-0.01, 0.01] mm^-1 of Sec. 2)
 #pragma once
 
+#include <climits>
 #include <cstdint>
 
 #include "hough.h"
@@ -79,32 +80,50 @@ __device__ __forceinline__ int rho_bin64(long long t, BinMagic m) {
   return bin_of_t((uint32_t)t, m);
 }
 
-// floor(a / b) for b > 0 given a float estimate q of a / b with relative error below
-// 2^-21: for |q| < 2^20 the estimate is within one of the quotient and an exact remainder
-// test fixes it; larger quotients take the 64-bit integer division.
-__device__ __forceinline__ long long floor_div_est(long long a, long long b, float q) {
-  if (fabsf(q) < 1048576.0f) {
-    int q0 = (int)floorf(q);
-    const long long r = a - (long long)q0 * b;
-    if (r < 0) q0 -= 1;
-    else if (r >= b) q0 += 1;
-    return q0;
-  }
-  long long q0 = a / b;
-  if ((a % b) != 0 && a < 0) q0 -= 1;
-  return q0;
+// floor(a / b) for b > 0.
+__device__ __forceinline__ long long floor_div(long long a, long long b) {
+  long long q = a / b;
+  if ((a % b) != 0 && a < 0) q -= 1;
+  return q;
 }
 
-// Conformal map of one hit. Returns 0, or HOUGH_F_BAD_HIT for r = 0 or a coordinate beyond 2^24 um.
-// The estimate uses x, y as floats (exact for |x|, |y| <= 2^24) and a rounded r^2.
-__device__ __forceinline__ int map_hit(int x, int y, long long& u, long long& v) {
-  if (x > kCoordMax || x < -kCoordMax || y > kCoordMax || y < -kCoordMax) return HOUGH_F_BAD_HIT;
+// Hits whose quotients the estimate does not settle: bad ones (x = LLONG_MIN), and any near the origin.
+static __device__ __noinline__ longlong2 map_hit_far(int x, int y) {
   const long long r2 = (long long)x * x + (long long)y * y;
-  if (r2 == 0) return HOUGH_F_BAD_HIT;
+  if (x > kCoordMax || x < -kCoordMax || y > kCoordMax || y < -kCoordMax || r2 == 0) return make_longlong2(LLONG_MIN, 0);
+  return make_longlong2(floor_div((long long)x * (1LL << 33), r2), floor_div((long long)y * (1LL << 33), r2));
+}
+
+// floor(2^33 x / r2) from a float estimate e of it, |e| < 2^16 and off by less than one half: the rounded-down
+// estimate is within one of the quotient, and the remainder (below 2 r2 in size, r2 <= 2^49, so 64-bit
+// arithmetic modulo 2^64 has it) settles it.
+__device__ __forceinline__ int floor_quotient(int x, float e, unsigned long long r2) {
+  int q = __float_as_int(__fadd_rd(e, 12582912.0f)) - 0x4B400000;  // rounded down: the low bits of 1.5 2^23 + e
+  const long long rem = (long long)(((unsigned long long)(unsigned)(2 * x) << 32) - (unsigned long long)(long long)q * r2);
+  if (rem < 0) --q;
+  else if (rem >= (long long)r2) ++q;
+  return q;
+}
+
+// Conformal map of one hit. Returns 0, or HOUGH_F_BAD_HIT for r = 0 or a coordinate beyond 2^24 um. The
+// estimate takes x, y as floats (exact for |x|, |y| <= 2^24), a rounded r^2 and the fast quotient (2 ulp): a
+// relative error below 2^-21, so below 1/32 for quotients below 2^16 (r above 131 mm).
+__device__ __forceinline__ int map_hit(int x, int y, long long& u, long long& v) {
   const float fx = (float)x, fy = (float)y;
-  const float s = 8589934592.0f / fmaf(fx, fx, fy * fy);  // 2^33 / r^2
-  u = floor_div_est((long long)x * (1LL << 33), r2, fx * s);
-  v = floor_div_est((long long)y * (1LL << 33), r2, fy * s);
+  const float s = __fdividef(8589934592.0f, fmaf(fx, fx, fy * fy));  // 2^33 / r^2
+  const float eu = fx * s, ev = fy * s;
+  const unsigned lim = 2u * kCoordMax;
+  if ((unsigned)(x + kCoordMax) <= lim && (unsigned)(y + kCoordMax) <= lim && fabsf(eu) < 65536.0f &&
+      fabsf(ev) < 65536.0f) {
+    const unsigned long long r2 = (unsigned long long)((long long)x * x + (long long)y * y);
+    u = floor_quotient(x, eu, r2);
+    v = floor_quotient(y, ev, r2);
+    return 0;
+  }
+  const longlong2 uv = map_hit_far(x, y);
+  if (uv.x == LLONG_MIN) return HOUGH_F_BAD_HIT;
+  u = uv.x;
+  v = uv.y;
   return 0;
 }
 

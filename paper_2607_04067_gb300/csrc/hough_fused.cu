@@ -121,7 +121,7 @@ __device__ unsigned long long block_sum_u64(unsigned long long v, unsigned long 
 // (compacted, order not kept). Valid hits beyond int32 set bit 0 of *s_flags, bad
 // hits bit 1.
 __device__ void stage_vote32(const int2* __restrict__ xy, long long base, int cn, int2* hb, int* s_nv, int* s_flags,
-                             long long lsq, uint16_t* idx) {
+                             unsigned lsq, uint16_t* idx) {
   const int lane = threadIdx.x & 31;
   // each thread's next hit is loaded one pass ahead, so the loads overlap the mapping
   int2 hn = threadIdx.x < cn ? xy[base + threadIdx.x] : make_int2(0, 0);
@@ -136,8 +136,10 @@ __device__ void stage_vote32(const int2* __restrict__ xy, long long base, int cn
       st = map_hit(h.x, h.y, u, v);
       ok = (st == 0);
     }
-    // fast path: int32 rho, and (mirror-pair layout) rho within one guard bin of the range
-    const bool f = ok && fits32(u, v) && (lsq == 0 || u * u + v * v <= lsq);
+    // fast path: int32 rho, and (mirror-pair layout) rho within one guard bin of the range; the squares of
+    // values within kFast32 add up below 2^32
+    const int u32 = (int)u, v32 = (int)v;
+    const bool f = ok && fits32(u, v) && (unsigned)(u32 * u32) + (unsigned)(v32 * v32) <= lsq;
     const unsigned bal = __ballot_sync(kFull, f);
     if (bal) {
       int slot = 0;
@@ -1249,6 +1251,7 @@ struct WorkItem {
   long long off[2];
   int item;  // >= n_items: none
   int event;
+  int left;  // items popped together with it and still to come
 };
 
 __device__ __forceinline__ void copy_async(void* smem, const void* gmem, int bytes) {
@@ -1261,6 +1264,8 @@ __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_
 struct ItemShared {
   WorkItem it[2];
   int nv, flags, wide, last, total, D, reuse, n_amb, n_low;
+  int staged;  // the event whose hits are staged whole (-1: none)
+  unsigned runs;  // of the queue
   int kept_tot;
   int tstart[129], tfrom[128];  // segments of the tile merge (2 a mirror-pair tile): starts, first records
   int tmp[32];
@@ -1711,7 +1716,7 @@ __device__ int merge_iterative(const Plan& pl, const FusedIO& io, unsigned char*
   int ucap = (int)((smem + pl.off_hits - reinterpret_cast<unsigned char*>(list)) / 10);
   if (ucap < max(1024, C >> 1)) {
     ucap = (int)((smem + pl.smem_bytes - reinterpret_cast<unsigned char*>(list)) / 10);
-    if (tid == 0) sh.reuse = 0;  // (read after the barriers below)
+    if (tid == 0) sh.reuse = 0, sh.staged = -1;  // (read after the barriers below)
   }
   ucap = min(32768, ucap) & ~15;
   const ListWindow lw{keys, colstart, NT, NR, pl.nms_radius, C, alive, surv};
@@ -1722,10 +1727,11 @@ __device__ int merge_iterative(const Plan& pl, const FusedIO& io, unsigned char*
 }
 
 // Steps 1-2 of a work item: clears the CTA's accumulator of theta tile t (with the halo columns,
-// the peak bitmap and the flags) and votes the event's hits [a, a + n) into it, chunk by chunk.
+// the peak bitmap and the flags) and votes the event's hits [a, a + n) into it, chunk by chunk. The event
+// number tells whether its hits are staged already.
 template <bool MP, bool ITER>
-__device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, long long a, int n,
-                          int t) {
+__device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, int event, long long a,
+                          int n, int t) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
   uint32_t* halo = reinterpret_cast<uint32_t*>(smem + pl.off_halo);
   int2* hb = reinterpret_cast<int2*>(smem + pl.off_hits);
@@ -1807,26 +1813,30 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     }
   }
 
-  // 2. map + vote, chunk by chunk
-  if (tid == 0) sh.reuse = (MP && n > 0 && n <= pl.hit_cap) ? 1 : 0;
+  // 2. map + vote, chunk by chunk. An event's next tile in the same CTA finds its hits staged (a tile of
+  // 1000 x 1000 spent 4.5 k of 30 k cycles on mapping them again).
+  const bool staged = T > 1 && sh.staged == event;
+  if (tid == 0 && !staged) sh.reuse = (MP && n > 0 && n <= pl.hit_cap) ? 1 : 0;
   for (int h0 = 0; h0 < n; h0 += pl.hit_cap) {
     const int cn = min(pl.hit_cap, n - h0);
     __syncthreads();
     HOUGH_PHASE(h0 == 0 ? HOUGH_PHASE_CLEAR : HOUGH_PHASE_VOTE);
     if (tid == 0) {
-      sh.nv = 0;
-      sh.wide = 0;
+      if (!staged) sh.nv = sh.wide = 0;
       sh.n_amb = 0;
     }
     __syncthreads();
-    stage_vote32(io.xy, a + h0, cn, hb, &sh.nv, &sh.wide, MP ? pl.mp_lsq : 0,
-                 MP ? reinterpret_cast<uint16_t*>(smem + pl.off_idx) : nullptr);
-    __syncthreads();
-    HOUGH_PHASE(HOUGH_PHASE_STAGE);
-    if (tid == 0) {
-      if (sh.wide & 2) sh.flags |= HOUGH_F_BAD_HIT;
-      if (sh.wide & 1) sh.reuse = 0;  // wide hits are not in the staged list
+    if (!staged) {
+      stage_vote32(io.xy, a + h0, cn, hb, &sh.nv, &sh.wide, MP ? (unsigned)pl.mp_lsq : 0xffffffffu,
+                   MP ? reinterpret_cast<uint16_t*>(smem + pl.off_idx) : nullptr);
+      __syncthreads();
+      if (tid == 0) {
+        if (sh.wide & 2) sh.flags |= HOUGH_F_BAD_HIT;
+        if (sh.wide & 1) sh.reuse = 0;  // wide hits are not in the staged list
+        sh.staged = sh.reuse ? event : -1;
+      }
     }
+    HOUGH_PHASE(HOUGH_PHASE_STAGE);
     if (MP && h0 == 0) edge_words(pl, aw, Wd, want_halo, sh.edge);  // for the scan (no hits: no candidates)
     if (!(sh.wide & 1)) {
       if (mp_halo) halo_mp32(pl, HL, hb, sh.nv);
@@ -1856,15 +1866,25 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
 
 }
 
-// Takes n items from the queue; the first one's index (at most INT_MAX, which is past the last item).
-__device__ __forceinline__ int pop_items(const FusedIO& io, int n) {
-  return (int)min(atomicAdd(io.queue, (unsigned long long)n), (unsigned long long)INT_MAX);
+// The queue hands out runs of pl.grab items (a tiled event's tiles, whose hits are then staged once), the same
+// number a CTA, and the rest, at least one a CTA, singly, so that no CTA is left with a run at the end. p: the
+// queue's count; runs: how many of them.
+__device__ __forceinline__ unsigned queue_runs(const Plan& pl, const FusedIO& io) {
+  const unsigned n = (unsigned)io.n_items, g = gridDim.x;
+  return pl.grab == 1 ? n : (n - min(n, g)) / g / (unsigned)pl.grab * g;
 }
 
-// The work item sh.it[cur]. more: the index of the item after it if that is known already (popped
-// together, or none), else -1 (popped here); sh.it[cur ^ 1] receives it.
+__device__ __forceinline__ void popped(const Plan& pl, const FusedIO& io, unsigned runs, unsigned long long p, int& item,
+                                       int& left) {
+  const unsigned q = (unsigned)min(p, (unsigned long long)io.n_items);
+  item = (int)min(q < runs ? (unsigned long long)q * pl.grab : (unsigned long long)runs * pl.grab + (q - runs),
+                  (unsigned long long)INT_MAX);
+  left = q < runs ? pl.grab - 1 : 0;
+}
+
+// The work item sh.it[cur]; with `queue`, sh.it[cur ^ 1] receives the one after it.
 template <bool MP, bool ITER>
-__device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, int cur, int more,
+__device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, int cur, bool queue,
                          bool do_cs) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
   uint32_t* halo = reinterpret_cast<uint32_t*>(smem + pl.off_halo);
@@ -1885,12 +1905,16 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   WorkItem& next = sh.it[cur ^ 1];
   // Not for the iterative finder on tiles: there an event's last tile takes much longer than the others, and an
   // item popped before it would wait for it instead of going to another CTA.
-  const bool fetch = io.persistent && tid == 0 && !(ITER && T > 1);
-  if (fetch && more < 0) more = pop_items(io, pl.grab);
+  const bool fetch = queue && tid == 0 && !(ITER && T > 1);
+  unsigned long long pop = 0;
+  if (fetch && sh.it[cur].left == 0) pop = atomicAdd(io.queue, 1ull);
   bool other = false;  // the next item exists and belongs to another event
   auto fetch_event = [&]() {
     if (!fetch) return;
+    int more = sh.it[cur].item + 1, left = sh.it[cur].left - 1;
+    if (left < 0) popped(pl, io, sh.runs, pop, more, left);
     next.item = more;
+    next.left = left;
     other = more < io.n_items;
     if (other && more - sh.it[cur].item + t < T) {  // items are popped in ascending order
       other = false;
@@ -1912,7 +1936,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
 
   {
     const long long a = sh.it[cur].off[0], nll = sh.it[cur].off[1] - a;
-    vote_tile<MP, ITER>(pl, io, smem, sh, a, nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll, t);
+    vote_tile<MP, ITER>(pl, io, smem, sh, (int)e, a, nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll, t);
   }
   fetch_event();
 
@@ -2163,7 +2187,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_MERGE);
-  if (io.persistent && !(ITER && T > 1) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
+  if (queue && !(ITER && T > 1) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
     const long long i = next.off[0] + 16LL * tid;
     if (i < next.off[1]) asm volatile("prefetch.global.L2 [%0];" ::"l"(io.xy + i));
   }
@@ -2201,26 +2225,33 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
   __syncthreads();  // the table is read before run_item's first barrier
   const bool do_cs = io.checksum != nullptr;
   const bool queue = io.persistent && io.n_items > gridDim.x;  // else an item a CTA, and none after it
-  auto fetch_item = [&](WorkItem& w, int it) {  // thread 0
+  auto fetch_item = [&](WorkItem& w, int it, int left) {  // thread 0
     w.item = it;
+    w.left = left;
     if (it >= io.n_items) return;
     const int e = io.order ? io.order[it / pl.tiles] : it / pl.tiles;
     w.event = e;
     w.off[0] = io.off[e];
     w.off[1] = io.off[e + 1];
   };
-  if (threadIdx.x == 0) fetch_item(sh.it[0], queue ? pop_items(io, pl.grab) : (int)blockIdx.x);
-  int left = 0;  // items popped together with the current one and still to come
+  if (threadIdx.x == 0) {
+    sh.staged = -1;
+    int it = blockIdx.x, left = 0;
+    sh.runs = queue_runs(pl, io);
+    if (queue) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left);
+    fetch_item(sh.it[0], it, left);
+  }
 #pragma unroll 1
   for (int cur = 0;; cur ^= 1) {
     __syncthreads();
-    const int it = sh.it[cur].item;
-    if (it >= io.n_items) break;
-    left = left > 0 ? left - 1 : pl.grab - 1;
-    const int more = !queue ? INT_MAX : left > 0 ? it + 1 : -1;
-    run_item<MP, ITER>(pl, io, smem, sh, cur, more, do_cs);
-    if (!io.persistent) break;
-    if (ITER && pl.tiles > 1 && threadIdx.x == 0) fetch_item(sh.it[cur ^ 1], more < 0 ? pop_items(io, pl.grab) : more);
+    if (sh.it[cur].item >= io.n_items) break;
+    run_item<MP, ITER>(pl, io, smem, sh, cur, queue, do_cs);
+    if (!queue) break;
+    if (ITER && pl.tiles > 1 && threadIdx.x == 0) {
+      int it = sh.it[cur].item + 1, left = sh.it[cur].left - 1;
+      if (left < 0) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left);
+      fetch_item(sh.it[cur ^ 1], it, left);
+    }
   }
 }
 
@@ -2259,6 +2290,7 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
     tc[j] = trig.c[j];
     tc[pl.n_theta + j] = trig.s[j];
   }
+  if (threadIdx.x == 0) sh.staged = -1;
   __syncthreads();
   const int T = pl.tiles, NT = pl.n_theta, NR = pl.n_rho, tid = threadIdx.x, bd = blockDim.x, lane = tid & 31;
   const uint32_t* acc = reinterpret_cast<const uint32_t*>(smem + pl.off_acc);
@@ -2269,7 +2301,7 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
     const int n = nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll;  // a too-large event is never deferred
     int flags = 0;
     for (int t = 0; t < T; ++t) {
-      vote_tile<MP, true>(pl, io, smem, sh, a, n, t);
+      vote_tile<MP, true>(pl, io, smem, sh, (int)e, a, n, t);
       const int j0 = t * pl.tile_w, wt = min(pl.tile_w, NT - j0), Wd = MP ? (wt >> 1) : 0,
                 aw = t * (pl.tile_w >> 1);
       if (MP) {
@@ -2305,6 +2337,7 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
       io.npeaks[e] = total;
       if (total > pl.max_peaks) flags |= HOUGH_F_PEAK_OVERFLOW;
       sh.reuse = 0;  // the staged hits were overwritten by the finder
+      sh.staged = -1;
     }
     __syncthreads();
     int kept = select_event(pl, io, smem, sh, tc, tc + NT, a, n, dst, min(total, pl.max_peaks), false);

@@ -227,6 +227,38 @@ def test_bad_hits_and_small_radii(h):
     assert np.all(u[idx[:15]] == np.iinfo(np.int64).min)
 
 
+def test_map_edges(h):
+    """The map's quotients about the radius where its float estimate gives way to plain division (2^16: 131 mm),
+    on the axes, at the largest coordinates and at the smallest radii, against Python integers."""
+    rng = np.random.default_rng(12)
+    r = np.concatenate([np.full(3000, 131072), rng.uniform(1, 400000, 3000), rng.uniform(4e5, 2 ** 24, 2000)])
+    a = rng.uniform(0, 2 * np.pi, len(r))
+    xy = np.stack([np.rint(r * np.cos(a)), np.rint(r * np.sin(a))], axis=1).astype(np.int32)
+    xy[:3000] += rng.integers(-3, 4, size=(3000, 2)).astype(np.int32)
+    xy = np.concatenate([xy, [[1, 0], [0, -1], [2 ** 24, 2 ** 24], [-2 ** 24, 1], [131072, 0], [0, 131073], [7, -7],
+                              [3 * 5 * 7 * 11, 4 * 5 * 7 * 11]]]).astype(np.int32)
+    xy = np.ascontiguousarray(xy[np.any(xy != 0, axis=1)])
+    off = torch.tensor([0, len(xy)], dtype=torch.int64, device="cuda")
+    st = h.new_status()
+    uq, vq = h.map_hits(torch.from_numpy(xy).cuda(), off, st)
+    assert h.status(st) == 0
+    exp = [((int(x) << 33) // (int(x) ** 2 + int(y) ** 2), (int(y) << 33) // (int(x) ** 2 + int(y) ** 2)) for x, y in xy]
+    assert to_np(uq).tolist() == [e[0] for e in exp] and to_np(vq).tolist() == [e[1] for e in exp]
+
+
+@pytest.mark.parametrize("name,n,tiles,grab", [("paper_1000", 200, 16, 0), ("paper_1000", 40, 16, 5), ("stress", 310, 4, 0),
+                                               ("batched", 700, 1, 3), ("plain_paper", 5, 2, 0)])
+def test_queue_runs(h, name, n, tiles, grab):
+    """Runs of tiles from the queue with their hits staged once, single items at the end, runs across events."""
+    cfg = gen.CONFIGS[name]
+    ev = gen.generate(cfg, n)
+    ref = oracle_of(cfg, ev)
+    xy, off = dev(ev)
+    out = h.run(xy, off, cfg_params(h, cfg, theta_tiles=tiles, events_per_cta=grab), checksum=True, batched=True)
+    assert h.status(out.status) == 0
+    assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
+
+
 def test_all_hits_small_radius_event(h):
     """Every hit on the int64 path, across several staging chunks."""
     rng = np.random.default_rng(4)
