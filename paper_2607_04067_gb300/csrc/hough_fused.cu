@@ -1188,58 +1188,139 @@ __device__ __forceinline__ bool sel_test_fp(const Plan& pl, float u, float v, in
   return (bm[d * pl.nrb_g + (p >> 5)] >> (p & 31)) & 1u;
 }
 
+// The same for four columns d .. d + 3 (past D: the last four again; with fewer than four, all of them), read and
+// tested side by side.
+__device__ __forceinline__ bool sel_test4(const Plan& pl, float u, float v, int d, int D, const float2* fab,
+                                          const int2* cs, const uint32_t* bm) {
+  bool m = false;
+  if (D >= 4) {
+    d = min(d, D - 4);
+    uint32_t hit = 0u;
+    bool clear = true;
+    const uint32_t* col = bm + d * pl.nrb_g;
+#pragma unroll
+    for (int i = 0; i < 4; ++i, col += pl.nrb_g) {
+      const float2 ab = fab[d + i];
+      const uint32_t y = __float_as_uint(__fmaf_rn(u, ab.x, __fmaf_rn(v, ab.y, pl.mp_c0)));
+      clear = clear & ((y & (uint32_t)pl.mp_amask) != 0u);
+      const uint32_t p = y >> pl.mp_F;  // the row in its low bits
+      hit |= __funnelshift_r(col[(p & (uint32_t)pl.mp_rmask) >> 5], 0u, p);  // (shifted by p mod 32)
+    }
+    if (clear) return (hit & 1u) != 0u;
+  }
+#pragma unroll 1
+  for (int i = 0; i < min(4, D); ++i) m = m || sel_test_fp(pl, u, v, (D >= 4 ? d : 0) + i, fab, cs, bm);
+  return m;
+}
+
+// Every staged hit against the D peak columns (the most populated first). (A) A lane a hit, the first kSelCap
+// columns, four at a time; the hits still open are listed. Then, while many are open, a lane a listed
+// hit over the next 24 columns, and again; once they are few, a warp a hit, 64 columns a step. A long list thus
+// costs a lane's tests a hit and column, and a short one no more than a few steps. (With a warp for every
+// open hit after A: 1000 x 1000 events, whose unkept hits, two fifths, meet all ~95 columns, 50.6 k cycles of 411 k;
+// iterative finder at 256 x 256 16.0 k; batched events 5.4 k. So 23.8 k, 10.1 k, 4.2 k.) zeroed: the mask holds 0
+// already. list: two lists of lcap entries; with more open hits than that after A, their bits in unres.
 __device__ int select_staged(const Plan& pl, const int2* hb, const uint16_t* idx, int nv, long long a,
                              uint8_t* __restrict__ mask, const int2* cs, const float2* fab, const uint32_t* bm, int D,
-                             uint32_t* unres) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+                             uint32_t* unres, uint16_t* list, int lcap, bool zeroed, int* cnt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, bd = blockDim.x;
   const int cap = min(D, kSelCap);
   const float* hf = reinterpret_cast<const float*>(hb);
   int kept = 0;
-  for (int i0 = 0; i0 < nv; i0 += blockDim.x) {
+#pragma unroll 1
+  for (int i0 = 0; i0 < nv; i0 += bd) {
     const int i = i0 + threadIdx.x;
-    bool hard = false;
-    if (i < nv) {
-      const float2 h = staged_hit(hf, i);
-      bool m = false;
-      for (int d = 0; d < cap && !m; ++d) m = sel_test_fp(pl, h.x, h.y, d, fab, cs, bm);
-      if (m) {
-        mask[a + idx[i]] = 1;
-        ++kept;
-      } else {
-        hard = cap < D;
-      }
+    const bool on = i < nv;
+    const float2 h = staged_hit(hf, on ? i : 0);
+    bool open = on;
+#pragma unroll 1
+    for (int d = 0; d < cap; d += 4) {
+      if (open) open = !sel_test4(pl, h.x, h.y, d, D, fab, cs, bm);
+      if (!__any_sync(kFull, open)) break;
     }
-    const unsigned hbits = __ballot_sync(kFull, hard);
-    if (lane == 0) unres[(i0 >> 5) + warp] = hbits;
+    if (on && !open) {
+      mask[a + idx[i]] = 1;
+      ++kept;
+    } else if (on && cap == D && !zeroed) {
+      mask[a + idx[i]] = 0;
+    }
+    if (cap < D) {
+      const unsigned bal = __ballot_sync(kFull, open);
+      if (lane == 0) unres[(i0 >> 5) + warp] = bal;
+      const int pos = warp_append(&cnt[0], open);
+      if (open && pos < lcap) list[pos] = (uint16_t)i;
+    }
   }
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_SEL_A);
-  if (D > cap) {
-    // Open hits come in runs (staging order follows the input), so warp w takes hit
-    // 32 j + w of every word j, sweeping 32 words per ballot: runs spread over all warps.
-    const int nw = (nv + 31) >> 5;
-    for (int wi0 = 0; wi0 < nw; wi0 += 32) {
-      for (int ws = warp; ws < 32; ws += nwarps) {
-        const uint32_t word = (wi0 + lane < nw) ? unres[wi0 + lane] : 0u;
-        uint32_t bits = __ballot_sync(kFull, (word >> ws) & 1u);
-        while (bits) {
-          const int i = ((wi0 + __ffs(bits) - 1) << 5) + ws;
-          bits &= bits - 1u;
-          const float2 h = staged_hit(hf, i);
-          bool m = false;
-          for (int d0 = cap; d0 < D && !m; d0 += 32) {
-            const int d = d0 + lane;
-            m = __any_sync(kFull, d < D && sel_test_fp(pl, h.x, h.y, d, fab, cs, bm));
-          }
-          if (lane == 0 && m) {
-            mask[a + idx[i]] = 1;
-            ++kept;
-          }
-        }
+  if (cap == D) return kept;
+  int n = cnt[0], d0 = cap, cur = 0;
+  if (n > lcap) {  // no room: every open hit in its place, all the remaining columns
+#pragma unroll 1
+    for (int i0 = 0; i0 < nv; i0 += bd) {
+      const int i = i0 + threadIdx.x;
+      bool open = i < nv && ((unres[(i0 >> 5) + warp] >> lane) & 1u);
+      const bool was = open;
+      const float2 h = staged_hit(hf, open ? i : 0);
+#pragma unroll 1
+      for (int d = d0; d < D; d += 4) {
+        if (open) open = !sel_test4(pl, h.x, h.y, d, D, fab, cs, bm);
+        if (!__any_sync(kFull, open)) break;
       }
+      if (was && !(open && zeroed)) mask[a + idx[i]] = open ? 0 : 1;
+      kept += was && !open;
+    }
+    n = 0;
+  }
+#pragma unroll 1
+  while (n >= 4 * nwarps && d0 < D) {  // uniform
+    const int d1 = min(D, d0 + 24);
+    const uint16_t* from = list + cur * lcap;
+    uint16_t* to = list + (cur ^ 1) * lcap;
+#pragma unroll 1
+    for (int t0 = threadIdx.x - lane; t0 < n; t0 += bd) {  // uniform a warp
+      const bool on = t0 + lane < n;
+      const int i = from[min(t0 + lane, n - 1)];
+      const float2 h = staged_hit(hf, i);
+      bool open = on;
+#pragma unroll 1
+      for (int d = d0; d < d1; d += 4) {
+        if (open) open = !sel_test4(pl, h.x, h.y, d, D, fab, cs, bm);
+        if (!__any_sync(kFull, open)) break;
+      }
+      if (on && !open) {
+        mask[a + idx[i]] = 1;
+        ++kept;
+      } else if (on && d1 == D && !zeroed) {
+        mask[a + idx[i]] = 0;
+      }
+      const int pos = warp_append(&cnt[cur + 1], open);
+      if (open) to[pos] = (uint16_t)i;
+    }
+    __syncthreads();
+    cur ^= 1;
+    d0 = d1;
+    n = cnt[cur == 1 ? 1 : 2];
+    if (threadIdx.x == 0) cnt[cur + 1] = 0;
+    __syncthreads();
+  }
+  if (d0 < D) {
+    const uint16_t* from = list + cur * lcap;
+#pragma unroll 1
+    for (int t = warp; t < n; t += nwarps) {
+      const int i = from[t];
+      const float2 h = staged_hit(hf, i);
+      bool m = false;
+#pragma unroll 1
+      for (int d = d0; d < D && !m; d += 64) {
+        const bool x = sel_test_fp(pl, h.x, h.y, min(d + lane, D - 1), fab, cs, bm);
+        const bool y = sel_test_fp(pl, h.x, h.y, min(d + 32 + lane, D - 1), fab, cs, bm);
+        m = __any_sync(kFull, x || y);
+      }
+      if (lane == 0 && (m || !zeroed)) mask[a + idx[i]] = m ? 1 : 0;
+      if (lane == 0) kept += m;
     }
   }
-  __syncthreads();
   return kept;
 }
 
@@ -1288,6 +1369,21 @@ __device__ __forceinline__ uint32_t dilated_word(const uint32_t* P, int W, int n
   for (int s = 1; s <= hw; ++s) d |= (p0 << s) | (pm >> (32 - s)) | (p0 >> s) | (pp << (32 - s));
   const int valid = NR - (W << 5);
   return valid < 32 ? d & ((1u << valid) - 1u) : d;
+}
+
+// The same with bit k + 1 for row k, and guard bits 0 and N_rho + 1 equal to rows 0 and N_rho - 1.
+__device__ __forceinline__ uint32_t dilated_guard_word(const uint32_t* P, int W, int nrb, int NR, int hw) {
+  const uint32_t pm = W > 0 ? P[W - 1] : 0u, p0 = W < nrb ? P[W] : 0u, pp = W + 1 < nrb ? P[W + 1] : 0u;
+  uint32_t d = (p0 << 1) | (pm >> 31);
+  for (int s = 1; s <= hw; ++s)  // rows s above (bits up by s + 1), and s below (down by s - 1); hw <= 31
+    d |= (s < 31 ? (p0 << (s + 1)) | (pm >> (31 - s)) : pm) | (s > 1 ? (p0 >> (s - 1)) | (pp << (33 - s)) : p0);
+  if (W == 0) d = (d & ~1u) | ((d >> 1) & 1u);
+  if (W == ((NR + 1) >> 5)) {
+    const int b = (NR + 1) & 31;
+    const uint32_t last = b ? (d >> (b - 1)) & 1u : (dilated_word(P, (NR - 1) >> 5, nrb, NR, hw) >> ((NR - 1) & 31)) & 1u;
+    d = (d & ~(1u << b)) | (last << b);
+  }
+  return d;
 }
 
 // Back-projection of every hit of event e against its stored peaks pk[0, S). With
@@ -1352,25 +1448,15 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
   const int D = sh.D;
   const int hw = pl.keep_hw;
   if (from_bits) {
-    for (int j = tid; j < NT; j += bd) {
-      if (colcnt[j] == 0) continue;
+    // word W of 32 columns a warp
+    const int lane = tid & 31, NG = (NT + 31) >> 5;
+#pragma unroll 1
+    for (int it = tid >> 5, W = 0; it < NG * nrb; it += bd >> 5) {
+      while (it - W * NG >= NG) ++W;
+      const int j = 32 * (it - W * NG) + lane;
+      if (j >= NT || colcnt[j] == 0) continue;
       const uint32_t* P = pbits + j * pl.nrb_p;
-      uint32_t* out = bm + colidx[j] * nrb;
-      if (!staged) {
-        for (int W = 0; W < nrb; ++W) out[W] = dilated_word(P, W, pl.nrb, NR, hw);
-      } else {
-        // bit k + 1 for row k; guard bits 0 and N_rho + 1 copy rows 0 and N_rho - 1
-        const uint32_t last = (dilated_word(P, (NR - 1) >> 5, pl.nrb, NR, hw) >> ((NR - 1) & 31)) & 1u;
-        uint32_t prev = 0u;
-        for (int W = 0; W < nrb; ++W) {
-          const uint32_t cur = dilated_word(P, W, pl.nrb, NR, hw);
-          uint32_t g = (cur << 1) | (prev >> 31);
-          if (W == 0) g |= cur & 1u;
-          if (W == ((NR + 1) >> 5)) g |= last << ((NR + 1) & 31);
-          out[W] = g;
-          prev = cur;
-        }
-      }
+      bm[colidx[j] * nrb + W] = staged ? dilated_guard_word(P, W, pl.nrb, NR, hw) : dilated_word(P, W, pl.nrb, NR, hw);
     }
   } else {
   for (int i = tid; i < D * nrb; i += bd) bm[i] = 0;
@@ -1398,11 +1484,16 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
     return 0;
   }
   if (staged) {
-    for (int i = tid; i < n; i += bd) io.mask[a + i] = 0;
+    const bool zeroed = sh.nv < n;  // bad hits are not among the staged ones
+    if (zeroed)
+      for (int i = tid; i < n; i += bd) io.mask[a + i] = 0;
+    if (tid < 3) sh.tmp[tid] = 0;
     __syncthreads();
+    // the peak bitmap and what follows it are free now
     return select_staged(pl, reinterpret_cast<const int2*>(smem + pl.off_hits),
-                         reinterpret_cast<const uint16_t*>(smem + pl.off_idx), sh.nv, a, io.mask, cs, fab, bm, D,
-                         unres);
+                         reinterpret_cast<const uint16_t*>(smem + pl.off_idx), sh.nv, a, io.mask, cs, fab, bm, D, unres,
+                         reinterpret_cast<uint16_t*>(smem + pl.off_pbits), (pl.smem_bytes - pl.off_pbits) >> 2, zeroed,
+                         sh.tmp);
   }
   int2* hb = reinterpret_cast<int2*>(smem + pl.off_hits);
   longlong2* hw64 = reinterpret_cast<longlong2*>(smem + pl.off_hits);

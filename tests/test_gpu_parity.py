@@ -762,3 +762,21 @@ def test_host_path_errors(h):
     with pytest.raises(h.HoughError) as ei:
         r(xy, bad)
     assert ei.value.code == h.EINVAL
+
+
+@pytest.mark.parametrize("nt,nr,thr,hw,tiles", [(256, 256, 60, 1, 1), (256, 94, 40, 31, 1), (128, 63, 60, 2, 1), (4, 4, 900, 1, 1),
+                                                (1000, 1000, 14, 0, 16), (64, 30, 120, 1, 1), (256, 256, 3000, 1, 1)])
+def test_selection_edges(h, nt, nr, thr, hw, tiles):
+    """Few peak columns (fewer than four, than twelve, none), many hits that meet every column, guard bits at
+    the ends of bitmap words, wide windows; events above the staged size and one of a single hit."""
+    ev = gen.generate("batched", 14)
+    k = int(ev.off[3])
+    xy = np.concatenate([ev.xy, ev.xy[:7500]])
+    off = np.concatenate([ev.off, [ev.off[-1] + 7500]]).astype(np.int64)
+    off[4] = k + 1  # the fourth event keeps one hit, the fifth gets the rest
+    ref = oracle.run(xy, off, oracle.params(nt, nr, thr, hw, 4096), threads=THREADS)
+    d_xy, d_off = torch.from_numpy(xy).cuda(), torch.from_numpy(off).cuda()
+    for batched in (False, True):
+        out = h.run(d_xy, d_off, h.params(nt, nr, thr, hw, 4096, theta_tiles=tiles), batched=batched)
+        assert h.status(out.status) == ref.status
+        assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off)
