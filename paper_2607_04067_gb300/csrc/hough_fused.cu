@@ -836,42 +836,55 @@ __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int thr, int 
   // the halves). Rows past the last one may be read (they only list a group in vain), inside the CTA's
   // shared memory.
   {
-    int g = 0, q = warp, c = 0;
-    uint32_t hit = 0, mine = 0;  // bit c of hit: the warp's c-th group; lane c keeps which one that is
-    while (q >= n4 && g < G) {
-      q -= n4;
-      ++g;
-    }
-    while (g < G) {
-      uint4 x[4];
-      int gs[4], qs[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {  // four independent loads (past the last group: row group 0, not counted)
-        gs[i] = g;
-        qs[i] = g < G ? q : 0;
-        x[i] = *(reinterpret_cast<const uint4*>(acc + mp_word(32 * (g < G ? g : 0), 1 + 4 * qs[i], rp)) + lane);
-        q += nwarps;
-        while (q >= n4 && g < G) {
-          q -= n4;
-          ++g;
+    const int per = (n4 - warp + nwarps - 1) / nwarps;  // the warp's row groups of each word group: warp, warp + nwarps, ...
+    uint32_t hit = 0;                                   // bit c: its (r0 + c)-th of all
+    int c = 0, r0 = 0;
+    auto test = [&](const uint4& x) {
+      const uint32_t top = vmax2(vmax2(x.x, x.y), vmax2(x.z, x.w));
+      if (__any_sync(kFull, ((top - TT + 0x80008000u) & 0x80008000u) != 0u)) hit |= 1u << c;
+      ++c;
+    };
+    auto flush = [&]() {
+      if (hit) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(n_list, __popc(hit));
+        at = __shfl_sync(kFull, at, 0) + __popc(hit & lanemask_lt());
+        if ((hit >> lane) & 1u) {
+          const int g = (r0 + lane) / per;
+          list[at] = (uint16_t)(g << 8 | (warp + (r0 + lane - g * per) * nwarps));
         }
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const uint32_t top = vmax2(vmax2(x[i].x, x[i].y), vmax2(x[i].z, x[i].w));
-        if (__any_sync(kFull, gs[i] < G && ((top - TT + 0x80008000u) & 0x80008000u) != 0u)) hit |= 1u << c;
-        if (lane == c) mine = (uint32_t)(gs[i] << 8 | qs[i]);
-        ++c;
+      hit = 0;
+      r0 += c;
+      c = 0;
+    };
+#pragma unroll 1
+    for (int g = 0; g < G; ++g) {
+      const uint4* row = reinterpret_cast<const uint4*>(acc + mp_word(32 * g, 1, rp)) + lane + (warp << 5);
+      int i = 0;
+#pragma unroll 1
+      for (; i + 3 < per; i += 4, row += nwarps << 7) {  // independent loads
+        const uint4 x0 = row[0], x1 = row[nwarps << 5], x2 = row[nwarps << 6], x3 = row[3 * (nwarps << 5)];
+        if (c > 28) flush();
+        test(x0);
+        test(x1);
+        test(x2);
+        test(x3);
       }
-      if (c == 32 || g >= G) {
-        int at = 0;
-        if (lane == 0 && hit) at = atomicAdd(n_list, __popc(hit));
-        at = __shfl_sync(kFull, at, 0) + __popc(hit & lanemask_lt());
-        if ((hit >> lane) & 1u) list[at] = (uint16_t)mine;
-        hit = 0;
-        c = 0;
+      if (i + 1 < per) {
+        const uint4 x0 = row[0], x1 = row[nwarps << 5];
+        if (c > 30) flush();
+        test(x0);
+        test(x1);
+        i += 2;
+        row += nwarps << 6;
+      }
+      if (i < per) {
+        if (c > 31) flush();
+        test(row[0]);
       }
     }
+    flush();
   }
   __syncthreads();
   // (2) Raster order runs over theta, then rho: the row above and the preceding column are
@@ -2171,6 +2184,10 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       for (int kb = key0; kb < key1; kb += 32) {
         const int key = kb + lane;
         uint32_t bits = key < key1 ? key_word(key) : 0u;
+        if (!__any_sync(kFull, bits != 0u)) {  // (most of a large tile's)
+          if (MP && T > 1 && key == key_hi) sh.n_low = base;
+          continue;
+        }
         const int np = __popc(bits);
         int pos = np;  // inclusive scan
 #pragma unroll
