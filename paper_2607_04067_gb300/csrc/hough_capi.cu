@@ -388,7 +388,8 @@ cudaError_t timed_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig
     e = cudaEventRecordWithFlags(g_ev_begin, st, cudaEventRecordExternal);
     if (e != cudaSuccess) return e;
   }
-  e = launch_fused(pl, io, trig, grid, st);
+  // the validation kernel stands right before only without the event between
+  e = launch_fused(pl, io, trig, grid, st, !io.solo && !(g_ev_begin && g_ev_end));
   if (e == cudaSuccess && g_ev_begin && g_ev_end) e = cudaEventRecordWithFlags(g_ev_end, st, cudaEventRecordExternal);
   return e;
 }
@@ -528,7 +529,9 @@ int hough_run(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int64_t
                          ws_bytes, d_status, cm);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = launch_prep(cm.io.off, n_events, n_hits, d_status, cm.io.queue, cm.io.tickets, nullptr, st);
+  cudaError_t e = cudaSuccess;
+  cm.io.solo = fused_solo(cm.pl, cm.io.n_items, (int)cm.io.n_items);
+  if (!cm.io.solo) e = launch_prep(cm.io.off, n_events, n_hits, d_status, cm.io.queue, cm.io.tickets, nullptr, st);
   if (e != cudaSuccess) return cuda_fail(e);
   if (cm.io.n_items == 0) return HOUGH_OK;
   TrigTable trig;
@@ -553,12 +556,14 @@ static int enqueue_batched(const Common& cm0, const hough_params* p, int64_t n_h
                            int32_t* d_status, int grid, cudaStream_t st) {
   Common cm = cm0;
   int* order = (int*)((char*)d_ws + cm.wl.order);
-  cudaError_t e = launch_prep(cm.io.off, n_events, n_hits, d_status, cm.io.queue, cm.io.tickets, order, st);
+  cudaError_t e = cudaSuccess;
+  cm.io.solo = fused_solo(cm.pl, cm.io.n_items, grid);
+  if (!cm.io.solo) e = launch_prep(cm.io.off, n_events, n_hits, d_status, cm.io.queue, cm.io.tickets, order, st);
   if (e != cudaSuccess) return cuda_fail(e);
   if (cm.io.n_items == 0) return HOUGH_OK;
   TrigTable trig;
   host_trig(p->n_theta, &trig);
-  cm.io.order = order;
+  cm.io.order = cm.io.solo ? nullptr : order;
   cm.io.persistent = 1;
   e = timed_fused(cm.pl, cm.io, trig, grid, st);
   return e == cudaSuccess ? HOUGH_OK : cuda_fail(e);

@@ -2319,16 +2319,38 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
 }
 
+// This thread's share of the check of a batch's offsets: off[0] = 0, none decreasing, off[ne] = nh.
+__device__ __forceinline__ int bad_offsets(const long long* off, long long ne, long long nh) {
+  int bad = 0;
+  for (long long e = threadIdx.x; e < ne; e += blockDim.x) {
+    const long long a = off[e], b = off[e + 1];
+    if (b < a || a < 0 || b > nh) bad = 1;
+  }
+  if (threadIdx.x == 0 && (off[0] != 0 || off[ne] != nh)) bad = 1;
+  return bad;
+}
+
 // One instance a layout (MP: mirror pairs) and peak finder, so that none carries the others' registers.
 template <bool MP, bool ITER>
 __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ItemShared sh;
-  if (io.status[1] != 0) return;  // offsets of this call failed validation
   int16_t* tc = reinterpret_cast<int16_t*>(smem + pl.off_trig);
   for (int j = threadIdx.x; j < pl.n_theta; j += blockDim.x) {
     tc[j] = trig.c[j];
     tc[pl.n_theta + j] = trig.s[j];
+  }
+  if (io.solo) {  // no validation kernel before: every CTA looks at all offsets (a few loads a thread)
+    const int bad = __syncthreads_or(bad_offsets(io.off, io.n_events, io.n_hits));
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      io.status[1] = bad;
+      if (bad) atomicOr(io.status, HOUGH_F_BAD_OFFSETS);
+    }
+    if (bad) return;
+  } else {
+    // launched before the validation kernel has ended: what it writes is read from here on
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (__ldcg(io.status + 1) != 0) return;  // offsets of this call failed validation
   }
   __syncthreads();  // the table is read before run_item's first barrier
   const bool do_cs = io.checksum != nullptr;
@@ -2468,13 +2490,8 @@ __global__ void __launch_bounds__(1024) prep_kernel(const long long* off, long l
                                                     unsigned long long* queue, int* tickets, int* order) {
   __shared__ int hist[2048];
   __shared__ int s_tmp[32];
-  int bad = 0;
-  for (long long e = threadIdx.x; e < ne; e += blockDim.x) {
-    const long long a = off[e], b = off[e + 1];
-    if (b < a || a < 0 || b > nh) bad = 1;
-  }
-  if (threadIdx.x == 0 && (off[0] != 0 || off[ne] != nh)) bad = 1;
-  bad = __syncthreads_or(bad);
+  asm volatile("griddepcontrol.launch_dependents;");  // the fused kernel's start overlaps with this one
+  const int bad = __syncthreads_or(bad_offsets(off, ne, nh));
   if (threadIdx.x == 0) {
     status[1] = bad;
     if (bad) atomicOr(status, HOUGH_F_BAD_OFFSETS);
@@ -2603,13 +2620,29 @@ int fused_max_ctas_per_sm(const Plan& pl) {
   return n;
 }
 
-cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st) {
+bool fused_solo(const Plan& pl, long long n_items, int grid) {
+  return pl.tiles == 1 && n_items > 0 && n_items <= grid && n_items <= pl.threads;
+}
+
+cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st,
+                         bool overlap) {
   const bool deferred = pl.peak_mode == HOUGH_PEAK_ITERATIVE && pl.tiles > 1;
   const FusedKernel fused = fused_of(pl), def = pl.mp ? deferred_kernel<true> : deferred_kernel<false>;
   cudaError_t err = set_smem((const void*)fused, pl.smem_bytes);
   if (err == cudaSuccess && deferred) err = set_smem((const void*)def, pl.smem_bytes);
   if (err != cudaSuccess) return err;
-  fused<<<grid, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)pl.threads);
+  cfg.dynamicSmemBytes = (size_t)pl.smem_bytes;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  err = cudaLaunchKernelEx(&cfg, fused, pl, io, trig);
+  if (err != cudaSuccess) return err;
   if (deferred) def<<<io.n_spill, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
   return cudaGetLastError();
 }

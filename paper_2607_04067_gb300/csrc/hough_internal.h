@@ -82,6 +82,7 @@ struct FusedIO {
   int n_spill;
   long long n_items;
   int persistent;
+  int solo;  // no validation kernel before the fused one, which checks the offsets itself
 };
 
 // Workspace carve-up (byte offsets inside the caller's buffer).
@@ -101,8 +102,14 @@ BinMagic host_magic(int n_rho);
 
 cudaError_t launch_prep(const long long* off, long long n_events, long long n_hits, int* status,
                         unsigned long long* queue, int* tickets, int* order, cudaStream_t st);
-cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st);
+// `overlap`: the validation kernel is what `st` holds last, and the fused kernel's start (its launch, shared memory
+// and trig table) overlaps with it; the kernel waits for its end before it reads anything written on the device.
+cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st,
+                         bool overlap);
 int fused_max_ctas_per_sm(const Plan& pl);
+// Whether a call takes the fused kernel alone: one tile an event (no tickets to reset), an item a CTA (no queue,
+// so no order), and so few events that each CTA's look at all offsets is one step a thread.
+bool fused_solo(const Plan& pl, long long n_items, int grid);
 
 cudaError_t launch_map(const int2* xy, long long n_hits, long long* uq, long long* vq, int* status, cudaStream_t st);
 cudaError_t launch_vote(const long long* uq, const long long* vq, const long long* off, long long n_events,

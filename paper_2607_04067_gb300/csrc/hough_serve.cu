@@ -250,8 +250,9 @@ cudaError_t launch_batch(Server& S, Slot& sl) {
   bind_workspace(S.plan, wl, ws, io);
   io.n_items = (long long)ne * S.plan.tiles;
   io.persistent = 0;
-  e = launch_prep(io.off, io.n_events, nh, io.status, io.queue, io.tickets, nullptr, st);
-  if (e == cudaSuccess) e = launch_fused(S.plan, io, S.trig, (int)io.n_items, st);
+  io.solo = fused_solo(S.plan, io.n_items, (int)io.n_items);
+  if (!io.solo) e = launch_prep(io.off, io.n_events, nh, io.status, io.queue, io.tickets, nullptr, st);
+  if (e == cudaSuccess) e = launch_fused(S.plan, io, S.trig, (int)io.n_items, st, !io.solo);
   // packed peaks go straight into pinned host memory when it is mapped (only the stored ones
   // cross the link), else into device memory and are copied back whole
   hough_peak* dense = sl.dense_mapped ? sl.dense_mapped : (hough_peak*)(sl.d + L.d_dense);

@@ -99,9 +99,10 @@ extern "C" int hough_run_batched_static(const int32_t* d_xy, int64_t n_hits, con
   io.n_items = n_events * (long long)pl.tiles;
   int* order = (int*)(ws + wl.order);
   cudaStream_t st = (cudaStream_t)stream;
-  e = launch_prep(io.off, n_events, n_hits, d_status, io.queue, io.tickets, order, st);
-  if (e != cudaSuccess) return fail(e);
-  if (io.n_items == 0) return HOUGH_OK;
+  if (io.n_items == 0) {
+    e = launch_prep(io.off, n_events, n_hits, d_status, io.queue, io.tickets, order, st);
+    return e == cudaSuccess ? HOUGH_OK : fail(e);
+  }
   int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -112,8 +113,13 @@ extern "C" int hough_run_batched_static(const int32_t* d_xy, int64_t n_hits, con
   if (grid > io.n_items) grid = io.n_items;
   TrigTable trig;
   host_trig(p->n_theta, &trig);
-  io.order = order;
+  io.solo = fused_solo(pl, io.n_items, (int)grid);
+  if (!io.solo) {
+    e = launch_prep(io.off, n_events, n_hits, d_status, io.queue, io.tickets, order, st);
+    if (e != cudaSuccess) return fail(e);
+    io.order = order;
+  }
   io.persistent = 1;
-  e = launch_fused(pl, io, trig, (int)grid, st);
+  e = launch_fused(pl, io, trig, (int)grid, st, !io.solo);
   return e == cudaSuccess ? HOUGH_OK : fail(e);
 }

@@ -306,6 +306,31 @@ def test_bad_offsets_write_nothing(h):
     assert h.status(st) == h.F_BAD_OFFSETS
 
 
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("n", [1, 2, 152, 153, 256, 257])
+def test_offsets_checked_by_either_kernel(h, n, batched):
+    """Few events: the fused kernel checks the offsets itself; more than the CTAs or a CTA's threads: a kernel before."""
+    ev = gen.generate("plain_small", n)
+    ref = oracle.run(ev.xy, ev.off, oracle.params(64, 64, 12, 1, 256), threads=THREADS)
+    xy, off = dev(ev)
+    p = h.params(64, 64, 12, 1, 256, block=256)
+    out = h.run(xy, off, p, batched=batched)
+    assert h.status(out.status) == ref.status
+    assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off)
+    for at, value in ((0, 1), (n, int(ev.off[-1]) + 1), (n // 2, -1), (n - 1, int(ev.off[-1]) + 1)):
+        bad = off.clone()
+        bad[at] = value
+        out.npeaks.fill_(-7)
+        out.status.zero_()
+        h.run(xy, bad, p, out=out, batched=batched)
+        assert h.status(out.status) == h.F_BAD_OFFSETS
+        assert torch.all(out.npeaks == -7)
+    out.status.zero_()
+    h.run(xy, off, p, out=out, batched=batched)  # a refused call leaves nothing behind
+    assert h.status(out.status) == ref.status
+    assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off)
+
+
 def test_peak_overflow_keeps_first_in_raster_order(h):
     cfg = gen.CONFIGS["plain_paper"]
     ev = gen.generate(cfg, 20)
