@@ -1,6 +1,8 @@
 // C ABI of libhough.so: argument checks, launch planning, workspace layout, CUDA-graph
 // replay of the batched path, status words. See include/hough.h for the contract.
 #include <cmath>
+#include <atomic>
+#include <climits>
 #include <cstring>
 #include <algorithm>
 #include <list>
@@ -88,7 +90,9 @@ void bind_workspace(const Plan& pl, const WsLayout& wl, char* ws, FusedIO& io) {
   io.n_spill = it_tiled ? wl.n_spill : 0;
 }
 
-static constexpr int kSmemBudget = 227 * 1024 - 2048;  // dynamic bytes; static shared memory stays below 2 KB
+static constexpr int kSmemStatic = 2048;  // static shared memory stays below
+static constexpr int kSmemBudget = 227 * 1024 - kSmemStatic;  // dynamic bytes
+static constexpr int kSmemPerSm = 228 * 1024, kSms = 152;
 
 static int round16(int x) { return (x + 15) & ~15; }
 
@@ -213,8 +217,23 @@ static void mp_consts(Plan& pl, int n_rho) {
   pl.mp_lsq = (long long)std::floor(L * L);
 }
 
-// Launch shape for parameters p.
-int make_plan(const hough_params* p, Plan& pl) {
+// Whether the table of n_theta (even) columns has c[N-1-j] = -c[j], s[N-1-j] = s[j]; looked at once each.
+static bool table_symmetric(int n_theta) {
+  static std::atomic<signed char> known[kMaxNTheta + 1];
+  signed char k = known[n_theta].load(std::memory_order_relaxed);
+  if (!k) {
+    TrigTable tt;
+    host_trig(n_theta, &tt);
+    k = 1;
+    for (int j = 0; j < n_theta && k > 0; ++j)
+      if (tt.c[n_theta - 1 - j] != -tt.c[j] || tt.s[n_theta - 1 - j] != tt.s[j]) k = -1;
+    known[n_theta].store(k, std::memory_order_relaxed);
+  }
+  return k > 0;
+}
+
+// Launch shape for parameters p, with at most max_cap staged hits a chunk (more where a CTA fills an SM in any case).
+int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
   int rc = check_params(p);
   if (rc) return rc;
   std::memset(&pl, 0, sizeof(pl));
@@ -241,14 +260,7 @@ int make_plan(const hough_params* p, Plan& pl) {
   }
   // Mirror pairs (columns j and N-1-j in one word) need an even N_theta and a table with
   // c[N-1-j] = -c[j], s[N-1-j] = s[j] (true for round-half-away-from-zero).
-  bool sym = false;
-  if (p->n_theta % 2 == 0) {
-    TrigTable tt;
-    host_trig(p->n_theta, &tt);
-    sym = true;
-    for (int j = 0; j < p->n_theta && sym; ++j)
-      sym = tt.c[p->n_theta - 1 - j] == -tt.c[j] && tt.s[p->n_theta - 1 - j] == tt.s[j];
-  }
+  const bool sym = p->n_theta % 2 == 0 && table_symmetric(p->n_theta);
   for (int T = (p->theta_tiles ? p->theta_tiles : 1); T <= (p->theta_tiles ? p->theta_tiles : 64); ++T) {
     // A mirror-pair tile owns WD = ceil(N/2 / T) words (columns [a, a + WD) and their mirrors;
     // the last tile fewer), in word groups of 32 lanes; other tiles W = ceil(N / T) columns.
@@ -330,7 +342,7 @@ int make_plan(const hough_params* p, Plan& pl) {
     // ones. No lists (one pass a peak) only where no number of staged hits leaves room for any.
     const bool whole = pl.peak_mode == HOUGH_PEAK_ITERATIVE && T == 1;
     for (int lists = whole ? 1 : 0; lists >= 0; --lists) {
-      for (int cap = 4096; cap >= 512; cap >>= 1) {
+      for (int cap = max_cap; cap >= 512; cap >>= 1) {
         pl.hit_cap = cap;
         for (int icap = !lists ? 0 : pl.mp ? 4096 : 8192; icap >= (!lists ? 0 : pl.mp ? 256 : 1024);
              icap = pl.mp && icap > 1024 ? icap - 512 : icap > 0 ? icap / 2 : -1) {
@@ -352,6 +364,48 @@ int make_plan(const hough_params* p, Plan& pl) {
     if (p->theta_tiles) return HOUGH_ESMEM;
   }
   return HOUGH_ESMEM;
+}
+
+// Launch shape of a call: make_plan's, but with fewer threads a CTA where the block is the library's to choose and
+// several CTAs fit an SM. One CTA of 1,024 threads fills an SM's registers, and on a small accumulator it spends
+// most of its time on barriers and on chains that 32 warps wait for together; CTAs of other events run in those
+// gaps. c CTAs of 1024 / c threads take kTurn[c] times as long as one (in twentieths; measured from 64 x 64 to
+// 160 x 160), so the c with the shortest time for all the events' turns is taken. Where events have few hits, fewer
+// staged hits (half as many again as the mean; an event with more takes several chunks) make room for more CTAs.
+// One CTA -> this rule, us: 64 x 64, 616 hits, 5,000 events 424 -> 177 and 500 events 59 -> 30; 100 x 100, 1,290
+// hits, 5,000 events 640 -> 365; 128 x 128, 2,022 hits, 1,000 events 167 -> 131, iterative finder 286 -> 218.
+// An accumulator of at most 8,192 cells takes half the threads in any case (64 x 64, 100 events: 18.2 -> 16.5):
+// its phases are shorter than what 32 warps add to each barrier.
+int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan& pl) {
+  const int rc = make_plan(p, pl);
+  if (rc || p->block || pl.tiles > 1 || n_events < 1) return rc;
+  static constexpr int kTurn[5] = {0, 20, 27, 38, 42};
+  hough_params q = *p;
+  q.theta_tiles = 1;
+  const bool small = pl.n_theta * pl.n_rho <= 8192 && pl.peak_mode == HOUGH_PEAK_LOCAL_MAX;
+  long long best = small ? LLONG_MAX : (n_events + kSms - 1) / kSms * kTurn[1];
+  int best_cap = 0;
+  Plan x = pl;
+  for (int cap = 4096; cap >= 2048; cap -= 1024) {
+    if (cap < 4096) {
+      hough_params w = q;
+      w.block = 0;
+      if (n_hits * 3 > n_events * cap * 2 || make_plan(&w, x, cap) != HOUGH_OK) break;
+    }
+    const int fit = kSmemPerSm / (x.smem_bytes + kSmemStatic + 1024);  // 1 KB a CTA is the system's
+    for (int c = 2; c <= std::min(fit, 4); ++c) {
+      const long long t = (n_events + kSms * c - 1) / (kSms * c) * kTurn[c];
+      const int block = 1024 / c / (x.groups * 32) * (x.groups * 32);
+      if (t < best && block) {
+        best = t;
+        best_cap = cap;
+        q.block = block;
+      }
+    }
+    if (fit >= 4) break;
+  }
+  if (best_cap && make_plan(&q, x, best_cap) == HOUGH_OK) pl = x;
+  return rc;
 }
 
 // ---- CUDA graph cache of the batched path ----
@@ -408,7 +462,7 @@ int prepare_fused(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int
   if (n_events > 0 && (!d_npeaks || !d_peaks || !d_nkept)) return HOUGH_EINVAL;
   if (n_hits > 0 && (!d_xy || !d_mask)) return HOUGH_EINVAL;
   if (((uintptr_t)d_xy & 7) || ((uintptr_t)d_peaks & 7) || ((uintptr_t)d_ws & 255)) return HOUGH_EINVAL;
-  int rc = make_plan(p, cm.pl);
+  int rc = make_plan(p, n_hits, n_events, cm.pl);
   if (rc) return rc;
   if ((long long)n_events * cm.pl.tiles > 0x7fffffffLL) return HOUGH_EINVAL;
   cm.wl = ws_layout(cm.pl, n_events);

@@ -28,7 +28,7 @@
 
 namespace hgpu {
 
-int make_plan(const hough_params* p, Plan& pl);
+int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096);
 
 namespace {
 

@@ -27,7 +27,7 @@
 
 namespace hgpu {
 
-int make_plan(const hough_params* p, Plan& pl);
+int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan& pl);
 void note_cuda_error(cudaError_t e);
 
 namespace {
@@ -74,7 +74,7 @@ extern "C" int hough_run_batched_static(const int32_t* d_xy, int64_t n_hits, con
   if (n_hits > 0 && (!d_xy || !d_mask)) return HOUGH_EINVAL;
   if (((uintptr_t)d_xy & 7) || ((uintptr_t)d_peaks & 7)) return HOUGH_EINVAL;
   Plan pl;
-  int rc = make_plan(p, pl);
+  int rc = make_plan(p, n_hits, n_events, pl);
   if (rc) return rc;
   if ((long long)n_events * pl.tiles > 0x7fffffffLL) return HOUGH_EINVAL;
   const WsLayout wl = ws_layout(pl, n_events);

@@ -331,6 +331,21 @@ def test_offsets_checked_by_either_kernel(h, n, batched):
     assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off)
 
 
+@pytest.mark.parametrize("n", [152, 153, 305, 609])
+@pytest.mark.parametrize("nt,nr", [(64, 64), (101, 63), (100, 100), (130, 64), (128, 160), (63, 131)])
+@pytest.mark.parametrize("iterative", [False, True])
+def test_several_ctas_an_sm(h, nt, nr, n, iterative):
+    """Small accumulators: four, three or two CTAs an SM where there are events for them."""
+    ev = gen.generate("plain_small", n)
+    kw = dict(peak_mode=1, rel_num=1, rel_den=2, nms_radius=2) if iterative else {}
+    ref = oracle.run(ev.xy, ev.off, oracle.params(nt, nr, 9, 1, 512, **kw), threads=THREADS)
+    xy, off = dev(ev)
+    for batched in (False, True):
+        out = h.run(xy, off, h.params(nt, nr, 9, 1, 512, **kw), checksum=True, batched=batched)
+        assert h.status(out.status) == ref.status
+        assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
+
+
 def test_peak_overflow_keeps_first_in_raster_order(h):
     cfg = gen.CONFIGS["plain_paper"]
     ev = gen.generate(cfg, 20)
