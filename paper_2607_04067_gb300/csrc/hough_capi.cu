@@ -217,7 +217,7 @@ static void mp_consts(Plan& pl, int n_rho) {
   pl.mp_lsq = (long long)std::floor(L * L);
 }
 
-// Whether the table of n_theta (even) columns has c[N-1-j] = -c[j], s[N-1-j] = s[j]; looked at once each.
+// Whether the table of n_theta columns has c[N-1-j] = -c[j], s[N-1-j] = s[j]; looked at once each.
 static bool table_symmetric(int n_theta) {
   static std::atomic<signed char> known[kMaxNTheta + 1];
   signed char k = known[n_theta].load(std::memory_order_relaxed);
@@ -230,6 +230,112 @@ static bool table_symmetric(int n_theta) {
     known[n_theta].store(k, std::memory_order_relaxed);
   }
   return k > 0;
+}
+
+// make_plan with T theta tiles, in mirror pairs or (mp false) columns; with `threads`, of so many (a multiple of 32),
+// the warps that make no full share of the words left out of the vote.
+static int plan_tiles(const hough_params* p, int T, bool mp, int max_cap, Plan& pl, int threads = 0) {
+  // A mirror-pair tile owns WD = ceil(N/2 / T) words (columns [a, a + WD) and their mirrors;
+  // the last tile fewer), in word groups of 32 lanes; other tiles W = ceil(N / T) columns.
+  int W;
+  if (mp) {
+    const int NW = (p->n_theta + 1) / 2, WD = (NW + T - 1) / T;
+    if ((T - 1) * WD >= NW) return HOUGH_ESMEM;  // every tile must own at least one word
+    W = 2 * WD;
+    pl.groups = 2 * ((WD + 31) / 32);
+  } else {
+    W = (p->n_theta + T - 1) / T;
+    if ((T - 1) * W >= p->n_theta) return HOUGH_ESMEM;  // every tile must own at least one column
+    pl.groups = (W + 31) / 32;
+  }
+  pl.tiles = T;
+  pl.tile_w = W;
+  if (p->events_per_cta == 0) pl.grab = T;  // a run of an event's tiles, whose hits are staged once
+  pl.nrho_pad = (p->n_rho + 1) & ~1;
+  const int halo = T > 1 ? 32 : 0;
+  if (threads) {
+    pl.split = (threads - halo) / (pl.groups * 32);
+    if (pl.split < 1) return HOUGH_ESMEM;
+  } else if (p->block) {
+    const int work = p->block - halo;
+    if (work <= 0 || work % (pl.groups * 32)) {
+      return p->theta_tiles ? HOUGH_EPARAM : HOUGH_ESMEM;  // this tile count cannot use the requested block
+    }
+    pl.split = work / (pl.groups * 32);
+  } else {
+    // as many warps as fit 1024 threads: with one CTA per SM (large accumulators) the
+    // extra warps hide the latency of the vote chains, the scan and the selection
+    int s = (1024 - halo) / (pl.groups * 32);
+    if (s < 1) s = 1;
+    pl.split = s;
+  }
+  pl.threads = threads ? threads : pl.groups * 32 * pl.split + halo;
+  if (pl.threads > 1024) {
+    return p->theta_tiles ? HOUGH_EPARAM : HOUGH_ESMEM;
+  }
+  pl.mp = mp ? 1 : 0;
+  if (pl.mp) mp_consts(pl, p->n_rho);
+  if (!pl.mp)
+  // Column layout: the power of two of row ranges that minimises the slowest warp's row steps, each
+  // unit (30 columns x one range) paying two extra rows to prime its window and about 16 rows' worth
+  // of setup.
+  {
+    const bool packed = (p->n_rho & 1) == 0;
+    const int nblk = (pl.tile_w + 29) / 30, nwarps = pl.threads / 32;
+    const int rows = packed ? p->n_rho / 2 : p->n_rho;
+    long best = -1;
+    for (int Rs = 0; (1 << Rs) <= 64 && (rows >> Rs) >= 2; ++Rs) {
+      const long R = 1L << Rs;
+      const long cost = ((nblk * R + nwarps - 1) / nwarps) * ((rows + R - 1) / R + 18);
+      if (best < 0 || cost < best) {
+        best = cost;
+        pl.scan_ranges = (int)R;
+        pl.scan_shift = Rs;
+      }
+    }
+  }
+  // keys of the peak records: (column, group of bitmap words), at most 4096 per CTA
+  {
+    int kg = 1, ks = 0;
+    while (kg < pl.nrb) {
+      kg <<= 1;
+      ++ks;
+    }
+    int gw = 1;
+    while (pl.groups * 32 * kg > 4096) {
+      kg >>= 1;
+      --ks;
+      gw <<= 1;
+    }
+    pl.key_groups = kg;
+    pl.key_shift = ks;
+    pl.key_words = gw;
+  }
+  // the most staged hits, then (iterative finder on a whole accumulator) the longest lists: mirror pairs,
+  // 4,096 to 256 undecided candidates; columns, 8,192 to 1,024 candidate keys and 2,048 to 256 undecided
+  // ones. No lists (one pass a peak) only where no number of staged hits leaves room for any.
+  const bool whole = pl.peak_mode == HOUGH_PEAK_ITERATIVE && T == 1;
+  for (int lists = whole ? 1 : 0; lists >= 0; --lists) {
+    for (int cap = max_cap; cap >= 512; cap >>= 1) {
+      pl.hit_cap = cap;
+      for (int icap = !lists ? 0 : pl.mp ? 4096 : 8192; icap >= (!lists ? 0 : pl.mp ? 256 : 1024);
+           icap = pl.mp && icap > 1024 ? icap - 512 : icap > 0 ? icap / 2 : -1) {
+        pl.iter_cap = icap;
+        for (int act = icap > 0 && !pl.mp ? 2048 : 0; act >= 0;
+             act = act > 1024 ? act - 512 : act > 256 ? act / 2 : act - 256) {  // 2048, 1536, 1024, 512, 256, 0
+          pl.iter_act = act;
+          // odd bitmap strides and the tiles' local maxima where there is room
+          for (bool local : {true, false})
+            for (pl.nrb_p = pl.nrb | 1; pl.nrb_p >= pl.nrb; --pl.nrb_p)
+              if (layout(pl, local)) {
+                stage_more(pl, local);
+                return HOUGH_OK;
+              }
+        }
+      }
+    }
+  }
+  return HOUGH_ESMEM;
 }
 
 // Launch shape for parameters p, with at most max_cap staged hits a chunk (more where a CTA fills an SM in any case).
@@ -258,114 +364,21 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
     pl.fp_dlo = (float)(delta - 0.5);
     pl.fp_dhi = (float)(-delta - 0.5);
   }
-  // Mirror pairs (columns j and N-1-j in one word) need an even N_theta and a table with
-  // c[N-1-j] = -c[j], s[N-1-j] = s[j] (true for round-half-away-from-zero).
-  const bool sym = p->n_theta % 2 == 0 && table_symmetric(p->n_theta);
+  // Mirror pairs (columns j and N-1-j in one word) need a table with c[N-1-j] = -c[j], s[N-1-j] = s[j] (true for
+  // round-half-away-from-zero). An odd N_theta takes them for the local maxima alone, in the tiles and threads that
+  // its columns take (so that a shape is accepted, and reported, as a column shape), else columns. (101 x 63, 500 events 118 -> 61 us; 199 x 200,
+  // 1,000 events 335 -> 204 us.)
+  const bool sym = table_symmetric(p->n_theta), odd = p->n_theta % 2 != 0;
   for (int T = (p->theta_tiles ? p->theta_tiles : 1); T <= (p->theta_tiles ? p->theta_tiles : 64); ++T) {
-    // A mirror-pair tile owns WD = ceil(N/2 / T) words (columns [a, a + WD) and their mirrors;
-    // the last tile fewer), in word groups of 32 lanes; other tiles W = ceil(N / T) columns.
-    int W;
-    if (sym) {
-      const int NW = p->n_theta / 2, WD = (NW + T - 1) / T;
-      if ((T - 1) * WD >= NW) continue;  // every tile must own at least one word
-      W = 2 * WD;
-      pl.groups = 2 * ((WD + 31) / 32);
-    } else {
-      W = (p->n_theta + T - 1) / T;
-      if ((T - 1) * W >= p->n_theta) continue;  // every tile must own at least one column
-      pl.groups = (W + 31) / 32;
+    rc = plan_tiles(p, T, sym && !odd, max_cap, pl);
+    if (rc == HOUGH_OK && odd && sym && p->peak_mode == HOUGH_PEAK_LOCAL_MAX) {
+      Plan mp = pl;
+      if (plan_tiles(p, T, true, max_cap, mp, pl.threads) == HOUGH_OK) pl = mp;
     }
-    pl.tiles = T;
-    pl.tile_w = W;
-    if (p->events_per_cta == 0) pl.grab = T;  // a run of an event's tiles, whose hits are staged once
-    pl.nrho_pad = (p->n_rho + 1) & ~1;
-    const int halo = T > 1 ? 32 : 0;
-    if (p->block) {
-      const int work = p->block - halo;
-      if (work <= 0 || work % (pl.groups * 32)) {
-        if (p->theta_tiles) return HOUGH_EPARAM;
-        continue;  // this tile count cannot use the requested block; try the next
-      }
-      pl.split = work / (pl.groups * 32);
-    } else {
-      // as many warps as fit 1024 threads: with one CTA per SM (large accumulators) the
-      // extra warps hide the latency of the vote chains, the scan and the selection
-      int s = (1024 - halo) / (pl.groups * 32);
-      if (s < 1) s = 1;
-      pl.split = s;
-    }
-    pl.threads = pl.groups * 32 * pl.split + halo;
-    if (pl.threads > 1024) {
-      if (p->theta_tiles) return HOUGH_EPARAM;
-      continue;
-    }
-    pl.mp = sym ? 1 : 0;
-    if (pl.mp) mp_consts(pl, p->n_rho);
-    if (!pl.mp)
-    // Column layout: the power of two of row ranges that minimises the slowest warp's row steps, each
-    // unit (30 columns x one range) paying two extra rows to prime its window and about 16 rows' worth
-    // of setup.
-    {
-      const bool packed = (p->n_rho & 1) == 0;
-      const int nblk = (pl.tile_w + 29) / 30, nwarps = pl.threads / 32;
-      const int rows = packed ? p->n_rho / 2 : p->n_rho;
-      long best = -1;
-      for (int Rs = 0; (1 << Rs) <= 64 && (rows >> Rs) >= 2; ++Rs) {
-        const long R = 1L << Rs;
-        const long cost = ((nblk * R + nwarps - 1) / nwarps) * ((rows + R - 1) / R + 18);
-        if (best < 0 || cost < best) {
-          best = cost;
-          pl.scan_ranges = (int)R;
-          pl.scan_shift = Rs;
-        }
-      }
-    }
-    // keys of the peak records: (column, group of bitmap words), at most 4096 per CTA
-    {
-      int kg = 1, ks = 0;
-      while (kg < pl.nrb) {
-        kg <<= 1;
-        ++ks;
-      }
-      int gw = 1;
-      while (pl.groups * 32 * kg > 4096) {
-        kg >>= 1;
-        --ks;
-        gw <<= 1;
-      }
-      pl.key_groups = kg;
-      pl.key_shift = ks;
-      pl.key_words = gw;
-    }
-    // the most staged hits, then (iterative finder on a whole accumulator) the longest lists: mirror pairs,
-    // 4,096 to 256 undecided candidates; columns, 8,192 to 1,024 candidate keys and 2,048 to 256 undecided
-    // ones. No lists (one pass a peak) only where no number of staged hits leaves room for any.
-    const bool whole = pl.peak_mode == HOUGH_PEAK_ITERATIVE && T == 1;
-    for (int lists = whole ? 1 : 0; lists >= 0; --lists) {
-      for (int cap = max_cap; cap >= 512; cap >>= 1) {
-        pl.hit_cap = cap;
-        for (int icap = !lists ? 0 : pl.mp ? 4096 : 8192; icap >= (!lists ? 0 : pl.mp ? 256 : 1024);
-             icap = pl.mp && icap > 1024 ? icap - 512 : icap > 0 ? icap / 2 : -1) {
-          pl.iter_cap = icap;
-          for (int act = icap > 0 && !pl.mp ? 2048 : 0; act >= 0;
-               act = act > 1024 ? act - 512 : act > 256 ? act / 2 : act - 256) {  // 2048, 1536, 1024, 512, 256, 0
-            pl.iter_act = act;
-            // odd bitmap strides and the tiles' local maxima where there is room
-            for (bool local : {true, false})
-              for (pl.nrb_p = pl.nrb | 1; pl.nrb_p >= pl.nrb; --pl.nrb_p)
-                if (layout(pl, local)) {
-                  stage_more(pl, local);
-                  return HOUGH_OK;
-                }
-          }
-        }
-      }
-    }
-    if (p->theta_tiles) return HOUGH_ESMEM;
+    if (rc == HOUGH_OK || p->theta_tiles) return rc;
   }
   return HOUGH_ESMEM;
 }
-
 // Launch shape of a call: make_plan's, but with fewer threads a CTA where the block is the library's to choose and
 // several CTAs fit an SM. One CTA of 1,024 threads fills an SM's registers, and on a small accumulator it spends
 // most of its time on barriers and on chains that 32 warps wait for together; CTAs of other events run in those

@@ -297,8 +297,10 @@ __device__ __forceinline__ void vote64(const Plan& pl, const VoteLane& L, const 
 }
 
 // ---- mirror-pair word layout (untiled events, N_theta a multiple of 64) ----
-// Word lane w in [0, N_theta/2) holds column w in its low half and column N_theta-1-w (its
-// mirror) in its high half, one word per physical row p = k + 1. Rows p = 0 and p = N_rho + 1
+// Word lane w in [0, (N_theta+1)/2) holds column w in its low half and column N_theta-1-w (its
+// mirror) in its high half, one word per physical row p = k + 1. With an odd N_theta the last word's column is
+// its own mirror (c = 0): the high half then repeats the low one. It serves as the neighbour of the column after it;
+// the scan and the fingerprint leave it out. Rows p = 0 and p = N_rho + 1
 // are guard rows: the fast path only takes hits whose rho stays within half a bin of the range,
 // so its unclamped bins fall in [-1, N_rho]; the guard rows are folded into rows 0 and
 // N_rho - 1 after the vote, which is what clamping would have done.
@@ -708,7 +710,7 @@ __device__ __forceinline__ HaloLane halo_lane(const Plan& pl, const int16_t* tc,
                                               const uint32_t* halo, int aw, int Wd) {
   const int side = threadIdx.x & 1, w = side ? aw + Wd : aw - 1;
   HaloLane h;
-  h.on = side ? w < (pl.n_theta >> 1) : w >= 0;
+  h.on = side ? w < ((pl.n_theta + 1) >> 1) : w >= 0;
   h.c = h.on ? tc[w] : 0;
   h.s = h.on ? ts[w] : 0;
   h.col = (uint32_t)__cvta_generic_to_shared(halo) + (uint32_t)(side * pl.rows_phys) * 4u;
@@ -785,7 +787,8 @@ struct EdgeWord {
 };
 
 // Edge words of the tile's groups (the CTA's last 2 G threads). Before word 0 lies the theta wrap (word 0, rows mirrored:
-// from the top down, halves swapped), after the middle word itself (halves swapped), else the halo
+// from the top down, halves swapped), after the middle word itself (halves swapped; with an odd N_theta the word
+// before it, which holds the column after the middle one), else the halo
 // (two contiguous columns of rows_phys words, of the words aw - 1 and aw + half; a tile owns words
 // [aw, aw + half), columns aw.. and their mirrors); without a halo, nothing (guard row 0, zero, throughout).
 __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, bool halo, EdgeWord* ew) {
@@ -795,10 +798,15 @@ __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, boo
   EdgeWord e{acc0, 32, 0};
   if (w >= 0 && w < half) {
     e.at += mp_word(w, 0, rp);
-  } else if (w < 0 ? aw == 0 : aw + half == (pl.n_theta >> 1)) {
-    e.at += w < 0 ? mp_word(0, pl.n_rho + 1, rp) : mp_word(half - 1, 0, rp);
+  } else if (w < 0 ? aw == 0 : aw + half == ((pl.n_theta + 1) >> 1)) {
+    const int at = half - 1 - (pl.n_theta & 1);
+    e.at += w < 0 ? mp_word(0, pl.n_rho + 1, rp) : mp_word(at, 0, rp);
     e.step = w < 0 ? -32 : 32;
     e.swap = 1;
+    if (w > 0 && at < 0) {  // the middle word alone: the one before it is the halo's
+      e.at = halo0;
+      e.step = 1;
+    }
   } else if (halo) {
     e.at = halo0 + (w < 0 ? 0 : rp);
     e.step = 1;
@@ -936,7 +944,8 @@ __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int thr, int 
     if (lane < n) {
       const uint32_t lo = (fl >> 12) & 15u, hi = fl >> 28;
       if (lo) atomicOr(&pbits[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
-      if (hi) atomicOr(&pbits[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
+      if (hi && (CAND || 2 * (aw + w) + 1 != pl.n_theta))
+        atomicOr(&pbits[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
     }
   }
 }
@@ -1418,10 +1427,11 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
   const int nrb = staged ? pl.nrb_g : pl.nrb;  // guard-bit bitmaps are one bit wider on each side
   const uint32_t* pbits = reinterpret_cast<const uint32_t*>(smem + pl.off_pbits);
   for (int i = tid; i < 64; i += bd) hist[i] = 0;
+  const int dup = pl.mp && (NT & 1) ? (NT + 1) >> 1 : NT;  // the bitmap's place of a middle column's repetition
   if (from_bits) {
     for (int j = tid; j < NT; j += bd) {
       int cc = 0;
-      for (int w = 0; w < pl.nrb; ++w) cc += __popc(pbits[j * pl.nrb_p + w]);
+      for (int w = 0; w < pl.nrb; ++w) cc += __popc(pbits[(j + (j >= dup)) * pl.nrb_p + w]);
       colcnt[j] = cc;
     }
   } else {
@@ -1468,7 +1478,7 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
       while (it - W * NG >= NG) ++W;
       const int j = 32 * (it - W * NG) + lane;
       if (j >= NT || colcnt[j] == 0) continue;
-      const uint32_t* P = pbits + j * pl.nrb_p;
+      const uint32_t* P = pbits + (j + (j >= dup)) * pl.nrb_p;
       bm[colidx[j] * nrb + W] = staged ? dilated_guard_word(P, W, pl.nrb, NR, hw) : dilated_word(P, W, pl.nrb, NR, hw);
     }
   } else {
@@ -1540,8 +1550,8 @@ __device__ __noinline__ unsigned long long tile_checksum(const uint32_t* acc, in
   for (int i = threadIdx.x; i < half * NR; i += blockDim.x) {
     const int k = i / half, w = i - k * half;
     const uint32_t x = acc[mp_word(w, k + 1, rp)];
-    cs += (unsigned long long)(x & 0xffffu) * mix64((unsigned long long)(aw + w) * NR + k + 1) +
-          (unsigned long long)(x >> 16) * mix64((unsigned long long)(NT - 1 - aw - w) * NR + k + 1);
+    cs += (unsigned long long)(x & 0xffffu) * mix64((unsigned long long)(aw + w) * NR + k + 1);
+    if (2 * (aw + w) + 1 != NT) cs += (unsigned long long)(x >> 16) * mix64((unsigned long long)(NT - 1 - aw - w) * NR + k + 1);
   }
   return cs;
 }
@@ -1845,7 +1855,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
   const int16_t* ts = tc + pl.n_theta;
   const int T = pl.tiles, NT = pl.n_theta, nrp = pl.nrho_pad;
   const int j0 = t * pl.tile_w;
-  const int wt = min(pl.tile_w, NT - j0);
+  const int wt = min(pl.tile_w, NT + (MP ? NT & 1 : 0) - j0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
   const int wpad = pl.groups * 32;
   const int rows_w = nrp >> 1;  // words per column
@@ -2001,7 +2011,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   const long long e = sh.it[cur].event;
   const int t = sh.it[cur].item % T;
   const int j0 = t * pl.tile_w;
-  const int wt = min(pl.tile_w, NT - j0);
+  const int wt = min(pl.tile_w, NT + (MP ? NT & 1 : 0) - j0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
   const int Wd = MP ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
 

@@ -346,6 +346,25 @@ def test_several_ctas_an_sm(h, nt, nr, n, iterative):
         assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
 
 
+@pytest.mark.parametrize("nt,nr,tiles", [(5, 40, 1), (5, 40, 2), (9, 33, 3), (63, 64, 1), (65, 30, 1), (65, 30, 2), (127, 96, 1),
+                                         (129, 61, 1), (129, 61, 4), (131, 64, 11), (199, 200, 0), (255, 256, 0), (257, 100, 3),
+                                         (511, 513, 0), (1023, 255, 0)])
+def test_odd_theta_edges(h, nt, nr, tiles):
+    """An odd column count in mirror pairs: the middle column alone, in a word group or a tile of its own, beside a halo."""
+    ev = gen.generate("plain_small", 12)
+    mid = [p for p in ((0, 3000), (0, -3000), (3000, 0), (1, 2500), (-1, 2500), (30000, 7)) for _ in range(40)]
+    wide = mid + [(2, 1), (-1, 2), (0, 1)] * 20  # 64-bit votes
+    xy = np.concatenate([ev.xy[: ev.off[-1]], np.array(mid + wide)]).astype(np.int32)
+    off = np.concatenate([ev.off, ev.off[-1] + np.array([240, 540])]).astype(np.int64)
+    t_xy, t_off = torch.from_numpy(xy).cuda(), torch.from_numpy(off).cuda()
+    for thr, maxp, hw in ((3, 4096, 1), (12, 60, 0), (30, 4096, 40)):
+        ref = oracle.run(xy, off, oracle.params(nt, nr, thr, hw, maxp), threads=THREADS)
+        for batched in (False, True):
+            out = h.run(t_xy, t_off, h.params(nt, nr, thr, hw, maxp, theta_tiles=tiles), checksum=True, batched=batched)
+            assert h.status(out.status) == ref.status
+            assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
+
+
 def test_peak_overflow_keeps_first_in_raster_order(h):
     cfg = gen.CONFIGS["plain_paper"]
     ev = gen.generate(cfg, 20)
