@@ -300,7 +300,7 @@ __device__ __forceinline__ void vote64(const Plan& pl, const VoteLane& L, const 
 // Word lane w in [0, (N_theta+1)/2) holds column w in its low half and column N_theta-1-w (its
 // mirror) in its high half, one word per physical row p = k + 1. With an odd N_theta the last word's column is
 // its own mirror (c = 0): the high half then repeats the low one. It serves as the neighbour of the column after it;
-// the scan and the fingerprint leave it out. Rows p = 0 and p = N_rho + 1
+// the peaks (run_item) and the fingerprint leave it out. Rows p = 0 and p = N_rho + 1
 // are guard rows: the fast path only takes hits whose rho stays within half a bin of the range,
 // so its unclamped bins fall in [-1, N_rho]; the guard rows are folded into rows 0 and
 // N_rho - 1 after the vote, which is what clamping would have done.
@@ -827,7 +827,7 @@ __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, boo
 // 100 instructions of set-up in each of 32 warps are about 1.3 k cycles): the first takes 11 instructions a
 // group, the second about 125. One pass in units of 30 words x 64 rows took 9.3 k cycles an event at 256 x 256
 // (the central rows' candidates fell to a few warps) and 10.0 k a tile at 1000 x 1000; units of 8 rows
-// 9.6 k and 7.5 k; this form 9.9 k and 3.9 k.
+// 9.6 k and 7.5 k; this form 9.3 k and 3.6 k.
 // list: room for (half + 31) / 32 * ((N_rho + 3) / 4) entries; *n_list zero beforehand.
 // cand (nullable): a second cleared bitmap for all cells that reach the threshold (the iterative finder's
 // candidates, of which the peaks are the 3x3 local maxima).
@@ -944,8 +944,7 @@ __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int thr, int 
     if (lane < n) {
       const uint32_t lo = (fl >> 12) & 15u, hi = fl >> 28;
       if (lo) atomicOr(&pbits[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
-      if (hi && (CAND || 2 * (aw + w) + 1 != pl.n_theta))
-        atomicOr(&pbits[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
+      if (hi) atomicOr(&pbits[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
     }
   }
 }
@@ -2139,6 +2138,10 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       HOUGH_PHASE(HOUGH_PHASE_FOLD);
       if (do_cs) csum = tile_checksum(acc, NT, NR, pl.rows_phys, aw, Wd);
       scan_mp<false>(pl, smem, pl.threshold, aw, Wd, sh.edge, pbits, nullptr, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb);
+      if ((NT & 1) && aw + Wd == (NT + 1) >> 1) {  // the middle column's repetition
+        __syncthreads();
+        for (int i = tid; i < pl.nrb; i += bd) pbits[Wd * pl.nrb_p + i] = 0u;
+      }
     } else if (packed) {
       scan_packed(pl, acc, halo, pbits, wt, T, j0, do_cs, csum);
     } else {
