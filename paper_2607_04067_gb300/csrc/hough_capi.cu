@@ -53,7 +53,7 @@ WsLayout ws_layout(const Plan& pl, long long n_events) {
   size_t o = 0;
   w.queue = o;
   o = align256(o + 64);
-  const long long T = pl.tiles;
+  const long long T = pl.ws_tiles;
   w.tickets = o;
   if (T > 1) o = align256(o + 4 * (size_t)n_events);
   w.tile_cnt = o;  // per tile: record count and low-segment count
@@ -77,7 +77,7 @@ WsLayout ws_layout(const Plan& pl, long long n_events) {
 }
 
 void bind_workspace(const Plan& pl, const WsLayout& wl, char* ws, FusedIO& io) {
-  const bool tiled = pl.tiles > 1, it_tiled = tiled && pl.peak_mode == HOUGH_PEAK_ITERATIVE;
+  const bool tiled = pl.tiles > 1 && !pl.cluster, it_tiled = tiled && pl.peak_mode == HOUGH_PEAK_ITERATIVE;
   io.queue = (unsigned long long*)(ws + wl.queue);
   io.defer_count = (unsigned*)(ws + wl.queue + 8);  // reset with the queue counter by the validation kernel
   io.tickets = tiled ? (int*)(ws + wl.tickets) : nullptr;
@@ -248,7 +248,7 @@ static int plan_tiles(const hough_params* p, int T, bool mp, int max_cap, Plan& 
     if ((T - 1) * W >= p->n_theta) return HOUGH_ESMEM;  // every tile must own at least one column
     pl.groups = (W + 31) / 32;
   }
-  pl.tiles = T;
+  pl.tiles = pl.ws_tiles = T;
   pl.tile_w = W;
   if (p->events_per_cta == 0) pl.grab = T;  // a run of an event's tiles, whose hits are staged once
   pl.nrho_pad = (p->n_rho + 1) & ~1;
@@ -379,7 +379,14 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
   }
   return HOUGH_ESMEM;
 }
-// Launch shape of a call: make_plan's, but with fewer threads a CTA where the block is the library's to choose and
+// Launch shape of a call: make_plan's, but for few events or many.
+// (1) Where tiles and block are the library's to choose and all CTAs of 2, 4 or 8 tiles an event find an SM at once, an
+// event's tiles are a cluster. (A cluster lies in one group of 16 to 20 SMs: 15 events of 8 tiles, 36 of 4 and 76 of
+// 2 were the most that ran together, and 48 us after 31.5 the step beyond; the line stays below them.) A tile
+// takes more than half a word group of 32 lanes, since fewer cost the vote the same (256 x 256 in 8 tiles 31.5, in 4
+// 31.8 us). Up to 20,000 cells the exchange costs what the tiles save (128 x 128: 21.6 us an event in one CTA, 23.1 in two).
+// 256 x 256: one event 31.7 -> 24.5 us, 16 46.8 -> 31.9, 64 52 -> 43.8; 512 x 512, 8 events 69 -> 44.
+// (2) Fewer threads a CTA where the block is the library's to choose and
 // several CTAs fit an SM. One CTA of 1,024 threads fills an SM's registers, and on a small accumulator it spends
 // most of its time on barriers and on chains that 32 warps wait for together; CTAs of other events run in those
 // gaps. c CTAs of 1024 / c threads take kTurn[c] times as long as one (in twentieths; measured from 64 x 64 to
@@ -391,7 +398,21 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
 // its phases are shorter than what 32 warps add to each barrier.
 int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan& pl) {
   const int rc = make_plan(p, pl);
-  if (rc || p->block || pl.tiles > 1 || n_events < 1) return rc;
+  if (rc || p->block || n_events < 1) return rc;
+  if (!p->theta_tiles && pl.mp && pl.peak_mode == HOUGH_PEAK_LOCAL_MAX && p->n_theta * p->n_rho > 20000) {
+    hough_params q = *p;
+    for (int T = 8; T >= 2 && T >= pl.tiles; T >>= 1) {
+      if (n_events > (T == 8 ? 12 : T == 4 ? 32 : 72) || (p->n_theta + 1) / 2 <= 32 * (T / 2)) continue;
+      Plan x;
+      q.theta_tiles = T;
+      if (make_plan(&q, x) != HOUGH_OK || !x.mp) continue;
+      x.cluster = 1;
+      x.ws_tiles = pl.ws_tiles;
+      pl = x;
+      return rc;
+    }
+  }
+  if (pl.tiles > 1) return rc;
   static constexpr int kTurn[5] = {0, 20, 27, 38, 42};
   hough_params q = *p;
   q.theta_tiles = 1;

@@ -1379,7 +1379,21 @@ struct ItemShared {
     int cnt4[128];  // the merge's counts (after both have been read)
   };
   int it_max, it_ok;  // iterative finder
+  // an event's tiles in a cluster: this one's records and low ones, its fingerprint, (tile 0) the hits kept
+  int2 cl_cnt;
+  unsigned long long cl_cs;
+  int cl_kept;
 };
+
+// Cluster barrier in two halves: what a thread wrote before `arrive` is seen after `wait`. A shared variable of the
+// cluster's CTA `rank` by the address of this CTA's own.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_address(const void* own, int rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(own)), "r"(rank));
+  return a;
+}
 
 // Word W of column P's peak rows dilated by +-hw (hw < 32) and cut to [0, N_rho): bit k is
 // set iff a peak lies within hw rows of k (0 outside the column's nrb words).
@@ -1996,7 +2010,11 @@ __device__ __forceinline__ void popped(const Plan& pl, const FusedIO& io, unsign
 }
 
 // The work item sh.it[cur]; with `queue`, sh.it[cur ^ 1] receives the one after it.
-template <bool MP, bool ITER>
+// CL: the event's T tiles are the CTAs of a cluster (tile t the CTA of rank t), which exchange their record counts, write their
+// records to their places and test a T-th of the hits each: for calls of so few events that SMs would stay idle.
+// An event of 256 x 256 alone took 31.7 us in one CTA, 24.5 us in four, of which the two exchanges and the share's
+// staging are about 3.
+template <bool MP, bool ITER, bool CL>
 __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, int cur, bool queue,
                          bool do_cs) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
@@ -2055,7 +2073,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
 
   // 3-4. peaks
   const int maxp = pl.max_peaks;
-  int total = 0, n_low = 0;
+  int total = 0, n_low = 0, ev_total = 0;
   unsigned long long cs_tile = 0;
   int tmax = 0;
   if (ITER && T == 1) {
@@ -2160,19 +2178,29 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       const int w = key & (KG - 1);
       return w < pl.nrb ? pbits[(key >> pl.key_shift) * pl.nrb_p + w] : 0u;
     };
+    const int key_hi = Wd << pl.key_shift;  // first key of the high columns
     int base = 0;  // records before this warp's keys
     if (G == 1) {
       // A warp counts and then writes one run of keys; its first position is the sum of the counts of
       // the warps before it: one barrier, where a block scan of the keys and a second read took five
       // and 3.3 k + 4.7 k cycles an event (batched).
-      int np = 0;
-      for (int key = key0 + lane; key < key1; key += 32) np += __popc(key_word(key));
+      int np = 0, low = 0;
+      for (int key = key0 + lane; key < key1; key += 32) {
+        const int x = __popc(key_word(key));
+        np += x;
+        if (CL && key < key_hi) low += x;
+      }
       np = __reduce_add_sync(kFull, np);
-      if (lane == 0) sh.tmp[warp] = np;
+      if (CL) low = __reduce_add_sync(kFull, low);
+      if (lane == 0) {
+        sh.tmp[warp] = np;
+        if (CL) sh.tfrom[warp] = low;
+      }
       __syncthreads();
       const int x = lane < nwarps ? sh.tmp[lane] : 0;
       base = __reduce_add_sync(kFull, lane < warp ? x : 0);
       total = __reduce_add_sync(kFull, x);
+      if (CL) n_low = __reduce_add_sync(kFull, lane < nwarps ? sh.tfrom[lane] : 0);
     } else {
       for (int key = tid; key < nkeys; key += bd) {
         const int c = key >> pl.key_shift, w0 = (key & (KG - 1)) * G, w1 = min(pl.nrb, w0 + G);
@@ -2185,12 +2213,31 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     }
     HOUGH_PHASE(HOUGH_PHASE_EXSCAN);
     // peaks of the tile's low columns (mirror-pair tiles: the high columns follow them)
-    const int key_hi = Wd << pl.key_shift;  // first key of the high columns
-    n_low = (MP && Wd < wt && G > 1) ? cnt[key_hi] : total;
+    if (!CL || G > 1) n_low = (MP && Wd < wt && G > 1) ? cnt[key_hi] : total;
+    int low_at = 0, high_at = 0;  // CL: of the tile's low and high records, places in the event's less those in the tile's
+    if (CL) {
+      cs_tile = do_cs ? block_sum_u64(csum, sh.red) : 0ull;
+      if (tid == 0) {
+        sh.cl_cnt = make_int2(total, n_low);
+        sh.cl_cs = cs_tile;
+        sh.cl_kept = 0;
+      }
+      cluster_arrive();
+      cluster_wait();
+      int all = 0, lo = 0;
+      if (lane < T) {
+        const uint32_t at = cluster_address(&sh.cl_cnt, lane);
+        asm volatile("ld.shared::cluster.v2.s32 {%0, %1}, [%2];" : "=r"(all), "=r"(lo) : "r"(at));
+      }
+      // raster order: the tiles' low segments, then (mirror pairs) their high ones from the last tile to the first
+      low_at = __reduce_add_sync(kFull, lane < t ? lo : 0);
+      high_at = __reduce_add_sync(kFull, lane > t ? all : lo) - n_low;
+      ev_total = __reduce_add_sync(kFull, all);
+    }
     // event column of tile-local column c: mirror-pair tiles hold [aw, aw + Wd) then
     // [N - aw - Wd, N - aw), both ascending; other tiles [j0, j0 + wt)
     const int hi0 = NT - aw - 2 * Wd;
-    hough_peak* dst = (T == 1) ? io.peaks + e * (long long)maxp : io.tile_peaks + (e * T + t) * (long long)maxp;
+    hough_peak* dst = (T == 1 || CL) ? io.peaks + e * (long long)maxp : io.tile_peaks + (e * T + t) * (long long)maxp;
     uint2* dst2 = reinterpret_cast<uint2*>(dst);  // records are 8-byte aligned (checked on the host)
     if (G == 1) {
       // a lane takes a key: its word's peaks, one a step, to the positions after the lanes before it
@@ -2198,7 +2245,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         const int key = kb + lane;
         uint32_t bits = key < key1 ? key_word(key) : 0u;
         if (!__any_sync(kFull, bits != 0u)) {  // (most of a large tile's)
-          if (MP && T > 1 && key == key_hi) sh.n_low = base;
+          if (MP && !CL && T > 1 && key == key_hi) sh.n_low = base;
           continue;
         }
         const int np = __popc(bits);
@@ -2211,7 +2258,8 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         const int step = __shfl_sync(kFull, pos, 31);
         pos += base - np;
         base += step;
-        if (MP && T > 1 && key == key_hi) sh.n_low = pos;
+        if (MP && !CL && T > 1 && key == key_hi) sh.n_low = pos;
+        if (CL) pos += key < key_hi ? low_at : high_at;
         const int c = key >> pl.key_shift, k0 = (key & (KG - 1)) << 5;
         const int col = MP ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
         while (bits && pos < maxp) {
@@ -2227,6 +2275,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       for (int key = tid; key < nkeys; key += bd) {
         const int c = key >> pl.key_shift, w0 = (key & (KG - 1)) * G, w1 = min(pl.nrb, w0 + G);
         int pos = cnt[key];
+        if (CL) pos += key < key_hi ? low_at : high_at;
         for (int w = w0; w < w1 && pos < maxp; ++w) {
           uint32_t bits = pbits[c * pl.nrb_p + w];
           while (bits && pos < maxp) {
@@ -2243,18 +2292,20 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         }
       }
     }
-    cs_tile = do_cs ? block_sum_u64(csum, sh.red) : 0ull;
-    __syncthreads();
-    if (G == 1 && MP && Wd < wt && T > 1) n_low = sh.n_low;
+    if (!CL) {
+      cs_tile = do_cs ? block_sum_u64(csum, sh.red) : 0ull;
+      __syncthreads();
+      if (G == 1 && MP && Wd < wt && T > 1) n_low = sh.n_low;
+    }
     HOUGH_PHASE(HOUGH_PHASE_RECORDS);
   }
 
   fetch_done();
 
   // 5. tiles: publish, and let the last tile of the event merge
-  int ev_total = total;
+  if (!CL) ev_total = total;
   unsigned long long ev_cs = cs_tile;
-  if (T > 1) {
+  if (T > 1 && !CL) {
     if (tid == 0) {
       io.tile_cnt[2 * (e * T + t)] = total;
       io.tile_cnt[2 * (e * T + t) + 1] = n_low;
@@ -2297,10 +2348,39 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
 
   // 6. event outputs and selection (single tile, or the last tile)
-  const long long a = sh.it[cur].off[0], nll = sh.it[cur].off[1] - a;
+  long long a = sh.it[cur].off[0];
+  const long long nll = sh.it[cur].off[1] - a;
   const bool too_large = nll > HOUGH_MAX_EVENT_HITS;
-  const int n = too_large ? 0 : (int)nll;
-  if (tid == 0) {
+  int n = too_large ? 0 : (int)nll;
+  if (CL) {
+    cluster_arrive();
+    // this tile's share of the hits, staged anew while the others write their records
+    const int h0 = (int)((long long)n * t / T), cn = (int)((long long)n * (t + 1) / T) - h0;
+    a += h0;
+    n = cn;
+    __syncthreads();  // sh.flags and sh.nv of the vote have been read
+    if (tid == 0) sh.nv = sh.wide = sh.reuse = 0;
+    __syncthreads();
+    if (MP && cn > 0 && cn <= pl.hit_cap) {
+      stage_vote32(io.xy, a, cn, reinterpret_cast<int2*>(smem + pl.off_hits), &sh.nv, &sh.wide, (unsigned)pl.mp_lsq,
+                   reinterpret_cast<uint16_t*>(smem + pl.off_idx));
+      __syncthreads();
+      if (tid == 0) sh.reuse = !(sh.wide & 1);
+    }
+    cluster_wait();
+    if (do_cs && t == 0 && warp == 0) {
+      unsigned long long x = 0;
+      if (lane < T) {
+        const uint32_t at = cluster_address(&sh.cl_cs, lane);
+        asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(x) : "r"(at));
+      }
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+      ev_cs = x;
+    }
+  }
+  if (tid == 0 && CL && t > 0) {
+    if (sh.flags) atomicOr(io.status, sh.flags);
+  } else if (tid == 0) {
     io.npeaks[e] = ev_total;
     if (io.checksum) io.checksum[e] = ev_cs;
     if (ev_total > maxp) sh.flags |= HOUGH_F_PEAK_OVERFLOW;
@@ -2314,7 +2394,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
   int kept = 0;
   if (too_large) {
-    for (long long i = tid; i < nll; i += bd) io.mask[a + i] = 0;
+    for (long long i = tid + (CL ? t * bd : 0); i < nll; i += CL ? T * bd : bd) io.mask[a + i] = 0;
   } else {
     kept = select_event(pl, io, smem, sh, tc, ts, a, n, io.peaks + e * (long long)maxp, min(ev_total, maxp),
                         !ITER && T == 1 && ev_total <= maxp && pl.keep_hw < 32);
@@ -2326,8 +2406,17 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   if (lane == 0 && kept) atomicAdd(&sh.kept_tot, kept);
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_SEL_B);
+  if (CL) {
+    if (tid == 0) {
+      const uint32_t at = cluster_address(&sh.cl_kept, 0);
+      asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(at), "r"(sh.kept_tot) : "memory");
+    }
+    cluster_arrive();
+    cluster_wait();
+    if (t > 0) return;
+  }
   if (tid == 0) {
-    io.nkept[e] = sh.kept_tot;
+    io.nkept[e] = CL ? sh.cl_kept : sh.kept_tot;
     if (sh.flags) atomicOr(io.status, sh.flags);
   }
 }
@@ -2343,8 +2432,8 @@ __device__ __forceinline__ int bad_offsets(const long long* off, long long ne, l
   return bad;
 }
 
-// One instance a layout (MP: mirror pairs) and peak finder, so that none carries the others' registers.
-template <bool MP, bool ITER>
+// One instance a layout (MP: mirror pairs), peak finder and (CL) use of clusters, so that none carries the others' registers.
+template <bool MP, bool ITER, bool CL>
 __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ItemShared sh;
@@ -2388,7 +2477,7 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
   for (int cur = 0;; cur ^= 1) {
     __syncthreads();
     if (sh.it[cur].item >= io.n_items) break;
-    run_item<MP, ITER>(pl, io, smem, sh, cur, queue, do_cs);
+    run_item<MP, ITER, CL>(pl, io, smem, sh, cur, queue, do_cs);
     if (!queue) break;
     if (ITER && pl.tiles > 1 && threadIdx.x == 0) {
       int it = sh.it[cur].item + 1, left = sh.it[cur].left - 1;
@@ -2620,8 +2709,9 @@ namespace {
 using FusedKernel = void (*)(const Plan, const FusedIO, const TrigTable);
 FusedKernel fused_of(const Plan& pl) {
   const bool it = pl.peak_mode == HOUGH_PEAK_ITERATIVE;
-  return pl.mp ? (it ? fused_kernel<true, true> : fused_kernel<true, false>)
-               : (it ? fused_kernel<false, true> : fused_kernel<false, false>);
+  if (pl.cluster) return fused_kernel<true, false, true>;
+  return pl.mp ? (it ? fused_kernel<true, true, false> : fused_kernel<true, false, false>)
+               : (it ? fused_kernel<false, true, false> : fused_kernel<false, false, false>);
 }
 }  // namespace
 
@@ -2634,7 +2724,7 @@ int fused_max_ctas_per_sm(const Plan& pl) {
 }
 
 bool fused_solo(const Plan& pl, long long n_items, int grid) {
-  return pl.tiles == 1 && n_items > 0 && n_items <= grid && n_items <= pl.threads;
+  return pl.cluster || (pl.tiles == 1 && n_items > 0 && n_items <= grid && n_items <= pl.threads);
 }
 
 cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st,
@@ -2645,15 +2735,21 @@ cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& tri
   if (err == cudaSuccess && deferred) err = set_smem((const void*)def, pl.smem_bytes);
   if (err != cudaSuccess) return err;
   cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
+  if (pl.cluster) {
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)pl.tiles;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  } else {
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)pl.threads);
   cfg.dynamicSmemBytes = (size_t)pl.smem_bytes;
   cfg.stream = st;
   cfg.attrs = &at;
-  cfg.numAttrs = overlap ? 1 : 0;
+  cfg.numAttrs = overlap || pl.cluster ? 1 : 0;
   err = cudaLaunchKernelEx(&cfg, fused, pl, io, trig);
   if (err != cudaSuccess) return err;
   if (deferred) def<<<io.n_spill, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);

@@ -38,6 +38,8 @@ struct Plan {
   int key_shift;    // log2(key_groups)
   int key_words;    // bitmap words per key
   int grab;       // persistent queue: items per pop
+  int cluster;    // an event's tiles are the CTAs of a cluster (mirror pairs, local maxima; no workspace)
+  int ws_tiles;   // the tiles that the workspace is laid out for: those of a large call
   int mp;         // 1: mirror-pair word layout (column j low half, N_theta-1-j high half, guard rows)
   int rows_phys;  // mirror-pair layout: physical rows per column (N_rho + 2)
   int mp_zoff;    // pattern of 1.5 2^23, plus 2^b
@@ -107,8 +109,8 @@ cudaError_t launch_prep(const long long* off, long long n_events, long long n_hi
 cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st,
                          bool overlap);
 int fused_max_ctas_per_sm(const Plan& pl);
-// Whether a call takes the fused kernel alone: one tile an event (no tickets to reset), an item a CTA (no queue,
-// so no order), and so few events that each CTA's look at all offsets is one step a thread.
+// Whether a call takes the fused kernel alone: one tile an event or tiles in clusters (no tickets to reset), an item a
+// CTA (no queue, so no order), and so few events that each CTA's look at all offsets is one step a thread.
 bool fused_solo(const Plan& pl, long long n_items, int grid);
 
 cudaError_t launch_map(const int2* xy, long long n_hits, long long* uq, long long* vq, int* status, cudaStream_t st);

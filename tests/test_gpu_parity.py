@@ -346,6 +346,41 @@ def test_several_ctas_an_sm(h, nt, nr, n, iterative):
         assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
 
 
+@pytest.mark.parametrize("n", [1, 12, 13, 32, 33, 72, 73])
+@pytest.mark.parametrize("nt,nr", [(66, 310), (130, 160), (131, 161), (256, 256), (258, 100), (512, 300), (640, 33)])
+def test_few_events_in_clusters(h, nt, nr, n):
+    """Calls of few events: their tiles as the CTAs of a cluster, at the last and first counts of 8, 4, 2 tiles and none."""
+    ev = gen.generate("plain_small", n)
+    k = int(ev.off[n // 2])
+    xy, off = ev.xy.copy(), ev.off.copy()
+    xy[k:k + 3] = ((2, 1), (0, 1), (0, 0))  # one event with 64-bit votes and a bad hit
+    off[-1:] = len(xy)
+    t_xy, t_off = torch.from_numpy(xy).cuda(), torch.from_numpy(off).cuda()
+    for thr, maxp, hw in ((4, 4096, 1), (6, 50, 0)):
+        ref = oracle.run(xy, off, oracle.params(nt, nr, thr, hw, maxp), threads=THREADS)
+        for batched in (False, True):
+            out = h.run(t_xy, t_off, h.params(nt, nr, thr, hw, maxp), checksum=True, batched=batched)
+            assert h.status(out.status) == ref.status
+            assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
+            out = h.run(t_xy, t_off, h.params(nt, nr, thr, hw, maxp), batched=batched)
+            assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off)
+
+
+@pytest.mark.parametrize("copies", [1, 12])
+def test_large_events_in_clusters(h, copies):
+    """Events in several staging chunks, one too large (skipped, flagged) and an empty one, in clusters of 4 and 2."""
+    ev = gen.generate("stress", 8)
+    sizes = [32767, 32768, 500, 0, 9000] * copies
+    xy = np.concatenate([np.concatenate([ev.xy] * 2)[:s] for s in sizes])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    ref = oracle.run(xy, off, oracle.params(256, 256, 100, 1, 4096), threads=THREADS)
+    assert ref.status == oracle.F_EVENT_TOO_LARGE
+    t_xy, t_off = torch.from_numpy(xy).cuda(), torch.from_numpy(off).cuda()
+    out = h.run(t_xy, t_off, h.params(256, 256, 100, 1, 4096), checksum=True, batched=True)
+    assert h.status(out.status) == h.F_EVENT_TOO_LARGE
+    assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
+
+
 @pytest.mark.parametrize("nt,nr,tiles", [(5, 40, 1), (5, 40, 2), (9, 33, 3), (63, 64, 1), (65, 30, 1), (65, 30, 2), (127, 96, 1),
                                          (129, 61, 1), (129, 61, 4), (131, 64, 11), (199, 200, 0), (255, 256, 0), (257, 100, 3),
                                          (511, 513, 0), (1023, 255, 0)])
