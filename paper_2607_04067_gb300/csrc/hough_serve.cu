@@ -138,7 +138,7 @@ struct Ring {
 
 // The loop thread's helpers for copies between the callers' buffers and pinned memory, the server's own: one
 // thread copies about 12 GB/s, and a burst of 4,000 requests of 2,022 hits (16 KB in, 15 KB out each) took
-// 10.2 ms, nearly all of it copies; with three helpers 4.2 ms. They sleep between copies, take a job only while it
+// 10.2 ms, nearly all of it copies; with three helpers 4.2 ms, with six 3.4. They sleep between copies, take a job only while it
 // is open, and the loop thread, which works on it too, waits for none that did not take it.
 class Crew {
  public:
@@ -614,7 +614,7 @@ int hough_serve_open(const hough_serve_config* c, void* d_buf, size_t d_bytes, v
       return HOUGH_ECUDA;
     }
   }
-  S->crew = std::make_unique<Crew>(std::min(3, (int)std::thread::hardware_concurrency() - 2));
+  S->crew = std::make_unique<Crew>(std::min(6, ((int)std::thread::hardware_concurrency() - 2) / 2));
   S->running.store(true);
   S->loop = std::thread(serve_loop, S);
   *server = S;
