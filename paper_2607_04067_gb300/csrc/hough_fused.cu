@@ -816,6 +816,88 @@ __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, boo
   ew[i] = e;
 }
 
+constexpr int kFoundGroups = 64;
+struct Found {
+  uint32_t* key;
+  int cap;
+  int* n;
+};
+// tile-local column, row, whether it is a 3x3 local maximum
+__device__ __forceinline__ uint32_t found_key(int c, int k, uint32_t lm) { return (uint32_t)(c << 11 | k << 1) | lm; }
+
+// Pass 2 of the peak scan (scan_mp) over nl listed groups; KEYS: with keys.
+template <bool CAND, bool KEYS>
+__device__ __forceinline__ void scan_groups(const Plan& pl, const uint32_t* sw, const uint32_t* acc, uint32_t TT, int aw, int half,
+                                            const EdgeWord* ew, uint32_t* pbits, uint32_t* cand, const uint16_t* list, int nl,
+                                            const Found& found) {
+  const int NR = pl.n_rho, rp = pl.rows_phys;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  // Raster order runs over theta, then rho: the row above and the preceding column are
+  // "before" a cell (strictly below it at a peak), the rest "after" (at most equal). The
+  // preceding column of the low half (column aw+w) is lane w-1's low half (the wrapped
+  // column N-1 at word 0: after, not before); of the high half (column N-1-aw-w) lane w+1's
+  // high half; lane w-1's high half follows it (except at word 0: the wrapped column 0).
+  // Strictness becomes +1 on that neighbour, so a cell is a peak iff C >= max(U + 1, D,
+  // VU + addU, VD + 0x10000, T) per half.
+  for (int it = warp; it < nl; it += nwarps) {
+    const int en = list[it], g = en >> 8, k = (en & 255) << 2, n = min(32, half - 32 * g), w = 32 * g + lane;
+    const uint32_t addU = (w != 0 || aw != 0) ? 1u : 0x10000u;
+    const uint32_t* ptr = acc + mp_word(w, k, rp);  // row k - 1 (lanes past the last word: zero words)
+    const uint32_t R[6] = {ptr[0], ptr[32], ptr[64], ptr[96], ptr[128], ptr[160]};
+    uint32_t EV[4] = {0u, 0u, 0u, 0u};  // 3-row maxima of the word beyond the group
+    if (lane == 0 || lane == min(n, 31)) {  // (n == 1: lanes 0 and 1)
+      const EdgeWord ed = ew[2 * g + (lane != 0)];
+      const int st = ed.step;
+      const uint32_t* q = sw + ed.at + st * k;
+      uint32_t e[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) e[i] = q[st * i];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) EV[i] = __byte_perm(vmax2(vmax2(e[i], e[i + 1]), e[i + 2]), 0u, ed.swap ? 0x1032u : 0x3210u);
+    }
+    uint32_t fl = 0u, cf = 0u;  // flags, the low column's in the low half, the newest row at bit 15 of each half
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (CAND) cf = (cf >> 1) | ((R[i + 1] - TT + 0x80008000u) & 0x80008000u);
+      uint32_t VM = vmax2(vmax2(R[i], R[i + 1]), R[i + 2]);
+      if (n < 32 && lane == n) VM = EV[i];
+      uint32_t VU = __shfl_up_sync(kFull, VM, 1), VD = __shfl_down_sync(kFull, VM, 1);
+      if (lane == 0) VU = EV[i];
+      if (lane == 31 && n == 32) VD = EV[i];
+      const uint32_t X = vmax2(vmax2(vmax2(R[i] + 0x00010001u, R[i + 2]), vmax2(VU + addU, VD + 0x10000u)), TT);
+      fl = (fl >> 1) | ((R[i + 1] - X + 0x80008000u) & 0x80008000u);
+    }
+    if (NR - k < 4) {  // rows past the last one
+      const uint32_t valid = ((1u << (NR - k)) - 1u) * 0x10001000u;
+      fl &= valid;
+      cf &= valid;
+    }
+    if (CAND && lane < n) {
+      const uint32_t lo = (cf >> 12) & 15u, hi = cf >> 28;
+      if (lo) atomicOr(&cand[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
+      if (hi) atomicOr(&cand[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
+    }
+    if (lane < n) {
+      const uint32_t lo = (fl >> 12) & 15u, hi = fl >> 28;
+      if (lo) atomicOr(&pbits[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
+      if (hi) atomicOr(&pbits[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
+    }
+    if (KEYS && lane < n) {
+      // bits 0-3 the low column's rows, 4-7 the high one's (a middle column's repetition left out)
+      const uint32_t x = CAND ? cf : fl, hmask = 2 * (aw + w) + 1 != pl.n_theta ? 0xf0u : 0u;
+      uint32_t bits = ((x >> 12) & 15u) | ((x >> 24) & hmask);
+      const uint32_t lms = CAND ? ((fl >> 12) & 15u) | ((fl >> 24) & 0xf0u) : 0u;
+      if (bits) {
+        int at = atomicAdd(found.n, __popc(bits));
+        for (; bits && at < found.cap; bits &= bits - 1u, ++at) {
+          const int b = __ffs(bits) - 1;
+          found.key[at] = found_key(b < 4 ? w : 2 * half - 1 - w, k + (b & 3), (lms >> b) & 1u);
+        }
+      }
+    }
+  }
+}
+
 // Peak scan of the mirror-pair layout, both columns of a word at once, in two passes. (1) Row groups (32
 // words x 4 rows: one 16-byte load a lane) in which some cell reaches the threshold are listed; about a
 // third of them at 256 x 256 and T = 16, a few per cent at 1000 x 1000 and T = 12. (2) Warps take listed
@@ -831,9 +913,11 @@ __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, boo
 // list: room for (half + 31) / 32 * ((N_rho + 3) / 4) entries; *n_list zero beforehand.
 // cand (nullable): a second cleared bitmap for all cells that reach the threshold (the iterative finder's
 // candidates, of which the peaks are the 3x3 local maxima).
+// found (tiles): with few listed groups, the peaks (CAND: the candidates) also as keys found_key in any order, counted in
+// found.n (zero beforehand; past found.cap, or with more groups, the count is and the keys are not complete).
 template <bool CAND>
 __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int thr, int aw, int half, const EdgeWord* ew,
-                        uint32_t* pbits, uint32_t* cand, uint16_t* list, int* n_list) {
+                        uint32_t* pbits, uint32_t* cand, uint16_t* list, int* n_list, const Found& found) {
   const int NR = pl.n_rho, rp = pl.rows_phys;
   const uint32_t* const sw = reinterpret_cast<const uint32_t*>(smem);
   const uint32_t* const acc = sw + (pl.off_acc >> 2);
@@ -895,57 +979,12 @@ __device__ void scan_mp(const Plan& pl, const unsigned char* smem, int thr, int 
     flush();
   }
   __syncthreads();
-  // (2) Raster order runs over theta, then rho: the row above and the preceding column are
-  // "before" a cell (strictly below it at a peak), the rest "after" (at most equal). The
-  // preceding column of the low half (column aw+w) is lane w-1's low half (the wrapped
-  // column N-1 at word 0: after, not before); of the high half (column N-1-aw-w) lane w+1's
-  // high half; lane w-1's high half follows it (except at word 0: the wrapped column 0).
-  // Strictness becomes +1 on that neighbour, so a cell is a peak iff C >= max(U + 1, D,
-  // VU + addU, VD + 0x10000, T) per half.
-  const int nl = *n_list;
-  for (int it = warp; it < nl; it += nwarps) {
-    const int en = list[it], g = en >> 8, k = (en & 255) << 2, n = min(32, half - 32 * g), w = 32 * g + lane;
-    const uint32_t addU = (w != 0 || aw != 0) ? 1u : 0x10000u;
-    const uint32_t* ptr = acc + mp_word(w, k, rp);  // row k - 1 (lanes past the last word: zero words)
-    const uint32_t R[6] = {ptr[0], ptr[32], ptr[64], ptr[96], ptr[128], ptr[160]};
-    uint32_t EV[4] = {0u, 0u, 0u, 0u};  // 3-row maxima of the word beyond the group
-    if (lane == 0 || lane == min(n, 31)) {  // (n == 1: lanes 0 and 1)
-      const EdgeWord ed = ew[2 * g + (lane != 0)];
-      const int st = ed.step;
-      const uint32_t* q = sw + ed.at + st * k;
-      uint32_t e[6];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) e[i] = q[st * i];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) EV[i] = __byte_perm(vmax2(vmax2(e[i], e[i + 1]), e[i + 2]), 0u, ed.swap ? 0x1032u : 0x3210u);
-    }
-    uint32_t fl = 0u, cf = 0u;  // flags, the low column's in the low half, the newest row at bit 15 of each half
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (CAND) cf = (cf >> 1) | ((R[i + 1] - TT + 0x80008000u) & 0x80008000u);
-      uint32_t VM = vmax2(vmax2(R[i], R[i + 1]), R[i + 2]);
-      if (n < 32 && lane == n) VM = EV[i];
-      uint32_t VU = __shfl_up_sync(kFull, VM, 1), VD = __shfl_down_sync(kFull, VM, 1);
-      if (lane == 0) VU = EV[i];
-      if (lane == 31 && n == 32) VD = EV[i];
-      const uint32_t X = vmax2(vmax2(vmax2(R[i] + 0x00010001u, R[i + 2]), vmax2(VU + addU, VD + 0x10000u)), TT);
-      fl = (fl >> 1) | ((R[i + 1] - X + 0x80008000u) & 0x80008000u);
-    }
-    if (NR - k < 4) {  // rows past the last one
-      const uint32_t valid = ((1u << (NR - k)) - 1u) * 0x10001000u;
-      fl &= valid;
-      cf &= valid;
-    }
-    if (CAND && lane < n) {
-      const uint32_t lo = (cf >> 12) & 15u, hi = cf >> 28;
-      if (lo) atomicOr(&cand[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
-      if (hi) atomicOr(&cand[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
-    }
-    if (lane < n) {
-      const uint32_t lo = (fl >> 12) & 15u, hi = fl >> 28;
-      if (lo) atomicOr(&pbits[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
-      if (hi) atomicOr(&pbits[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
-    }
+  const int nl = *n_list;  // (2)
+  if (found.cap > 0 && nl <= kFoundGroups) {
+    scan_groups<CAND, true>(pl, sw, acc, TT, aw, half, ew, pbits, cand, list, nl, found);
+  } else {
+    if (threadIdx.x == 0) *found.n = INT_MAX;
+    scan_groups<CAND, false>(pl, sw, acc, TT, aw, half, ew, pbits, cand, list, nl, found);
   }
 }
 
@@ -1349,6 +1388,8 @@ __device__ int select_staged(const Plan& pl, const int2* hb, const uint16_t* idx
 // memory, the current one and the next: in a persistent launch the next is popped before the current one's
 // vote, and its event's index and offsets are read by asynchronous copies issued between the phases, so that
 // no barrier waits for their latency (3.5 k cycles an event in a chain after the last item).
+constexpr int kFoundMax = 128;  // keys that are ranked one by one
+
 struct WorkItem {
   long long off[2];
   int item;  // >= n_items: none
@@ -1365,7 +1406,7 @@ __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_
 
 struct ItemShared {
   WorkItem it[2];
-  int nv, flags, wide, last, total, D, reuse, n_amb, n_low;
+  int nv, flags, wide, last, total, D, reuse, n_amb, n_low, n_found;
   int staged;  // the event whose hits are staged whole (-1: none)
   unsigned runs;  // of the queue
   int kept_tot;
@@ -2081,7 +2122,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // extraction, which clears the cells it suppresses; records in extraction order
     if (MP) {
       mp_fold(pl, acc, Wd, nullptr);
-      if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
+      if (tid == 0) sh.n_amb = sh.n_found = 0;  // the scan's counts of listed groups and of keys
       __syncthreads();
       HOUGH_PHASE(HOUGH_PHASE_FOLD);
     }
@@ -2105,7 +2146,8 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       const int tq = (int)max((long long)pl.threshold, ((long long)pl.rel_num * amax + pl.rel_den - 1) / pl.rel_den);
       uint32_t* cand = pbits + pl.groups * 32 * pl.nrb_p;
       uint32_t* list = cand + pl.groups * 32 * pl.nrb_p;
-      scan_mp<true>(pl, smem, tq, 0, Wd, sh.edge, pbits, cand, reinterpret_cast<uint16_t*>(list), &sh.n_amb);
+      scan_mp<true>(pl, smem, tq, 0, Wd, sh.edge, pbits, cand, reinterpret_cast<uint16_t*>(list), &sh.n_amb,
+                    Found{nullptr, 0, &sh.n_found});
       __syncthreads();
       const WholeWindow ww{acc, Wd, pl.rows_phys, NT, NR, pl.nms_radius, pl.nrb_p, cand, pbits};
       const int nk = resolve_kept(ww, list, pl.iter_cap, reinterpret_cast<uint16_t*>(list + 2 * pl.iter_cap), sh.tmp);
@@ -2134,10 +2176,12 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // the neighbour columns of other tiles count as empty there)
     unsigned long long csum = 0;
     const bool packed = !MP && (NR & 1) == 0;
+    Found found{nullptr, 0, &sh.n_found};  // after the scan's list of groups
+    const int gate = (((Wd + 31) >> 5) * ((NR + 3) >> 2) + 1) >> 1;
     uint32_t* local = pl.off_local ? reinterpret_cast<uint32_t*>(smem + pl.off_local) : pbits;  // no room: none marked
     if (ITER && MP) {
       mp_fold(pl, acc, Wd, nullptr);
-      if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
+      if (tid == 0) sh.n_amb = sh.n_found = 0;  // the scan's counts of listed groups and of keys
       if (pl.off_local)
         for (int i = tid; i < pl.groups * 32 * pl.nrb_p; i += bd) local[i] = 0u;
       __syncthreads();
@@ -2145,17 +2189,20 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       tmax = acc_max_mp(pl, acc, Wd, &sh.it_max);
       if (do_cs) csum = tile_checksum(acc, NT, NR, pl.rows_phys, aw, Wd);
       const int tq = (int)max((long long)pl.threshold, ((long long)pl.rel_num * tmax + pl.rel_den - 1) / pl.rel_den);
-      scan_mp<true>(pl, smem, tq, aw, Wd, sh.edge, local, pbits, reinterpret_cast<uint16_t*>(halo), &sh.n_amb);
+      found = Found{halo + gate, min(kFoundMax, 2 * pl.rows_phys - gate), &sh.n_found};
+      scan_mp<true>(pl, smem, tq, aw, Wd, sh.edge, local, pbits, reinterpret_cast<uint16_t*>(halo), &sh.n_amb, found);
     } else if (ITER) {
       tmax = tile_max_cs(pl, acc, wt, j0, do_cs, &sh.it_max, csum);
       tile_candidate_bits(pl, acc, pbits, wt, (int)max((long long)pl.threshold, ((long long)pl.rel_num * tmax + pl.rel_den - 1) / pl.rel_den));
     } else if (MP) {
       mp_fold(pl, acc, Wd, T > 1 ? halo : nullptr);
-      if (tid == 0) sh.n_amb = 0;  // the scan's count of listed groups
+      if (tid == 0) sh.n_amb = sh.n_found = 0;  // the scan's counts of listed groups and of keys
       __syncthreads();
       HOUGH_PHASE(HOUGH_PHASE_FOLD);
       if (do_cs) csum = tile_checksum(acc, NT, NR, pl.rows_phys, aw, Wd);
-      scan_mp<false>(pl, smem, pl.threshold, aw, Wd, sh.edge, pbits, nullptr, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb);
+      if (T > 1 && !CL)
+        found = Found{reinterpret_cast<uint32_t*>(cnt) + gate, min(kFoundMax, pl.groups * 32 * pl.key_groups - gate), &sh.n_found};
+      scan_mp<false>(pl, smem, pl.threshold, aw, Wd, sh.edge, pbits, nullptr, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb, found);
       if ((NT & 1) && aw + Wd == (NT + 1) >> 1) {  // the middle column's repetition
         __syncthreads();
         for (int i = tid; i < pl.nrb; i += bd) pbits[Wd * pl.nrb_p + i] = 0u;
@@ -2180,7 +2227,12 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     };
     const int key_hi = Wd << pl.key_shift;  // first key of the high columns
     int base = 0;  // records before this warp's keys
-    if (G == 1) {
+    const bool ranked = MP && T > 1 && !CL && sh.n_found <= found.cap;
+    if (ranked) {
+      total = sh.n_found;
+      for (int j = 0; j < total; j += 32)
+        n_low += __popc(__ballot_sync(kFull, j + lane < total && found.key[j + lane] < found_key(Wd, 0, 0u)));
+    } else if (G == 1) {
       // A warp counts and then writes one run of keys; its first position is the sum of the counts of
       // the warps before it: one barrier, where a block scan of the keys and a second read took five
       // and 3.3 k + 4.7 k cycles an event (batched).
@@ -2213,7 +2265,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     }
     HOUGH_PHASE(HOUGH_PHASE_EXSCAN);
     // peaks of the tile's low columns (mirror-pair tiles: the high columns follow them)
-    if (!CL || G > 1) n_low = (MP && Wd < wt && G > 1) ? cnt[key_hi] : total;
+    if (!ranked && (!CL || G > 1)) n_low = (MP && Wd < wt && G > 1) ? cnt[key_hi] : total;
     int low_at = 0, high_at = 0;  // CL: of the tile's low and high records, places in the event's less those in the tile's
     if (CL) {
       cs_tile = do_cs ? block_sum_u64(csum, sh.red) : 0ull;
@@ -2239,7 +2291,21 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     const int hi0 = NT - aw - 2 * Wd;
     hough_peak* dst = (T == 1 || CL) ? io.peaks + e * (long long)maxp : io.tile_peaks + (e * T + t) * (long long)maxp;
     uint2* dst2 = reinterpret_cast<uint2*>(dst);  // records are 8-byte aligned (checked on the host)
-    if (G == 1) {
+    if (ranked) {
+      // Few records: a warp a key, its place the number of smaller ones. (A tile of 1000 x 1000 has seven, and the
+      // keys of its 2,048 bitmap words took 3.4 k cycles of 23 k: 1,000 events 1405 -> 1357 us, the iterative
+      // finder 841 -> 804. Not for whole events: 64 x 64, 126 records, 16.4 us by bitmap words, 18.4 so.)
+      for (int i = warp; i < total; i += nwarps) {
+        const uint32_t key = found.key[i];
+        int pos = 0;
+        for (int j = 0; j < total; j += 32)
+          pos += __popc(__ballot_sync(kFull, j + lane < total && found.key[j + lane] < key));
+        const int c = (int)(key >> 11), k = (int)(key >> 1) & 1023;
+        if (lane == 0 && pos < maxp)
+          dst2[pos] = make_uint2((uint32_t)(c < Wd ? aw + c : hi0 + c) | ((uint32_t)k << 16),
+                                 (uint32_t)mp_get(acc, c, k, Wd, pl) | (pl.off_local ? (key & 1u) << 16 : 0u));
+      }
+    } else if (G == 1) {
       // a lane takes a key: its word's peaks, one a step, to the positions after the lanes before it
       for (int kb = key0; kb < key1; kb += 32) {
         const int key = kb + lane;
@@ -2295,7 +2361,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     if (!CL) {
       cs_tile = do_cs ? block_sum_u64(csum, sh.red) : 0ull;
       __syncthreads();
-      if (G == 1 && MP && Wd < wt && T > 1) n_low = sh.n_low;
+      if (!ranked && G == 1 && MP && Wd < wt && T > 1) n_low = sh.n_low;
     }
     HOUGH_PHASE(HOUGH_PHASE_RECORDS);
   }

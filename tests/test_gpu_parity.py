@@ -366,6 +366,23 @@ def test_few_events_in_clusters(h, nt, nr, n):
             assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off)
 
 
+@pytest.mark.parametrize("nt,nr,tiles", [(64, 64, 1), (64, 64, 2), (63, 65, 1), (256, 256, 0), (512, 257, 4), (1000, 1000, 0), (1001, 900, 0)])
+def test_records_by_keys(h, nt, nr, tiles):
+    """Tiles of few records, ranked one by one: thresholds from a record an event to more than are ranked."""
+    ev = gen.generate("plain_paper", 5)
+    xy, off = dev(ev)
+    for iterative in (False, True):
+        if iterative and nt % 2 and tiles == 0:
+            continue
+        kw = dict(peak_mode=1, rel_num=1, rel_den=3, nms_radius=2) if iterative else {}
+        for thr, maxp in ((40, 512), (16, 512), (8, 7), (4, 8192)):
+            ref = oracle.run(ev.xy, ev.off, oracle.params(nt, nr, thr, 1, maxp, **kw), threads=THREADS)
+            for batched in (False, True):
+                out = h.run(xy, off, h.params(nt, nr, thr, 1, maxp, theta_tiles=tiles, **kw), checksum=True, batched=batched)
+                assert h.status(out.status) == ref.status
+                assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
+
+
 @pytest.mark.parametrize("copies", [1, 12])
 def test_large_events_in_clusters(h, copies):
     """Events in several staging chunks, one too large (skipped, flagged) and an empty one, in clusters of 4 and 2."""
