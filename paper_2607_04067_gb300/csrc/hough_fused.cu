@@ -1395,6 +1395,7 @@ struct WorkItem {
   int item;  // >= n_items: none
   int event;
   int left;  // items popped together with it and still to come
+  int run;   // popped in a run of grab items
 };
 
 __device__ __forceinline__ void copy_async(void* smem, const void* gmem, int bytes) {
@@ -2043,11 +2044,12 @@ __device__ __forceinline__ unsigned queue_runs(const Plan& pl, const FusedIO& io
 }
 
 __device__ __forceinline__ void popped(const Plan& pl, const FusedIO& io, unsigned runs, unsigned long long p, int& item,
-                                       int& left) {
+                                       int& left, int& run) {
   const unsigned q = (unsigned)min(p, (unsigned long long)io.n_items);
   item = (int)min(q < runs ? (unsigned long long)q * pl.grab : (unsigned long long)runs * pl.grab + (q - runs),
                   (unsigned long long)INT_MAX);
-  left = q < runs ? pl.grab - 1 : 0;
+  run = q < runs;
+  left = run ? pl.grab - 1 : 0;
 }
 
 // The work item sh.it[cur]; with `queue`, sh.it[cur ^ 1] receives the one after it.
@@ -2083,10 +2085,11 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   bool other = false;  // the next item exists and belongs to another event
   auto fetch_event = [&]() {
     if (!fetch) return;
-    int more = sh.it[cur].item + 1, left = sh.it[cur].left - 1;
-    if (left < 0) popped(pl, io, sh.runs, pop, more, left);
+    int more = sh.it[cur].item + 1, left = sh.it[cur].left - 1, run = sh.it[cur].run;
+    if (left < 0) popped(pl, io, sh.runs, pop, more, left, run);
     next.item = more;
     next.left = left;
+    next.run = run;
     other = more < io.n_items;
     if (other && more - sh.it[cur].item + t < T) {  // items are popped in ascending order
       other = false;
@@ -2378,15 +2381,20 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       if (do_cs) io.tile_cs[e * T + t] = cs_tile;
       if (io.tile_max) io.tile_max[e * T + t] = tmax;
     }
-    __threadfence();
+    // A run is all of an event's tiles in this CTA: they end in order, and what its threads wrote is seen after a
+    // barrier. (A fence and a ticket cost each tile of 1000 x 1000 1.4 k cycles of 26.)
+    const bool own = sh.it[cur].run && pl.grab == T;
+    if (!own) __threadfence();
     __syncthreads();
-    if (tid == 0) sh.last = (atomicAdd(&io.tickets[e], 1) == T - 1);
-    __syncthreads();
-    if (!sh.last) {
+    if (!own) {
+      if (tid == 0) sh.last = (atomicAdd(&io.tickets[e], 1) == T - 1);
+      __syncthreads();
+    }
+    if (own ? t < T - 1 : !sh.last) {
       if (tid == 0 && sh.flags) atomicOr(io.status, sh.flags);
       return;
     }
-    __threadfence();
+    if (!own) __threadfence();
     // Raster order of the event: the tiles' low segments in tile order, then (mirror-pair
     // tiles) their high segments in reverse tile order. Segment s < T is tile s's records
     // [0, lo); segment T + i is tile T-1-i's records [lo, all).
@@ -2523,9 +2531,10 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
   __syncthreads();  // the table is read before run_item's first barrier
   const bool do_cs = io.checksum != nullptr;
   const bool queue = io.persistent && io.n_items > gridDim.x;  // else an item a CTA, and none after it
-  auto fetch_item = [&](WorkItem& w, int it, int left) {  // thread 0
+  auto fetch_item = [&](WorkItem& w, int it, int left, int run) {  // thread 0
     w.item = it;
     w.left = left;
+    w.run = run;
     if (it >= io.n_items) return;
     const int e = io.order ? io.order[it / pl.tiles] : it / pl.tiles;
     w.event = e;
@@ -2534,10 +2543,10 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
   };
   if (threadIdx.x == 0) {
     sh.staged = -1;
-    int it = blockIdx.x, left = 0;
+    int it = blockIdx.x, left = 0, run = 0;
     sh.runs = queue_runs(pl, io);
-    if (queue) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left);
-    fetch_item(sh.it[0], it, left);
+    if (queue) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left, run);
+    fetch_item(sh.it[0], it, left, run);
   }
 #pragma unroll 1
   for (int cur = 0;; cur ^= 1) {
@@ -2546,9 +2555,9 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
     run_item<MP, ITER, CL>(pl, io, smem, sh, cur, queue, do_cs);
     if (!queue) break;
     if (ITER && pl.tiles > 1 && threadIdx.x == 0) {
-      int it = sh.it[cur].item + 1, left = sh.it[cur].left - 1;
-      if (left < 0) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left);
-      fetch_item(sh.it[cur ^ 1], it, left);
+      int it = sh.it[cur].item + 1, left = sh.it[cur].left - 1, run = sh.it[cur].run;
+      if (left < 0) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left, run);
+      fetch_item(sh.it[cur ^ 1], it, left, run);
     }
   }
 }
