@@ -232,8 +232,7 @@ static bool table_symmetric(int n_theta) {
   return k > 0;
 }
 
-// make_plan with T theta tiles, in mirror pairs or (mp false) columns; with `threads`, of so many (a multiple of 32),
-// the warps that make no full share of the words left out of the vote.
+// make_plan with T theta tiles, in mirror pairs or (mp false) columns; with `threads`, of so many (a multiple of 32).
 static int plan_tiles(const hough_params* p, int T, bool mp, int max_cap, Plan& pl, int threads = 0) {
   // A mirror-pair tile owns WD = ceil(N/2 / T) words (columns [a, a + WD) and their mirrors;
   // the last tile fewer), in word groups of 32 lanes; other tiles W = ceil(N / T) columns.
@@ -254,8 +253,7 @@ static int plan_tiles(const hough_params* p, int T, bool mp, int max_cap, Plan& 
   pl.nrho_pad = (p->n_rho + 1) & ~1;
   const int halo = T > 1 ? 32 : 0;
   if (threads) {
-    pl.split = (threads - halo) / (pl.groups * 32);
-    if (pl.split < 1) return HOUGH_ESMEM;
+    pl.split = 1;
   } else if (p->block) {
     const int work = p->block - halo;
     if (work <= 0 || work % (pl.groups * 32)) {
@@ -274,6 +272,10 @@ static int plan_tiles(const hough_params* p, int T, bool mp, int max_cap, Plan& 
     return p->theta_tiles ? HOUGH_EPARAM : HOUGH_ESMEM;
   }
   pl.mp = mp ? 1 : 0;
+  if (mp) {
+    pl.vote_p = (pl.threads - halo) / 32 / (pl.groups / 2);
+    if (pl.vote_p < 1) return HOUGH_ESMEM;
+  }
   if (pl.mp) mp_consts(pl, p->n_rho);
   if (!pl.mp)
   // Column layout: the power of two of row ranges that minimises the slowest warp's row steps, each
@@ -365,15 +367,18 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
     pl.fp_dhi = (float)(-delta - 0.5);
   }
   // Mirror pairs (columns j and N-1-j in one word) need a table with c[N-1-j] = -c[j], s[N-1-j] = s[j] (true for
-  // round-half-away-from-zero). An odd N_theta takes them for the local maxima alone, in the tiles and threads that
-  // its columns take (so that a shape is accepted, and reported, as a column shape), else columns. (101 x 63, 500 events 118 -> 61 us; 199 x 200,
-  // 1,000 events 335 -> 204 us.)
+  // round-half-away-from-zero). An odd N_theta takes them in the tiles and threads that its columns take (so
+  // that a shape is accepted, and reported, as a column shape), else columns. (101 x 63, 500 events 118 -> 60 us; 199 x 200,
+  // 1,000 events 335 -> 204 us; iterative finder, 553 x 54, 196 events 529 -> 280 us.)
   const bool sym = table_symmetric(p->n_theta), odd = p->n_theta % 2 != 0;
   for (int T = (p->theta_tiles ? p->theta_tiles : 1); T <= (p->theta_tiles ? p->theta_tiles : 64); ++T) {
     rc = plan_tiles(p, T, sym && !odd, max_cap, pl);
-    if (rc == HOUGH_OK && odd && sym && p->peak_mode == HOUGH_PEAK_LOCAL_MAX) {
+    if (rc == HOUGH_OK && odd && sym) {
       Plan mp = pl;
-      if (plan_tiles(p, T, true, max_cap, mp, pl.threads) == HOUGH_OK) pl = mp;
+      // not where a whole accumulator leaves the iterative finder no room for lists
+      if (plan_tiles(p, T, true, max_cap, mp, pl.threads) == HOUGH_OK &&
+          !(mp.peak_mode == HOUGH_PEAK_ITERATIVE && T == 1 && mp.iter_cap == 0))
+        pl = mp;
     }
     if (rc == HOUGH_OK || p->theta_tiles) return rc;
   }
@@ -417,7 +422,7 @@ int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan&
   hough_params q = *p;
   q.theta_tiles = 1;
   const bool small = pl.n_theta * pl.n_rho <= 8192 && pl.peak_mode == HOUGH_PEAK_LOCAL_MAX;
-  long long best = small ? LLONG_MAX : (n_events + kSms - 1) / kSms * kTurn[1];
+  long long best = small ? LLONG_MAX : (n_events + kSms - 1) / kSms * kTurn[1] * 1024 / pl.threads;
   int best_cap = 0;
   Plan x = pl;
   for (int cap = 4096; cap >= 2048; cap -= 1024) {
@@ -428,9 +433,10 @@ int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan&
     }
     const int fit = kSmemPerSm / (x.smem_bytes + kSmemStatic + 1024);  // 1 KB a CTA is the system's
     for (int c = 2; c <= std::min(fit, 4); ++c) {
-      const long long t = (n_events + kSms * c - 1) / (kSms * c) * kTurn[c];
       const int block = 1024 / c / (x.groups * 32) * (x.groups * 32);
-      if (t < best && block) {
+      if (!block) break;
+      const long long t = (n_events + kSms * c - 1) / (kSms * c) * kTurn[c] * (1024 / c) / block;
+      if (t < best) {
         best = t;
         best_cap = cap;
         q.block = block;

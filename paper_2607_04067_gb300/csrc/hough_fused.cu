@@ -300,7 +300,7 @@ __device__ __forceinline__ void vote64(const Plan& pl, const VoteLane& L, const 
 // Word lane w in [0, (N_theta+1)/2) holds column w in its low half and column N_theta-1-w (its
 // mirror) in its high half, one word per physical row p = k + 1. With an odd N_theta the last word's column is
 // its own mirror (c = 0): the high half then repeats the low one. It serves as the neighbour of the column after it;
-// the peaks (run_item) and the fingerprint leave it out. Rows p = 0 and p = N_rho + 1
+// it has no place in the bitmaps, and the fingerprint and the finder's passes leave it out. Rows p = 0 and p = N_rho + 1
 // are guard rows: the fast path only takes hits whose rho stays within half a bin of the range,
 // so its unclamped bins fall in [-1, N_rho]; the guard rows are folded into rows 0 and
 // N_rho - 1 after the vote, which is what clamping would have done.
@@ -309,11 +309,11 @@ __device__ __forceinline__ int mp_word(int w, int p, int rows_phys) {
   return (((w >> 5) * rows_phys + p) << 5) + (w & 31);
 }
 
-// Cell (c, k) of a mirror-pair tile of Wd words; tile-local column c < Wd is word c's low half,
-// c >= Wd word 2 Wd - 1 - c's high half.
-__device__ __forceinline__ int mp_get(const uint32_t* acc, int c, int k, int Wd, const Plan& pl) {
+// Cell (c, k) of a mirror-pair tile of wt columns in Wd = (wt + 1) / 2 words; tile-local column c < Wd is word c's low
+// half, c >= Wd word wt - 1 - c's high half.
+__device__ __forceinline__ int mp_get(const uint32_t* acc, int c, int k, int Wd, int wt, const Plan& pl) {
   const bool hi = c >= Wd;
-  const uint32_t x = acc[mp_word(hi ? 2 * Wd - 1 - c : c, k + 1, pl.rows_phys)];
+  const uint32_t x = acc[mp_word(hi ? wt - 1 - c : c, k + 1, pl.rows_phys)];
   return hi ? (int)(x >> 16) : (int)(x & 0xffffu);
 }
 
@@ -321,11 +321,11 @@ __device__ __forceinline__ int mp_get(const uint32_t* acc, int c, int k, int Wd,
 // 16-bit store of zero into the cell's half of its word, which leaves the other half of the word alone.
 template <bool MP>
 struct FusedCells {
-  static constexpr bool kPairs = MP;  // word w holds columns w and 2 Wd - 1 - w
+  static constexpr bool kPairs = MP;  // word w holds columns w and NT - 1 - w
   uint32_t* acc;
-  int Wd, nrp, rp;  // tile words, padded rows (other layouts), rows with guards (mirror-pair)
+  int Wd, NT, nrp, rp;  // words, columns, padded rows (other layouts), rows with guards (mirror-pair)
   __device__ int words() const { return Wd; }
-  __device__ int mirror_col(int w) const { return 2 * Wd - 1 - w; }
+  __device__ int mirror_col(int w) const { return NT - 1 - w; }
   __device__ uint32_t word(int w, int k) const { return acc[mp_word(w, k + 1, rp)]; }
   // words w4 .. w4 + 3 of row k (w4 a multiple of 4: all four in one 32-word group, 16-byte aligned;
   // words past the tile's own are zero)
@@ -335,7 +335,7 @@ struct FusedCells {
   __device__ int get(int j, int k) const {
     if (MP) {
       const bool hi = j >= Wd;
-      const uint32_t x = acc[mp_word(hi ? 2 * Wd - 1 - j : j, k + 1, rp)];
+      const uint32_t x = acc[mp_word(hi ? NT - 1 - j : j, k + 1, rp)];
       return hi ? (int)(x >> 16) : (int)(x & 0xffffu);
     }
     return acc_get(acc, j, k, nrp);
@@ -343,7 +343,7 @@ struct FusedCells {
   __device__ void clear(int j, int k) {
     if (MP) {
       const bool hi = j >= Wd;
-      reinterpret_cast<uint16_t*>(acc)[2 * mp_word(hi ? 2 * Wd - 1 - j : j, k + 1, rp) + (hi ? 1 : 0)] = 0;
+      reinterpret_cast<uint16_t*>(acc)[2 * mp_word(hi ? NT - 1 - j : j, k + 1, rp) + (hi ? 1 : 0)] = 0;
     } else {
       reinterpret_cast<uint16_t*>(acc)[2 * acc_index(j, k, nrp) + (k & 1)] = 0;
     }
@@ -390,7 +390,7 @@ struct WholeWindow {
   }
   __device__ uint16_t* cell(int j, int k) const {
     const bool hi = j >= half;
-    return reinterpret_cast<uint16_t*>(acc + mp_word(hi ? 2 * half - 1 - j : j, k + 1, rp)) + (hi ? 1 : 0);
+    return reinterpret_cast<uint16_t*>(acc + mp_word(hi ? NT - 1 - j : j, k + 1, rp)) + (hi ? 1 : 0);
   }
   __device__ bool live(uint32_t jk) const { return *cell((int)(jk >> 16), (int)(jk & 0xffffu)) != 0; }
   // Rank within a window in 32 bits: votes (15 bits), then the place of the column in raster order (9 bits; a
@@ -642,7 +642,7 @@ __device__ __forceinline__ void vote_last(const Plan& pl, const int16_t* tc, con
 template <int W, int U>
 __device__ __forceinline__ void vote_words(const Plan& pl, unsigned char* smem, const int16_t* tc, const int16_t* ts,
                                            uint32_t acc_s, int aw, int Wd, int nv, const AmbList& L) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = pl.groups >> 1, P2 = 2 * pl.split;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = pl.groups >> 1, P2 = pl.vote_p;
   const int P = P2 * W, w0 = (warp / P) * (32 * W) + lane, np = nv >> 1;
   const float4* hb4 = reinterpret_cast<const float4*>(smem + pl.off_hits);
   if (warp < G * P2 && w0 < Wd) {
@@ -839,6 +839,8 @@ __device__ __forceinline__ void scan_groups(const Plan& pl, const uint32_t* sw, 
   // high half; lane w-1's high half follows it (except at word 0: the wrapped column 0).
   // Strictness becomes +1 on that neighbour, so a cell is a peak iff C >= max(U + 1, D,
   // VU + addU, VD + 0x10000, T) per half.
+  const bool mid = 2 * (aw + half) - 1 == pl.n_theta;  // the last word's column is the middle one, which has one place
+  const int last = 2 * half - 1 - mid;                  // the tile's last column
   for (int it = warp; it < nl; it += nwarps) {
     const int en = list[it], g = en >> 8, k = (en & 255) << 2, n = min(32, half - 32 * g), w = 32 * g + lane;
     const uint32_t addU = (w != 0 || aw != 0) ? 1u : 0x10000u;
@@ -872,26 +874,26 @@ __device__ __forceinline__ void scan_groups(const Plan& pl, const uint32_t* sw, 
       fl &= valid;
       cf &= valid;
     }
+    if (mid && w == last - w) fl &= 0xffffu, cf &= 0xffffu;
     if (CAND && lane < n) {
       const uint32_t lo = (cf >> 12) & 15u, hi = cf >> 28;
       if (lo) atomicOr(&cand[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
-      if (hi) atomicOr(&cand[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
+      if (hi) atomicOr(&cand[(last - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
     }
     if (lane < n) {
       const uint32_t lo = (fl >> 12) & 15u, hi = fl >> 28;
       if (lo) atomicOr(&pbits[w * pl.nrb_p + (k >> 5)], lo << (k & 31));
-      if (hi) atomicOr(&pbits[(2 * half - 1 - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
+      if (hi) atomicOr(&pbits[(last - w) * pl.nrb_p + (k >> 5)], hi << (k & 31));
     }
     if (KEYS && lane < n) {
-      // bits 0-3 the low column's rows, 4-7 the high one's (a middle column's repetition left out)
-      const uint32_t x = CAND ? cf : fl, hmask = 2 * (aw + w) + 1 != pl.n_theta ? 0xf0u : 0u;
-      uint32_t bits = ((x >> 12) & 15u) | ((x >> 24) & hmask);
+      const uint32_t x = CAND ? cf : fl;  // bits 0-3 the low column's rows, 4-7 the high one's
+      uint32_t bits = ((x >> 12) & 15u) | ((x >> 24) & 0xf0u);
       const uint32_t lms = CAND ? ((fl >> 12) & 15u) | ((fl >> 24) & 0xf0u) : 0u;
       if (bits) {
         int at = atomicAdd(found.n, __popc(bits));
         for (; bits && at < found.cap; bits &= bits - 1u, ++at) {
           const int b = __ffs(bits) - 1;
-          found.key[at] = found_key(b < 4 ? w : 2 * half - 1 - w, k + (b & 3), (lms >> b) & 1u);
+          found.key[at] = found_key(b < 4 ? w : last - w, k + (b & 3), (lms >> b) & 1u);
         }
       }
     }
@@ -1482,11 +1484,10 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
   const int nrb = staged ? pl.nrb_g : pl.nrb;  // guard-bit bitmaps are one bit wider on each side
   const uint32_t* pbits = reinterpret_cast<const uint32_t*>(smem + pl.off_pbits);
   for (int i = tid; i < 64; i += bd) hist[i] = 0;
-  const int dup = pl.mp && (NT & 1) ? (NT + 1) >> 1 : NT;  // the bitmap's place of a middle column's repetition
   if (from_bits) {
     for (int j = tid; j < NT; j += bd) {
       int cc = 0;
-      for (int w = 0; w < pl.nrb; ++w) cc += __popc(pbits[(j + (j >= dup)) * pl.nrb_p + w]);
+      for (int w = 0; w < pl.nrb; ++w) cc += __popc(pbits[j * pl.nrb_p + w]);
       colcnt[j] = cc;
     }
   } else {
@@ -1533,7 +1534,7 @@ __device__ int select_event(const Plan& pl, const FusedIO& io, unsigned char* sm
       while (it - W * NG >= NG) ++W;
       const int j = 32 * (it - W * NG) + lane;
       if (j >= NT || colcnt[j] == 0) continue;
-      const uint32_t* P = pbits + (j + (j >= dup)) * pl.nrb_p;
+      const uint32_t* P = pbits + j * pl.nrb_p;
       bm[colidx[j] * nrb + W] = staged ? dilated_guard_word(P, W, pl.nrb, NR, hw) : dilated_word(P, W, pl.nrb, NR, hw);
     }
   } else {
@@ -1605,9 +1606,12 @@ __device__ __noinline__ unsigned long long tile_checksum(const uint32_t* acc, in
   for (int i = threadIdx.x; i < half * NR; i += blockDim.x) {
     const int k = i / half, w = i - k * half;
     const uint32_t x = acc[mp_word(w, k + 1, rp)];
-    cs += (unsigned long long)(x & 0xffffu) * mix64((unsigned long long)(aw + w) * NR + k + 1);
-    if (2 * (aw + w) + 1 != NT) cs += (unsigned long long)(x >> 16) * mix64((unsigned long long)(NT - 1 - aw - w) * NR + k + 1);
+    cs += (unsigned long long)(x & 0xffffu) * mix64((unsigned long long)(aw + w) * NR + k + 1) +
+          (unsigned long long)(x >> 16) * mix64((unsigned long long)(NT - 1 - aw - w) * NR + k + 1);
   }
+  if (2 * (aw + half) - 1 == NT)  // the middle column once
+    for (int k = threadIdx.x; k < NR; k += blockDim.x)
+      cs -= (unsigned long long)(acc[mp_word(half - 1, k + 1, rp)] >> 16) * mix64((unsigned long long)(NT >> 1) * NR + k + 1);
   return cs;
 }
 
@@ -1910,26 +1914,23 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
   const int16_t* ts = tc + pl.n_theta;
   const int T = pl.tiles, NT = pl.n_theta, nrp = pl.nrho_pad;
   const int j0 = t * pl.tile_w;
-  const int wt = min(pl.tile_w, NT + (MP ? NT & 1 : 0) - j0);
+  const int wt = min(pl.tile_w, NT - j0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
   const int wpad = pl.groups * 32;
   const int rows_w = nrp >> 1;  // words per column
   // mirror-pair tiles: words [aw, aw + Wd), i.e. columns [aw, aw + Wd) and their mirrors
   // (full tiles own tile_w / 2 words, the last one possibly fewer)
-  const int Wd = MP ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
+  const int Wd = MP ? (wt + 1) >> 1 : 0, aw = t * (pl.tile_w >> 1);
 
   // lane roles of the vote
   VoteLane L;
-  L.halo = warp >= pl.groups * pl.split;
+  L.halo = !MP && warp >= pl.groups * pl.split;
   L.on = false;
   L.cj = L.sj = 0;
   L.col1 = L.col2 = 0;
   const uint32_t acc_s = (uint32_t)__cvta_generic_to_shared(acc);
   const bool want_halo = !ITER;  // only the 3x3 test reads the halo
-  if (L.halo && MP) {
-    L.p = 0;  // no words of its own (every thread votes halo hits)
-    L.P = 1;
-  } else if (L.halo) {
+  if (L.halo) {
     const int jh = lane < 16 ? (j0 - 1 + NT) % NT : (j0 + wt) % NT;
     L.on = want_halo;
     L.cj = tc[jh];
@@ -1938,7 +1939,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
     L.p = 0;
     L.P = 1;
   } else if (MP) {
-    const int P2 = 2 * pl.split, gpair = warp / P2;
+    const int P2 = pl.vote_p, gpair = warp / P2;  // (past the last group: no words)
     L.p = warp % P2;
     L.P = P2;
     const int c1 = gpair * 32 + lane;
@@ -2071,9 +2072,9 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   const long long e = sh.it[cur].event;
   const int t = sh.it[cur].item % T;
   const int j0 = t * pl.tile_w;
-  const int wt = min(pl.tile_w, NT + (MP ? NT & 1 : 0) - j0);
+  const int wt = min(pl.tile_w, NT - j0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
-  const int Wd = MP ? (wt >> 1) : 0, aw = t * (pl.tile_w >> 1);
+  const int Wd = MP ? (wt + 1) >> 1 : 0, aw = t * (pl.tile_w >> 1);
 
   // the next item, in steps whose latencies pass behind the phases between them (thread 0)
   WorkItem& next = sh.it[cur ^ 1];
@@ -2132,7 +2133,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     if (do_cs) {
       unsigned long long cs = 0;
       for (int c = tid; c < NT * NR; c += bd) {
-        const int j = c / NR, k = c - j * NR, v = MP ? mp_get(acc, j, k, Wd, pl) : acc_get(acc, j, k, nrp);
+        const int j = c / NR, k = c - j * NR, v = MP ? mp_get(acc, j, k, Wd, wt, pl) : acc_get(acc, j, k, nrp);
         if (v) cs += (unsigned long long)v * mix64((unsigned long long)c + 1);
       }
       cs_tile = block_sum_u64(cs, sh.red);
@@ -2162,13 +2163,17 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // No bitmaps, or more peaks than the list ranks. (One pass a peak lists a kept set's cells in rank order
     // too: the dropped candidates are zero, the cells that are none below the threshold.)
     if (total < 0) {
+      if (MP && (NT & 1)) {  // a middle column's repetition
+        for (int k = tid; k < NR; k += bd) reinterpret_cast<uint16_t*>(acc)[2 * mp_word(Wd - 1, k + 1, pl.rows_phys) + 1] = 0;
+        __syncthreads();
+      }
       auto general = [&](auto cells) {
         const int st_words = (((NT * NR + 15) >> 4) + 31) & ~31;  // 2 bits a cell, whole 32-word blocks
         return extract_iterative(cells, NT, NR, kIterSliceRows, pl.threshold, pl.rel_num, pl.rel_den, pl.nms_radius,
                                  maxp, pbits, MP ? 0 : pl.iter_cap, nullptr, st_words, dst, sh.tmp,
                                  reinterpret_cast<uint16_t*>(pbits + pl.iter_cap + st_words), pl.iter_act);
       };
-      total = MP ? general(FusedCells<true>{acc, Wd, nrp, pl.rows_phys}) : general(FusedCells<false>{acc, Wd, nrp, pl.rows_phys});
+      total = MP ? general(FusedCells<true>{acc, Wd, NT, nrp, pl.rows_phys}) : general(FusedCells<false>{acc, Wd, NT, nrp, pl.rows_phys});
     }
     n_low = total;
   } else {
@@ -2206,10 +2211,6 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       if (T > 1 && !CL)
         found = Found{reinterpret_cast<uint32_t*>(cnt) + gate, min(kFoundMax, pl.groups * 32 * pl.key_groups - gate), &sh.n_found};
       scan_mp<false>(pl, smem, pl.threshold, aw, Wd, sh.edge, pbits, nullptr, reinterpret_cast<uint16_t*>(cnt), &sh.n_amb, found);
-      if ((NT & 1) && aw + Wd == (NT + 1) >> 1) {  // the middle column's repetition
-        __syncthreads();
-        for (int i = tid; i < pl.nrb; i += bd) pbits[Wd * pl.nrb_p + i] = 0u;
-      }
     } else if (packed) {
       scan_packed(pl, acc, halo, pbits, wt, T, j0, do_cs, csum);
     } else {
@@ -2291,7 +2292,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     }
     // event column of tile-local column c: mirror-pair tiles hold [aw, aw + Wd) then
     // [N - aw - Wd, N - aw), both ascending; other tiles [j0, j0 + wt)
-    const int hi0 = NT - aw - 2 * Wd;
+    const int hi0 = NT - aw - wt;
     hough_peak* dst = (T == 1 || CL) ? io.peaks + e * (long long)maxp : io.tile_peaks + (e * T + t) * (long long)maxp;
     uint2* dst2 = reinterpret_cast<uint2*>(dst);  // records are 8-byte aligned (checked on the host)
     if (ranked) {
@@ -2306,7 +2307,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         const int c = (int)(key >> 11), k = (int)(key >> 1) & 1023;
         if (lane == 0 && pos < maxp)
           dst2[pos] = make_uint2((uint32_t)(c < Wd ? aw + c : hi0 + c) | ((uint32_t)k << 16),
-                                 (uint32_t)mp_get(acc, c, k, Wd, pl) | (pl.off_local ? (key & 1u) << 16 : 0u));
+                                 (uint32_t)mp_get(acc, c, k, Wd, wt, pl) | (pl.off_local ? (key & 1u) << 16 : 0u));
       }
     } else if (G == 1) {
       // a lane takes a key: its word's peaks, one a step, to the positions after the lanes before it
@@ -2334,7 +2335,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         while (bits && pos < maxp) {
           const int k = k0 + __ffs(bits) - 1;
           bits &= bits - 1u;
-          const int votes = MP ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
+          const int votes = MP ? mp_get(acc, c, k, Wd, wt, pl) : acc_get(acc, c, k, nrp);
           uint32_t lm = 0u;
           if (ITER && MP && pl.off_local) lm = (local[c * pl.nrb_p + (k >> 5)] >> (k & 31)) & 1u;
           dst2[pos++] = make_uint2((uint32_t)col | ((uint32_t)k << 16), (uint32_t)votes | (lm << 16));
@@ -2351,7 +2352,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
             const int bb = __ffs(bits) - 1;
             bits &= bits - 1u;
             const int k = (w << 5) + bb;
-            const int votes = MP ? mp_get(acc, c, k, Wd, pl) : acc_get(acc, c, k, nrp);
+            const int votes = MP ? mp_get(acc, c, k, Wd, wt, pl) : acc_get(acc, c, k, nrp);
             const int col = MP ? (c < Wd ? aw + c : hi0 + c) : j0 + c;
             uint32_t lm = 0u;
             if (ITER && MP && pl.off_local) lm = (local[c * pl.nrb_p + w] >> bb) & 1u;
@@ -2609,7 +2610,7 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
     int flags = 0;
     for (int t = 0; t < T; ++t) {
       vote_tile<MP, true>(pl, io, smem, sh, (int)e, a, n, t);
-      const int j0 = t * pl.tile_w, wt = min(pl.tile_w, NT - j0), Wd = MP ? (wt >> 1) : 0,
+      const int j0 = t * pl.tile_w, wt = min(pl.tile_w, NT - j0), Wd = MP ? (wt + 1) >> 1 : 0,
                 aw = t * (pl.tile_w >> 1);
       if (MP) {
         mp_fold(pl, const_cast<uint32_t*>(acc), Wd, nullptr);

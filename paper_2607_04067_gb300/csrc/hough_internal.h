@@ -39,6 +39,7 @@ struct Plan {
   int key_words;    // bitmap words per key
   int grab;       // persistent queue: items per pop
   int cluster;    // an event's tiles are the CTAs of a cluster (mirror pairs, local maxima; no workspace)
+  int vote_p;     // mirror pairs: warps that share a word group's votes
   int ws_tiles;   // the tiles that the workspace is laid out for: those of a large call
   int mp;         // 1: mirror-pair word layout (column j low half, N_theta-1-j high half, guard rows)
   int rows_phys;  // mirror-pair layout: physical rows per column (N_rho + 2)

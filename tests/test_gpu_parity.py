@@ -409,10 +409,17 @@ def test_odd_theta_edges(h, nt, nr, tiles):
     xy = np.concatenate([ev.xy[: ev.off[-1]], np.array(mid + wide)]).astype(np.int32)
     off = np.concatenate([ev.off, ev.off[-1] + np.array([240, 540])]).astype(np.int64)
     t_xy, t_off = torch.from_numpy(xy).cuda(), torch.from_numpy(off).cuda()
-    for thr, maxp, hw in ((3, 4096, 1), (12, 60, 0), (30, 4096, 40)):
-        ref = oracle.run(xy, off, oracle.params(nt, nr, thr, hw, maxp), threads=THREADS)
+    it = dict(peak_mode=1, rel_num=1, rel_den=3)
+    for thr, maxp, hw, kw in ((3, 4096, 1, {}), (12, 60, 0, {}), (30, 4096, 40, {}), (3, 4096, 1, dict(it, nms_radius=1)),
+                              (2, 4096, 0, dict(it, nms_radius=min(5, (nt - 1) // 2)))):
+        ref = oracle.run(xy, off, oracle.params(nt, nr, thr, hw, maxp, **kw), threads=THREADS)
         for batched in (False, True):
-            out = h.run(t_xy, t_off, h.params(nt, nr, thr, hw, maxp, theta_tiles=tiles), checksum=True, batched=batched)
+            try:
+                p = h.resolve(h.params(nt, nr, thr, hw, maxp, theta_tiles=tiles, **kw))
+            except h.HoughError:
+                assert kw  # the iterative finder refuses some tilings
+                continue
+            out = h.run(t_xy, t_off, h.params(nt, nr, thr, hw, maxp, theta_tiles=tiles, **kw), checksum=True, batched=batched)
             assert h.status(out.status) == ref.status
             assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
 
