@@ -82,7 +82,8 @@ extern "C" {
 #define HOUGH_MAX_EVENT_HITS 32767
 #define HOUGH_RHO_HALF_RANGE 703687442LL /* H */
 
-/* Algorithm and launch parameters. Zero in a launch field means "choose". */
+/* Algorithm and launch parameters. Zero in a launch field means "choose": by these parameters and by a call's events
+ * and hits. No result depends on a launch field. */
 typedef struct hough_params {
   int32_t n_theta;        /* N_theta in [4, 1024] */
   int32_t n_rho;          /* N_rho in [4, 1024] */
@@ -90,7 +91,7 @@ typedef struct hough_params {
   int32_t keep_halfwidth; /* rho-bin half-width of the selection window, >= 0 */
   int32_t max_peaks;      /* stored peaks per event, in [1, 65536] */
   int32_t theta_tiles;    /* theta tiles per event (0 = auto); each tile is one CTA */
-  int32_t events_per_cta; /* persistent queue: work items taken per pop (0 = auto) */
+  int32_t events_per_cta; /* persistent queue: work items taken per pop (0 = auto: an event's tiles) */
   int32_t block;          /* threads per CTA (0 = auto) */
   /* Peak finder (Sec. 2). HOUGH_PEAK_LOCAL_MAX (0, the default): one pass of 3x3 local maxima
    * >= threshold, listed in raster order. HOUGH_PEAK_ITERATIVE (1): the paper's own finder. A
@@ -99,8 +100,7 @@ typedef struct hough_params {
    * that is not yet suppressed (ties: the first in raster order) becomes the next peak, and
    * every cell within nms_radius of it in theta and rho is suppressed. Theta wraps with rho
    * mirrored, and rows beyond the rho edges are skipped. Peaks are listed in extraction order.
-   * The iterative finder needs the whole accumulator in one CTA on the fused paths
-   * (theta_tiles 1); the stepwise hough_peaks takes any size. */
+   * Fused paths take it on whole accumulators and on theta tiles, the stepwise hough_peaks at any size. */
   int32_t peak_mode;
   int32_t rel_num;        /* mode 1: numerator of the relative threshold, 0 <= rel_num <= rel_den */
   int32_t rel_den;        /* mode 1: denominator, >= 1 */
@@ -375,7 +375,7 @@ int hough_run_batched_static(const int32_t* d_xy, int64_t n_hits, const int64_t*
 /* Autotuner of the batched path: times hough_run_batched's kernels on the sample batch
  * (d_xy, d_off: device, the caller's representative events) for every feasible launch shape
  * -- theta tiles in {1, 2, 4, 8, 16}, threads per CTA in {256, 512, 1024} (or the widest the
- * tiling allows), queue items per pop (events_per_cta) in {1, 2, 4} -- and writes the fastest
+ * tiling allows), queue items per pop (events_per_cta) in {1, 2, 4, tiles} -- and writes the fastest
  * into *p (theta_tiles, block, events_per_cta; the algorithm fields are untouched). d_scratch
  * holds outputs and workspace of every candidate: hough_autotune_scratch_size bytes, 256-byte
  * aligned. Results are cached per (parameters, device, SM count, hits per event in octaves);
@@ -384,7 +384,8 @@ size_t hough_autotune_scratch_size(const hough_params* p, int64_t n_hits, int64_
 int hough_autotune(hough_params* p, const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int64_t n_events,
                    void* d_scratch, size_t scratch_bytes, int32_t* d_status, void* stream, float* best_ms);
 
-/* Launch shape the library would use for these parameters: fills the zero launch fields
+/* Launch shape the library would use for these parameters in a large call (calls of few events, or of many with small
+ * accumulators, take other tiles or threads where those are left to it): fills the zero launch fields
  * of *p (theta_tiles, events_per_cta, block) and returns HOUGH_OK or an error. */
 int hough_resolve_params(hough_params* p);
 

@@ -766,20 +766,21 @@ int hough_autotune(hough_params* p, const int32_t* d_xy, int64_t n_hits, const i
   bool found = false;
   for (int T = 1; T <= 16; T *= 2) {
     for (int threads : {256, 512, 1024}) {
-      for (int grab : {1, 2, 4}) {
+      bool have_t = false;
+      for (int grab : {1, 2, 4, T}) {  // (T: an event's tiles in a run)
+        if (grab == T && T <= 4 && have_t) continue;
+        have_t = have_t || grab == T;
         hough_params q = *p;
         q.theta_tiles = T;
         q.events_per_cta = grab;
         Plan probe;
         q.block = 0;
         if (make_plan(&q, probe) != HOUGH_OK) continue;
-        const int halo = T > 1 ? 32 : 0;
-        const int lanes = probe.groups * 32;
-        if (threads - halo <= 0 || (threads - halo) % lanes) {
+        q.block = threads;
+        Plan exact;
+        if (make_plan(&q, exact) != HOUGH_OK) {
           if (threads != 1024) continue;
           q.block = probe.threads;  // the widest block this tiling allows
-        } else {
-          q.block = threads;
         }
         Common cm;
         if (prepare_fused(d_xy, n_hits, d_off, n_events, &q, (int32_t*)(s + L.npeaks), (hough_peak*)(s + L.peaks),

@@ -8,12 +8,13 @@
 //     Lane l's cells live in shared-memory bank l only: word ((g * rows + row) * 32 + l),
 //     rows = N_rho / 2 packed int16 pairs, so the column-parallel
 //     vote is free of bank conflicts whatever rho bins the hits hit; warps sharing
-//     columns split the hits and add with red.shared. With an even N_theta a lane owns
+//     columns split the hits and add with red.shared. In mirror pairs a lane owns
 //     column j and its mirror N_theta-1-j (th -> pi - th: c -> -c, s -> s), so one pair
 //     of products gives both rho values;
-//   - for tiled events one extra warp votes the two neighbour columns of the tile
-//     (halo), so the 3x3 peak test is exact on tile edges; the last tile CTA of an
-//     event (ticket counter) merges the tiles' peak lists in tile order and selects.
+//   - for tiled events the neighbour columns of the tile are voted too (halo: mirror pairs by every thread,
+//     columns by one extra warp), so the 3x3 peak test is exact on tile edges; the last tile CTA of an
+//     event (ticket counter; a run of all tiles in one CTA needs none) merges the tiles' peak lists in tile order
+//     and selects. Events of small calls take the tiles of a cluster, which merge without a workspace.
 #include <climits>
 #include <map>
 #include <mutex>
@@ -217,7 +218,7 @@ __device__ void stage_sel64(const int2* __restrict__ xy, long long base, int cn,
 // Which columns a worker lane owns, and where their row-0 words live.
 struct VoteLane {
   bool on;          // lane votes
-  bool halo;        // lane of the halo warp (tiles > 1)
+  bool halo;        // columns: lane of the halo warp (tiles > 1)
   int p, P;         // hit partition of this warp, partitions per column set
   int cj, sj;       // trig of the (first) column
   uint32_t col1;    // shared address of column 1, row 0

@@ -23,8 +23,8 @@ struct Plan {
   int tiles;      // theta tiles per event
   int tile_w;     // columns per tile (last tile may be narrower)
   int groups;     // 32-column groups per tile
-  int split;      // warps voting each column group (hit partitions)
-  int threads;    // CTA size: groups * split * 32 (+ 32 halo lanes when tiles > 1)
+  int split;      // columns: warps voting each column group (hit partitions)
+  int threads;    // CTA size: groups * split * 32 (+ 32 halo lanes when tiles > 1), an odd N_theta's as its columns'
   int nrho_pad;   // rows allocated per column
   int nrb;        // 32-bit bitmap words per column
   int nrb_p;      // words a column takes in the peak bitmap: nrb made odd where there is room, so that

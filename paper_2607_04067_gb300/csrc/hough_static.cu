@@ -19,7 +19,7 @@
 // device afterwards. Every call shares the same array and leaves its
 // contents behind, so calls that overlap on the GPU (other streams, other host threads) race
 // and must be serialised by the caller. Everything that has to start at zero (the queue
-// counter and the per-event tile tickets) is cleared by the validation kernel of each call.
+// counter and the per-event tile tickets) is cleared by the validation kernel of each call that uses it.
 #include <cstring>
 #include <mutex>
 

@@ -383,6 +383,18 @@ def test_records_by_keys(h, nt, nr, tiles):
                 assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
 
 
+@pytest.mark.parametrize("nt", [65, 101, 513])
+def test_autotune_odd_theta(h, nt):
+    """A shape for an odd column count, in mirror pairs or columns, that the run then accepts."""
+    ev = gen.generate("plain_small", 40)
+    xy, off = dev(ev)
+    tuned, _ = h.autotune(xy, off, h.params(nt, 200, 9, 1, 512))
+    ref = oracle.run(ev.xy, ev.off, oracle.params(nt, 200, 9, 1, 512), threads=THREADS)
+    out = h.run(xy, off, tuned, checksum=True, batched=True)
+    assert h.status(out.status) == ref.status
+    assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
+
+
 @pytest.mark.parametrize("copies", [1, 12])
 def test_large_events_in_clusters(h, copies):
     """Events in several staging chunks, one too large (skipped, flagged) and an empty one, in clusters of 4 and 2."""
