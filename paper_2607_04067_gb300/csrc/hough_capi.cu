@@ -642,7 +642,7 @@ static int batched_grid(const Common& cm) {
   const int per_sm = fused_max_ctas_per_sm(cm.pl);
   if (per_sm < 1) return -1;
   long long grid = (long long)sms * per_sm;
-  if (grid > cm.io.n_items) grid = cm.io.n_items;
+  if (grid > cm.io.n_items || cm.pl.cluster) grid = cm.io.n_items;  // clusters are whole and take no queue
   return (int)(grid > 0 ? grid : 1);
 }
 

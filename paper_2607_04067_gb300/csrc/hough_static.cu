@@ -110,7 +110,7 @@ extern "C" int hough_run_batched_static(const int32_t* d_xy, int64_t n_hits, con
   const int per_sm = fused_max_ctas_per_sm(pl);
   if (per_sm < 1) return HOUGH_ESMEM;
   long long grid = (long long)sms * per_sm;
-  if (grid > io.n_items) grid = io.n_items;
+  if (grid > io.n_items || pl.cluster) grid = io.n_items;  // clusters are whole and take no queue
   TrigTable trig;
   host_trig(p->n_theta, &trig);
   io.solo = fused_solo(pl, io.n_items, (int)grid);
