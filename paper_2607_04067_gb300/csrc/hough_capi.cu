@@ -399,8 +399,9 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
 // staged hits (half as many again as the mean; an event with more takes several chunks) make room for more CTAs.
 // One CTA -> this rule, us: 64 x 64, 616 hits, 5,000 events 424 -> 177 and 500 events 59 -> 30; 100 x 100, 1,290
 // hits, 5,000 events 640 -> 365; 128 x 128, 2,022 hits, 1,000 events 167 -> 131, iterative finder 286 -> 218.
-// An accumulator of at most 8,192 cells takes half the threads in any case (64 x 64, 100 events: 18.2 -> 16.5):
-// its phases are shorter than what 32 warps add to each barrier.
+// An accumulator of at most 8,192 cells with up to 1,024 hits an event takes half the threads in any case (64 x 64, 616
+// hits, 100 events: 18.2 -> 16.5; with 4,720 hits, two events, 50.3 -> 51.6, hence the line): its phases are shorter
+// than what 32 warps add to each barrier.
 int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan& pl) {
   const int rc = make_plan(p, pl);
   if (rc || p->block || n_events < 1) return rc;
@@ -421,7 +422,7 @@ int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan&
   static constexpr int kTurn[5] = {0, 20, 27, 38, 42};
   hough_params q = *p;
   q.theta_tiles = 1;
-  const bool small = pl.n_theta * pl.n_rho <= 8192 && pl.peak_mode == HOUGH_PEAK_LOCAL_MAX;
+  const bool small = pl.n_theta * pl.n_rho <= 8192 && pl.peak_mode == HOUGH_PEAK_LOCAL_MAX && n_hits <= 1024 * n_events;
   long long best = small ? LLONG_MAX : (n_events + kSms - 1) / kSms * kTurn[1] * 1024 / pl.threads;
   int best_cap = 0;
   Plan x = pl;
