@@ -400,7 +400,7 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
 // One CTA -> this rule, us: 64 x 64, 616 hits, 5,000 events 424 -> 177 and 500 events 59 -> 30; 100 x 100, 1,290
 // hits, 5,000 events 640 -> 365; 128 x 128, 2,022 hits, 1,000 events 167 -> 131, iterative finder 286 -> 218.
 // An accumulator of at most 8,192 cells with up to 1,024 hits an event takes half the threads in any case (64 x 64, 616
-// hits, 100 events: 18.2 -> 16.5; with 4,720 hits, two events, 50.3 -> 51.6, hence the line): its phases are shorter
+// hits, 100 events: 18.2 -> 16.5; 64 x 74, 4,720 hits, two events: 45.2 -> 51.6, hence the line): its phases are shorter
 // than what 32 warps add to each barrier.
 int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan& pl) {
   const int rc = make_plan(p, pl);
