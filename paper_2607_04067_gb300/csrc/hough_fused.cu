@@ -1388,9 +1388,12 @@ __device__ int select_staged(const Plan& pl, const int2* hb, const uint16_t* idx
 }
 
 // A work item: tile item % T of event `event`, whose hits are [off[0], off[1]). Two of them in shared
-// memory, the current one and the next: in a persistent launch the next is popped before the current one's
+// memory, the current one and the next: in a persistent launch the next is popped after the current one's
 // vote, and its event's index and offsets are read by asynchronous copies issued between the phases, so that
-// no barrier waits for their latency (3.5 k cycles an event in a chain after the last item).
+// no barrier waits for their latency (3.5 k cycles an event in a chain after the last item). Not earlier: the CTAs
+// start with the largest events, and those that pop as they start pair them with the next largest; half-way through
+// an item, those with small events come first, as they will at its end. (256 x 256, 160 events of 2,022 hits: 83.1 us popped
+// before the vote, 63.5 after it; 200 events 84.8 and 70.6; 20,000 events 4,678 and 4,656.)
 constexpr int kFoundMax = 128;  // keys that are ranked one by one
 
 struct WorkItem {
@@ -2054,6 +2057,16 @@ __device__ __forceinline__ void popped(const Plan& pl, const FusedIO& io, unsign
   left = run ? pl.grab - 1 : 0;
 }
 
+// Whether the item after `item` is popped at its end and not after its vote: the iterative finder on tiles, where an
+// event's last tile takes much longer than the others and an item popped before it would wait for it instead of going
+// to another CTA; and on whole events in the last two turns, since two thirds of an event come after its vote and not in
+// proportion to its hits (256 x 256, half the maximum, R = 3, 160 events of 1,290 hits: 93.4 us popped after the vote, 81.0
+// so; the chain costs 3.5 k of 119 k cycles an item, in those turns alone).
+template <bool ITER>
+__device__ __forceinline__ bool pops_late(const Plan& pl, const FusedIO& io, int item) {
+  return ITER && (pl.tiles > 1 || item + 2LL * gridDim.x >= io.n_items);
+}
+
 // The work item sh.it[cur]; with `queue`, sh.it[cur ^ 1] receives the one after it.
 // CL: the event's T tiles are the CTAs of a cluster (tile t the CTA of rank t), which exchange their record counts, write their
 // records to their places and test a T-th of the hits each: for calls of so few events that SMs would stay idle.
@@ -2079,12 +2092,13 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
 
   // the next item, in steps whose latencies pass behind the phases between them (thread 0)
   WorkItem& next = sh.it[cur ^ 1];
-  // Not for the iterative finder on tiles: there an event's last tile takes much longer than the others, and an
-  // item popped before it would wait for it instead of going to another CTA.
-  const bool fetch = queue && tid == 0 && !(ITER && T > 1);
+  const bool ahead = queue && !pops_late<ITER>(pl, io, sh.it[cur].item);
+  const bool fetch = ahead && tid == 0;
   unsigned long long pop = 0;
-  if (fetch && sh.it[cur].left == 0) pop = atomicAdd(io.queue, 1ull);
   bool other = false;  // the next item exists and belongs to another event
+  auto fetch_pop = [&]() {
+    if (fetch && sh.it[cur].left == 0) pop = atomicAdd(io.queue, 1ull);
+  };
   auto fetch_event = [&]() {
     if (!fetch) return;
     int more = sh.it[cur].item + 1, left = sh.it[cur].left - 1, run = sh.it[cur].run;
@@ -2115,7 +2129,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     const long long a = sh.it[cur].off[0], nll = sh.it[cur].off[1] - a;
     vote_tile<MP, ITER>(pl, io, smem, sh, (int)e, a, nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll, t);
   }
-  fetch_event();
+  fetch_pop();
 
   // 3-4. peaks
   const int maxp = pl.max_peaks;
@@ -2141,7 +2155,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       __syncthreads();
     }
     HOUGH_PHASE(HOUGH_PHASE_SCAN);
-    fetch_offsets();
+    fetch_event();
     hough_peak* dst = io.peaks + e * (long long)maxp;
     total = -1;
     if (MP && pl.iter_cap > 0) {
@@ -2154,6 +2168,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       scan_mp<true>(pl, smem, tq, 0, Wd, sh.edge, pbits, cand, reinterpret_cast<uint16_t*>(list), &sh.n_amb,
                     Found{nullptr, 0, &sh.n_found});
       __syncthreads();
+      fetch_offsets();
       const WholeWindow ww{acc, Wd, pl.rows_phys, NT, NR, pl.nms_radius, pl.nrb_p, cand, pbits};
       const int nk = resolve_kept(ww, list, pl.iter_cap, reinterpret_cast<uint16_t*>(list + 2 * pl.iter_cap), sh.tmp);
       if (nk <= ranked_room(2 * pl.iter_cap)) {
@@ -2164,6 +2179,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // No bitmaps, or more peaks than the list ranks. (One pass a peak lists a kept set's cells in rank order
     // too: the dropped candidates are zero, the cells that are none below the threshold.)
     if (total < 0) {
+      if (!MP || pl.iter_cap == 0) fetch_offsets();
       if (MP && (NT & 1)) {  // a middle column's repetition
         for (int k = tid; k < NR; k += bd) reinterpret_cast<uint16_t*>(acc)[2 * mp_word(Wd - 1, k + 1, pl.rows_phys) + 1] = 0;
         __syncthreads();
@@ -2219,7 +2235,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     }
     __syncthreads();
     HOUGH_PHASE(HOUGH_PHASE_SCAN);
-    fetch_offsets();
+    fetch_event();
 
     // 4. raster-order positions and peak records: keys (column, group of key_words bitmap words)
     // in raster order, counted from the peak bitmap
@@ -2269,6 +2285,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       total = block_exscan(cnt, nkeys, sh.tmp);
     }
     HOUGH_PHASE(HOUGH_PHASE_EXSCAN);
+    fetch_offsets();
     // peaks of the tile's low columns (mirror-pair tiles: the high columns follow them)
     if (!ranked && (!CL || G > 1)) n_low = (MP && Wd < wt && G > 1) ? cnt[key_hi] : total;
     int low_at = 0, high_at = 0;  // CL: of the tile's low and high records, places in the event's less those in the tile's
@@ -2464,7 +2481,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_MERGE);
-  if (queue && !(ITER && T > 1) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
+  if (ahead && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
     const long long i = next.off[0] + 16LL * tid;
     if (i < next.off[1]) asm volatile("prefetch.global.L2 [%0];" ::"l"(io.xy + i));
   }
@@ -2556,7 +2573,7 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
     if (sh.it[cur].item >= io.n_items) break;
     run_item<MP, ITER, CL>(pl, io, smem, sh, cur, queue, do_cs);
     if (!queue) break;
-    if (ITER && pl.tiles > 1 && threadIdx.x == 0) {
+    if (pops_late<ITER>(pl, io, sh.it[cur].item) && threadIdx.x == 0) {
       int it = sh.it[cur].item + 1, left = sh.it[cur].left - 1, run = sh.it[cur].run;
       if (left < 0) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left, run);
       fetch_item(sh.it[cur ^ 1], it, left, run);

@@ -331,6 +331,47 @@ def test_offsets_checked_by_either_kernel(h, n, batched):
     assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off)
 
 
+def best_us(f, stream, reps=10, rounds=7):
+    """Time of one of `reps` calls back to back, the best of `rounds`."""
+    for _ in range(3):
+        f()
+    stream.synchronize()
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = float("inf")
+    for _ in range(rounds):
+        a.record(stream)
+        for _ in range(reps):
+            f()
+        b.record(stream)
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / reps * 1e3)
+    return best
+
+
+def time_run(h, xy, off, p, stream, batched=True):
+    t_xy, t_off = torch.from_numpy(np.ascontiguousarray(xy)).cuda(), torch.from_numpy(off).cuda()
+    out = h.alloc_outputs(len(xy), len(off) - 1, p)
+    torch.cuda.synchronize()
+    return best_us(lambda: h.run(t_xy, t_off, p, out=out, batched=batched, stream=stream), stream)
+
+
+def test_uneven_events_in_two_turns(h):
+    """A CTA an event, half of them large, and eight small events more. Two small ones one after the other (1,500 hits) end
+    before a large one (6,000), so the eight should cost next to nothing beside eight empty ones; behind large ones they
+    cost a small event's time, which a call of small ones bounds from above."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ev = gen.generate("stress", 200)
+    p = h.params(256, 256, 40, 1, 4096, theta_tiles=1)
+    s = torch.cuda.Stream()
+
+    def call(large, small, extra):
+        sizes = np.array([large] * (sms // 2) + [small] * (sms - sms // 2) + [extra] * 8)
+        off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        return time_run(h, np.resize(ev.xy, (int(off[-1]), 2)), off, p, s)
+
+    assert call(6000, 1500, 1500) - call(6000, 1500, 0) < 0.5 * call(1500, 1500, 0)
+
+
 @pytest.mark.parametrize("n", [152, 153, 305, 609])
 @pytest.mark.parametrize("nt,nr", [(64, 64), (101, 63), (100, 100), (130, 64), (128, 160), (63, 131)])
 @pytest.mark.parametrize("iterative", [False, True])
