@@ -88,13 +88,15 @@ __device__ __forceinline__ long long floor_div(long long a, long long b) {
 }
 
 // Hits whose quotients the estimate does not settle: bad ones (x = LLONG_MIN), and any near the origin.
-static __device__ __noinline__ longlong2 map_hit_far(int x, int y) {
+__device__ __forceinline__ longlong2 map_hit_far(int x, int y) {
+  if (x > kCoordMax || x < -kCoordMax || y > kCoordMax || y < -kCoordMax) return make_longlong2(LLONG_MIN, 0);
   const long long r2 = (long long)x * x + (long long)y * y;
-  if (x > kCoordMax || x < -kCoordMax || y > kCoordMax || y < -kCoordMax || r2 == 0) return make_longlong2(LLONG_MIN, 0);
+  if (r2 == 0) return make_longlong2(LLONG_MIN, 0);
   return make_longlong2(floor_div((long long)x * (1LL << 33), r2), floor_div((long long)y * (1LL << 33), r2));
 }
+static __device__ __noinline__ longlong2 map_hit_far_call(int x, int y) { return map_hit_far(x, y); }
 
-// floor(2^33 x / r2) from a float estimate e of it, |e| < 2^16 and off by less than one half: the rounded-down
+// floor(2^33 x / r2) from a float estimate e of it, |e| < 2^20 and off by less than one: the rounded-down
 // estimate is within one of the quotient, and the remainder (below 2 r2 in size, r2 <= 2^49, so 64-bit
 // arithmetic modulo 2^64 has it) settles it.
 __device__ __forceinline__ int floor_quotient(int x, float e, unsigned long long r2) {
@@ -107,20 +109,24 @@ __device__ __forceinline__ int floor_quotient(int x, float e, unsigned long long
 
 // Conformal map of one hit. Returns 0, or HOUGH_F_BAD_HIT for r = 0 or a coordinate beyond 2^24 um. The
 // estimate takes x, y as floats (exact for |x|, |y| <= 2^24), a rounded r^2 and the fast quotient (2 ulp): a
-// relative error below 2^-21, so below 1/32 for quotients below 2^16 (r above 131 mm).
+// relative error below 2^-21, so below one half for quotients below 2^20 (all of r above 8.2 mm; with the line at 2^16,
+// 131 mm, events nearer took the 64-bit divisions: 1,000 events of 2,000 hits at 8-100 mm, 740 us, so 698; 4.2 M hits mapped by
+// the stepwise call 67 us, so 32).
+// FarCall: the far path by a call, for kernels whose registers it would take.
+template <bool FarCall = true>
 __device__ __forceinline__ int map_hit(int x, int y, long long& u, long long& v) {
   const float fx = (float)x, fy = (float)y;
   const float s = __fdividef(8589934592.0f, fmaf(fx, fx, fy * fy));  // 2^33 / r^2
   const float eu = fx * s, ev = fy * s;
   const unsigned lim = 2u * kCoordMax;
-  if ((unsigned)(x + kCoordMax) <= lim && (unsigned)(y + kCoordMax) <= lim && fabsf(eu) < 65536.0f &&
-      fabsf(ev) < 65536.0f) {
+  if ((unsigned)(x + kCoordMax) <= lim && (unsigned)(y + kCoordMax) <= lim && fabsf(eu) < 1048576.0f &&
+      fabsf(ev) < 1048576.0f) {
     const unsigned long long r2 = (unsigned long long)((long long)x * x + (long long)y * y);
     u = floor_quotient(x, eu, r2);
     v = floor_quotient(y, ev, r2);
     return 0;
   }
-  const longlong2 uv = map_hit_far(x, y);
+  const longlong2 uv = FarCall ? map_hit_far_call(x, y) : map_hit_far(x, y);
   if (uv.x == LLONG_MIN) return HOUGH_F_BAD_HIT;
   u = uv.x;
   v = uv.y;

@@ -24,7 +24,7 @@ __global__ void map_kernel(const int2* __restrict__ xy, long long n, long long* 
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int2 h = xy[i];
     long long u = 0, v = 0;
-    if (map_hit(h.x, h.y, u, v)) {
+    if (map_hit<false>(h.x, h.y, u, v)) {
       u = v = LLONG_MIN;
       bad = 1;
     }

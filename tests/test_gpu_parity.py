@@ -562,6 +562,32 @@ def test_vote_edges(h, n_theta, n_rho, tiles):
         assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
 
 
+@pytest.mark.parametrize("r0", [8192, 131072, 1024, 200000])
+def test_map_where_the_estimate_ends(h, r0):
+    """Quotients around 2^20 (where the float estimate ends), 2^16, far above and in the ordinary range, against integers."""
+    rng = np.random.default_rng(r0)
+    r, a = rng.uniform(0.97 * r0, 1.03 * r0, 100_000), rng.uniform(0, 2 * np.pi, 100_000)
+    xy = np.stack([r * np.cos(a), r * np.sin(a)], 1).astype(np.int32)
+    xy[:8] = [(r0, 0), (-r0, 0), (0, r0), (0, -r0), (r0 - 1, 1), (r0 + 1, -1), (-r0 + 1, 0), (0, -r0 - 1)]
+    x, y = xy[:, 0].astype(np.int64), xy[:, 1].astype(np.int64)
+    uq, vq = h.map_hits(torch.from_numpy(xy).cuda(), torch.tensor([0, len(xy)], dtype=torch.int64, device="cuda"), h.new_status())
+    assert np.array_equal(to_np(uq), (x << 33) // (x * x + y * y)) and np.array_equal(to_np(vq), (y << 33) // (x * x + y * y))
+
+
+def test_near_hits_map_as_fast_as_far_ones(h):
+    """The quotients of hits at 9 to 100 mm are settled by the same few operations as those at 200 to 800 mm, so the same
+    number of them takes the same time (1.5 leaves room for the clock; the 64-bit divisions take twice as long)."""
+    rng = np.random.default_rng(5)
+    n, s, us = 1 << 22, torch.cuda.current_stream(), []
+    for lo, hi in ((9e3, 100e3), (200e3, 800e3)):
+        r, a = rng.uniform(lo, hi, n), rng.uniform(0, 2 * np.pi, n)
+        xy = torch.from_numpy(np.stack([r * np.cos(a), r * np.sin(a)], 1).astype(np.int32)).cuda()
+        off, st = torch.tensor([0, n], dtype=torch.int64, device="cuda"), h.new_status()
+        uq, vq = h.map_hits(xy, off, st)
+        us.append(best_us(lambda: h.map_hits(xy, off, st, uq, vq), s))
+    assert us[0] < 1.5 * us[1]
+
+
 # ---------------------------------------------------------------- exhaustive bin function
 
 @pytest.mark.parametrize("n_rho", [4, 63, 64, 256, 512, 1000, 1024])
