@@ -118,8 +118,8 @@ __device__ __forceinline__ int map_hit(int x, int y, long long& u, long long& v)
   const float fx = (float)x, fy = (float)y;
   const float s = __fdividef(8589934592.0f, fmaf(fx, fx, fy * fy));  // 2^33 / r^2
   const float eu = fx * s, ev = fy * s;
-  const unsigned lim = 2u * kCoordMax;
-  if ((unsigned)(x + kCoordMax) <= lim && (unsigned)(y + kCoordMax) <= lim && fabsf(eu) < 1048576.0f &&
+  const unsigned lim = 2u * kCoordMax;  // (unsigned sums: any int32 may come in)
+  if ((unsigned)x + kCoordMax <= lim && (unsigned)y + kCoordMax <= lim && fabsf(eu) < 1048576.0f &&
       fabsf(ev) < 1048576.0f) {
     const unsigned long long r2 = (unsigned long long)((long long)x * x + (long long)y * y);
     u = floor_quotient(x, eu, r2);

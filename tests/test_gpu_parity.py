@@ -227,9 +227,24 @@ def test_bad_hits_and_small_radii(h):
     assert np.all(u[idx[:15]] == np.iinfo(np.int64).min)
 
 
+def test_coordinates_of_any_int32(h):
+    """Coordinates up to the ends of int32 are bad hits like any other beyond 2^24, and the last good ones are good."""
+    ev = gen.generate("plain_small", 3)
+    ends = [-2 ** 31, -2 ** 31 + 1, -2 ** 31 + 2 ** 24, -2 ** 24 - 1, 2 ** 24 + 1, 2 ** 31 - 2 ** 24, 2 ** 31 - 1]
+    bad = [(c, 5) for c in ends] + [(-5, c) for c in ends] + [(c, d) for c in ends for d in ends]
+    xy = np.concatenate([ev.xy, np.array(bad + [(2 ** 24, -2 ** 24), (-2 ** 24, 2 ** 24)], np.int64).astype(np.int32)])
+    off = np.append(ev.off, len(xy))
+    ref = oracle.run(xy, off, oracle.params(64, 64, 12, 1, 256), threads=THREADS)
+    t_xy, t_off = torch.from_numpy(xy).cuda(), torch.from_numpy(off).cuda()
+    out = h.run(t_xy, t_off, h.params(64, 64, 12, 1, 256), checksum=True)
+    assert h.status(out.status) == ref.status == h.F_BAD_HIT
+    assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
+    uq, _ = h.map_hits(t_xy, t_off, h.new_status())
+    assert np.array_equal(to_np(uq)[len(ev.xy):] == np.iinfo(np.int64).min, [True] * len(bad) + [False] * 2)
+
+
 def test_map_edges(h):
-    """The map's quotients about the radius where its float estimate gives way to plain division (2^16: 131 mm),
-    on the axes, at the largest coordinates and at the smallest radii, against Python integers."""
+    """The map's quotients at radii up to 400 mm (the float estimate gives way to plain division at 2^20, 8 mm), on the axes, at the largest coordinates and at the smallest radii, against Python integers."""
     rng = np.random.default_rng(12)
     r = np.concatenate([np.full(3000, 131072), rng.uniform(1, 400000, 3000), rng.uniform(4e5, 2 ** 24, 2000)])
     a = rng.uniform(0, 2 * np.pi, len(r))
