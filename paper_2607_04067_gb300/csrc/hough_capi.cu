@@ -402,7 +402,16 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
 // An accumulator of at most 8,192 cells with up to 1,024 hits an event takes half the threads in any case (64 x 64, 616
 // hits, 100 events: 18.2 -> 16.5; 64 x 74, 4,720 hits, two events: 45.2 -> 51.6, hence the line): its phases are shorter
 // than what 32 warps add to each barrier.
-int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan& pl) {
+// A call's sizes do not tell how even its events are, and one event with many times the others' hits takes longer in a CTA of
+// fewer threads (8,000 hits: 1.2 times with 512, 1.9 times with 256; 64 x 64, 608 events of 600 hits, ten of 8,000: 113 us,
+// 75 with a block of 1,024). Among events of 500 to 4,700 hits that loses only where one CTA an SM has a few events left after the
+// first turn, the smallest ones: so calls of at most one and a half turns, with more than 1,500 hits an event (with fewer its
+// fixed part counts most) and more than one word group (64 columns: 35.8 us in two CTAs an SM, 37.9 in one), launch both
+// shapes, and the events choose (is_uneven). The launch that finds nothing to do costs 2.2 us; behind the validation
+// kernel of larger calls it would be 4.
+int make_plan(const hough_params* p, long long n_hits, long long n_events, CallPlan& cp) {
+  cp.two = false;
+  Plan& pl = cp.pl;
   const int rc = make_plan(p, pl);
   if (rc || p->block || n_events < 1) return rc;
   if (!p->theta_tiles && pl.mp && pl.peak_mode == HOUGH_PEAK_LOCAL_MAX && p->n_theta * p->n_rho > 20000) {
@@ -445,7 +454,10 @@ int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan&
     }
     if (fit >= 4) break;
   }
-  if (best_cap && make_plan(&q, x, best_cap) == HOUGH_OK) pl = x;
+  if (!best_cap || make_plan(&q, x, best_cap) != HOUGH_OK) return rc;
+  cp.two = n_events > kSms && n_events * 2 <= kSms * 3 && n_hits > 1500 * n_events && pl.groups > 2;
+  cp.one = pl;
+  pl = x;
   return rc;
 }
 
@@ -476,21 +488,12 @@ using namespace hgpu;
 
 namespace {
 
-cudaError_t timed_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st) {
-  cudaError_t e;
-  // External records become real event-record nodes when the stream is being captured.
-  if (g_ev_begin && g_ev_end) {
-    e = cudaEventRecordWithFlags(g_ev_begin, st, cudaEventRecordExternal);
-    if (e != cudaSuccess) return e;
-  }
-  // the validation kernel stands right before only without the event between
-  e = launch_fused(pl, io, trig, grid, st, !io.solo && !(g_ev_begin && g_ev_end));
-  if (e == cudaSuccess && g_ev_begin && g_ev_end) e = cudaEventRecordWithFlags(g_ev_end, st, cudaEventRecordExternal);
-  return e;
-}
+// External records become real event-record nodes when the stream is being captured.
+cudaError_t mark_begin(cudaStream_t st) { return cudaEventRecordWithFlags(g_ev_begin, st, cudaEventRecordExternal); }
+cudaError_t mark_end(cudaStream_t st) { return cudaEventRecordWithFlags(g_ev_end, st, cudaEventRecordExternal); }
 
 struct Common {
-  Plan pl;
+  CallPlan cp;
   WsLayout wl;
   FusedIO io;
 };
@@ -503,10 +506,11 @@ int prepare_fused(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int
   if (n_events > 0 && (!d_npeaks || !d_peaks || !d_nkept)) return HOUGH_EINVAL;
   if (n_hits > 0 && (!d_xy || !d_mask)) return HOUGH_EINVAL;
   if (((uintptr_t)d_xy & 7) || ((uintptr_t)d_peaks & 7) || ((uintptr_t)d_ws & 255)) return HOUGH_EINVAL;
-  int rc = make_plan(p, n_hits, n_events, cm.pl);
+  int rc = make_plan(p, n_hits, n_events, cm.cp);
   if (rc) return rc;
-  if ((long long)n_events * cm.pl.tiles > 0x7fffffffLL) return HOUGH_EINVAL;
-  cm.wl = ws_layout(cm.pl, n_events);
+  const Plan& pl = cm.cp.pl;
+  if ((long long)n_events * pl.tiles > 0x7fffffffLL) return HOUGH_EINVAL;
+  cm.wl = ws_layout(pl, n_events);
   if (ws_bytes < cm.wl.total) return HOUGH_EWORKSPACE;
   char* ws = (char*)d_ws;
   FusedIO& io = cm.io;
@@ -521,8 +525,8 @@ int prepare_fused(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int
   io.nkept = d_nkept;
   io.checksum = (unsigned long long*)d_checksum;
   io.status = d_status;
-  bind_workspace(cm.pl, cm.wl, ws, io);
-  io.n_items = n_events * (long long)cm.pl.tiles;
+  bind_workspace(pl, cm.wl, ws, io);
+  io.n_items = n_events * (long long)pl.tiles;
   return HOUGH_OK;
 }
 
@@ -616,6 +620,27 @@ int hough_resolve_params(hough_params* p) {
   return HOUGH_OK;
 }
 
+// (grid 0: not to be had)
+static CallGrid batched_grid(const Common& cm) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return CallGrid{};
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return CallGrid{};
+  return call_grid(cm.cp, cm.io.n_items, sms);
+}
+
+static int enqueue(const Common& cm, const hough_params* p, const CallGrid& g, int* order, cudaStream_t st) {
+  TrigTable trig;
+  host_trig(p->n_theta, &trig);
+  const bool timed = g_ev_begin && g_ev_end;
+  const cudaError_t e = launch_call(cm.cp, cm.io, trig, g, order, st, timed ? mark_begin : nullptr, timed ? mark_end : nullptr);
+  return e == cudaSuccess ? HOUGH_OK : cuda_fail(e);
+}
+
+static int enqueue_batched(Common cm, const hough_params* p, void* d_ws, const CallGrid& g, cudaStream_t st) {
+  cm.io.persistent = 1;
+  return enqueue(cm, p, g, (int*)((char*)d_ws + cm.wl.order), st);
+}
+
 int hough_run(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int64_t n_events, const hough_params* p,
               int32_t* d_npeaks, hough_peak* d_peaks, uint8_t* d_mask, int32_t* d_nkept, uint64_t* d_checksum,
               void* d_ws, size_t ws_bytes, int32_t* d_status, void* stream) {
@@ -624,44 +649,11 @@ int hough_run(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int64_t
                          ws_bytes, d_status, cm);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = cudaSuccess;
-  cm.io.solo = fused_solo(cm.pl, cm.io.n_items, (int)cm.io.n_items);
-  if (!cm.io.solo) e = launch_prep(cm.io.off, n_events, n_hits, d_status, cm.io.queue, cm.io.tickets, nullptr, st);
-  if (e != cudaSuccess) return cuda_fail(e);
-  if (cm.io.n_items == 0) return HOUGH_OK;
-  TrigTable trig;
-  host_trig(p->n_theta, &trig);
-  cm.io.persistent = 0;
-  e = timed_fused(cm.pl, cm.io, trig, (int)cm.io.n_items, st);
-  return e == cudaSuccess ? HOUGH_OK : cuda_fail(e);
-}
-
-static int batched_grid(const Common& cm) {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return -1;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-  const int per_sm = fused_max_ctas_per_sm(cm.pl);
-  if (per_sm < 1) return -1;
-  long long grid = (long long)sms * per_sm;
-  if (grid > cm.io.n_items || cm.pl.cluster) grid = cm.io.n_items;  // clusters are whole and take no queue
-  return (int)(grid > 0 ? grid : 1);
-}
-
-static int enqueue_batched(const Common& cm0, const hough_params* p, int64_t n_hits, int64_t n_events, void* d_ws,
-                           int32_t* d_status, int grid, cudaStream_t st) {
-  Common cm = cm0;
-  int* order = (int*)((char*)d_ws + cm.wl.order);
-  cudaError_t e = cudaSuccess;
-  cm.io.solo = fused_solo(cm.pl, cm.io.n_items, grid);
-  if (!cm.io.solo) e = launch_prep(cm.io.off, n_events, n_hits, d_status, cm.io.queue, cm.io.tickets, order, st);
-  if (e != cudaSuccess) return cuda_fail(e);
-  if (cm.io.n_items == 0) return HOUGH_OK;
-  TrigTable trig;
-  host_trig(p->n_theta, &trig);
-  cm.io.order = cm.io.solo ? nullptr : order;
-  cm.io.persistent = 1;
-  e = timed_fused(cm.pl, cm.io, trig, grid, st);
-  return e == cudaSuccess ? HOUGH_OK : cuda_fail(e);
+  if (cm.cp.two) {
+    const CallGrid g = batched_grid(cm);
+    return g.grid < 1 || g.one < 1 ? HOUGH_ESMEM : enqueue_batched(cm, p, d_ws, g, st);
+  }
+  return enqueue(cm, p, CallGrid{(int)cm.io.n_items, 0}, nullptr, st);
 }
 
 // ---- autotuner ----
@@ -788,11 +780,11 @@ int hough_autotune(hough_params* p, const int32_t* d_xy, int64_t n_hits, const i
                           (uint8_t*)(s + L.mask), (int32_t*)(s + L.nkept), nullptr, s + L.ws,
                           scratch_bytes - L.ws, d_status, cm) != HOUGH_OK)
           continue;
-        const int grid = batched_grid(cm);
-        if (grid < 1) continue;
-        if (enqueue_batched(cm, &q, n_hits, n_events, s + L.ws, d_status, grid, st) != HOUGH_OK) continue;
+        const CallGrid grid = batched_grid(cm);
+        if (grid.grid < 1) continue;
+        if (enqueue_batched(cm, &q, s + L.ws, grid, st) != HOUGH_OK) continue;
         cudaEventRecord(e0, st);
-        for (int r = 0; r < 2; ++r) enqueue_batched(cm, &q, n_hits, n_events, s + L.ws, d_status, grid, st);
+        for (int r = 0; r < 2; ++r) enqueue_batched(cm, &q, s + L.ws, grid, st);
         cudaEventRecord(e1, st);
         if (cudaEventSynchronize(e1) != cudaSuccess) continue;
         float ms = 0.f;
@@ -829,9 +821,9 @@ int hough_run_batched(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off,
                          ws_bytes, d_status, cm);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  const int grid = batched_grid(cm);
-  if (grid < 1) return HOUGH_ESMEM;
-  if (st == nullptr) return enqueue_batched(cm, p, n_hits, n_events, d_ws, d_status, grid, st);  // legacy stream: no capture
+  const CallGrid grid = batched_grid(cm);
+  if (grid.grid < 1 || (cm.cp.two && grid.one < 1)) return HOUGH_ESMEM;
+  if (st == nullptr) return enqueue_batched(cm, p, d_ws, grid, st);  // legacy stream: no capture
   GraphKey key;
   std::memset(&key, 0, sizeof(key));
   key.xy = d_xy;
@@ -862,7 +854,7 @@ int hough_run_batched(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off,
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(e);
-  rc = enqueue_batched(cm, p, n_hits, n_events, d_ws, d_status, grid, st);
+  rc = enqueue_batched(cm, p, d_ws, grid, st);
   e = cudaStreamEndCapture(st, &graph);
   if (rc) {
     if (graph) cudaGraphDestroy(graph);

@@ -15,6 +15,7 @@
 //     columns by one extra warp), so the 3x3 peak test is exact on tile edges; the last tile CTA of an
 //     event (ticket counter; a run of all tiles in one CTA needs none) merges the tiles' peak lists in tile order
 //     and selects. Events of small calls take the tiles of a cluster, which merge without a workspace.
+#include <algorithm>
 #include <climits>
 #include <map>
 #include <mutex>
@@ -2525,6 +2526,54 @@ __device__ __forceinline__ int bad_offsets(const long long* off, long long ne, l
   return bad;
 }
 
+// Whether a call's events are too uneven for two CTAs an SM instead of one; s: two shared ints, every thread calls it. An event of
+// 4,700 hits takes 1.13 times as long with 512 threads as with 1,024, which is worth it only where one CTA an SM would end
+// later anyway: with its share of all hits, or after two of the smallest events (an event's fixed part counts as 1,800
+// hits). 128 x 128, 160 events: of about 1,290 hits each 48.0 us in one CTA an SM, 33.8 in two; of 500 to 4,700 hits 42.4
+// and 46.3 (iterative finder 65 and 78).
+__device__ __forceinline__ bool is_uneven(const FusedIO& io, int ctas, int* s) {
+  constexpr int kFixed = 1800;
+  if (threadIdx.x == 0) {
+    s[0] = 0;
+    s[1] = INT_MAX;
+  }
+  __syncthreads();
+  int most = 0, fewest = HOUGH_MAX_EVENT_HITS;
+  for (long long e = threadIdx.x; e < io.n_events; e += blockDim.x) {
+    const int n = (int)min(io.off[e + 1] - io.off[e], (long long)HOUGH_MAX_EVENT_HITS);
+    most = max(most, n);
+    fewest = min(fewest, n);
+  }
+  most = __reduce_max_sync(kFull, most);
+  fewest = __reduce_min_sync(kFull, fewest);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&s[0], most);
+    atomicMin(&s[1], fewest);
+  }
+  __syncthreads();
+  const long long top = s[0] + kFixed, share = (io.n_hits + io.n_events * kFixed) / ctas;
+  return 23 * top > 20 * max(max(top, share), 2LL * (s[1] + kFixed));
+}
+
+// What the validation kernel does for a launch with a queue, by the CTAs of the launch before it: CTA b puts event b at its place
+// among the events, largest first, and the first one resets the queue. s: a shared int.
+__device__ __forceinline__ void order_event(const FusedIO& io, int* s) {
+  const long long e = blockIdx.x, c = io.off[e + 1] - io.off[e];
+  if (threadIdx.x == 0) *s = 0;
+  __syncthreads();
+  int before = 0;
+  for (long long i = threadIdx.x; i < io.n_events; i += blockDim.x) {
+    const long long x = io.off[i + 1] - io.off[i];
+    before += x > c || (x == c && i < e);
+  }
+  before = __reduce_add_sync(kFull, before);
+  if ((threadIdx.x & 31) == 0) atomicAdd(s, before);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  io.next_order[*s] = (int)e;
+  if (e == 0) io.queue[0] = 0ull;
+}
+
 // One instance a layout (MP: mirror pairs), peak finder and (CL) use of clusters, so that none carries the others' registers.
 template <bool MP, bool ITER, bool CL>
 __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
@@ -2536,16 +2585,22 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
     tc[pl.n_theta + j] = trig.s[j];
   }
   if (io.solo) {  // no validation kernel before: every CTA looks at all offsets (a few loads a thread)
+    const bool first = !CL && io.part == 1;
+    if (first) asm volatile("griddepcontrol.launch_dependents;");  // the second launch's CTAs may take SMs that are done
     const int bad = __syncthreads_or(bad_offsets(io.off, io.n_events, io.n_hits));
+    const bool uneven = first && !bad && is_uneven(io, io.part_ctas, sh.tmp);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       io.status[1] = bad;
+      if (first) io.status[2] = uneven;
       if (bad) atomicOr(io.status, HOUGH_F_BAD_OFFSETS);
     }
-    if (bad) return;
+    if (uneven) order_event(io, sh.tmp + 2);
+    if (bad || uneven) return;
   } else {
-    // launched before the validation kernel has ended: what it writes is read from here on
+    // launched before the validation kernel (or the first launch) has ended: what it writes is read from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (__ldcg(io.status + 1) != 0) return;  // offsets of this call failed validation
+    if (!CL && io.part == 2 && __ldcg(io.status + 2) == 0) return;
   }
   __syncthreads();  // the table is read before run_item's first barrier
   const bool do_cs = io.checksum != nullptr;
@@ -2848,6 +2903,39 @@ cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& tri
   if (err != cudaSuccess) return err;
   if (deferred) def<<<io.n_spill, pl.threads, pl.smem_bytes, st>>>(pl, io, trig);
   return cudaGetLastError();
+}
+
+CallGrid call_grid(const CallPlan& cp, long long n_items, int sms) {
+  auto grid = [&](const Plan& pl) {
+    const long long g = (long long)sms * fused_max_ctas_per_sm(pl);
+    if (g < 1) return 0;
+    return (int)std::max(1LL, g > n_items || pl.cluster ? n_items : g);  // clusters are whole and take no queue
+  };
+  return CallGrid{grid(cp.pl), cp.two ? grid(cp.one) : 0};
+}
+
+cudaError_t launch_call(const CallPlan& cp, FusedIO io, const TrigTable& trig, const CallGrid& g, int* order, cudaStream_t st,
+                        Mark before, Mark after) {
+  cudaError_t e = cudaSuccess;
+  io.solo = fused_solo(cp.pl, io.n_items, g.grid);
+  if (!io.solo) e = launch_prep(io.off, io.n_events, io.n_hits, io.status, io.queue, io.tickets, order, st);
+  if (e != cudaSuccess || io.n_items == 0) return e;
+  if (before) e = before(st);
+  const bool two = cp.two && io.solo && g.one > 0;
+  io.order = io.solo ? nullptr : order;
+  io.part = two;
+  io.part_ctas = g.one;
+  io.next_order = order;
+  // the validation kernel stands right before only without a mark between
+  if (e == cudaSuccess) e = launch_fused(cp.pl, io, trig, g.grid, st, !io.solo && !before);
+  if (e == cudaSuccess && two) {
+    io.part = 2;
+    io.solo = 0;
+    io.order = order;
+    e = launch_fused(cp.one, io, trig, g.one, st, true);
+  }
+  if (e == cudaSuccess && after) e = after(st);
+  return e;
 }
 
 }  // namespace hgpu

@@ -59,6 +59,13 @@ struct Plan {
   BinMagic magic;
 };
 
+// Launch shape of a call. With `two`, pl has two CTAs an SM, and `one`, with one, is launched behind it: the events' sizes say on
+// the device which of the two works (is_uneven).
+struct CallPlan {
+  Plan pl, one;
+  bool two;
+};
+
 struct FusedIO {
   const int2* xy;
   long long n_hits;
@@ -86,6 +93,9 @@ struct FusedIO {
   long long n_items;
   int persistent;
   int solo;  // no validation kernel before the fused one, which checks the offsets itself
+  int part;  // of a call's two launches: 1 the first, solo, for even events, 2 that for uneven ones; 0: there is one
+  int part_ctas;    // part 1: CTAs of part 2
+  int* next_order;  // part 1: room for the order of the events in part 2
 };
 
 // Workspace carve-up (byte offsets inside the caller's buffer).
@@ -105,14 +115,26 @@ BinMagic host_magic(int n_rho);
 
 cudaError_t launch_prep(const long long* off, long long n_events, long long n_hits, int* status,
                         unsigned long long* queue, int* tickets, int* order, cudaStream_t st);
-// `overlap`: the validation kernel is what `st` holds last, and the fused kernel's start (its launch, shared memory
-// and trig table) overlaps with it; the kernel waits for its end before it reads anything written on the device.
+// `overlap`: the validation kernel (or the first of two fused ones) is what `st` holds last, and the fused kernel's start
+// (its launch, shared memory and trig table) overlaps with it; the kernel waits for its end before it reads anything
+// written on the device.
 cudaError_t launch_fused(const Plan& pl, const FusedIO& io, const TrigTable& trig, int grid, cudaStream_t st,
                          bool overlap);
 int fused_max_ctas_per_sm(const Plan& pl);
 // Whether a call takes the fused kernel alone: one tile an event or tiles in clusters (no tickets to reset), an item a
 // CTA (no queue, so no order), and so few events that each CTA's look at all offsets is one step a thread.
 bool fused_solo(const Plan& pl, long long n_items, int grid);
+// CTAs of a call's persistent launch and, with cp.two, of the second one (0: no CTA fits).
+struct CallGrid {
+  int grid, one;
+};
+CallGrid call_grid(const CallPlan& cp, long long n_items, int sms);
+// All kernels of a call, whose launch of cp.pl has g.grid CTAs (io without order and solo). order: the workspace's, null where
+// CTAs take the items by their places. before, after (nullable): called around the fused ones.
+using Mark = cudaError_t (*)(cudaStream_t);
+cudaError_t launch_call(const CallPlan& cp, FusedIO io, const TrigTable& trig, const CallGrid& g, int* order, cudaStream_t st,
+                        Mark before = nullptr, Mark after = nullptr);
+int make_plan(const hough_params* p, long long n_hits, long long n_events, CallPlan& cp);
 
 cudaError_t launch_map(const int2* xy, long long n_hits, long long* uq, long long* vq, int* status, cudaStream_t st);
 cudaError_t launch_vote(const long long* uq, const long long* vq, const long long* off, long long n_events,

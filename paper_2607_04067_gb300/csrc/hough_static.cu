@@ -27,7 +27,6 @@
 
 namespace hgpu {
 
-int make_plan(const hough_params* p, long long n_hits, long long n_events, Plan& pl);
 void note_cuda_error(cudaError_t e);
 
 namespace {
@@ -73,9 +72,10 @@ extern "C" int hough_run_batched_static(const int32_t* d_xy, int64_t n_hits, con
   if (n_events > 0 && (!d_npeaks || !d_peaks || !d_nkept)) return HOUGH_EINVAL;
   if (n_hits > 0 && (!d_xy || !d_mask)) return HOUGH_EINVAL;
   if (((uintptr_t)d_xy & 7) || ((uintptr_t)d_peaks & 7)) return HOUGH_EINVAL;
-  Plan pl;
-  int rc = make_plan(p, n_hits, n_events, pl);
+  CallPlan cp;
+  int rc = make_plan(p, n_hits, n_events, cp);
   if (rc) return rc;
+  const Plan& pl = cp.pl;
   if ((long long)n_events * pl.tiles > 0x7fffffffLL) return HOUGH_EINVAL;
   const WsLayout wl = ws_layout(pl, n_events);
   if (wl.total > (size_t)HOUGH_STATIC_SCRATCH_BYTES) return HOUGH_EWORKSPACE;  // batch too large for the array
@@ -97,29 +97,15 @@ extern "C" int hough_run_batched_static(const int32_t* d_xy, int64_t n_hits, con
   io.status = d_status;
   bind_workspace(pl, wl, ws, io);
   io.n_items = n_events * (long long)pl.tiles;
-  int* order = (int*)(ws + wl.order);
-  cudaStream_t st = (cudaStream_t)stream;
-  if (io.n_items == 0) {
-    e = launch_prep(io.off, n_events, n_hits, d_status, io.queue, io.tickets, order, st);
-    return e == cudaSuccess ? HOUGH_OK : fail(e);
-  }
+  io.persistent = 1;
   int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return fail(e);
-  const int per_sm = fused_max_ctas_per_sm(pl);
-  if (per_sm < 1) return HOUGH_ESMEM;
-  long long grid = (long long)sms * per_sm;
-  if (grid > io.n_items || pl.cluster) grid = io.n_items;  // clusters are whole and take no queue
+  const CallGrid grid = call_grid(cp, io.n_items, sms);
+  if (io.n_items > 0 && (grid.grid < 1 || (cp.two && grid.one < 1))) return HOUGH_ESMEM;
   TrigTable trig;
   host_trig(p->n_theta, &trig);
-  io.solo = fused_solo(pl, io.n_items, (int)grid);
-  if (!io.solo) {
-    e = launch_prep(io.off, n_events, n_hits, d_status, io.queue, io.tickets, order, st);
-    if (e != cudaSuccess) return fail(e);
-    io.order = order;
-  }
-  io.persistent = 1;
-  e = launch_fused(pl, io, trig, (int)grid, st, !io.solo);
+  e = launch_call(cp, io, trig, grid, (int*)(ws + wl.order), (cudaStream_t)stream);
   return e == cudaSuccess ? HOUGH_OK : fail(e);
 }

@@ -402,6 +402,55 @@ def test_several_ctas_an_sm(h, nt, nr, n, iterative):
         assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
 
 
+def uneven_batch(n, small, large, n_large, seed=6):
+    """n events, n_large of them of `large` hits, the others of about `small`."""
+    rng = np.random.default_rng(seed)
+    sizes = rng.integers(small - small // 8, small + small // 8 + 1, n)
+    sizes[rng.choice(n, n_large, replace=False)] = large
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    return np.resize(gen.generate("stress", 300).xy, (int(off[-1]), 2)), off
+
+
+@pytest.mark.parametrize("n,small,large,n_large", [(153, 1600, 5000, 1), (160, 1600, 8000, 5), (200, 1600, 1700, 5), (228, 1600, 5000, 30),
+                                                   (228, 0, 20000, 100), (229, 1600, 5000, 30), (608, 40, 3000, 10), (1000, 40, 3000, 10)])
+@pytest.mark.parametrize("nt,nr", [(64, 64), (101, 63), (128, 128)])
+@pytest.mark.parametrize("iterative", [False, True])
+def test_uneven_events_on_small_accumulators(h, nt, nr, n, small, large, n_large, iterative):
+    """Few more events than SMs with many hits each on small accumulators, where two launches look whether the events are even:
+    even, uneven, mostly empty ones, one event more than that, bad offsets; and uneven events of larger calls."""
+    kw = dict(peak_mode=1, rel_num=1, rel_den=2, nms_radius=2) if iterative else {}
+    xy, off = uneven_batch(n, small, large, n_large)
+    off[1] = 0  # the first event is empty, the second has its hits too
+    ref = oracle.run(xy, off, oracle.params(nt, nr, 9, 1, 512, **kw), threads=THREADS)
+    t_xy, t_off = torch.from_numpy(np.ascontiguousarray(xy)).cuda(), torch.from_numpy(off).cuda()
+    p = h.params(nt, nr, 9, 1, 512, **kw)
+    for batched in (False, True):
+        out = h.run(t_xy, t_off, p, checksum=True, batched=batched)
+        assert h.status(out.status) == ref.status
+        assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
+        bad = t_off.clone()
+        bad[n // 2] = -1
+        out.npeaks.fill_(-7)
+        out.status.zero_()
+        h.run(t_xy, bad, p, out=out, batched=batched)
+        assert h.status(out.status) == h.F_BAD_OFFSETS
+        assert torch.all(out.npeaks == -7)
+    out = h.alloc_outputs(len(xy), n, p, checksum=True)
+    h.run_static(t_xy, t_off, p, out)
+    assert h.status(out.status) == ref.status
+    assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
+
+
+@pytest.mark.parametrize("nt", [100, 128])
+def test_uneven_events_take_one_cta_an_sm(h, nt):
+    """160 events of 500 to 4,700 hits: the few beyond an event an SM are small and end behind small ones, while two CTAs
+    an SM, of half the threads, would take a fifth longer for the large ones (iterative finder)."""
+    ev = gen.generate("batched", 160)
+    kw, s = dict(theta_tiles=1, peak_mode=1, rel_num=1, rel_den=2, nms_radius=3), torch.cuda.Stream()
+    one = time_run(h, ev.xy, ev.off, h.params(nt, nt, 8, 1, 4096, block=1024, **kw), s)
+    assert time_run(h, ev.xy, ev.off, h.params(nt, nt, 8, 1, 4096, **kw), s) < 1.1 * one
+
+
 @pytest.mark.parametrize("n", [1, 12, 13, 32, 33, 72, 73])
 @pytest.mark.parametrize("nt,nr", [(66, 310), (130, 160), (131, 161), (256, 256), (258, 100), (512, 300), (640, 33)])
 def test_few_events_in_clusters(h, nt, nr, n):
