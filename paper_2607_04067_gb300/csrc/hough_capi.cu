@@ -615,7 +615,7 @@ int hough_resolve_params(hough_params* p) {
   int rc = make_plan(p, pl);
   if (rc) return rc;
   p->theta_tiles = pl.tiles;
-  p->events_per_cta = p->events_per_cta > 0 ? p->events_per_cta : 1;
+  p->events_per_cta = pl.grab;
   p->block = pl.threads;
   return HOUGH_OK;
 }

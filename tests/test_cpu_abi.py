@@ -57,6 +57,15 @@ def test_resolve_and_reject_params():
     assert h.resolve(h.params(512, 512, 20, peak_mode=1, rel_num=1, rel_den=2)).theta_tiles == 4
 
 
+def test_resolve_reports_the_run_length():
+    """The queue hands out an event's tiles in a run unless the caller says otherwise."""
+    for nt, nr, tiles in ((64, 64, 1), (512, 512, 4), (1000, 1000, 16), (1001, 900, 11)):
+        r = h.resolve(h.params(nt, nr, 16))
+        assert (r.theta_tiles, r.events_per_cta) == (tiles, tiles)
+        assert h.resolve(h.params(nt, nr, 16, events_per_cta=3)).events_per_cta == 3
+        assert h.resolve(r).events_per_cta == tiles
+
+
 def test_workspace_sizes(lib):
     small = h.workspace_size(h.params(256, 256, 16, max_peaks=4096), 1000)
     big = h.workspace_size(h.params(256, 256, 16, max_peaks=4096), 100000)
