@@ -376,9 +376,11 @@ int hough_run_batched_static(const int32_t* d_xy, int64_t n_hits, const int64_t*
  * (d_xy, d_off: device, the caller's representative events) for every feasible launch shape
  * -- theta tiles in {1, 2, 4, 8, 16}, threads per CTA in {256, 512, 1024} (or the widest the
  * tiling allows), queue items per pop (events_per_cta) in {1, 2, 4, tiles} -- and writes the fastest
- * into *p (theta_tiles, block, events_per_cta; the algorithm fields are untouched). d_scratch
+ * into *p (theta_tiles, block, events_per_cta; the algorithm fields are untouched). Where zero launch fields give
+ * such a batch a shape that no others do, that one is timed too, and the three fields are 0 if it is the fastest. d_scratch
  * holds outputs and workspace of every candidate: hough_autotune_scratch_size bytes, 256-byte
- * aligned. Results are cached per (parameters, device, SM count, hits per event in octaves);
+ * aligned. Results are cached per (parameters, device, SM count, hits per event in octaves, events in classes: up to
+ * 12, 32, 72, then by turns of the SMs up to 16);
  * a cached answer returns at once with *best_ms = -1. Synchronises `stream`. */
 size_t hough_autotune_scratch_size(const hough_params* p, int64_t n_hits, int64_t n_events);
 int hough_autotune(hough_params* p, const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int64_t n_events,

@@ -664,7 +664,7 @@ namespace {
 // only for the same kind of work (the peak finder included).
 struct TuneKey {
   int n_theta, n_rho, threshold, keep_hw, max_peaks, peak_mode, rel_num, rel_den, nms_radius, device, sms,
-      hits_bucket;
+      hits_bucket, events_bucket;
   bool operator<(const TuneKey& o) const { return std::memcmp(this, &o, sizeof(TuneKey)) < 0; }
 };
 
@@ -738,6 +738,9 @@ int hough_autotune(hough_params* p, const int32_t* d_xy, int64_t n_hits, const i
     int b = 0;
     while (b < 20 && (double)(1 << (b + 1)) <= hpe) ++b;
     key.hits_bucket = b;
+    // a call of few events takes clusters, one of a few turns several CTAs an SM
+    const long long turns = (n_events + kSms - 1) / kSms;
+    key.events_bucket = n_events <= 12 ? 0 : n_events <= 32 ? 1 : n_events <= 72 ? 2 : (int)std::min(turns, 16LL) + 2;
   }
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -757,6 +760,28 @@ int hough_autotune(hough_params* p, const int32_t* d_xy, int64_t n_hits, const i
   hough_params best = *p;
   float best_t = 1e30f;
   bool found = false;
+  auto time_shape = [&](const hough_params& q) {
+    Common cm;
+    if (prepare_fused(d_xy, n_hits, d_off, n_events, &q, (int32_t*)(s + L.npeaks), (hough_peak*)(s + L.peaks),
+                      (uint8_t*)(s + L.mask), (int32_t*)(s + L.nkept), nullptr, s + L.ws, scratch_bytes - L.ws, d_status,
+                      cm) != HOUGH_OK)
+      return;
+    const CallGrid grid = batched_grid(cm);
+    if (grid.grid < 1) return;
+    if (enqueue_batched(cm, &q, s + L.ws, grid, st) != HOUGH_OK) return;
+    cudaEventRecord(e0, st);
+    for (int r = 0; r < 2; ++r) enqueue_batched(cm, &q, s + L.ws, grid, st);
+    cudaEventRecord(e1, st);
+    if (cudaEventSynchronize(e1) != cudaSuccess) return;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    ms *= 0.5f;
+    if (ms < best_t) {
+      best_t = ms;
+      best = q;
+      found = true;
+    }
+  };
   for (int T = 1; T <= 16; T *= 2) {
     for (int threads : {256, 512, 1024}) {
       bool have_t = false;
@@ -775,28 +800,21 @@ int hough_autotune(hough_params* p, const int32_t* d_xy, int64_t n_hits, const i
           if (threads != 1024) continue;
           q.block = probe.threads;  // the widest block this tiling allows
         }
-        Common cm;
-        if (prepare_fused(d_xy, n_hits, d_off, n_events, &q, (int32_t*)(s + L.npeaks), (hough_peak*)(s + L.peaks),
-                          (uint8_t*)(s + L.mask), (int32_t*)(s + L.nkept), nullptr, s + L.ws,
-                          scratch_bytes - L.ws, d_status, cm) != HOUGH_OK)
-          continue;
-        const CallGrid grid = batched_grid(cm);
-        if (grid.grid < 1) continue;
-        if (enqueue_batched(cm, &q, s + L.ws, grid, st) != HOUGH_OK) continue;
-        cudaEventRecord(e0, st);
-        for (int r = 0; r < 2; ++r) enqueue_batched(cm, &q, s + L.ws, grid, st);
-        cudaEventRecord(e1, st);
-        if (cudaEventSynchronize(e1) != cudaSuccess) continue;
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        ms *= 0.5f;
-        if (ms < best_t) {
-          best_t = ms;
-          best = q;
-          found = true;
-        }
+        time_shape(q);
       }
     }
+  }
+  // the shape of zero fields, where no explicit ones give it: clusters, fewer staged hits, a choice by the events' sizes
+  hough_params q = *p;
+  q.theta_tiles = q.block = q.events_per_cta = 0;
+  CallPlan cp;
+  if (make_plan(&q, n_hits, n_events, cp) == HOUGH_OK) {
+    hough_params w = *p;
+    w.theta_tiles = cp.pl.tiles;
+    w.block = cp.pl.threads;
+    w.events_per_cta = 0;
+    Plan x;
+    if (cp.two || cp.pl.cluster || make_plan(&w, x) != HOUGH_OK || x.hit_cap != cp.pl.hit_cap) time_shape(q);
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

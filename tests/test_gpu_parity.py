@@ -693,6 +693,26 @@ def test_autotuned_shape_gives_identical_results(h):
     assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off, checksum=out.checksum)
 
 
+@pytest.mark.parametrize("n", [1, 16])
+def test_autotuned_few_events_are_no_slower_than_untuned(h, n):
+    """A call of few events takes the CTAs of clusters when its launch fields are zero, a quarter faster than any shape with
+    them: the autotuner finds it, also after a large batch of the same parameters has been tuned."""
+    ev = gen.generate("batched", 1000)
+    p = h.params(256, 256, 18, 1, 4096)
+    xy, off = dev(ev)
+    _, ms = h.autotune(xy, off, p)
+    few, few_off = xy[: int(ev.off[n])].contiguous(), off[: n + 1].contiguous()
+    tuned, ms_few = h.autotune(few, few_off, p)
+    assert ms_few > 0  # not the large batch's
+    ref = oracle.run(ev.xy[: ev.off[n]], ev.off[: n + 1], oracle.params(256, 256, 18, 1, 4096), threads=THREADS)
+    out = h.run(few, few_off, tuned, checksum=True, batched=True)
+    assert h.status(out.status) == ref.status
+    assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, ev.off[: n + 1], checksum=out.checksum)
+    s = torch.cuda.Stream()
+    us = [time_run(h, ev.xy[: ev.off[n]], ev.off[: n + 1], q, s) for q in (tuned, p)]
+    assert us[0] < 1.1 * us[1]
+
+
 def test_autotune_cache_keys_the_peak_finder(h):
     """The autotuner writes only the launch shape, and its cache tells the peak finders apart:
     tuning the 3x3 finder first must not hand the iterative finder's tuning the 3x3 parameters.
