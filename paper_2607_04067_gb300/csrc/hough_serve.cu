@@ -21,9 +21,9 @@
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <mutex>
-#include <system_error>
 #include <thread>
 #include <type_traits>
 #include <vector>
@@ -144,8 +144,9 @@ class Crew {
  public:
   explicit Crew(int helpers) {
     try {
+      threads_.reserve((size_t)std::max(0, helpers));  // so that a thread that has started has its place
       for (int i = 0; i < helpers; ++i) threads_.emplace_back([this] { help(); });
-    } catch (const std::system_error&) {  // fewer, or none
+    } catch (const std::exception&) {  // no thread or no memory: fewer, or none
     }
   }
   ~Crew() {
