@@ -154,6 +154,30 @@ def test_replayed_poisson_stream_matches_oracle(h):
     assert stats["passes"] > 0 and stats["stall_ns"] == 1_000_000
 
 
+@pytest.mark.parametrize("iterative", [False, True])
+def test_burst_copied_by_the_helpers_matches_oracle(h, iterative):
+    """Two bursts of 1,500 requests in micro-batches of 256 events, 4 MB of hits each, which the helper threads copy in and out
+    (they take part from 2 MB): every request's mask, peaks and counts, the second burst after the first has drained."""
+    cfg = gen.CONFIGS["served"]
+    pool = gen.generate(cfg, 700, with_truth=False)
+    maxp, n = cfg.max_peaks, 1500
+    ref = oracle_ref(cfg, pool, iterative)
+    ev_of = np.arange(n) % pool.n_events
+    moff = np.concatenate([[0], np.cumsum(np.diff(pool.off)[ev_of])])
+    with h.Server(cfg_params(h, cfg, iterative), slots=4, max_batch_events=256, flush_us=50) as srv:
+        for _ in range(2):
+            mask, peaks = np.full(int(moff[-1]), 7, np.uint8), np.zeros((n, maxp, 4), np.int16)
+            res = h.Server.result_array(n)
+            srv.replay(pool.xy, pool.off, np.zeros(n, np.int64), mask_out=mask, peaks_out=peaks, results_out=res)
+            srv.drain(60)
+            assert np.array_equal(res["id"], np.arange(n)) and np.all(res["status"] == 0)
+            for i in range(n):
+                assert_matches_oracle(ref, pool, int(ev_of[i]), int(res["npeaks"][i]), int(res["nkept"][i]),
+                                      mask[moff[i]:moff[i + 1]], peaks[i], maxp)
+        _, rec = srv.trace()
+    assert np.sum(8 * rec["n_hits"] >= 2 << 20) >= 4
+
+
 def test_replay_results_into_caller_array(h):
     """With a result array, the replay's requests deliver their records there (by request id),
     nothing reaches poll(), and the counts equal the oracle's for every request."""
