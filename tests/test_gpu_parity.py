@@ -477,8 +477,6 @@ def test_records_by_keys(h, nt, nr, tiles):
     ev = gen.generate("plain_paper", 5)
     xy, off = dev(ev)
     for iterative in (False, True):
-        if iterative and nt % 2 and tiles == 0:
-            continue
         kw = dict(peak_mode=1, rel_num=1, rel_den=3, nms_radius=2) if iterative else {}
         for thr, maxp in ((40, 512), (16, 512), (8, 7), (4, 8192)):
             ref = oracle.run(ev.xy, ev.off, oracle.params(nt, nr, thr, 1, maxp, **kw), threads=THREADS)
@@ -531,11 +529,6 @@ def test_odd_theta_edges(h, nt, nr, tiles):
                               (2, 4096, 0, dict(it, nms_radius=min(5, (nt - 1) // 2)))):
         ref = oracle.run(xy, off, oracle.params(nt, nr, thr, hw, maxp, **kw), threads=THREADS)
         for batched in (False, True):
-            try:
-                p = h.resolve(h.params(nt, nr, thr, hw, maxp, theta_tiles=tiles, **kw))
-            except h.HoughError:
-                assert kw  # the iterative finder refuses some tilings
-                continue
             out = h.run(t_xy, t_off, h.params(nt, nr, thr, hw, maxp, theta_tiles=tiles, **kw), checksum=True, batched=batched)
             assert h.status(out.status) == ref.status
             assert_event_outputs_equal(ref, out.npeaks, out.peaks, out.mask, out.nkept, off, checksum=out.checksum)
