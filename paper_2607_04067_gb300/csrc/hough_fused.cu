@@ -298,7 +298,7 @@ __device__ __forceinline__ void vote64(const Plan& pl, const VoteLane& L, const 
   }
 }
 
-// ---- mirror-pair word layout (untiled events, N_theta a multiple of 64) ----
+// ---- mirror-pair word layout (even column counts; odd ones where it fits the tiles and threads of their columns) ----
 // Word lane w in [0, (N_theta+1)/2) holds column w in its low half and column N_theta-1-w (its
 // mirror) in its high half, one word per physical row p = k + 1. With an odd N_theta the last word's column is
 // its own mirror (c = 0): the high half then repeats the low one. It serves as the neighbour of the column after it;
@@ -323,17 +323,8 @@ __device__ __forceinline__ int mp_get(const uint32_t* acc, int c, int k, int Wd,
 // 16-bit store of zero into the cell's half of its word, which leaves the other half of the word alone.
 template <bool MP>
 struct FusedCells {
-  static constexpr bool kPairs = MP;  // word w holds columns w and NT - 1 - w
   uint32_t* acc;
-  int Wd, NT, nrp, rp;  // words, columns, padded rows (other layouts), rows with guards (mirror-pair)
-  __device__ int words() const { return Wd; }
-  __device__ int mirror_col(int w) const { return NT - 1 - w; }
-  __device__ uint32_t word(int w, int k) const { return acc[mp_word(w, k + 1, rp)]; }
-  // words w4 .. w4 + 3 of row k (w4 a multiple of 4: all four in one 32-word group, 16-byte aligned;
-  // words past the tile's own are zero)
-  __device__ uint4 words4(int w4, int k) const {
-    return *reinterpret_cast<const uint4*>(acc + mp_word(w4, k + 1, rp));
-  }
+  int Wd, NT, nrp, rp;  // words, columns, padded rows (columns), rows with guards (mirror pairs)
   __device__ int get(int j, int k) const {
     if (MP) {
       const bool hi = j >= Wd;
@@ -1414,7 +1405,7 @@ __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_
 
 struct ItemShared {
   WorkItem it[2];
-  int nv, flags, wide, last, total, D, reuse, n_amb, n_low, n_found;
+  int nv, flags, wide, last, D, reuse, n_amb, n_low, n_found;
   int staged;  // the event whose hits are staged whole (-1: none)
   unsigned runs;  // of the queue
   int kept_tot;
@@ -2185,13 +2176,16 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
         for (int k = tid; k < NR; k += bd) reinterpret_cast<uint16_t*>(acc)[2 * mp_word(Wd - 1, k + 1, pl.rows_phys) + 1] = 0;
         __syncthreads();
       }
-      auto general = [&](auto cells) {
+      FusedCells<MP> cells{acc, Wd, NT, nrp, pl.rows_phys};
+      if constexpr (MP) {
+        total = extract_iterative_passes(cells, NT, NR, kIterSliceRows, pl.threshold, pl.rel_num, pl.rel_den, pl.nms_radius, maxp,
+                                         pbits, dst, sh.tmp);
+      } else {
         const int st_words = (((NT * NR + 15) >> 4) + 31) & ~31;  // 2 bits a cell, whole 32-word blocks
-        return extract_iterative(cells, NT, NR, kIterSliceRows, pl.threshold, pl.rel_num, pl.rel_den, pl.nms_radius,
-                                 maxp, pbits, MP ? 0 : pl.iter_cap, nullptr, st_words, dst, sh.tmp,
-                                 reinterpret_cast<uint16_t*>(pbits + pl.iter_cap + st_words), pl.iter_act);
-      };
-      total = MP ? general(FusedCells<true>{acc, Wd, NT, nrp, pl.rows_phys}) : general(FusedCells<false>{acc, Wd, NT, nrp, pl.rows_phys});
+        total = extract_iterative(cells, NT, NR, kIterSliceRows, pl.threshold, pl.rel_num, pl.rel_den, pl.nms_radius, maxp,
+                                  pbits, pl.iter_cap, nullptr, st_words, dst, sh.tmp,
+                                  reinterpret_cast<uint16_t*>(pbits + pl.iter_cap + st_words), pl.iter_act);
+      }
     }
     n_low = total;
   } else {
@@ -2639,7 +2633,6 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
 // Accumulator of one deferred event in HBM (int32 cells, raster order) for the iterative finder;
 // suppressed cells are kept in a shared bitmap.
 struct SpillCells {
-  static constexpr bool kPairs = false;
   const int* A;
   uint32_t* gone;
   int NR;
