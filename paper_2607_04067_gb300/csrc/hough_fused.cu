@@ -1379,15 +1379,16 @@ __device__ int select_staged(const Plan& pl, const int2* hb, const uint16_t* idx
   return kept;
 }
 
-// A work item: tile item % T of event `event`, whose hits are [off[0], off[1]). Two of them in shared
-// memory, the current one and the next: in a persistent launch the next is popped after the current one's
-// vote, and its event's index and offsets are read by asynchronous copies issued between the phases, so that
-// no barrier waits for their latency (3.5 k cycles an event in a chain after the last item). Not earlier: the CTAs
-// start with the largest events, and those that pop as they start pair them with the next largest; half-way through
-// an item, those with small events come first, as they will at its end. (256 x 256, 160 events of 2,022 hits: 83.1 us popped
-// before the vote, 63.5 after it; 200 events 84.8 and 70.6; 20,000 events 4,678 and 4,656.)
 constexpr int kFoundMax = 128;  // keys that are ranked one by one
 
+// A work item: tile item % T of event `event`, whose hits are [off[0], off[1]). Two of them in shared
+// memory, the current one and the next: in a persistent launch the next is popped while the current one runs, and its
+// event's index and offsets are read by asynchronous copies issued between the phases, so that no barrier waits
+// for their latency (3.5 k cycles an event in a chain after the last item). It is popped after the vote: the CTAs start with the
+// largest events, and those that pop as they start pair them with the next largest; half-way through an item, those
+// with small events come first, as they will at its end. (256 x 256, 160 events of 2,022 hits: 83.1 us popped before
+// the vote, 63.5 after it; 200 events 84.8 and 70.6; 20,000 events 4,678 and 4,626.) The iterative finder pops before
+// the vote (after it 1 % slower, 5,000 events) but for the last two turns (pops_late).
 struct WorkItem {
   long long off[2];
   int item;  // >= n_items: none
@@ -2049,11 +2050,11 @@ __device__ __forceinline__ void popped(const Plan& pl, const FusedIO& io, unsign
   left = run ? pl.grab - 1 : 0;
 }
 
-// Whether the item after `item` is popped at its end and not after its vote: the iterative finder on tiles, where an
-// event's last tile takes much longer than the others and an item popped before it would wait for it instead of going
-// to another CTA; and on whole events in the last two turns, since two thirds of an event come after its vote and not in
-// proportion to its hits (256 x 256, half the maximum, R = 3, 160 events of 1,290 hits: 93.4 us popped after the vote, 81.0
-// so; the chain costs 3.5 k of 119 k cycles an item, in those turns alone).
+// Whether the item after `item` is popped at its end: the iterative finder on tiles, where an event's last tile takes
+// much longer than the others and an item popped before it would wait for it instead of going to another CTA; and on whole
+// events in the last two turns, since two thirds of an event come after its vote and not in proportion to its hits
+// (256 x 256, half the maximum, R = 3, 160 events of 1,290 hits: 93.4 us popped after the vote, 81.0 so; the chain costs 3.5 k of
+// 119 k cycles an item, in those turns alone).
 template <bool ITER>
 __device__ __forceinline__ bool pops_late(const Plan& pl, const FusedIO& io, int item) {
   return ITER && (pl.tiles > 1 || item + 2LL * gridDim.x >= io.n_items);
@@ -2084,8 +2085,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
 
   // the next item, in steps whose latencies pass behind the phases between them (thread 0)
   WorkItem& next = sh.it[cur ^ 1];
-  const bool ahead = queue && !pops_late<ITER>(pl, io, sh.it[cur].item);
-  const bool fetch = ahead && tid == 0;
+  const bool fetch = queue && tid == 0 && !pops_late<ITER>(pl, io, sh.it[cur].item);
   unsigned long long pop = 0;
   bool other = false;  // the next item exists and belongs to another event
   auto fetch_pop = [&]() {
@@ -2117,11 +2117,13 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     if (fetch && other) copy_async_wait();
   };
 
+  if (ITER) fetch_pop();
   {
     const long long a = sh.it[cur].off[0], nll = sh.it[cur].off[1] - a;
     vote_tile<MP, ITER>(pl, io, smem, sh, (int)e, a, nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll, t);
   }
-  fetch_pop();
+  if (ITER) fetch_event();
+  else fetch_pop();
 
   // 3-4. peaks
   const int maxp = pl.max_peaks;
@@ -2147,7 +2149,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       __syncthreads();
     }
     HOUGH_PHASE(HOUGH_PHASE_SCAN);
-    fetch_event();
+    fetch_offsets();
     hough_peak* dst = io.peaks + e * (long long)maxp;
     total = -1;
     if (MP && pl.iter_cap > 0) {
@@ -2160,7 +2162,6 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
       scan_mp<true>(pl, smem, tq, 0, Wd, sh.edge, pbits, cand, reinterpret_cast<uint16_t*>(list), &sh.n_amb,
                     Found{nullptr, 0, &sh.n_found});
       __syncthreads();
-      fetch_offsets();
       const WholeWindow ww{acc, Wd, pl.rows_phys, NT, NR, pl.nms_radius, pl.nrb_p, cand, pbits};
       const int nk = resolve_kept(ww, list, pl.iter_cap, reinterpret_cast<uint16_t*>(list + 2 * pl.iter_cap), sh.tmp);
       if (nk <= ranked_room(2 * pl.iter_cap)) {
@@ -2171,7 +2172,6 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
     // No bitmaps, or more peaks than the list ranks. (One pass a peak lists a kept set's cells in rank order
     // too: the dropped candidates are zero, the cells that are none below the threshold.)
     if (total < 0) {
-      if (!MP || pl.iter_cap == 0) fetch_offsets();
       if (MP && (NT & 1)) {  // a middle column's repetition
         for (int k = tid; k < NR; k += bd) reinterpret_cast<uint16_t*>(acc)[2 * mp_word(Wd - 1, k + 1, pl.rows_phys) + 1] = 0;
         __syncthreads();
@@ -2476,7 +2476,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_MERGE);
-  if (ahead && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
+  if (queue && !pops_late<ITER>(pl, io, sh.it[cur].item) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
     const long long i = next.off[0] + 16LL * tid;
     if (i < next.off[1]) asm volatile("prefetch.global.L2 [%0];" ::"l"(io.xy + i));
   }
@@ -2525,7 +2525,7 @@ __device__ __forceinline__ int bad_offsets(const long long* off, long long ne, l
 // later anyway: with its share of all hits, or after two of the smallest events (an event's fixed part counts as 1,800
 // hits). 128 x 128, 160 events: of about 1,290 hits each 48.0 us in one CTA an SM, 33.8 in two; of 500 to 4,700 hits 42.4
 // and 46.3 (iterative finder 65 and 78).
-__device__ __forceinline__ bool is_uneven(const FusedIO& io, int ctas, int* s) {
+__device__ __noinline__ bool is_uneven(const FusedIO& io, int ctas, int* s) {
   constexpr int kFixed = 1800;
   if (threadIdx.x == 0) {
     s[0] = 0;
@@ -2551,7 +2551,7 @@ __device__ __forceinline__ bool is_uneven(const FusedIO& io, int ctas, int* s) {
 
 // What the validation kernel does for a launch with a queue, by the CTAs of the launch before it: CTA b puts event b at its place
 // among the events, largest first, and the first one resets the queue. s: a shared int.
-__device__ __forceinline__ void order_event(const FusedIO& io, int* s) {
+__device__ __noinline__ void order_event(const FusedIO& io, int* s) {
   const long long e = blockIdx.x, c = io.off[e + 1] - io.off[e];
   if (threadIdx.x == 0) *s = 0;
   __syncthreads();
