@@ -451,6 +451,14 @@ def test_uneven_events_take_one_cta_an_sm(h, nt):
     assert time_run(h, ev.xy, ev.off, h.params(nt, nt, 8, 1, 4096, **kw), s) < 1.1 * one
 
 
+def test_uneven_events_in_one_turn_are_staged_whole(h):
+    """400 events of 500 to 4,700 hits at 128 x 128: a third CTA an SM would have room only with 3,072 staged hits, so the events
+    that end the call would take two chunks and a fifth longer than with two CTAs of 512 threads."""
+    ev, s = gen.generate("batched", 400), torch.cuda.Stream()
+    two = time_run(h, ev.xy, ev.off, h.params(128, 128, 8, 1, 4096, theta_tiles=1, block=512), s)
+    assert time_run(h, ev.xy, ev.off, h.params(128, 128, 8, 1, 4096), s) < 1.1 * two
+
+
 @pytest.mark.parametrize("n", [1, 12, 13, 32, 33, 72, 73])
 @pytest.mark.parametrize("nt,nr", [(66, 310), (130, 160), (131, 161), (256, 256), (258, 100), (512, 300), (640, 33)])
 def test_few_events_in_clusters(h, nt, nr, n):
@@ -895,6 +903,9 @@ def test_iterative_stepwise_large_accumulator(h):
     (256, 200, 4, 1, 4, 8, 64),   # 128 segments to merge
     (250, 64, 3, 1, 3, 1, 8),     # tiles of uneven width
     (255, 64, 3, 1, 3, 4, 5),     # column tiles: no local maxima marked
+    (459, 206, 12, 1, 2, 3, 1),   # whole columns that leave no room for lists: one pass a peak
+    (467, 204, 12, 1, 3, 2, 1),   # whole columns with the shortest list: events past it
+    (467, 204, 40, 3, 4, 1, 1),   # and within it
 ])
 def test_iterative_edges(h, nt, nr, thr, num, den, R, tiles):
     """Whole and tiled finders where their lists, windows and merges have their edges; two events of one and
