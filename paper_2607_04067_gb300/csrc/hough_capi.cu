@@ -396,9 +396,9 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
 // most of its time on barriers and on chains that 32 warps wait for together; CTAs of other events run in those
 // gaps. c CTAs of 1024 / c threads take kTurn[c] times as long as one (in twentieths; measured from 64 x 64 to
 // 160 x 160), so the c with the shortest time for all the events' turns is taken. Where events have few hits, fewer
-// staged hits (half as many again as the mean; an event with more takes several chunks) make room for more CTAs; more than two
-// in a single turn only with twice the mean (128 x 128, events of 500 to 4,700 hits, 400 of them: three CTAs 72.4 us, two 60.8;
-// 64 x 64, 608 of them: four 61.0, three 63.9).
+// staged hits (half as many again as the mean; an event with more takes several chunks) make room for more CTAs; but not for
+// more than two in a single turn of events of more than 1,500 hits (128 x 128, events of 500 to 4,700 hits, 400 of them: three
+// CTAs 72.4 us, two 60.8; 64 x 64, 608 of them: four 61.0, three 63.9; 100 x 100, 500 of about 1,290: four 57.7, 66.5 with 4,096 staged hits).
 // One CTA -> this rule, us: 64 x 64, 616 hits, 5,000 events 424 -> 177 and 500 events 59 -> 30; 100 x 100, 1,290
 // hits, 5,000 events 640 -> 365; 128 x 128, 2,022 hits, 1,000 events 167 -> 131, iterative finder 286 -> 218.
 // An accumulator of at most 8,192 cells with up to 1,024 hits an event takes half the threads in any case (64 x 64, 616
@@ -448,7 +448,7 @@ int make_plan(const hough_params* p, long long n_hits, long long n_events, CallP
       const int block = 1024 / c / (x.groups * 32) * (x.groups * 32);
       if (!block) break;
       // in one turn the largest events end the call, and those above the staged hits take chunks
-      if (c > 2 && n_events <= kSms * c && n_hits * 2 > n_events * cap) continue;
+      if (c > 2 && cap < 4096 && n_events <= kSms * c && n_hits > 1500 * n_events) continue;
       const long long t = (n_events + kSms * c - 1) / (kSms * c) * kTurn[c] * (1024 / c) / block;
       if (t < best) {
         best = t;
