@@ -1103,27 +1103,33 @@ __device__ inline int resolve_walk(int NT, int NR, int R, int maxp, uint32_t* ke
   return n;
 }
 
-// The iterative finder: the candidate form where it applies (cap > 0): resolved in rounds when
-// st_words > 0, else (or when the rounds give up) by the walk; otherwise one pass per peak.
-// scratch (shared): max(iter_scratch_words(NT, NR, SH), cap + max(ceil(NT NR / 32), st_words))
-// words when sup is null: the candidate keys, then the walk's bitmap, or the rounds' states
-// (st_words >= ceil(NT NR / 16) rounded up to 32 words). With sup given (a shared bitmap of NT NR
-// bits, left set) the walk uses it, and scratch needs max(iter_scratch_words, cap + st_words).
+// The iterative finder in candidate form where it applies (else -1, nothing written): resolved in rounds when
+// st_words > 0, else (or when the rounds give up) by the walk.
+// scratch (shared): cap + max(ceil(NT NR / 32), st_words) words when sup is null: the candidate keys, then the walk's
+// bitmap, or the rounds' states (st_words >= ceil(NT NR / 16) rounded up to 32 words). With sup given (a shared bitmap
+// of NT NR bits, left set) the walk uses it, and scratch needs cap + st_words.
+template <class Cells>
+__device__ int extract_candidates(Cells& cells, int NT, int NR, int thr, int rel_num, int rel_den, int R, int maxp,
+                                  uint32_t* scratch, int cap, uint32_t* sup, int st_words, hough_peak* dst, int* s,
+                                  uint16_t* act = nullptr, int act_cap = 0) {
+  int tq = 0;
+  const int C = collect_candidates(cells, NT, NR, thr, rel_num, rel_den, scratch, cap, s, &tq);
+  if (C < 0) return -1;
+  if (st_words > 0) {
+    const int n = resolve_rounds(cells, NT, NR, R, tq, maxp, scratch, C, scratch + cap, st_words, act, act_cap, dst, s);
+    if (n >= 0) return n;
+  }
+  return resolve_walk(NT, NR, R, maxp, scratch, C, sup ? sup : scratch + cap, dst, s);
+}
+
+// The iterative finder: the candidate form where it applies (cap > 0), else one pass a peak (scratch: at least
+// iter_scratch_words(NT, NR, SH) words too).
 template <class Cells>
 __device__ int extract_iterative(Cells& cells, int NT, int NR, int SH, int thr, int rel_num, int rel_den, int R,
-                                 int maxp, uint32_t* scratch, int cap, uint32_t* sup, int st_words,
-                                 hough_peak* dst, int* s, uint16_t* act = nullptr, int act_cap = 0) {
+                                 int maxp, uint32_t* scratch, int cap, uint32_t* sup, hough_peak* dst, int* s) {
   if (cap > 0) {
-    int tq = 0;
-    const int C = collect_candidates(cells, NT, NR, thr, rel_num, rel_den, scratch, cap, s, &tq);
-    if (C >= 0) {
-      if (st_words > 0) {
-        const int n =
-            resolve_rounds(cells, NT, NR, R, tq, maxp, scratch, C, scratch + cap, st_words, act, act_cap, dst, s);
-        if (n >= 0) return n;
-      }
-      return resolve_walk(NT, NR, R, maxp, scratch, C, sup ? sup : scratch + cap, dst, s);
-    }
+    const int n = extract_candidates(cells, NT, NR, thr, rel_num, rel_den, R, maxp, scratch, cap, sup, 0, dst, s);
+    if (n >= 0) return n;
   }
   return extract_iterative_passes(cells, NT, NR, SH, thr, rel_num, rel_den, R, maxp, scratch, dst, s);
 }

@@ -328,7 +328,7 @@ __global__ void peaks_iterative_kernel(const int16_t* __restrict__ acc, int NT, 
   __syncthreads();
   GlobalCells cells{acc + e * (long long)NT * NR, gone, NR};
   const int n =
-      extract_iterative(cells, NT, NR, SH, thr, rel_num, rel_den, R, maxp, cm, cap, gone, 0, peaks + e * maxp, s_sel);
+      extract_iterative(cells, NT, NR, SH, thr, rel_num, rel_den, R, maxp, cm, cap, gone, peaks + e * maxp, s_sel);
   if (threadIdx.x == 0) {
     npeaks[e] = n;
     if (n > maxp) atomicOr(status, HOUGH_F_PEAK_OVERFLOW);
