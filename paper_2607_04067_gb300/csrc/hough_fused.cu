@@ -806,8 +806,8 @@ __device__ __forceinline__ void edge_words(const Plan& pl, int aw, int half, boo
     e.step = w < 0 ? -32 : 32;
     e.swap = 1;
     if (w > 0 && at < 0) {  // the middle word alone: the one before it is the halo's
-      e.at = halo0;
-      e.step = 1;
+      e.at = halo ? halo0 : acc0;
+      e.step = halo ? 1 : 0;
     }
   } else if (halo) {
     e.at = halo0 + (w < 0 ? 0 : rp);
