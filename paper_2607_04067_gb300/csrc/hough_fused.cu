@@ -1397,7 +1397,7 @@ constexpr int kFoundMax = 128;  // keys that are ranked one by one
 // largest events, and those that pop as they start pair them with the next largest; half-way through an item, those
 // with small events come first, as they will at its end. (256 x 256, 160 events of 2,022 hits: 83.1 us popped before
 // the vote, 63.5 after it; 200 events 84.8 and 70.6; 20,000 events 4,678 and 4,626.) The iterative finder pops before
-// the vote (after it 1 % slower, 5,000 events) but for the last two turns (pops_late).
+// the vote (after it 1 % slower, 5,000 events) but for the last two turns (late_items).
 struct WorkItem {
   long long off[2];
   int item;  // >= n_items: none
@@ -1418,6 +1418,7 @@ struct ItemShared {
   int nv, flags, wide, last, D, reuse, n_amb, n_low, n_found;
   int staged;  // the event whose hits are staged whole (-1: none)
   unsigned runs;  // of the queue
+  int late;       // first of the items after which the next one is popped (late_items)
   int kept_tot;
   int tstart[129], tfrom[128];  // segments of the tile merge (2 a mirror-pair tile): starts, first records
   int tmp[32];
@@ -1908,7 +1909,7 @@ __device__ int merge_iterative(const Plan& pl, const FusedIO& io, unsigned char*
 // Steps 1-2 of a work item: clears the CTA's accumulator of theta tile t (with the halo columns,
 // the peak bitmap and the flags) and votes the event's hits [a, a + n) into it, chunk by chunk. The event
 // number tells whether its hits are staged already.
-template <bool MP, bool ITER>
+template <bool MP, bool ITER, bool WHOLE>
 __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, int event, long long a,
                           int n, int t) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
@@ -1918,7 +1919,7 @@ __device__ void vote_tile(const Plan& pl, const FusedIO& io, unsigned char* smem
   uint32_t* pbits = reinterpret_cast<uint32_t*>(smem + pl.off_pbits);
   const int16_t* tc = reinterpret_cast<const int16_t*>(smem + pl.off_trig);
   const int16_t* ts = tc + pl.n_theta;
-  const int T = pl.tiles, NT = pl.n_theta, nrp = pl.nrho_pad;
+  const int T = WHOLE ? 1 : pl.tiles, NT = pl.n_theta, nrp = pl.nrho_pad;
   const int j0 = t * pl.tile_w;
   const int wt = min(pl.tile_w, NT - j0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bd = blockDim.x;
@@ -2059,14 +2060,18 @@ __device__ __forceinline__ void popped(const Plan& pl, const FusedIO& io, unsign
   left = run ? pl.grab - 1 : 0;
 }
 
-// Whether the item after `item` is popped at its end: the iterative finder on tiles, where an event's last tile takes
-// much longer than the others and an item popped before it would wait for it instead of going to another CTA; and on whole
-// events in the last two turns, since two thirds of an event come after its vote and not in proportion to its hits
-// (256 x 256, half the maximum, R = 3, 160 events of 1,290 hits: 93.4 us popped after the vote, 81.0 so; the chain costs 3.5 k of
-// 119 k cycles an item, in those turns alone).
+// First of the items at whose end, not after whose vote, the next one is popped. Those of the last two turns on tiles, since
+// one of an event's tiles goes on with the merge and the selection, and an item popped before would wait for them instead of
+// going to another CTA (512 x 512, events of 4,720 hits: 40 of them 125.5 us popped after the vote, 104.7 so; 449 x 528, 74 of
+// them 263.8 and 239.2), but not with more than eight tiles an event, short ones (1000 x 1000, 40 events: 111.1 and 117.1);
+// all for the iterative finder on tiles, whose merge takes longest; and those of the last two turns for it on whole
+// events, since two thirds of an event come after its vote and not in proportion to its hits (256 x 256, half the maximum, R = 3,
+// 160 events of 1,290 hits: 93.4 us popped after the vote, 81.0 so; the chain costs 3.5 k of 119 k cycles an item, in those
+// turns alone).
 template <bool ITER>
-__device__ __forceinline__ bool pops_late(const Plan& pl, const FusedIO& io, int item) {
-  return ITER && (pl.tiles > 1 || item + 2LL * gridDim.x >= io.n_items);
+__device__ __forceinline__ int late_items(const Plan& pl, const FusedIO& io) {
+  if (!ITER && (pl.tiles == 1 || pl.tiles > 8)) return INT_MAX;
+  return pl.tiles > 1 && ITER ? 0 : max(0, (int)io.n_items - 2 * (int)gridDim.x);
 }
 
 // The work item sh.it[cur]; with `queue`, sh.it[cur ^ 1] receives the one after it.
@@ -2074,7 +2079,7 @@ __device__ __forceinline__ bool pops_late(const Plan& pl, const FusedIO& io, int
 // records to their places and test a T-th of the hits each: for calls of so few events that SMs would stay idle.
 // An event of 256 x 256 alone took 31.7 us in one CTA, 24.5 us in four, of which the two exchanges and the share's
 // staging are about 3.
-template <bool MP, bool ITER, bool CL>
+template <bool MP, bool ITER, bool CL, bool WHOLE>
 __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem, ItemShared& sh, int cur, bool queue,
                          bool do_cs) {
   uint32_t* acc = reinterpret_cast<uint32_t*>(smem + pl.off_acc);
@@ -2084,7 +2089,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   const int16_t* tc = reinterpret_cast<const int16_t*>(smem + pl.off_trig);
   const int16_t* ts = tc + pl.n_theta;
 
-  const int T = pl.tiles, NT = pl.n_theta, NR = pl.n_rho, nrp = pl.nrho_pad;
+  const int T = WHOLE ? 1 : pl.tiles, NT = pl.n_theta, NR = pl.n_rho, nrp = pl.nrho_pad;
   const long long e = sh.it[cur].event;
   const int t = sh.it[cur].item % T;
   const int j0 = t * pl.tile_w;
@@ -2094,7 +2099,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
 
   // the next item, in steps whose latencies pass behind the phases between them (thread 0)
   WorkItem& next = sh.it[cur ^ 1];
-  const bool fetch = queue && tid == 0 && !pops_late<ITER>(pl, io, sh.it[cur].item);
+  const bool fetch = queue && tid == 0 && (WHOLE || sh.it[cur].item < sh.late);
   unsigned long long pop = 0;
   bool other = false;  // the next item exists and belongs to another event
   auto fetch_pop = [&]() {
@@ -2129,7 +2134,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   if (ITER) fetch_pop();
   {
     const long long a = sh.it[cur].off[0], nll = sh.it[cur].off[1] - a;
-    vote_tile<MP, ITER>(pl, io, smem, sh, (int)e, a, nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll, t);
+    vote_tile<MP, ITER, WHOLE>(pl, io, smem, sh, (int)e, a, nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll, t);
   }
   if (ITER) fetch_event();
   else fetch_pop();
@@ -2487,7 +2492,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_MERGE);
-  if (queue && !pops_late<ITER>(pl, io, sh.it[cur].item) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
+  if (queue && (WHOLE || sh.it[cur].item < sh.late) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
     const long long i = next.off[0] + 16LL * tid;
     if (i < next.off[1]) asm volatile("prefetch.global.L2 [%0];" ::"l"(io.xy + i));
   }
@@ -2579,8 +2584,29 @@ __device__ __noinline__ void order_event(const FusedIO& io, int* s) {
   if (e == 0) io.queue[0] = 0ull;
 }
 
-// One instance a layout (MP: mirror pairs), peak finder and (CL) use of clusters, so that none carries the others' registers.
-template <bool MP, bool ITER, bool CL>
+// Item `it` of the queue or of the CTA's place, with its event and offsets (thread 0).
+__device__ __forceinline__ void fetch_item(const Plan& pl, const FusedIO& io, WorkItem& w, int it, int left, int run) {
+  w.item = it;
+  w.left = left;
+  w.run = run;
+  if (it >= io.n_items) return;
+  const int e = io.order ? io.order[it / pl.tiles] : it / pl.tiles;
+  w.event = e;
+  w.off[0] = io.off[e];
+  w.off[1] = io.off[e + 1];
+}
+
+// The item after sh.it[cur], popped at its end (thread 0).
+__device__ __forceinline__ void fetch_late(const Plan& pl, const FusedIO& io, ItemShared& sh, int cur) {
+  int it = sh.it[cur].item + 1, left = sh.it[cur].left - 1, run = sh.it[cur].run;
+  if (left < 0) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left, run);
+  fetch_item(pl, io, sh.it[cur ^ 1], it, left, run);
+}
+
+// One instance a layout (MP: mirror pairs), peak finder and (CL) use of clusters, so that none carries the others' registers;
+// WHOLE: of events in one tile (mirror pairs, local maxima: 20,000 events of 256 x 256 took 4,620 us with the tiles' merge in it and
+// 4,731 with their late pops too, 4,501 so).
+template <bool MP, bool ITER, bool CL, bool WHOLE>
 __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ItemShared sh;
@@ -2610,33 +2636,22 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
   __syncthreads();  // the table is read before run_item's first barrier
   const bool do_cs = io.checksum != nullptr;
   const bool queue = io.persistent && io.n_items > gridDim.x;  // else an item a CTA, and none after it
-  auto fetch_item = [&](WorkItem& w, int it, int left, int run) {  // thread 0
-    w.item = it;
-    w.left = left;
-    w.run = run;
-    if (it >= io.n_items) return;
-    const int e = io.order ? io.order[it / pl.tiles] : it / pl.tiles;
-    w.event = e;
-    w.off[0] = io.off[e];
-    w.off[1] = io.off[e + 1];
-  };
   if (threadIdx.x == 0) {
     sh.staged = -1;
     int it = blockIdx.x, left = 0, run = 0;
     sh.runs = queue_runs(pl, io);
+    sh.late = late_items<ITER>(pl, io);
     if (queue) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left, run);
-    fetch_item(sh.it[0], it, left, run);
+    fetch_item(pl, io, sh.it[0], it, left, run);
   }
 #pragma unroll 1
   for (int cur = 0;; cur ^= 1) {
     __syncthreads();
     if (sh.it[cur].item >= io.n_items) break;
-    run_item<MP, ITER, CL>(pl, io, smem, sh, cur, queue, do_cs);
+    run_item<MP, ITER, CL, WHOLE>(pl, io, smem, sh, cur, queue, do_cs);
     if (!queue) break;
-    if (pops_late<ITER>(pl, io, sh.it[cur].item) && threadIdx.x == 0) {
-      int it = sh.it[cur].item + 1, left = sh.it[cur].left - 1, run = sh.it[cur].run;
-      if (left < 0) popped(pl, io, sh.runs, atomicAdd(io.queue, 1ull), it, left, run);
-      fetch_item(sh.it[cur ^ 1], it, left, run);
+    if (!WHOLE && sh.it[cur].item >= sh.late) {
+      if (threadIdx.x == 0) fetch_late(pl, io, sh, cur);
     }
   }
 }
@@ -2686,7 +2701,7 @@ __global__ void __launch_bounds__(1024) deferred_kernel(const Plan pl, const Fus
     const int n = nll > HOUGH_MAX_EVENT_HITS ? 0 : (int)nll;  // a too-large event is never deferred
     int flags = 0;
     for (int t = 0; t < T; ++t) {
-      vote_tile<MP, true>(pl, io, smem, sh, (int)e, a, n, t);
+      vote_tile<MP, true, false>(pl, io, smem, sh, (int)e, a, n, t);
       const int j0 = t * pl.tile_w, wt = min(pl.tile_w, NT - j0), Wd = MP ? (wt + 1) >> 1 : 0,
                 aw = t * (pl.tile_w >> 1);
       if (MP) {
@@ -2862,9 +2877,9 @@ namespace {
 using FusedKernel = void (*)(const Plan, const FusedIO, const TrigTable);
 FusedKernel fused_of(const Plan& pl) {
   const bool it = pl.peak_mode == HOUGH_PEAK_ITERATIVE;
-  if (pl.cluster) return fused_kernel<true, false, true>;
-  return pl.mp ? (it ? fused_kernel<true, true, false> : fused_kernel<true, false, false>)
-               : (it ? fused_kernel<false, true, false> : fused_kernel<false, false, false>);
+  if (pl.cluster) return fused_kernel<true, false, true, false>;
+  if (!pl.mp) return it ? fused_kernel<false, true, false, false> : fused_kernel<false, false, false, false>;
+  return it ? fused_kernel<true, true, false, false> : pl.tiles == 1 ? fused_kernel<true, false, false, true> : fused_kernel<true, false, false, false>;
 }
 }  // namespace
 

@@ -411,6 +411,22 @@ def uneven_batch(n, small, large, n_large, seed=6):
     return np.resize(gen.generate("stress", 300).xy, (int(off[-1]), 2)), off
 
 
+def test_tiles_of_a_second_turn_go_to_ctas_without_a_merge(h):
+    """Equal events in four tiles, as many that each CTA has one and a half of them. The CTA of an event's last tile merges and
+    selects; with half the CTAs free for a second tile nobody needs to take one after that, while in two full turns a
+    quarter must. So the call takes a turn and a half and not two: nine tenths of the two at most."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ev, s = gen.generate("stress", 80), torch.cuda.Stream()
+    p = h.params(512, 512, 20, 1, 16384)
+    assert h.resolve(p).theta_tiles == 4
+
+    def call(n):
+        off = np.arange(n + 1, dtype=np.int64) * 4720
+        return time_run(h, np.resize(ev.xy, (int(off[-1]), 2)), off, p, s)
+
+    assert call(3 * sms // 8) < 0.9 * call(sms // 2)
+
+
 @pytest.mark.parametrize("n,small,large,n_large", [(153, 1600, 5000, 1), (160, 1600, 8000, 5), (200, 1600, 1700, 5), (228, 1600, 5000, 30),
                                                    (228, 0, 20000, 100), (229, 1600, 5000, 30), (608, 40, 3000, 10), (1000, 40, 3000, 10)])
 @pytest.mark.parametrize("nt,nr", [(64, 64), (101, 63), (128, 128)])
