@@ -634,7 +634,7 @@ static CallGrid batched_grid(const Common& cm) {
 
 static int enqueue(const Common& cm, const hough_params* p, const CallGrid& g, int* order, cudaStream_t st) {
   TrigTable trig;
-  host_trig(p->n_theta, &trig);
+  if (cm.io.n_items > 0) host_trig(p->n_theta, &trig);
   const bool timed = g_ev_begin && g_ev_end;
   const cudaError_t e = launch_call(cm.cp, cm.io, trig, g, order, st, timed ? mark_begin : nullptr, timed ? mark_end : nullptr);
   return e == cudaSuccess ? HOUGH_OK : cuda_fail(e);

@@ -2099,7 +2099,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
 
   // the next item, in steps whose latencies pass behind the phases between them (thread 0)
   WorkItem& next = sh.it[cur ^ 1];
-  const bool fetch = queue && tid == 0 && (WHOLE || sh.it[cur].item < sh.late);
+  const bool fetch = queue && tid == 0 && ((WHOLE && !ITER) || sh.it[cur].item < sh.late);
   unsigned long long pop = 0;
   bool other = false;  // the next item exists and belongs to another event
   auto fetch_pop = [&]() {
@@ -2492,7 +2492,7 @@ __device__ void run_item(const Plan& pl, const FusedIO& io, unsigned char* smem,
   }
   __syncthreads();
   HOUGH_PHASE(HOUGH_PHASE_MERGE);
-  if (queue && (WHOLE || sh.it[cur].item < sh.late) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
+  if (queue && ((WHOLE && !ITER) || sh.it[cur].item < sh.late) && next.item < io.n_items) {  // the next event's hits into the L2 (16 a line)
     const long long i = next.off[0] + 16LL * tid;
     if (i < next.off[1]) asm volatile("prefetch.global.L2 [%0];" ::"l"(io.xy + i));
   }
@@ -2605,7 +2605,7 @@ __device__ __forceinline__ void fetch_late(const Plan& pl, const FusedIO& io, It
 
 // One instance a layout (MP: mirror pairs), peak finder and (CL) use of clusters, so that none carries the others' registers;
 // WHOLE: of events in one tile (mirror pairs, local maxima: 20,000 events of 256 x 256 took 4,620 us with the tiles' merge in it and
-// 4,731 with their late pops too, 4,501 so).
+// 4,731 with their late pops too, 4,501 so; iterative finder, 5,000 events 1,907 and 1,846).
 template <bool MP, bool ITER, bool CL, bool WHOLE>
 __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedIO io, const TrigTable trig) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -2650,7 +2650,7 @@ __global__ void __launch_bounds__(1024) fused_kernel(const Plan pl, const FusedI
     if (sh.it[cur].item >= io.n_items) break;
     run_item<MP, ITER, CL, WHOLE>(pl, io, smem, sh, cur, queue, do_cs);
     if (!queue) break;
-    if (!WHOLE && sh.it[cur].item >= sh.late) {
+    if ((!WHOLE || ITER) && sh.it[cur].item >= sh.late) {
       if (threadIdx.x == 0) fetch_late(pl, io, sh, cur);
     }
   }
@@ -2879,7 +2879,8 @@ FusedKernel fused_of(const Plan& pl) {
   const bool it = pl.peak_mode == HOUGH_PEAK_ITERATIVE;
   if (pl.cluster) return fused_kernel<true, false, true, false>;
   if (!pl.mp) return it ? fused_kernel<false, true, false, false> : fused_kernel<false, false, false, false>;
-  return it ? fused_kernel<true, true, false, false> : pl.tiles == 1 ? fused_kernel<true, false, false, true> : fused_kernel<true, false, false, false>;
+  if (it) return pl.tiles == 1 ? fused_kernel<true, true, false, true> : fused_kernel<true, true, false, false>;
+  return pl.tiles == 1 ? fused_kernel<true, false, false, true> : fused_kernel<true, false, false, false>;
 }
 }  // namespace
 
