@@ -168,7 +168,8 @@ size_t hough_workspace_size(const hough_params* p, int64_t n_events);
  * sum over cells c = j*n_rho + k of acc[c] * splitmix64_finalizer(c + 1) mod 2^64.
  * d_ws: workspace of ws_bytes >= hough_workspace_size(p, n_events), 256-byte aligned.
  * d_xy and d_peaks must be 8-byte aligned (each record is written as one 8-byte store);
- * otherwise HOUGH_EINVAL. One CTA per (event, theta tile). */
+ * otherwise HOUGH_EINVAL. One CTA per (event, theta tile); a call of a few more events than SMs may be
+ * scheduled as in hough_run_batched where that ends sooner. */
 int hough_run(const int32_t* d_xy, int64_t n_hits, const int64_t* d_off, int64_t n_events, const hough_params* p,
               int32_t* d_npeaks, hough_peak* d_peaks, uint8_t* d_mask, int32_t* d_nkept, uint64_t* d_checksum,
               void* d_ws, size_t ws_bytes, int32_t* d_status, void* stream);
@@ -220,8 +221,9 @@ int hough_host_stage_ms(float* ms, int32_t n);
 
 /* Measurement hook for the calling host thread: when both are non-NULL, later fused and
  * batched calls record the CUDA events begin/end (cudaEvent_t passed as void*) on their
- * stream immediately before and after the main fused kernel, so its duration can be read
- * with cudaEventElapsedTime. NULL, NULL turns it off. Graph replays are cached per pair. */
+ * stream immediately before and after the main fused kernel (both, where a call launches two),
+ * so its duration can be read with cudaEventElapsedTime. NULL, NULL turns it off. Graph replays
+ * are cached per pair. */
 void hough_set_stage_events(void* begin, void* end);
 
 /* ---- serving loop (continuous batching) ---- */

@@ -397,7 +397,7 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
 // gaps. c CTAs of 1024 / c threads take kTurn[c] times as long as one (in twentieths; measured from 64 x 64 to
 // 160 x 160), so the c with the shortest time for all the events' turns is taken. Where events have few hits, fewer
 // staged hits (half as many again as the mean; an event with more takes several chunks) make room for more CTAs; but not for
-// more than two in a single turn of events of more than 1,500 hits (128 x 128, events of 500 to 4,700 hits, 400 of them: three
+// more than two in a single turn of events of more than 1,500 hits (128 x 128, events of 500 to 3,650 hits, 400 of them: three
 // CTAs 72.4 us, two 60.8; 64 x 64, 608 of them: four 61.0, three 63.9; 100 x 100, 500 of about 1,290: four 57.7, 66.5 with 4,096 staged hits).
 // One CTA -> this rule, us: 64 x 64, 616 hits, 5,000 events 424 -> 177 and 500 events 59 -> 30; 100 x 100, 1,290
 // hits, 5,000 events 640 -> 365; 128 x 128, 2,022 hits, 1,000 events 167 -> 131, iterative finder 286 -> 218.
@@ -406,7 +406,7 @@ int make_plan(const hough_params* p, Plan& pl, int max_cap = 4096) {
 // than what 32 warps add to each barrier.
 // A call's sizes do not tell how even its events are, and one event with many times the others' hits takes longer in a CTA of
 // fewer threads (8,000 hits: 1.2 times with 512, 1.9 times with 256; 64 x 64, 608 events of 600 hits, ten of 8,000: 113 us,
-// 75 with a block of 1,024). Among events of 500 to 4,700 hits that loses only where one CTA an SM has a few events left after the
+// 75 with a block of 1,024). Among events of 500 to 3,650 hits that loses only where one CTA an SM has a few events left after the
 // first turn, the smallest ones: so calls of at most one and a half turns, with more than 1,500 hits an event (with fewer its
 // fixed part counts most) and more than one word group (64 columns: 35.8 us in two CTAs an SM, 37.9 in one), launch both
 // shapes, and the events choose (is_uneven). The launch that finds nothing to do costs 2.2 us; behind the validation

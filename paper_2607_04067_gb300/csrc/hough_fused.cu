@@ -2536,11 +2536,11 @@ __device__ __forceinline__ int bad_offsets(const long long* off, long long ne, l
   return bad;
 }
 
-// Whether a call's events are too uneven for two CTAs an SM instead of one; s: two shared ints, every thread calls it. An event of
-// 4,700 hits takes 1.13 times as long with 512 threads as with 1,024, which is worth it only where one CTA an SM would end
-// later anyway: with its share of all hits, or after two of the smallest events (an event's fixed part counts as 1,800
-// hits). 128 x 128, 160 events: of about 1,290 hits each 48.0 us in one CTA an SM, 33.8 in two; of 500 to 4,700 hits 42.4
-// and 46.3 (iterative finder 65 and 78).
+// Whether a call's events are too uneven for two CTAs an SM instead of one; s: two shared ints, every thread calls it. A large
+// event takes longer with 512 threads than with 1,024 (alone on an SM, 128 x 128: 4,000 hits 1.07 times, 8,000 hits 1.15;
+// beside another one more), which is worth it only where one CTA an SM would end later anyway: with its share of all
+// hits, or after two of the smallest events (an event's fixed part counts as 1,800 hits). 128 x 128, 160 events: of about
+// 1,290 hits each 48.0 us in one CTA an SM, 33.8 in two; of 500 to 3,650 hits 42.4 and 46.3 (iterative finder 65 and 78).
 __device__ __noinline__ bool is_uneven(const FusedIO& io, int ctas, int* s) {
   constexpr int kFixed = 1800;
   if (threadIdx.x == 0) {

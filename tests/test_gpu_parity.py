@@ -459,7 +459,7 @@ def test_uneven_events_on_small_accumulators(h, nt, nr, n, small, large, n_large
 
 @pytest.mark.parametrize("nt", [100, 128])
 def test_uneven_events_take_one_cta_an_sm(h, nt):
-    """160 events of 500 to 4,700 hits: the few beyond an event an SM are small and end behind small ones, while two CTAs
+    """160 events of 500 to 3,650 hits: the few beyond an event an SM are small and end behind small ones, while two CTAs
     an SM, of half the threads, would take a fifth longer for the large ones (iterative finder)."""
     ev = gen.generate("batched", 160)
     kw, s = dict(theta_tiles=1, peak_mode=1, rel_num=1, rel_den=2, nms_radius=3), torch.cuda.Stream()
@@ -468,7 +468,7 @@ def test_uneven_events_take_one_cta_an_sm(h, nt):
 
 
 def test_uneven_events_in_one_turn_are_staged_whole(h):
-    """400 events of 500 to 4,700 hits at 128 x 128: a third CTA an SM would have room only with 3,072 staged hits, so the events
+    """400 events of 500 to 3,650 hits at 128 x 128: a third CTA an SM would have room only with 3,072 staged hits, so the events
     that end the call would take two chunks and a fifth longer than with two CTAs of 512 threads."""
     ev, s = gen.generate("batched", 400), torch.cuda.Stream()
     two = time_run(h, ev.xy, ev.off, h.params(128, 128, 8, 1, 4096, theta_tiles=1, block=512), s)
